@@ -62,12 +62,13 @@ int derive(const kvm_params* p, Dims& d) {
     return KVM_OK;
 }
 
-inline size_t score_row_bytes(const Dims& d) {
-    return d.dtype == KVM_BF16 ? score_tc_scratch_bytes_per_row() : sizeof(float);
+// scratch of the score step: the bf16 path's side tensor, or the fp32 path's states, partial sums and split planes
+inline size_t score_bytes(const Dims& d) {
+    return d.dtype == KVM_BF16 ? (size_t)d.B * d.Hq * d.S * score_tc_scratch_bytes_per_row() : score_f32_scratch_bytes(d);
 }
 
 struct Workspace {
-    float* lse;         // row-pass output: [B,Hq,S] fp32 (fp32 path) or [B,Hq,S,16] bf16 side tensor (bf16 path)
+    float* lse;         // score scratch: [B,Hq,S,16] bf16 side tensor (bf16), or states and partial sums (fp32)
     float* scores;      // [U,S]
     float* sim;         // [U,S]
     int32_t* set_start; // [U,cap+1]
@@ -81,7 +82,7 @@ Workspace carve(const Dims& d, void* base) {
     Workspace w;
     size_t off = 0;
     auto take = [&](size_t n) { size_t o = off; off += align_up(n); return (char*)base + o; };
-    w.lse = (float*)take((size_t)d.B * d.Hq * d.S * score_row_bytes(d));
+    w.lse = (float*)take(score_bytes(d));
     w.scores = (float*)take((size_t)d.U * d.S * sizeof(float));
     w.sim = (float*)take((size_t)d.U * d.S * sizeof(float));
     w.set_start = (int32_t*)take((size_t)d.U * (d.cap + 1) * sizeof(int32_t));
@@ -102,18 +103,13 @@ int check_ws(const Dims& d, void* ws, size_t ws_bytes, Workspace& w) {
     return KVM_OK;
 }
 
-// sim_out (nullable): where the neighbour-key similarities are wanted.  *sim_done tells whether the score
-// step produced them on the side (bf16 path) or the caller still has to launch the similarity kernel.
+// sim_out (nullable): where the neighbour-key similarities are wanted, which the score step produces on the side.
 cudaError_t run_score(const Dims& d, const void* Q, const void* K, const float* lse_in, float* scores,
-                      const Workspace& w, kvm_stats* stats, cudaStream_t st, float* sim_out = nullptr,
-                      bool* sim_done = nullptr) {
-    // bf16: tensor cores (tcgen05); fp32: plain FMA, since tensor-core input rounding cannot hold the score tolerance
-    if (d.dtype == KVM_BF16) {
-        if (sim_done) *sim_done = sim_out != nullptr;
-        return launch_score_tc(d, Q, K, lse_in, w.lse, scores, stats, st, sim_out);
-    }
-    if (sim_done) *sim_done = false;
-    return launch_score_simt(d, Q, K, lse_in, w.lse, scores, st);
+                      const Workspace& w, kvm_stats* stats, cudaStream_t st, float* sim_out = nullptr) {
+    // fp32 tensors enter the tensor cores as exact sums of three bf16 planes: rounding them would not hold the
+    // score tolerance
+    return d.dtype == KVM_BF16 ? launch_score_tc(d, Q, K, lse_in, w.lse, scores, stats, st, sim_out)
+                               : launch_score_f32(d, Q, K, lse_in, w.lse, scores, stats, st, sim_out);
 }
 
 }  // namespace
@@ -185,16 +181,10 @@ int kvm_row_lse(const kvm_params* p, const void* Q, const void* K, float* lse_ou
     Workspace w;
     if ((rc = check_ws(d, ws, ws_bytes, w)) != KVM_OK) return rc;
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    if (d.dtype == KVM_BF16)
-        return launch_score_tc(d, Q, K, nullptr, w.lse, nullptr, nullptr, st, nullptr, lse_out) == cudaSuccess
-                   ? KVM_OK
-                   : KVM_E_CUDA;
-    // fp32 path: its row pass leaves the natural-log lse in the workspace as it is
-    if (launch_score_simt(d, Q, K, nullptr, w.lse, nullptr, st) != cudaSuccess) return KVM_E_CUDA;
-    return cudaMemcpyAsync(lse_out, w.lse, (size_t)d.B * d.Hq * d.S * sizeof(float), cudaMemcpyDeviceToDevice, st) ==
-                   cudaSuccess
-               ? KVM_OK
-               : KVM_E_CUDA;
+    const cudaError_t e = d.dtype == KVM_BF16
+                              ? launch_score_tc(d, Q, K, nullptr, w.lse, nullptr, nullptr, st, nullptr, lse_out)
+                              : launch_score_f32(d, Q, K, nullptr, w.lse, nullptr, nullptr, st, nullptr, lse_out);
+    return e == cudaSuccess ? KVM_OK : KVM_E_CUDA;
 }
 
 int kvm_segment(const kvm_params* p, const void* K, const float* scores, int32_t* set_id, int32_t* set_start,
@@ -326,11 +316,7 @@ int kvm_compress_with_lse(const kvm_params* p, const void* Q, const void* K, con
     cudaStream_t st = (cudaStream_t)cuda_stream;
     float* scores = scores_out ? scores_out : w.scores;
     const bool want_sim = d.set_rule == KVM_SETS_ADJACENT;
-    bool sim_done = false;
-    if (run_score(d, Q, K, lse_in, scores, w, stats, st, want_sim ? w.sim : nullptr, &sim_done) != cudaSuccess)
-        return KVM_E_CUDA;
-    if (want_sim && !sim_done)
-        if (launch_similarity(d, K, w.sim, st) != cudaSuccess) return KVM_E_CUDA;
+    if (run_score(d, Q, K, lse_in, scores, w, stats, st, want_sim ? w.sim : nullptr) != cudaSuccess) return KVM_E_CUDA;
     if (d.set_rule == KVM_SETS_ANCHOR)
         if (launch_anchor_runs(d, K, w.sim, (float*)w.set_id, st) != cudaSuccess) return KVM_E_CUDA;
     if (launch_segment(d, scores, w.sim, w.set_id, w.set_start, out_pos, out_len, stats, st) != cudaSuccess)
@@ -544,9 +530,11 @@ int kvm_score_static(const kvm_params* p, const void* Q, const void* K, float* s
     if (rc != KVM_OK) return rc;
     if (!Q || !K || !scores) return KVM_E_NULL;
     if (misaligned(Q) || misaligned(K) || misaligned(scores)) return KVM_E_ALIGN;
-    // the row pass leaves 4 bytes per query row for fp32 tensors and 32 bytes for bf16 ones
-    if ((unsigned long long)d.B * d.Hq * d.S * score_row_bytes(d) > (unsigned long long)KVM_STATIC_SCORE_ROWS * sizeof(float))
+    // 32 bytes per query row for bf16 tensors; fp32 ones need 4 where work items stay whole, and no more than the
+    // array where they are split (so that both entry points run the same plan)
+    if (d.dtype == KVM_F32 && (unsigned long long)d.B * d.Hq * d.S > (unsigned long long)KVM_STATIC_SCORE_ROWS)
         return KVM_E_STATIC_LIMIT;
+    if (score_bytes(d) > sizeof(g_static_score_scratch)) return KVM_E_STATIC_LIMIT;
     unsigned char* base = (unsigned char*)static_scratch_for_current_device();
     if (!base) return KVM_E_CUDA;
     cudaStream_t st = (cudaStream_t)cuda_stream;

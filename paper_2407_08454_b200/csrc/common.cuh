@@ -79,8 +79,10 @@ cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, si
 }
 
 // Launchers (each enqueues on the stream and returns the launch status).
-cudaError_t launch_score_simt(const Dims& d, const void* Q, const void* K, const float* lse_in, float* lse_ws,
-                              float* scores, cudaStream_t st);
+cudaError_t launch_score_f32(const Dims& d, const void* Q, const void* K, const float* lse_in, void* scratch,
+                             float* scores, kvm_stats* stats, cudaStream_t st, float* sim_out = nullptr,
+                             float* lse_out = nullptr);
+size_t score_f32_scratch_bytes(const Dims& d);
 cudaError_t launch_score_tc(const Dims& d, const void* Q, const void* K, const float* lse_in, float* lse_ws,
                             float* scores, kvm_stats* stats, cudaStream_t st, float* sim_out = nullptr,
                             float* lse_out = nullptr);
