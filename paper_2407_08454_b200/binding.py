@@ -61,6 +61,30 @@ class KvmError(RuntimeError):
 
 
 _lib = None
+_F = {}          # entry points of the loaded library, argument types declared
+
+_P, _I, _Z = ctypes.c_void_p, ctypes.c_int32, ctypes.c_size_t
+_PARAMS = ctypes.POINTER(KvmParams)
+# Argument types as in include/kvm.h: with them declared, pointers pass as plain integers (a ctypes object per argument
+# costs more than the call).
+_ARGTYPES = {
+    "kvm_sizes": (_PARAMS, ctypes.POINTER(_I), ctypes.POINTER(_I), ctypes.POINTER(_I)),
+    "kvm_workspace_bytes": (_PARAMS, ctypes.POINTER(_Z)),
+    "kvm_host_staging_bytes": (_PARAMS, ctypes.POINTER(_Z)),
+    "kvm_score": (_PARAMS, _P, _P, _P, _P, _P, _Z, _P),
+    "kvm_row_lse": (_PARAMS, _P, _P, _P, _P, _Z, _P),
+    "kvm_score_static": (_PARAMS, _P, _P, _P, _P),
+    "kvm_segment": (_PARAMS, _P, _P, _P, _P, _P, _P, _P, _P, _P, _Z, _P),
+    "kvm_layer_ratio": (_PARAMS, _P, _P, _P, _P, _Z, _P),
+    "kvm_attend": (_PARAMS, _P, _P, _P, _I, _P, _P, _P, _Z, _P),
+    "kvm_prefill_attend": (_PARAMS, _P, _P, _P, _P, _P, _P, _P),
+    "kvm_output_perturbation": (_PARAMS,) + (_P,) * 11 + (_Z, _P),
+    "kvm_merge_compact": (_PARAMS,) + (_P,) * 9 + (_Z, _P),
+    "kvm_compress": (_PARAMS,) + (_P,) * 10 + (_Z, _P),
+    "kvm_compress_with_lse": (_PARAMS,) + (_P,) * 11 + (_Z, _P),
+    "kvm_compress_layers": (_PARAMS, _I) + (_P,) * 10 + (_Z, _P),
+    "kvm_compress_host": (_PARAMS,) + (_P,) * 8 + (_Z, _P),
+}
 
 
 def lib() -> ctypes.CDLL:
@@ -76,8 +100,22 @@ def lib() -> ctypes.CDLL:
         L.kvm_status_string.argtypes = [ctypes.c_int]
         for name in EXPORTS:
             getattr(L, name)
+        # (a handle of its own: whoever takes lib() declares or converts arguments as they like)
+        own = ctypes.CDLL(LIB_PATH)
+        for name, types in _ARGTYPES.items():
+            fn = getattr(own, name)
+            fn.argtypes = types
+            _F[name] = fn
         _lib = L
     return _lib
+
+
+def _call(name: str, p: KvmParams, *args) -> None:
+    if _lib is None:
+        lib()
+    rc = _F[name](p, *args)
+    if rc != KVM_OK:
+        raise KvmError(rc, name)
 
 
 def status_string(status: int) -> str:
@@ -102,22 +140,23 @@ def make_params(batch: int, n_q_heads: int, n_kv_heads: int, seq: int, head_dim:
                      pivot_rule, weight_rule, set_rule, key_ptr)
 
 
-def _ptr(t: Optional[torch.Tensor]) -> ctypes.c_void_p:
+def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
     if t is None:
-        return ctypes.c_void_p(0)
+        return None
     assert t.is_contiguous(), "tensors must be contiguous"
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
-def _stream(stream) -> ctypes.c_void_p:
+# The current stream's handle without the Stream object around it.
+_device, _raw_stream = torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream
+
+
+def _stream(stream) -> int:
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
-
-
-def _check(rc: int, where: str) -> None:
-    if rc != KVM_OK:
-        raise KvmError(rc, where)
+        if not torch.cuda.is_initialized():
+            torch.cuda.init()
+        return _raw_stream(_device())
+    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
 def kvm_version() -> int:
@@ -126,97 +165,82 @@ def kvm_version() -> int:
 
 def kvm_sizes(p: KvmParams):
     cap, nr, nh = ctypes.c_int32(), ctypes.c_int32(), ctypes.c_int32()
-    _check(lib().kvm_sizes(ctypes.byref(p), ctypes.byref(cap), ctypes.byref(nr), ctypes.byref(nh)), "kvm_sizes")
+    _call("kvm_sizes", p, cap, nr, nh)
     return cap.value, nr.value, nh.value
 
 
 def kvm_workspace_bytes(p: KvmParams) -> int:
     n = ctypes.c_size_t()
-    _check(lib().kvm_workspace_bytes(ctypes.byref(p), ctypes.byref(n)), "kvm_workspace_bytes")
+    _call("kvm_workspace_bytes", p, n)
     return n.value
 
 
 def kvm_host_staging_bytes(p: KvmParams) -> int:
     n = ctypes.c_size_t()
-    _check(lib().kvm_host_staging_bytes(ctypes.byref(p), ctypes.byref(n)), "kvm_host_staging_bytes")
+    _call("kvm_host_staging_bytes", p, n)
     return n.value
 
 
 def kvm_score(p: KvmParams, Q, K, lse_in, scores, ws, stream=None) -> None:
-    _check(lib().kvm_score(ctypes.byref(p), _ptr(Q), _ptr(K), _ptr(lse_in), _ptr(scores), _ptr(ws),
-                           ctypes.c_size_t(ws.numel() * ws.element_size()), _stream(stream)), "kvm_score")
+    _call("kvm_score", p, _ptr(Q), _ptr(K), _ptr(lse_in), _ptr(scores), _ptr(ws), ws.nbytes, _stream(stream))
 
 
 def kvm_row_lse(p: KvmParams, Q, K, lse_out, ws, stream=None) -> None:
-    _check(lib().kvm_row_lse(ctypes.byref(p), _ptr(Q), _ptr(K), _ptr(lse_out), _ptr(ws),
-                             ctypes.c_size_t(ws.numel() * ws.element_size()), _stream(stream)), "kvm_row_lse")
+    _call("kvm_row_lse", p, _ptr(Q), _ptr(K), _ptr(lse_out), _ptr(ws), ws.nbytes, _stream(stream))
 
 
 def kvm_score_static(p: KvmParams, Q, K, scores, stream=None) -> None:
     """kvm_score on the library's built-in scratch: for callers that cannot allocate a workspace.
     batch * n_q_heads * seq must not exceed KVM_STATIC_SCORE_ROWS (fp32) or an eighth of it (bf16); calls on one
     device must not overlap."""
-    _check(lib().kvm_score_static(ctypes.byref(p), _ptr(Q), _ptr(K), _ptr(scores), _stream(stream)),
-           "kvm_score_static")
+    _call("kvm_score_static", p, _ptr(Q), _ptr(K), _ptr(scores), _stream(stream))
 
 
 def kvm_segment(p: KvmParams, K, scores, set_id, set_start, pivot, out_len, sim_out, stats, ws, stream=None) -> None:
-    _check(lib().kvm_segment(ctypes.byref(p), _ptr(K), _ptr(scores), _ptr(set_id), _ptr(set_start), _ptr(pivot),
-                             _ptr(out_len), _ptr(sim_out), _ptr(stats), _ptr(ws),
-                             ctypes.c_size_t(ws.numel() * ws.element_size()), _stream(stream)), "kvm_segment")
+    _call("kvm_segment", p, _ptr(K), _ptr(scores), _ptr(set_id), _ptr(set_start), _ptr(pivot), _ptr(out_len),
+          _ptr(sim_out), _ptr(stats), _ptr(ws), ws.nbytes, _stream(stream))
 
 
 def kvm_layer_ratio(p: KvmParams, K, ratio, sim_out, ws, stream=None) -> None:
-    _check(lib().kvm_layer_ratio(ctypes.byref(p), _ptr(K), _ptr(ratio), _ptr(sim_out), _ptr(ws),
-                                 ctypes.c_size_t(ws.numel() * ws.element_size()), _stream(stream)), "kvm_layer_ratio")
+    _call("kvm_layer_ratio", p, _ptr(K), _ptr(ratio), _ptr(sim_out), _ptr(ws), ws.nbytes, _stream(stream))
 
 
 def kvm_attend(p: KvmParams, q, K, V, rows: int, length, out, ws, stream=None) -> None:
-    _check(lib().kvm_attend(ctypes.byref(p), _ptr(q), _ptr(K), _ptr(V), ctypes.c_int32(rows), _ptr(length), _ptr(out),
-                            _ptr(ws), ctypes.c_size_t(ws.numel() * ws.element_size()), _stream(stream)), "kvm_attend")
+    _call("kvm_attend", p, _ptr(q), _ptr(K), _ptr(V), rows, _ptr(length), _ptr(out), _ptr(ws), ws.nbytes,
+          _stream(stream))
 
 
 def kvm_prefill_attend(p: KvmParams, Q, K, V, O, lse, stats=None, stream=None) -> None:
     """Causal attention over the whole prompt: O [B,Hq,S,D] bf16 and the rows' natural-log log-sum-exp [B,Hq,S]."""
-    _check(lib().kvm_prefill_attend(ctypes.byref(p), _ptr(Q), _ptr(K), _ptr(V), _ptr(O), _ptr(lse), _ptr(stats),
-                                    _stream(stream)), "kvm_prefill_attend")
+    _call("kvm_prefill_attend", p, _ptr(Q), _ptr(K), _ptr(V), _ptr(O), _ptr(lse), _ptr(stats), _stream(stream))
 
 
 def kvm_output_perturbation(p: KvmParams, q, K, V, K_c, V_c, len_c, out_full, out_comp, err, ref, ws,
                             stream=None) -> None:
-    _check(lib().kvm_output_perturbation(ctypes.byref(p), _ptr(q), _ptr(K), _ptr(V), _ptr(K_c), _ptr(V_c),
-                                         _ptr(len_c), _ptr(out_full), _ptr(out_comp), _ptr(err), _ptr(ref), _ptr(ws),
-                                         ctypes.c_size_t(ws.numel() * ws.element_size()), _stream(stream)),
-           "kvm_output_perturbation")
+    _call("kvm_output_perturbation", p, _ptr(q), _ptr(K), _ptr(V), _ptr(K_c), _ptr(V_c), _ptr(len_c), _ptr(out_full),
+          _ptr(out_comp), _ptr(err), _ptr(ref), _ptr(ws), ws.nbytes, _stream(stream))
 
 
 def kvm_merge_compact(p: KvmParams, K, V, set_start, pivot, out_len, K_out, V_out, out_size, ws, stream=None) -> None:
-    _check(lib().kvm_merge_compact(ctypes.byref(p), _ptr(K), _ptr(V), _ptr(set_start), _ptr(pivot), _ptr(out_len),
-                                   _ptr(K_out), _ptr(V_out), _ptr(out_size), _ptr(ws),
-                                   ctypes.c_size_t(ws.numel() * ws.element_size()), _stream(stream)),
-           "kvm_merge_compact")
+    _call("kvm_merge_compact", p, _ptr(K), _ptr(V), _ptr(set_start), _ptr(pivot), _ptr(out_len), _ptr(K_out),
+          _ptr(V_out), _ptr(out_size), _ptr(ws), ws.nbytes, _stream(stream))
 
 
 def kvm_compress(p: KvmParams, Q, K, V, K_out, V_out, out_len, out_pos, scores_out, stats, ws, stream=None) -> None:
-    _check(lib().kvm_compress(ctypes.byref(p), _ptr(Q), _ptr(K), _ptr(V), _ptr(K_out), _ptr(V_out), _ptr(out_len),
-                              _ptr(out_pos), _ptr(scores_out), _ptr(stats), _ptr(ws),
-                              ctypes.c_size_t(ws.numel() * ws.element_size()), _stream(stream)), "kvm_compress")
+    _call("kvm_compress", p, _ptr(Q), _ptr(K), _ptr(V), _ptr(K_out), _ptr(V_out), _ptr(out_len), _ptr(out_pos),
+          _ptr(scores_out), _ptr(stats), _ptr(ws), ws.nbytes, _stream(stream))
 
 
 def kvm_compress_with_lse(p: KvmParams, Q, K, V, lse_in, K_out, V_out, out_len, out_pos, scores_out, stats, ws,
                           stream=None) -> None:
-    _check(lib().kvm_compress_with_lse(ctypes.byref(p), _ptr(Q), _ptr(K), _ptr(V), _ptr(lse_in), _ptr(K_out),
-                                       _ptr(V_out), _ptr(out_len), _ptr(out_pos), _ptr(scores_out), _ptr(stats),
-                                       _ptr(ws), ctypes.c_size_t(ws.numel() * ws.element_size()), _stream(stream)),
-           "kvm_compress_with_lse")
+    _call("kvm_compress_with_lse", p, _ptr(Q), _ptr(K), _ptr(V), _ptr(lse_in), _ptr(K_out), _ptr(V_out),
+          _ptr(out_len), _ptr(out_pos), _ptr(scores_out), _ptr(stats), _ptr(ws), ws.nbytes, _stream(stream))
 
 
 def kvm_compress_host(p: KvmParams, Q, K, V, K_out, V_out, out_len, out_pos, dev, stream=None) -> None:
     """Q..out_pos are HOST tensors (pin them for asynchronous copies); `dev` is a device byte buffer."""
-    _check(lib().kvm_compress_host(ctypes.byref(p), _ptr(Q), _ptr(K), _ptr(V), _ptr(K_out), _ptr(V_out),
-                                   _ptr(out_len), _ptr(out_pos), _ptr(dev),
-                                   ctypes.c_size_t(dev.numel() * dev.element_size()), _stream(stream)),
-           "kvm_compress_host")
+    _call("kvm_compress_host", p, _ptr(Q), _ptr(K), _ptr(V), _ptr(K_out), _ptr(V_out), _ptr(out_len), _ptr(out_pos),
+          _ptr(dev), dev.nbytes, _stream(stream))
 
 
 # ----------------------------------------------------------------------------- convenience
@@ -266,21 +290,25 @@ def compress_layers(p: KvmParams, layers, sim_thresholds=None, device="cuda", st
     similarity threshold per layer (Section 3.2: thresholds chosen layer by layer), through kvm_compress_layers.
     Returns, per layer, a `Compressed` holding the outputs, and the layer's compression ratio mean(out_len) / S."""
     n = len(layers)
-    comps = [Compressor(p, device=device) for _ in range(n)]
-    ptrs = lambda ts: (ctypes.c_void_p * n)(*[t.data_ptr() for t in ts])
-    for Q, K, V in layers:
-        assert Q.is_contiguous() and K.is_contiguous() and V.is_contiguous()
+    B, H, cap, D = p.batch, p.n_kv_heads, kvm_sizes(p)[0], p.head_dim
+    dt = torch.bfloat16 if p.dtype == KVM_BF16 else torch.float32
+    # one allocation per kind for the whole stack (each layer's tensors are views of it) and one zero fill
+    ws = torch.empty(kvm_workspace_bytes(p), dtype=torch.uint8, device=device)
+    kv = torch.zeros(2, n, B, H, cap, D, dtype=dt, device=device)
+    ints = torch.zeros(n * B * H * (cap + 1), dtype=torch.int32, device=device)
+    out_len, out_pos = ints[:n * B * H].view(n, B, H), ints[n * B * H:].view(n, B, H, cap)
+
+    def rows(t):            # the layers' addresses within a stacked tensor
+        step = t[0].numel() * t.element_size()
+        return (ctypes.c_void_p * n)(*range(t.data_ptr(), t.data_ptr() + n * step, step))
+
+    ptrs = lambda i: (ctypes.c_void_p * n)(*[_ptr(l[i]) for l in layers])
     eps = None
     if sim_thresholds is not None:
         assert len(sim_thresholds) == n
         eps = (ctypes.c_float * n)(*[float(e) for e in sim_thresholds])
-    ws = comps[0].ws
-    _check(lib().kvm_compress_layers(ctypes.byref(p), ctypes.c_int32(n), eps, ptrs([l[0] for l in layers]),
-                                     ptrs([l[1] for l in layers]), ptrs([l[2] for l in layers]),
-                                     ptrs([c.K_out for c in comps]), ptrs([c.V_out for c in comps]),
-                                     ptrs([c.out_len for c in comps]), ptrs([c.out_pos for c in comps]),
-                                     ctypes.c_void_p(0), _ptr(ws), ctypes.c_size_t(ws.numel()), _stream(stream)),
-           "kvm_compress_layers")
-    out = [Compressed(c.K_out, c.V_out, c.out_len, c.out_pos, None, c.cap) for c in comps]
-    ratios = [float(c.out_len.float().mean() / p.seq) for c in comps]
+    _call("kvm_compress_layers", p, n, eps, ptrs(0), ptrs(1), ptrs(2), rows(kv[0]), rows(kv[1]), rows(out_len),
+          rows(out_pos), None, ws.data_ptr(), ws.nbytes, _stream(stream))
+    out = [Compressed(kv[0, l], kv[1, l], out_len[l], out_pos[l], None, cap) for l in range(n)]
+    ratios = (out_len.cpu().float().mean((1, 2)) / p.seq).tolist()      # the one read-back of the call
     return out, ratios
