@@ -3,138 +3,550 @@
 // perturbation |O_t - O_t*| of Definition 2.1 between the full and the
 // compressed cache.
 //
-// Bandwidth-bound: every K and V row of the cache is read once per query head
-// (the G query heads of a KV head read the same rows within a short time, so
-// the repeats are L2 hits).  The rows of one (batch, query head) are split into
-// chunks sized so that the blocks fill the GPU in one wave, one block per chunk; inside a block a group of LPR
-// lanes owns a row at a time and keeps an online-softmax state (max, sum,
-// weighted V sum) in registers; groups, then chunks, are combined in a fixed
-// order, so results are reproducible.
-#include "common.cuh"
+// Bandwidth-bound: K and V rows are read once from HBM.  What it takes to get there:
+//   - the query heads of a KV head share a row's one way through shared memory (up to eight at a time; one block per
+//     query head read everything G times through L2: 206 us against 72 us on 8 x 32/8 heads x 12288 rows on average);
+//   - one persistent block per SM takes an equal share of all the rows there are (lengths differ; the shares are cut by
+//     a prefix sum over the units' lengths, so that no SM idles while another finishes a long unit);
+//   - the rows come by bulk copies into a ring of 16 KB + 16 KB stages, 128 KB in flight per SM, issued by a warp of
+//     its own; eight warps compute.
+// A group of LPR lanes owns four rows of a stage.  Its products (rows x heads) are summed across the lanes by a
+// transposing butterfly that leaves each lane one (row, head) to exponentiate; the weights come back by shuffle for
+// the second product.  The reference maximum moves only when it has been outgrown by 8 (log2 units).
+// A unit's rows that fall into several blocks' shares leave partial states (weighted V sum, maximum, sum), combined in a
+// fixed order by a second kernel: results are reproducible.
+#include <mutex>
+
+#include "tc_common.cuh"
 
 namespace kvm {
 namespace {
 
-constexpr int ATT_NT = 256;
-constexpr int ATT_MIN_CHUNK = 64;           // fewest cache rows a block is given (bounds the number of chunks)
-constexpr int ATT_BLOCKS_PER_SM = 4;        // resident blocks per SM (register-limited): the chunk count aims at one wave
+using namespace tc;
+
+constexpr int ATT_WARPS = 8;                // computing warps; one more issues the copies
+constexpr int ATT_NT = (ATT_WARPS + 1) * 32;
+constexpr int ATT_STAGES = 4;
+constexpr int ATT_STAGE_BYTES = 16384;      // of K, and as much of V
+constexpr int ATT_MIN_SHARE = 64;           // fewest rows a block is given (bounds the number of pieces)
+constexpr int RPI = 4;                      // rows of a stage per lane group
 constexpr float LOG2E = 1.4426950408889634f;
+constexpr float REF_STEP = 8.f;             // the reference maximum follows in steps of at least this (log2 units)
 
 // Weight of a partial state with maximum m when the overall maximum is M (an empty state has m = -inf).
 __device__ __forceinline__ float rescale(float m, float M) { return m == -INFINITY ? 0.f : exp2f(m - M); }
-
-// part layout per (bh, split): D weighted sums, then the maximum and the sum (log2 domain).
-template <typename T, int D>
-__global__ void __launch_bounds__(ATT_NT) attend_partial_kernel(const T* __restrict__ q, const T* __restrict__ K,
-                                                                const T* __restrict__ V,
-                                                                const int32_t* __restrict__ len,
-                                                                float* __restrict__ part, int rows, int chunk, int G,
-                                                                int Hq, int Hkv, float scale_log2e) {
-    constexpr int N = Vec<T>::N, LPR = D / N, NGRP = ATT_NT / LPR;
-    __shared__ float sm_m[NGRP], sm_l[NGRP];
-    __shared__ __align__(16) float sm_acc[NGRP][D];
-    const int split = blockIdx.x, nsplit = gridDim.x;
-    const int bh = blockIdx.y;
-    const int b = bh / Hq, h = bh % Hq;
-    const long long u = (long long)b * Hkv + h / G;
-    const int n = len ? max(0, min(len[u], rows)) : rows;
-    const int r0 = split * chunk, r1 = min(r0 + chunk, n);
-    const int grp = threadIdx.x / LPR, lane = threadIdx.x % LPR;
-    const unsigned gmask = (LPR == 32) ? 0xffffffffu : (((1u << LPR) - 1u) << ((threadIdx.x % 32) / LPR * LPR));
-    const T* Ku = K + (size_t)u * rows * D;
-    const T* Vu = V + (size_t)u * rows * D;
-
-    float qf[N];
-    Vec<T>::unpack(ldg16(q + (size_t)bh * D + lane * N), qf);
-    float m = -INFINITY, l = 0.f, acc[N];
-#pragma unroll
-    for (int e = 0; e < N; ++e) acc[e] = 0.f;
-    // RPI rows per iteration: their loads are independent and in flight together; one rescale per iteration
-#ifndef KVM_ATT_RPI
-#define KVM_ATT_RPI 4
-#endif
-    constexpr int RPI = KVM_ATT_RPI;
-    for (int r = r0 + grp * RPI; r < r1; r += NGRP * RPI) {
-        uint4 kraw[RPI], vraw[RPI];
-#pragma unroll
-        for (int i = 0; i < RPI; ++i) {
-            const int ri = min(r + i, r1 - 1);                   // clamped rows are loaded but given no weight
-            kraw[i] = ldg16(Ku + (size_t)ri * D + lane * N);
-            vraw[i] = ldg16(Vu + (size_t)ri * D + lane * N);
+// The block's walk over the items of its share.  Item = (unit, group of GH query heads), in that order; `start` counts
+// rows over all items.
+struct Item {
+    unsigned long long start;    // rows of all items before this one
+    int id, n;                   // item, rows of its unit
+    int off, cnt;                // this block's part: rows [off, off + cnt)
+};
+struct Work {
+    const int32_t* len;
+    int rows, HG, items;
+    unsigned long long q, f, f_end;      // rows per block; this block's share [f, f_end)
+    __device__ __forceinline__ int rows_of(int item) const { return len ? max(0, min(__ldg(len + item / HG), rows)) : rows; }
+    // moves to the part of item `it` that belongs to the share (skipping empty items); false when the share is done
+    __device__ __forceinline__ bool settle(Item& it) const {
+        while (f < f_end && it.id < items) {
+            if (it.start + it.n > f) {
+                it.off = (int)(f - it.start);
+                it.cnt = (int)min((unsigned long long)(it.n - it.off), f_end - f);
+                return true;
+            }
+            it.start += it.n;
+            if (++it.id < items) it.n = rows_of(it.id);
         }
-        float s[RPI];
-#pragma unroll
-        for (int i = 0; i < RPI; ++i) {
-            float kf[N];
-            Vec<T>::unpack(kraw[i], kf);
-            float dot = 0.f;
-#pragma unroll
-            for (int e = 0; e < N; ++e) dot = fmaf(qf[e], kf[e], dot);
-            s[i] = dot;
-        }
-#pragma unroll
-        for (int off = 1; off < LPR; off <<= 1) {
-#pragma unroll
-            for (int i = 0; i < RPI; ++i) s[i] += __shfl_xor_sync(gmask, s[i], off);
-        }
-        float mn = m;
-#pragma unroll
-        for (int i = 0; i < RPI; ++i) {
-            s[i] = (r + i < r1) ? s[i] * scale_log2e : -INFINITY;
-            mn = fmaxf(mn, s[i]);
-        }
-        const float corr = exp2f(m - mn);                        // first iteration: exp2(-inf) = 0
-        l *= corr;
-#pragma unroll
-        for (int e = 0; e < N; ++e) acc[e] *= corr;
-#pragma unroll
-        for (int i = 0; i < RPI; ++i) {
-            const float pj = exp2f(s[i] - mn);                   // 0 for a clamped row
-            float vf[N];
-            Vec<T>::unpack(vraw[i], vf);
-            l += pj;
-#pragma unroll
-            for (int e = 0; e < N; ++e) acc[e] = fmaf(pj, vf[e], acc[e]);
-        }
-        m = mn;
+        return false;
     }
-    if (lane == 0) { sm_m[grp] = m; sm_l[grp] = l; }
+};
+
+// This block's share, cut by a prefix sum over the items' rows (all threads of the block; false: nothing to do).
+struct ShareSmem {
+    unsigned long long wsum[ATT_WARPS + 1], start;
+    int id;
+};
+__device__ __forceinline__ bool take_share(Work& w, Item& it, ShareSmem& sh) {
+    const int warp = threadIdx.x >> 5, wl = threadIdx.x & 31;
+    const int E = (w.items + ATT_NT - 1) / ATT_NT, i0 = min(w.items, (int)threadIdx.x * E), i1 = min(w.items, i0 + E);
+    unsigned long long mine = 0;
+    for (int i = i0; i < i1; ++i) mine += w.rows_of(i);
+    unsigned long long inc = mine;
 #pragma unroll
-    for (int e = 0; e < N; ++e) sm_acc[grp][lane * N + e] = acc[e];
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long t = __shfl_up_sync(0xffffffffu, inc, o);
+        if (wl >= o) inc += t;
+    }
+    if (wl == 31) sh.wsum[warp] = inc;
     __syncthreads();
-    if (threadIdx.x < D) {
-        float M = -INFINITY;
+    unsigned long long total = 0, before = inc - mine;
 #pragma unroll
-        for (int g = 0; g < NGRP; ++g) M = fmaxf(M, sm_m[g]);
-        float L = 0.f, o = 0.f;
+    for (int x = 0; x <= ATT_WARPS; ++x) {
+        if (x < warp) before += sh.wsum[x];
+        total += sh.wsum[x];
+    }
+    w.q = max((total + gridDim.x - 1) / gridDim.x, (unsigned long long)ATT_MIN_SHARE);
+    w.f = min(total, w.q * blockIdx.x);
+    w.f_end = min(total, w.f + w.q);
+    if (w.f == w.f_end) return false;
+    if (before <= w.f && w.f < before + mine) {                    // true in exactly one thread
+        unsigned long long st = before;
+        int id = i0, n = w.rows_of(id);
+        while (st + n <= w.f) { st += n; n = w.rows_of(++id); }
+        sh.start = st;
+        sh.id = id;
+    }
+    __syncthreads();
+    it.start = sh.start; it.id = sh.id; it.n = w.rows_of(it.id);
+    return true;
+}
+
+// Piece end: the warps' states (sm_m, sm_l, sm_acc [warp][GH][D]) in a fixed order -> the piece's state of `heads` heads;
+// and, from the block that holds the item's first row, how many pieces it has.
+template <int D, int GH>
+__device__ __forceinline__ void store_piece(const Work& w, const Item& it, const float (*sm_m)[GH], const float (*sm_l)[GH],
+                                            const float* sm_acc, bool bad, float* part, int32_t* pieces, int max_pieces,
+                                            int heads, int stride) {
+    const int first = (int)(it.start / w.q);
+    float* dst = part + ((size_t)it.id * max_pieces + (blockIdx.x - first)) * stride * (D + 2);
+    for (int i = threadIdx.x; i < heads * D; i += ATT_WARPS * 32) {
+        const int h = i / D;
+        float M = -INFINITY, L = 0.f, o = 0.f;
 #pragma unroll
-        for (int g = 0; g < NGRP; ++g) {
-            const float w = rescale(sm_m[g], M);
-            L = fmaf(sm_l[g], w, L);
-            o = fmaf(sm_acc[g][threadIdx.x], w, o);
+        for (int x = 0; x < ATT_WARPS; ++x) M = fmaxf(M, sm_m[x][h]);
+#pragma unroll
+        for (int x = 0; x < ATT_WARPS; ++x) {
+            const float a = rescale(sm_m[x][h], M);
+            L = fmaf(sm_l[x][h], a, L);
+            o = fmaf(sm_acc[(x * GH + h) * D + i % D], a, o);
         }
-        float* dst = part + ((size_t)bh * nsplit + split) * (D + 2);
-        dst[threadIdx.x] = o;
-        if (threadIdx.x == 0) { dst[D] = M; dst[D + 1] = L; }
+        dst[h * (D + 2) + i % D] = bad ? NAN : o;
+        if (i % D == 0) { dst[h * (D + 2) + D] = M; dst[h * (D + 2) + D + 1] = L; }
+    }
+    if (threadIdx.x == 0 && (int)blockIdx.x == first) pieces[it.id] = (int)((it.start + it.n - 1) / w.q) - first + 1;
+}
+
+// part: per item and piece, for each of the GH heads D weighted sums, the maximum and the sum (log2 units); pieces:
+// per item, how many there are.
+template <typename T, int D, int GH>
+__global__ void __launch_bounds__(ATT_NT, 1)
+attend_partial_fma_kernel(const T* __restrict__ q, const T* __restrict__ K, const T* __restrict__ V,
+                      const int32_t* __restrict__ len, float* __restrict__ part, int32_t* __restrict__ pieces, int rows, int G,
+                      int U, int max_pieces, float scale_log2e) {
+    constexpr int N = Vec<T>::N, LPR = D / N, GPW = 32 / LPR;      // elements per 16 bytes, lanes per row, groups per warp
+    constexpr int SROWS = ATT_STAGE_BYTES / (D * (int)sizeof(T));  // rows per stage
+    static_assert(SROWS == ATT_WARPS * GPW * RPI, "a stage is one round of every group");
+    constexpr int NV = RPI * GH, CNT = NV > LPR ? NV / LPR : 1;    // products per lane, and how many it keeps
+    constexpr int REP = NV < LPR ? LPR / NV : 1, RL = RPI / CNT;   // lanes holding the same product; lanes per head's rows
+    static_assert(CNT <= RPI, "a lane's products belong to one head");
+    extern __shared__ __align__(128) uint8_t smem[];
+    uint8_t* ring = smem;                                          // [stage][K | V][SROWS][D]
+    float* sm_acc = reinterpret_cast<float*>(smem + ATT_STAGES * 2 * ATT_STAGE_BYTES);   // [warp][GH][D]
+    __shared__ __align__(8) uint64_t full[ATT_STAGES], empty[ATT_STAGES];
+    __shared__ float sm_m[ATT_WARPS][GH], sm_l[ATT_WARPS][GH];
+    __shared__ ShareSmem sh;
+    __shared__ volatile int s_bad;
+
+    const int warp = threadIdx.x >> 5, wl = threadIdx.x & 31;
+    Work w;
+    w.len = len; w.rows = rows; w.HG = (G + GH - 1) / GH; w.items = U * w.HG;
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < ATT_STAGES; ++i) {
+            mbar_init(&full[i], 1);
+            mbar_init(&empty[i], ATT_WARPS);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        s_bad = 0;
+    }
+    grid_dependency_wait();
+    Item it;
+    if (!take_share(w, it, sh)) return;
+
+    if (warp == ATT_WARPS) {
+        // ---- copies
+        if (wl == 0) {
+            uint32_t k = 0;
+            bool ok = true;
+            while (ok && w.settle(it)) {
+                const size_t r0 = (size_t)(it.id / w.HG) * rows + it.off;
+                for (int r = 0; r < it.cnt; r += SROWS, ++k) {
+                    const int s = k % ATT_STAGES;
+                    ok = mbar_wait(&empty[s], ((k / ATT_STAGES) & 1) ^ 1, &s_bad);
+                    if (!ok) break;
+                    const uint32_t bytes = (uint32_t)min(SROWS, it.cnt - r) * D * sizeof(T);
+                    const uint32_t dst = smem_u32(ring + s * 2 * ATT_STAGE_BYTES), bar = smem_u32(&full[s]);
+                    mbar_expect_tx(&full[s], 2 * bytes);
+                    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                                 ::"r"(dst), "l"(K + (r0 + r) * D), "r"(bytes), "r"(bar) : "memory");
+                    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                                 ::"r"(dst + ATT_STAGE_BYTES), "l"(V + (r0 + r) * D), "r"(bytes), "r"(bar) : "memory");
+                }
+                w.f += it.cnt;
+            }
+        }
+        return;
+    }
+    // ---- arithmetic
+    const int lane = wl % LPR, g = wl / LPR;                       // lane within the row, group within the warp
+    const int head = lane / (RL * REP);                            // the head whose products this lane finishes
+    const int rl = (lane / REP) % RL;                              // ... for rows rl * CNT .. + CNT of the group's four
+    const int lb = g * LPR;                                        // the group's first lane
+    uint32_t k = 0;
+    while (w.settle(it)) {
+        const int u = it.id / w.HG, h0 = (it.id % w.HG) * GH;
+        uint64_t qp[GH][N / 2], acc[GH][N / 2];
+#pragma unroll
+        for (int h = 0; h < GH; ++h) {
+            float f[N];
+            Vec<T>::unpack(ldg16(q + ((size_t)u * G + min(h0 + h, G - 1)) * D + lane * N), f);
+#pragma unroll
+            for (int e = 0; e < N / 2; ++e) { qp[h][e] = pack2(f[2 * e], f[2 * e + 1]); acc[h][e] = 0ull; }
+        }
+        float m = -INFINITY, l = 0.f;                              // of this lane's head (l: of this lane's rows)
+        for (int r = 0; r < it.cnt; r += SROWS, ++k) {
+            const int s = k % ATT_STAGES;
+            // (the block's own copies always complete; a wait that ran out all the same makes the outputs NaN)
+            if (!__all_sync(0xffffffffu, mbar_wait(&full[s], (k / ATT_STAGES) & 1, &s_bad))) break;
+            const int row = (warp * GPW + g) * RPI, live = it.cnt - r - row;      // rows of the group that exist
+            const uint4* sk = reinterpret_cast<const uint4*>(ring + s * 2 * ATT_STAGE_BYTES) + row * LPR + lane;
+            const uint4* sv = reinterpret_cast<const uint4*>(ring + s * 2 * ATT_STAGE_BYTES + ATT_STAGE_BYTES) + row * LPR + lane;
+            float v[NV];                                           // product of head h, row i: v[h * RPI + i]
+#pragma unroll
+            for (int i = 0; i < RPI; ++i) {
+                float f[N];
+                Vec<T>::unpack(sk[i * LPR], f);
+#pragma unroll
+                for (int h = 0; h < GH; ++h) {
+                    uint64_t a = 0ull;
+#pragma unroll
+                    for (int e = 0; e < N / 2; ++e) a = ffma2(qp[h][e], pack2(f[2 * e], f[2 * e + 1]), a);
+                    float lo, hi;
+                    unpack2(a, lo, hi);
+                    v[h * RPI + i] = lo + hi;
+                }
+            }
+#pragma unroll
+            for (int o = LPR / 2, c = NV; o > 0; o >>= 1) {
+                if (c > 1) {
+                    c >>= 1;
+                    const bool up = (lane & o) != 0;
+#pragma unroll
+                    for (int i = 0; i < NV / 2; ++i) {
+                        if (i >= c) break;
+                        const float keep = up ? v[i + c] : v[i], give = up ? v[i] : v[i + c];
+                        v[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+                    }
+                } else {
+                    v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+                }
+            }
+            float p[CNT], mx = -INFINITY;
+#pragma unroll
+            for (int i = 0; i < CNT; ++i) {
+                p[i] = rl * CNT + i < live ? v[i] * scale_log2e : -INFINITY;
+                mx = fmaxf(mx, p[i]);
+            }
+#pragma unroll
+            for (int o = REP; o < REP * RL; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+            const bool grow = mx > m + REF_STEP || (m == -INFINITY && mx > -INFINITY);
+            if (__any_sync(0xffffffffu, grow)) {
+                const float alpha = grow ? exp2f(m - mx) : 1.f;
+                if (grow) m = mx;
+                l *= alpha;
+#pragma unroll
+                for (int h = 0; h < GH; ++h) {
+                    const float a = __shfl_sync(0xffffffffu, alpha, lb + h * RL * REP);
+                    const uint64_t a2 = pack2(a, a);
+#pragma unroll
+                    for (int e = 0; e < N / 2; ++e) acc[h][e] = ffma2(acc[h][e], a2, 0ull);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < CNT; ++i) {
+                p[i] = p[i] == -INFINITY ? 0.f : exp2f(p[i] - m);
+                l += p[i];
+            }
+#pragma unroll
+            for (int i = 0; i < RPI; ++i) {
+                uint4 raw = sv[i * LPR];
+                if (i >= live) raw = make_uint4(0, 0, 0, 0);       // (a stage's unwritten rows may hold anything)
+                float f[N];
+                Vec<T>::unpack(raw, f);
+#pragma unroll
+                for (int h = 0; h < GH; ++h) {
+                    const float a = __shfl_sync(0xffffffffu, p[i % CNT], lb + (h * RL + i / CNT) * REP);
+                    const uint64_t a2 = pack2(a, a);
+#pragma unroll
+                    for (int e = 0; e < N / 2; ++e) acc[h][e] = ffma2(a2, pack2(f[2 * e], f[2 * e + 1]), acc[h][e]);
+                }
+            }
+            __syncwarp();
+            if (wl == 0) mbar_arrive(&empty[s]);
+        }
+        // ---- piece end: the warp's groups, then the warps, in a fixed order
+#pragma unroll
+        for (int o = REP; o < REP * RL; o <<= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+        float M = m;
+#pragma unroll
+        for (int o = LPR; o < 32; o <<= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+        const float wgt = rescale(m, M);
+        l *= wgt;
+#pragma unroll
+        for (int o = LPR; o < 32; o <<= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+        if (g == 0 && lane == head * RL * REP) { sm_m[warp][head] = M; sm_l[warp][head] = l; }
+#pragma unroll
+        for (int h = 0; h < GH; ++h) {
+            const float a = __shfl_sync(0xffffffffu, wgt, lb + h * RL * REP);
+#pragma unroll
+            for (int e = 0; e < N / 2; ++e) {
+                float x[2];
+                unpack2(acc[h][e], x[0], x[1]);
+#pragma unroll
+                for (int z = 0; z < 2; ++z) {
+                    x[z] *= a;
+#pragma unroll
+                    for (int o = LPR; o < 32; o <<= 1) x[z] += __shfl_xor_sync(0xffffffffu, x[z], o);
+                }
+                if (g == 0) *reinterpret_cast<float2*>(sm_acc + (warp * GH + h) * D + lane * N + 2 * e) = make_float2(x[0], x[1]);
+            }
+        }
+        named_bar(1, ATT_WARPS * 32);
+        store_piece<D, GH>(w, it, sm_m, sm_l, sm_acc, s_bad != 0, part, pieces, max_pieces, GH, GH);
+        named_bar(1, ATT_WARPS * 32);
+        w.f += it.cnt;
     }
 }
 
+// ------------------------------------------------------------------ bf16 caches: the same on warp-level matrix products
+// With bf16 rows the FMA kernel spends 420 instructions per warp and stage on unpacking, multiplying and shuffling; the
+// matrix instructions take a fifth of that, and up to eight query heads for the price of one.  (The work is a stream of
+// K and V past a handful of queries: bandwidth-bound, so the warp-level instructions' rate is no limit, and their
+// operands need neither tensor memory nor a barrier between the two products.)
+//   S = K q^T   16 rows x 8 heads per product chain (K rows as they lie, q as the constant operand)
+//   O^T += V^T P  16 channels x 8 heads per product; P enters as three bf16 terms (24 bits, exact), V is bf16 already,
+//               and every 16 rows' products start from zero and are added in fp32, so that nothing is rounded earlier
+//               than in fp32 arithmetic
+// Rows come by TMA with the 128-byte swizzle (ldmatrix without bank conflicts).
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ldsm4_t(uint32_t (&r)[4], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ uint32_t transpose8x8(uint32_t x) {
+    uint32_t r;
+    asm("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(r) : "r"(x));
+    return r;
+}
+
+constexpr int MMA_GH = 8;                   // query heads of a product
+
 template <int D>
-__global__ void __launch_bounds__(D) attend_combine_kernel(const float* __restrict__ part, float* __restrict__ out,
-                                                           int nsplit) {
-    grid_dependency_wait();     // the partial states come from the kernel before this one
-    const int bh = blockIdx.x;
-    const float* p = part + (size_t)bh * nsplit * (D + 2);
-    float M = -INFINITY;
-    for (int s = 0; s < nsplit; ++s) M = fmaxf(M, p[(size_t)s * (D + 2) + D]);
-    float L = 0.f, o = 0.f;
-    for (int s = 0; s < nsplit; ++s) {
-        const float* ps = p + (size_t)s * (D + 2);
-        const float w = rescale(ps[D], M);
-        L = fmaf(ps[D + 1], w, L);
-        o = fmaf(ps[threadIdx.x], w, o);
+__global__ void __launch_bounds__(ATT_NT, 1)
+attend_partial_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
+                          const __nv_bfloat16* __restrict__ q, const int32_t* __restrict__ len, float* __restrict__ part,
+                          int32_t* __restrict__ pieces, int rows, int G, int U, int max_pieces, float scale_log2e) {
+    constexpr int KCH = D / 64;                                    // 64-channel (128-byte) column chunks
+    constexpr int SROWS = ATT_STAGE_BYTES / (D * 2);               // rows per stage (64 or 128)
+    constexpr int CHUNK = SROWS * 128;                             // bytes of a column chunk of a stage
+    constexpr int NB = SROWS / 16;                                 // 16-row blocks per stage, one per warp
+    static_assert(ATT_WARPS % NB == 0, "stages are dealt to whole sets of NB warps");
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    uint8_t* ring = smem_raw + (base - smem_u32(smem_raw));        // [stage][K | V][KCH][SROWS][128 B]
+    float* sm_acc = reinterpret_cast<float*>(ring + ATT_STAGES * 2 * ATT_STAGE_BYTES);   // [warp][MMA_GH][D]
+    __shared__ __align__(8) uint64_t full[ATT_STAGES], empty[ATT_STAGES];
+    __shared__ float sm_m[ATT_WARPS][MMA_GH], sm_l[ATT_WARPS][MMA_GH];
+    __shared__ ShareSmem sh;
+    __shared__ volatile int s_bad;
+
+    const int warp = threadIdx.x >> 5, wl = threadIdx.x & 31;
+    const int stride = min(G, MMA_GH);                             // heads a piece's state is laid out for
+    Work w;
+    w.len = len; w.rows = rows; w.HG = (G + MMA_GH - 1) / MMA_GH; w.items = U * w.HG;
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < ATT_STAGES; ++i) {
+            mbar_init(&full[i], 1);
+            mbar_init(&empty[i], NB);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        s_bad = 0;
     }
-    out[(size_t)bh * D + threadIdx.x] = L > 0.f ? o / L : 0.f;     // an empty cache attends to nothing
+    grid_dependency_wait();
+    Item it;
+    if (!take_share(w, it, sh)) return;
+
+    if (warp == ATT_WARPS) {
+        // ---- copies (a stage's rows past the piece are rows of the next pieces, or zeros past the tensor: masked)
+        if (wl == 0) {
+            uint32_t k = 0;
+            bool ok = true;
+            while (ok && w.settle(it)) {
+                const int r0 = it.off, u = it.id / w.HG;
+                for (int r = 0; r < it.cnt; r += SROWS, ++k) {
+                    const int s = k % ATT_STAGES;
+                    ok = mbar_wait(&empty[s], ((k / ATT_STAGES) & 1) ^ 1, &s_bad);
+                    if (!ok) break;
+                    mbar_expect_tx(&full[s], 2 * ATT_STAGE_BYTES);
+                    uint8_t* st = ring + s * 2 * ATT_STAGE_BYTES;
+#pragma unroll
+                    for (int c = 0; c < KCH; ++c) {
+                        tma_load_3d(st + c * CHUNK, &map_k, &full[s], c * 64, r0 + r, u);
+                        tma_load_3d(st + ATT_STAGE_BYTES + c * CHUNK, &map_v, &full[s], c * 64, r0 + r, u);
+                    }
+                }
+                w.f += it.cnt;
+            }
+        }
+        return;
+    }
+    // ---- arithmetic.  gid, tig: row and column pair of this lane in the 8x8 fragments
+    const int gid = wl >> 2, tig = wl & 3, blk = warp % NB;
+    const int sset = warp / NB;                                    // takes the stages k with k % (ATT_WARPS / NB) == sset
+    // ldmatrix addresses: K rows 0..15 x two 16-byte pieces; V (transposed) rows 0..7, 8..15 x two pieces
+    const int krow = blk * 16 + (wl & 15), kpc = wl >> 4;
+    const int vrow = blk * 16 + (wl & 7) + ((wl >> 4) << 3), vpc = (wl >> 3) & 1;
+    uint32_t k = 0;
+    while (w.settle(it)) {
+        const int u = it.id / w.HG, h0 = (it.id % w.HG) * MMA_GH, heads = min(G - h0, MMA_GH);
+        uint32_t qf[D / 16][2];                                    // q^T as B fragments: channels 2 tig.. (+8), head gid
+#pragma unroll
+        for (int ks = 0; ks < D / 16; ++ks)
+#pragma unroll
+            for (int x = 0; x < 2; ++x)
+                qf[ks][x] = gid < heads ? __ldg(reinterpret_cast<const uint32_t*>(q + ((size_t)u * G + h0 + gid) * D + ks * 16 + x * 8) + tig) : 0u;
+        float o[D / 16][4];                                        // channel dt * 16 + gid (+8), heads 2 tig, 2 tig + 1
+#pragma unroll
+        for (int dt = 0; dt < D / 16; ++dt)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) o[dt][e] = 0.f;
+        float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};    // of heads 2 tig, 2 tig + 1 (l: of this lane's rows)
+        for (int r = 0; r < it.cnt; r += SROWS, ++k) {
+            if ((int)(k % (ATT_WARPS / NB)) != sset) continue;
+            const int s = k % ATT_STAGES;
+            // (the block's own copies always complete; a wait that ran out all the same makes the outputs NaN)
+            if (!__all_sync(0xffffffffu, mbar_wait(&full[s], (k / ATT_STAGES) & 1, &s_bad))) break;
+            const int live = it.cnt - r - blk * 16;                // rows of the block that exist
+            if (live > 0) {
+                const uint32_t kb = base + s * 2 * ATT_STAGE_BYTES, vb = kb + ATT_STAGE_BYTES;
+                float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                for (int ks = 0; ks < D / 16; ++ks) {
+                    uint32_t a[4];
+                    ldsm4(a, kb + (ks / 4) * CHUNK + krow * 128 + ((((ks % 4) * 2 + kpc) ^ (krow & 7)) << 4));
+                    mma16816(ks & 1 ? c1 : c0, a, qf[ks][0], qf[ks][1]);
+                }
+                float x[4];                                        // rows gid, gid + 8 x heads 2 tig, 2 tig + 1
+#pragma unroll
+                for (int e = 0; e < 4; ++e) x[e] = gid + (e >> 1) * 8 < live ? (c0[e] + c1[e]) * scale_log2e : -INFINITY;
+                const float mx[2] = {fmaxf(x[0], x[2]), fmaxf(x[1], x[3])};
+                if (__any_sync(0xffffffffu, mx[0] > m[0] + REF_STEP || mx[1] > m[1] + REF_STEP)) {
+                    float alpha[2];
+#pragma unroll
+                    for (int y = 0; y < 2; ++y) {
+                        float t = mx[y];
+#pragma unroll
+                        for (int z = 4; z < 32; z <<= 1) t = fmaxf(t, __shfl_xor_sync(0xffffffffu, t, z));
+                        const float mn = t > m[y] + REF_STEP ? t : m[y];
+                        alpha[y] = rescale(m[y], mn);
+                        m[y] = mn;
+                        l[y] *= alpha[y];
+                    }
+#pragma unroll
+                    for (int dt = 0; dt < D / 16; ++dt)
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) o[dt][e] *= alpha[e & 1];
+                }
+                // weights, as three bf16 terms each, in the B operand's layout (rows 2 tig.. of head gid)
+                float p[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    p[e] = rescale(x[e], m[e & 1]);
+                    l[e & 1] += p[e];
+                }
+                uint32_t pb[3][2];
+#pragma unroll
+                for (int t = 0; t < 3; ++t)
+#pragma unroll
+                    for (int y = 0; y < 2; ++y) {
+                        const uint32_t pk = Vec<__nv_bfloat16>::pack2(p[2 * y], p[2 * y + 1]);
+                        p[2 * y] -= __uint_as_float(pk << 16);     // exact
+                        p[2 * y + 1] -= __uint_as_float(pk & 0xffff0000u);
+                        pb[t][y] = transpose8x8(pk);
+                    }
+                // rows that do not exist may hold anything: their V becomes zero (masks of the operand's rows 2 tig.. + 8)
+                uint32_t mask[2] = {0xffffffffu, 0xffffffffu};
+                if (live < 16)
+#pragma unroll
+                    for (int y = 0; y < 2; ++y)
+                        mask[y] = (2 * tig + y * 8 < live ? 0xffffu : 0u) | (2 * tig + 1 + y * 8 < live ? 0xffff0000u : 0u);
+#pragma unroll
+                for (int dt = 0; dt < D / 16; ++dt) {
+                    uint32_t a[4];
+                    ldsm4_t(a, vb + (dt / 4) * CHUNK + vrow * 128 + ((((dt % 4) * 2 + vpc) ^ (vrow & 7)) << 4));
+                    if (live < 16) { a[0] &= mask[0]; a[1] &= mask[0]; a[2] &= mask[1]; a[3] &= mask[1]; }
+                    float c[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                    for (int t = 2; t >= 0; --t) mma16816(c, a, pb[t][0], pb[t][1]);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) o[dt][e] += c[e];
+                }
+            }
+            __syncwarp();
+            if (wl == 0) mbar_arrive(&empty[s]);
+        }
+#pragma unroll
+        for (int y = 0; y < 2; ++y)
+#pragma unroll
+            for (int z = 4; z < 32; z <<= 1) l[y] += __shfl_xor_sync(0xffffffffu, l[y], z);
+        if (gid == 0) {
+            sm_m[warp][2 * tig] = m[0]; sm_m[warp][2 * tig + 1] = m[1];
+            sm_l[warp][2 * tig] = l[0]; sm_l[warp][2 * tig + 1] = l[1];
+        }
+#pragma unroll
+        for (int dt = 0; dt < D / 16; ++dt)
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (2 * tig + (e & 1) < heads) sm_acc[(warp * MMA_GH + 2 * tig + (e & 1)) * D + dt * 16 + gid + (e >> 1) * 8] = o[dt][e];
+        named_bar(1, ATT_WARPS * 32);
+        store_piece<D, MMA_GH>(w, it, sm_m, sm_l, sm_acc, s_bad != 0, part, pieces, max_pieces, heads, stride);
+        named_bar(1, ATT_WARPS * 32);
+        w.f += it.cnt;
+    }
+}
+
+// One block per query head: its pieces' states in order.
+template <int D>
+__global__ void __launch_bounds__(D) attend_combine_kernel(const float* __restrict__ part, const int32_t* __restrict__ pieces,
+                                                           const int32_t* __restrict__ len, float* __restrict__ out, int rows,
+                                                           int G, int gh, int max_pieces) {
+    const int u = blockIdx.x / G, h = blockIdx.x % G;              // b * Hq + h = unit * G + head of the group
+    const int item = u * ((G + gh - 1) / gh) + h / gh;
+    grid_dependency_wait();     // the partial states come from the kernel before this one
+    const int n = len ? min(__ldg(len + u), rows) : rows;
+    float o = 0.f, L = 0.f;
+    if (n > 0) {                                                   // an empty cache attends to nothing
+        const int np = __ldcg(pieces + item);
+        const float* p = part + ((size_t)item * max_pieces * gh + h % gh) * (D + 2);
+        float M = -INFINITY;
+#pragma unroll 4
+        for (int s = 0; s < np; ++s) {
+            const float* ps = p + (size_t)s * gh * (D + 2);
+            const float ms = __ldcg(ps + D), ls = __ldcg(ps + D + 1), os = __ldcg(ps + threadIdx.x);
+            const float mn = fmaxf(M, ms), a = rescale(M, mn), c = rescale(ms, mn);
+            L = fmaf(ls, c, L * a);
+            o = fmaf(os, c, o * a);
+            M = mn;
+        }
+    }
+    out[(size_t)blockIdx.x * D + threadIdx.x] = L > 0.f || L != L ? o / L : 0.f;
 }
 
 // err = |O - O*|_2 and ref = |O|_2 per (batch, query head).
@@ -162,40 +574,101 @@ __global__ void __launch_bounds__(D) perturbation_kernel(const float* __restrict
     }
 }
 
-template <typename T, int D>
-cudaError_t launch_t(const Dims& d, const void* q, const void* K, const void* V, int rows, const int32_t* len,
-                     float* out, float* part, cudaStream_t st) {
-    // as many chunks per head as keep every SM's resident blocks busy in a single wave, within the scratch bound
-    int dev = 0, sms = 0;
-    cudaError_t e0 = cudaGetDevice(&dev);
-    if (e0 == cudaSuccess) e0 = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e0 != cudaSuccess) return e0;
-    int want = (ATT_BLOCKS_PER_SM * sms) / (d.B * d.Hq);
-    want = want < 1 ? 1 : (want > attend_splits(rows) ? attend_splits(rows) : want);
-    const int chunk = (rows + want - 1) / want;
-    const int nsplit = (rows + chunk - 1) / chunk;
-    attend_partial_kernel<T, D><<<dim3(nsplit, d.B * d.Hq), ATT_NT, 0, st>>>(
-        (const T*)q, (const T*)K, (const T*)V, len, part, rows, chunk, d.G, d.Hq, d.Hkv, d.scale * LOG2E);
-    cudaError_t e = cudaGetLastError();
+// Query heads that share a pass over the rows.
+inline int head_group(const Dims& d) {
+    if (d.dtype == KVM_BF16) return d.G < MMA_GH ? d.G : MMA_GH;
+    return d.G >= 5 ? 8 : (d.G >= 3 ? 4 : d.G);
+}
+// Pieces an item can fall into: shares are at least ATT_MIN_SHARE rows.
+inline int most_pieces(int rows) { return (rows + ATT_MIN_SHARE - 2) / ATT_MIN_SHARE + 1; }
+
+// SM count of the current device; the kernel's shared-memory opt-in, once per device.
+template <typename... KArgs>
+cudaError_t prepare_kernel(void (*kernel)(KArgs...), int smem, int (&sms_of)[KVM_MAX_DEVICES], std::mutex& mu, int& sms) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    return launch_dependent(attend_combine_kernel<D>, dim3(d.B * d.Hq), dim3(D), 0, st, (const float*)part, out, nsplit);
+    if (dev < 0 || dev >= KVM_MAX_DEVICES) return cudaErrorInvalidDevice;
+    std::lock_guard<std::mutex> lock(mu);
+    if (!sms_of[dev]) {
+        if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
+        if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+        sms_of[dev] = sms;
+    }
+    sms = sms_of[dev];
+    return cudaSuccess;
+}
+
+struct Scratch {
+    int items, gh, mp;
+    int32_t* pieces;
+    float* states;
+    unsigned grid(int sms, int rows) const {
+        const long long most = ((long long)items * rows + ATT_MIN_SHARE - 1) / ATT_MIN_SHARE;
+        return (unsigned)(most < sms ? most : sms);
+    }
+};
+
+template <typename T, int D, int GH>
+cudaError_t launch_fma(const Dims& d, const void* q, const void* K, const void* V, int rows, const int32_t* len,
+                       const Scratch& sc, cudaStream_t st) {
+    constexpr int smem = ATT_STAGES * 2 * ATT_STAGE_BYTES + ATT_WARPS * GH * D * (int)sizeof(float);
+    static std::mutex mu;
+    static int sms_of[KVM_MAX_DEVICES] = {};
+    int sms = 0;
+    const cudaError_t e = prepare_kernel(attend_partial_fma_kernel<T, D, GH>, smem, sms_of, mu, sms);
+    if (e != cudaSuccess) return e;
+    return launch_dependent(attend_partial_fma_kernel<T, D, GH>, dim3(sc.grid(sms, rows)), dim3(ATT_NT), smem, st, (const T*)q,
+                            (const T*)K, (const T*)V, len, sc.states, sc.pieces, rows, d.G, d.U, sc.mp, d.scale * LOG2E);
+}
+template <int D>
+cudaError_t launch_mma(const Dims& d, const void* q, const void* K, const void* V, int rows, const int32_t* len,
+                       const Scratch& sc, cudaStream_t st) {
+    constexpr int smem = 1024 + ATT_STAGES * 2 * ATT_STAGE_BYTES + ATT_WARPS * MMA_GH * D * (int)sizeof(float);
+    static std::mutex mu;
+    static int sms_of[KVM_MAX_DEVICES] = {};
+    int sms = 0;
+    const cudaError_t e = prepare_kernel(attend_partial_mma_kernel<D>, smem, sms_of, mu, sms);
+    if (e != cudaSuccess) return e;
+    CUtensorMap mk, mv;
+    if (!make_map(&mk, K, d.U, rows, D, ATT_STAGE_BYTES / (2 * D)) || !make_map(&mv, V, d.U, rows, D, ATT_STAGE_BYTES / (2 * D)))
+        return cudaErrorNotSupported;
+    return launch_dependent(attend_partial_mma_kernel<D>, dim3(sc.grid(sms, rows)), dim3(ATT_NT), smem, st, mk, mv,
+                            (const __nv_bfloat16*)q, len, sc.states, sc.pieces, rows, d.G, d.U, sc.mp, d.scale * LOG2E);
+}
+
+template <int D>
+cudaError_t launch_t(const Dims& d, const void* q, const void* K, const void* V, int rows, const int32_t* len, float* out,
+                     float* part, cudaStream_t st) {
+    Scratch sc;
+    sc.gh = head_group(d);
+    sc.items = d.U * ((d.G + sc.gh - 1) / sc.gh);
+    sc.mp = most_pieces(rows);
+    sc.pieces = reinterpret_cast<int32_t*>(part);
+    sc.states = part + (sc.items + 3) / 4 * 4;
+    auto fn = d.dtype == KVM_BF16 ? launch_mma<D>
+              : sc.gh == 1        ? launch_fma<float, D, 1>
+              : sc.gh == 2        ? launch_fma<float, D, 2>
+              : sc.gh == 4        ? launch_fma<float, D, 4>
+                                  : launch_fma<float, D, 8>;
+    const cudaError_t e = fn(d, q, K, V, rows, len, sc, st);
+    if (e != cudaSuccess) return e;
+    return launch_dependent(attend_combine_kernel<D>, dim3(d.B * d.Hq), dim3(D), 0, st, (const float*)sc.states,
+                            (const int32_t*)sc.pieces, len, out, rows, d.G, sc.gh, sc.mp);
 }
 
 }  // namespace
 
-// Upper bound on the chunks per head (what the scratch is sized for).
-int attend_splits(int rows) { return (rows + ATT_MIN_CHUNK - 1) / ATT_MIN_CHUNK; }
-
-size_t attend_scratch_floats(const Dims& d) { return (size_t)d.B * d.Hq * attend_splits(d.S) * (d.D + 2); }
+// States of every item's pieces and the items' piece counts.
+size_t attend_scratch_floats(const Dims& d) {
+    const int gh = head_group(d);
+    const size_t items = (size_t)d.U * ((d.G + gh - 1) / gh);
+    return (items + 3) / 4 * 4 + items * most_pieces(d.S) * gh * (d.D + 2);
+}
 
 cudaError_t launch_attend(const Dims& d, const void* q, const void* K, const void* V, int rows, const int32_t* len,
                           float* out, float* part, cudaStream_t st) {
-    if (d.dtype == KVM_BF16) {
-        return d.D == 128 ? launch_t<__nv_bfloat16, 128>(d, q, K, V, rows, len, out, part, st)
-                          : launch_t<__nv_bfloat16, 64>(d, q, K, V, rows, len, out, part, st);
-    }
-    return d.D == 128 ? launch_t<float, 128>(d, q, K, V, rows, len, out, part, st)
-                      : launch_t<float, 64>(d, q, K, V, rows, len, out, part, st);
+    return d.D == 128 ? launch_t<128>(d, q, K, V, rows, len, out, part, st) : launch_t<64>(d, q, K, V, rows, len, out, part, st);
 }
 
 cudaError_t launch_perturbation(const Dims& d, const float* O, const float* Os, float* err, float* ref,

@@ -108,7 +108,6 @@ cudaError_t launch_gather(const Dims& d, const void* K, const void* V, const int
                           cudaStream_t st);
 
 // Decode-step attention over a ragged cache and the full-vs-compressed output difference.
-int attend_splits(int rows);
 size_t attend_scratch_floats(const Dims& d);
 cudaError_t launch_attend(const Dims& d, const void* q, const void* K, const void* V, int rows, const int32_t* len,
                           float* out, float* part, cudaStream_t st);

@@ -221,13 +221,13 @@ inline EncodeTiledFn encode_fn() {
     return fn;
 }
 
-// [heads, S, D] bf16, boxes of [1, 128 rows, 64 channels], 128-byte swizzle, zero fill past S.
-inline bool make_map(CUtensorMap* map, const void* ptr, int heads, int S, int D) {
+// [heads, S, D] bf16, boxes of [1, box_rows rows, 64 channels], 128-byte swizzle, zero fill past S.
+inline bool make_map(CUtensorMap* map, const void* ptr, int heads, int S, int D, int box_rows = 128) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
     cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)S, (cuuint64_t)heads};
     cuuint64_t strides[2] = {(cuuint64_t)D * 2, (cuuint64_t)S * D * 2};
-    cuuint32_t box[3] = {64, 128, 1};
+    cuuint32_t box[3] = {64, (cuuint32_t)box_rows, 1};
     cuuint32_t estr[3] = {1, 1, 1};
     return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,

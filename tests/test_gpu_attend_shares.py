@@ -1,0 +1,42 @@
+"""Decode attention where the rows are split over the blocks: shares that cut units anywhere, groups of every size,
+empty units, rows that no block of rows divides, against fp64."""
+import pytest
+import torch
+
+import paper_2407_08454_b200 as kvm
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("B,G,Hkv,rows,D", [
+    (1, 1, 1, 1, 128),         # one row
+    (1, 3, 2, 15, 64),         # less than a 16-row block
+    (2, 5, 2, 65, 128),        # one row past a stage
+    (1, 8, 1, 700, 64),        # one unit over many blocks
+    (1, 9, 3, 333, 128),       # more query heads than one pass takes
+    (3, 2, 37, 97, 64),        # more units than blocks need, shares cut in the middle of units
+    (1, 1, 300, 70, 128),      # more units than SMs
+])
+def test_attend_against_fp64(B, G, Hkv, rows, D, dtype):
+    g = torch.Generator().manual_seed(rows * G + D)
+    q = (torch.randn(B, Hkv * G, D, generator=g) * 3).to(dtype).cuda()
+    K = torch.randn(B, Hkv, rows, D, generator=g).to(dtype).cuda()
+    V = torch.randn(B, Hkv, rows, D, generator=g).to(dtype).cuda()
+    n = torch.randint(0, rows + 1, (B, Hkv), generator=g, dtype=torch.int32)
+    n.view(-1)[-1] = rows
+    p = kvm.make_params(B, Hkv * G, Hkv, rows, D, dtype, budget=1.0, recent_ratio=0.0, heavy_ratio=0.0)
+    ws = torch.full((kvm.kvm_workspace_bytes(p),), 255, dtype=torch.uint8, device="cuda")
+    for length in (None, n):
+        Kc, Vc = K.clone(), V.clone()
+        dead = (torch.arange(rows) >= (n[..., None] if length is not None else torch.full_like(n, rows)[..., None]))
+        Kc[dead.cuda()], Vc[dead.cuda()] = float("nan"), float("nan")      # rows past a unit's length may hold anything
+        out = torch.full((B, Hkv * G, D), 7.0, device="cuda")
+        kvm.kvm_attend(p, q, Kc, Vc, rows, None if length is None else length.cuda(), out, ws)
+        L = (q.double().view(B, Hkv, G, D) @ K.double().transpose(-1, -2)) / D ** 0.5
+        L = L.masked_fill(dead.cuda()[:, :, None], float("-inf"))
+        ref = torch.nan_to_num(torch.softmax(L, -1)) @ V.double()
+        # a logit of at most ~20 is off by (D + few) * 2^-24 of |q||k| c; weights and sums add 2^-20 of the largest value
+        qk = (q.double().norm(dim=-1).max() * K.double().norm(dim=-1).max() / D ** 0.5).item()
+        tol = (2 * (D / 16 + 4) * 2.0 ** -23 * qk + 2.0 ** -20) * V.double().abs().max().item()
+        assert (out.double().view_as(ref) - ref).abs().max().item() <= tol
