@@ -313,7 +313,8 @@ int kvm_output_perturbation(const kvm_params* p, const void* q, const void* K, c
  * not acceptable -- and that has no spare buffer to lend as a workspace.
  *
  * Instead of a caller workspace, the row log-sum-exp scratch lives in a fixed
- * array built into the library image: KVM_STATIC_SCORE_ROWS floats (4 MiB).  Every
+ * array built into the library image: KVM_STATIC_SCORE_ROWS floats (4 MiB), and
+ * 1.25 MiB for the partial results of work items that are cut.  Every
  * GPU on which the CUDA runtime loads the library's device code holds that array
  * from then (at the latest from this function's first call there) until the process
  * exits, whether or not the function is called again.

@@ -25,7 +25,7 @@ def sources():
 # wait limit and a producer that leaves out one stage, so that a wait runs out, the kernel returns and reports
 # it.  It is never loaded by the package itself.
 WAITTEST_LIB = os.path.join(_PKG, "libkvm_waittest.so")
-WAITTEST_FLAGS = ("-DKVM_TEST_WAIT_LIMIT_CLOCKS=4000000ll", "-DKVM_TEST_DROP_B_STAGE=3")
+WAITTEST_FLAGS = ("-DKVM_TEST_WAIT_LIMIT_CLOCKS=4000000ll", "-DKVM_TEST_DROP_B_STAGE=3", "-DKVM_TEST_DROP_SCORE_STEP=0")
 
 
 def _stale(lib: str = LIB) -> bool:

@@ -5,7 +5,7 @@
 
 #include <mutex>
 
-#include "common.cuh"
+#include "score_plan.cuh"
 
 namespace kvm {
 namespace {
@@ -64,11 +64,11 @@ int derive(const kvm_params* p, Dims& d) {
 
 // scratch of the score step: the bf16 path's side tensor, or the fp32 path's states, partial sums and split planes
 inline size_t score_bytes(const Dims& d) {
-    return d.dtype == KVM_BF16 ? (size_t)d.B * d.Hq * d.S * score_tc_scratch_bytes_per_row() : score_f32_scratch_bytes(d);
+    return d.dtype == KVM_BF16 ? score_tc_scratch_bytes(d) : score_f32_scratch_bytes(d);
 }
 
 struct Workspace {
-    float* lse;         // score scratch: [B,Hq,S,16] bf16 side tensor (bf16), or states and partial sums (fp32)
+    float* lse;         // score scratch
     float* scores;      // [U,S]
     float* sim;         // [U,S]
     int32_t* set_start; // [U,cap+1]
@@ -105,10 +105,11 @@ int check_ws(const Dims& d, void* ws, size_t ws_bytes, Workspace& w) {
 
 // sim_out (nullable): where the neighbour-key similarities are wanted, which the score step produces on the side.
 cudaError_t run_score(const Dims& d, const void* Q, const void* K, const float* lse_in, float* scores,
-                      const Workspace& w, kvm_stats* stats, cudaStream_t st, float* sim_out = nullptr) {
+                      const Workspace& w, kvm_stats* stats, cudaStream_t st, float* sim_out = nullptr,
+                      ScorePart* parts = nullptr) {
     // fp32 tensors enter the tensor cores as exact sums of three bf16 planes: rounding them would not hold the
     // score tolerance
-    return d.dtype == KVM_BF16 ? launch_score_tc(d, Q, K, lse_in, w.lse, scores, stats, st, sim_out)
+    return d.dtype == KVM_BF16 ? launch_score_tc(d, Q, K, lse_in, w.lse, scores, stats, st, sim_out, nullptr, parts)
                                : launch_score_f32(d, Q, K, lse_in, w.lse, scores, stats, st, sim_out);
 }
 
@@ -205,7 +206,7 @@ int kvm_segment(const kvm_params* p, const void* K, const float* scores, int32_t
     } else if (d.set_rule == KVM_SETS_ADJACENT || sim_out) {
         if (launch_similarity(d, K, sim, st) != cudaSuccess) return KVM_E_CUDA;
     }
-    if (launch_segment(d, scores, sim, set_id, set_start, pivot, out_len, stats, st) != cudaSuccess)
+    if (launch_segment(d, const_cast<float*>(scores), ScorePart{}, sim, set_id, set_start, pivot, out_len, stats, st) != cudaSuccess)
         return KVM_E_CUDA;
     return KVM_OK;
 }
@@ -316,10 +317,11 @@ int kvm_compress_with_lse(const kvm_params* p, const void* Q, const void* K, con
     cudaStream_t st = (cudaStream_t)cuda_stream;
     float* scores = scores_out ? scores_out : w.scores;
     const bool want_sim = d.set_rule == KVM_SETS_ADJACENT;
-    if (run_score(d, Q, K, lse_in, scores, w, stats, st, want_sim ? w.sim : nullptr) != cudaSuccess) return KVM_E_CUDA;
+    ScorePart parts;
+    if (run_score(d, Q, K, lse_in, scores, w, stats, st, want_sim ? w.sim : nullptr, &parts) != cudaSuccess) return KVM_E_CUDA;
     if (d.set_rule == KVM_SETS_ANCHOR)
         if (launch_anchor_runs(d, K, w.sim, (float*)w.set_id, st) != cudaSuccess) return KVM_E_CUDA;
-    if (launch_segment(d, scores, w.sim, w.set_id, w.set_start, out_pos, out_len, stats, st) != cudaSuccess)
+    if (launch_segment(d, scores, parts, w.sim, w.set_id, w.set_start, out_pos, out_len, stats, st) != cudaSuccess)
         return KVM_E_CUDA;
     if (d.weight_rule == KVM_WEIGHT_PIVOT_ONLY)
         return launch_gather(d, K, V, w.set_start, out_pos, out_len, K_out, V_out, nullptr, st) == cudaSuccess
@@ -505,9 +507,10 @@ namespace {
 
 constexpr int kMaxDevices = KVM_MAX_DEVICES;
 
-// The row pass's output for up to KVM_STATIC_SCORE_ROWS fp32 rows.  In HOST code this name is only a stand-in
+// The row pass's output for up to KVM_STATIC_SCORE_ROWS fp32 rows, and room for what cut work items leave (for 2^17 bf16
+// rows at most 0.6 MiB over all shapes; the fp32 path's share the 4 MiB).  In HOST code this name is only a stand-in
 // for the device symbol; its device address comes from cudaGetSymbolAddress below.
-static __device__ __align__(256) unsigned char g_static_score_scratch[(size_t)KVM_STATIC_SCORE_ROWS * sizeof(float)];
+static __device__ __align__(256) unsigned char g_static_score_scratch[(size_t)KVM_STATIC_SCORE_ROWS * sizeof(float) + (5u << 18)];
 
 void* g_static_ptr[kMaxDevices];   // device address of the array, per device; set once
 
@@ -530,9 +533,9 @@ int kvm_score_static(const kvm_params* p, const void* Q, const void* K, float* s
     if (rc != KVM_OK) return rc;
     if (!Q || !K || !scores) return KVM_E_NULL;
     if (misaligned(Q) || misaligned(K) || misaligned(scores)) return KVM_E_ALIGN;
-    // 32 bytes per query row for bf16 tensors; fp32 ones need 4 where work items stay whole, and no more than the
-    // array where they are split (so that both entry points run the same plan)
-    if (d.dtype == KVM_F32 && (unsigned long long)d.B * d.Hq * d.S > (unsigned long long)KVM_STATIC_SCORE_ROWS)
+    // 32 bytes per query row for bf16 tensors; fp32 ones need 4 where work items stay whole, and what fits the array
+    // where they are split (so that both entry points run the same plan)
+    if ((unsigned long long)d.B * d.Hq * d.S > (unsigned long long)KVM_STATIC_SCORE_ROWS / (d.dtype == KVM_BF16 ? 8 : 1))
         return KVM_E_STATIC_LIMIT;
     if (score_bytes(d) > sizeof(g_static_score_scratch)) return KVM_E_STATIC_LIMIT;
     unsigned char* base = (unsigned char*)static_scratch_for_current_device();

@@ -83,14 +83,15 @@ cudaError_t launch_score_f32(const Dims& d, const void* Q, const void* K, const 
                              float* scores, kvm_stats* stats, cudaStream_t st, float* sim_out = nullptr,
                              float* lse_out = nullptr);
 size_t score_f32_scratch_bytes(const Dims& d);
-cudaError_t launch_score_tc(const Dims& d, const void* Q, const void* K, const float* lse_in, float* lse_ws,
+struct ScorePart;             // partial column sums left for the segment kernel (score_plan.cuh)
+cudaError_t launch_score_tc(const Dims& d, const void* Q, const void* K, const float* lse_in, void* scratch,
                             float* scores, kvm_stats* stats, cudaStream_t st, float* sim_out = nullptr,
-                            float* lse_out = nullptr);
-size_t score_tc_scratch_bytes_per_row();
+                            float* lse_out = nullptr, ScorePart* parts = nullptr);
+size_t score_tc_scratch_bytes(const Dims& d);
 cudaError_t launch_prefill_attend(const Dims& d, const void* Q, const void* K, const void* V, void* O, float* lse,
                                   kvm_stats* stats, cudaStream_t st);
 cudaError_t launch_similarity(const Dims& d, const void* K, float* sim, cudaStream_t st);
-cudaError_t launch_segment(const Dims& d, const float* scores, const float* sim, int32_t* set_id,
+cudaError_t launch_segment(const Dims& d, float* scores, const ScorePart& parts, const float* sim, int32_t* set_id,
                            int32_t* set_start, int32_t* pivot, int32_t* out_len, kvm_stats* stats, cudaStream_t st);
 size_t segment_max_smem();
 cudaError_t launch_anchor_runs(const Dims& d, const void* K, float* run_out, float* inv_norm, cudaStream_t st);

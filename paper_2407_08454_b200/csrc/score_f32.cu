@@ -38,6 +38,7 @@
 
 #include <mutex>
 
+#include "score_plan.cuh"
 #include "similarity_core.cuh"
 #include "tc_common.cuh"
 
@@ -45,8 +46,11 @@ namespace kvm {
 namespace {
 
 using namespace tc;
+using plan::Plan;
+using plan::Walk;
+using plan::add_state;
 
-constexpr int TILE = 128;
+constexpr int TILE = plan::TILE;
 constexpr int KCHUNK = 64;                         // channels per 128-byte swizzled bf16 row
 constexpr int NPLANE = 3;
 constexpr uint32_t PLANE_BYTES = TILE * 128;       // [128 rows x 64 bf16]
@@ -56,103 +60,22 @@ constexpr int NACC = 2;                            // accumulator pairs: 2 x (12
 constexpr int NEPI = 8, NCONV = 7;                // warps; with the MMA warp sixteen, i.e. 128 registers a thread
 constexpr int NTHREADS = (NEPI + NCONV + 1) * 32;
 constexpr int NSLOT = 8;                           // piece-end buffers in rotation
-constexpr int PLAN_CTAS = 148;                     // the split of the work is a function of the shape alone
 constexpr size_t SPLIT_BYTES_MAX = (size_t)KVM_STATIC_SCORE_ROWS * sizeof(float);
 constexpr float LOG2E = 1.4426950408889634f, LN2 = 0.6931471805599453f;
 
-// ------------------------------------------------------------------ the split of the work
-struct Plan {
-    int NH, U, G, T;         // query heads and units in total, query heads per unit, 128-row tiles per head
-    unsigned steps, q;       // steps of a pass (the same for both), steps per CTA
-    int split;               // items may be cut
-    int pr, pc;              // most pieces of a row-pass item / a column-pass item
-    __host__ __device__ unsigned tri() const { return (unsigned)T * (unsigned)(T + 1) / 2; }
-    // first step of an item, steps of an item, and how many CTAs share it
-    __host__ __device__ unsigned row_start(int head, int tile) const { return (unsigned)head * tri() + (unsigned)tile * (unsigned)(tile + 1) / 2; }
-    __host__ __device__ unsigned col_start(int u, int tile) const {
-        const unsigned jr = (unsigned)(T - 1 - tile);
-        return (unsigned)G * ((unsigned)u * tri() + jr * (jr + 1) / 2);
-    }
-    __host__ __device__ int row_pieces(int head, int tile) const {
-        const unsigned f = row_start(head, tile);
-        return (int)((f + (unsigned)tile) / q - f / q) + 1;
-    }
-    __host__ __device__ int col_pieces(int u, int tile) const {
-        const unsigned f = col_start(u, tile);
-        return (int)((f + (unsigned)(G * (T - tile)) - 1) / q - f / q) + 1;
-    }
-};
-
+// Items are cut where the pieces' results fit 4 MiB (large problems balance well with whole ones); one rule for both passes.
+size_t split_bytes(const Dims& d, const Plan& p) {
+    return (size_t)p.NH * d.S * p.pieces(p.T) * sizeof(float2) + (size_t)p.U * d.S * p.pieces(p.G * p.T) * sizeof(float);
+}
 bool make_plan(const Dims& d, Plan& p) {
-    p.NH = d.B * d.Hq; p.U = d.U; p.G = d.G; p.T = (d.S + TILE - 1) / TILE;
-    const long long steps = (long long)p.NH * p.T * (p.T + 1) / 2;
-    if (steps + PLAN_CTAS >= (1ll << 31)) return false;      // (more than fits a GPU's memory)
-    p.steps = (unsigned)steps;
-    p.q = (p.steps + PLAN_CTAS - 1) / PLAN_CTAS;
-    auto pieces = [&](int len) { const int n = (len - 1 + (int)p.q - 1) / (int)p.q + 1; return n < len ? n : len; };
-    p.pr = pieces(p.T);
-    p.pc = pieces(p.G * p.T);
-    const unsigned long long rows = (unsigned long long)p.NH * d.S, keys = (unsigned long long)p.U * d.S;
-    p.split = rows * p.pr * sizeof(float2) + keys * p.pc * sizeof(float) <= SPLIT_BYTES_MAX;
-    if (!p.split) p.pr = p.pc = 1;
+    if (!plan::make(d, p)) return false;
+    if (split_bytes(d, p) <= SPLIT_BYTES_MAX) {
+        p.split_row = p.split_col = 1;
+        p.pr = p.pieces(p.T);
+        p.pc = p.pieces(p.G * p.T);
+    }
     return true;
 }
-
-__device__ __forceinline__ unsigned tri_root(unsigned x) {       // largest t with t (t + 1) / 2 <= x
-    unsigned t = (unsigned)((sqrtf(8.f * (float)x + 1.f) - 1.f) * 0.5f);
-    while (t * (t + 1) / 2 > x) --t;
-    while ((t + 1) * (t + 2) / 2 <= x) ++t;
-    return t;
-}
-
-// A CTA's pieces, one after the other.  head: query head (pass 1) or unit (pass 2); tile: the A tile; the piece is
-// steps [i0, i0 + n) of the item; B tile of step i: key tile i (pass 1), query tile tile + i % (T - tile) of query head
-// i / (T - tile) of the group (pass 2).
-template <int PASS>
-struct Walk {
-    unsigned f, f_end;
-    int head, tile, i0, n, len;
-    __device__ __forceinline__ void locate(const Plan& p) {
-        if (PASS == 1) {
-            head = (int)(f / p.tri());
-            const unsigned r = f - (unsigned)head * p.tri();
-            tile = (int)tri_root(r);
-            i0 = (int)(r - (unsigned)tile * (unsigned)(tile + 1) / 2);
-            len = tile + 1;
-        } else {
-            const unsigned gt = (unsigned)p.G * p.tri();
-            head = (int)(f / gt);
-            const unsigned r = f - (unsigned)head * gt, jr = tri_root(r / (unsigned)p.G);
-            tile = p.T - 1 - (int)jr;
-            i0 = (int)(r - (unsigned)p.G * (jr * (jr + 1) / 2));
-            len = p.G * (int)(jr + 1);
-        }
-    }
-    // where CTA c's share begins: step c q, or the first item that starts there or later when items stay whole
-    __device__ __forceinline__ unsigned boundary(const Plan& p, unsigned c) {
-        f = min(c * p.q, p.steps);
-        if (!p.split && f < p.steps) {
-            locate(p);
-            if (i0) f += (unsigned)(len - i0);
-        }
-        return f;
-    }
-    __device__ __forceinline__ void init(const Plan& p) {
-        f_end = boundary(p, blockIdx.x + 1);
-        f = boundary(p, blockIdx.x);
-        if (f >= f_end) return;
-        locate(p);
-        n = (int)min((unsigned)(len - i0), f_end - f);
-    }
-    __device__ __forceinline__ bool valid() const { return f < f_end; }
-    __device__ __forceinline__ void next(const Plan& p) {
-        f += (unsigned)n;
-        i0 = 0;
-        if (PASS == 1) { if (++tile == p.T) { tile = 0; ++head; } len = tile + 1; }
-        else { if (--tile < 0) { tile = p.T - 1; ++head; } len = p.G * (p.T - tile); }
-        n = (int)min((unsigned)len, f_end - f);
-    }
-};
 
 struct alignas(16) Shared {
     uint64_t full_a[2], empty_a, full_b[NSTAGE], empty_b[NSTAGE], acc_full[NACC], acc_empty[NACC];
@@ -164,13 +87,6 @@ struct alignas(16) Shared {
 };
 
 static_assert(offsetof(Shared, nl) % 16 == 0, "read four at a time");
-
-// Folds a partial (maximum, sum) of a query row into (M, L); log2 units.
-__device__ __forceinline__ void add_state(float& M, float& L, float2 st) {
-    const float mn = fmaxf(M, st.x);
-    if (mn > -INFINITY) L = L * exp2f(M - mn) + st.y * exp2f(st.x - mn);
-    M = mn;
-}
 
 // A 128-row x 64-channel chunk of a [S, D] fp32 matrix on its way to three bf16 planes, in units of eight channels:
 // unit u = t + k * (converter threads) is the eight channels u % 8 of row u / 8.
@@ -473,17 +389,15 @@ score_f32_kernel(const float* __restrict__ Q, const float* __restrict__ K, float
                     if (PASS == 1) {
                         const float M = fmaxf(m0, m1);
                         const float L = bad ? NAN : (m0 > -INFINITY ? l0 * exp2f(m0 - M) : 0.f) + (m1 > -INFINITY ? l1 * exp2f(m1 - M) : 0.f);
-                        if (plan.split) {
-                            const unsigned piece = blockIdx.x - plan.row_start(w.head, w.tile) / plan.q;
-                            states[(size_t)piece * rows + at] = make_float2(M, L);
+                        if (plan.split_row) {
+                            states[(size_t)w.piece(plan) * rows + at] = make_float2(M, L);
                         } else {
                             out[at] = M + log2f(L);
                         }
                     } else {
                         const float a = bad ? NAN : l0 + l1;
-                        if (plan.split) {
-                            const unsigned piece = blockIdx.x - plan.col_start(w.head, w.tile) / plan.q;
-                            out[(size_t)piece * plan.U * S + at] = a;
+                        if (plan.split_col) {
+                            out[(size_t)w.piece(plan) * plan.U * S + at] = a;
                         } else {
                             out[at] = a / (float)plan.G;
                         }
@@ -516,20 +430,12 @@ __global__ void __launch_bounds__(256) row_lse_kernel(const float2* __restrict__
     lse[r] = (M + log2f(L)) * LN2;
 }
 
-// Partial column sums -> the score of key j of unit u, in piece order.
-__device__ __forceinline__ void combine_token(const float* __restrict__ part, float* __restrict__ scores, const Plan& plan,
-                                              int S, int u, int j) {
-    const size_t keys = (size_t)plan.U * S, k = (size_t)u * S + j;
-    const int np = plan.col_pieces(u, j / TILE);
-    float a = 0.f;
-    for (int x = 0; x < np; ++x) a += __ldcg(part + (size_t)x * keys + k);
-    scores[k] = a / (float)plan.G;
-}
+// Partial column sums -> scores.
 __global__ void __launch_bounds__(256) combine_kernel(const float* __restrict__ part, float* __restrict__ scores,
                                                       const Plan plan, int S) {
     grid_dependency_wait();
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j < S) combine_token(part, scores, plan, S, blockIdx.y, j);
+    if (j < S) scores[(size_t)blockIdx.y * S + j] = plan::column_sum(part, plan, S, blockIdx.y, j);
 }
 // The same beside the neighbour similarities (Eq. 2, which need K alone and run while the column pass drains).
 constexpr int SIM_RUN = 8;                         // consecutive tokens per lane group
@@ -547,13 +453,13 @@ __global__ void __launch_bounds__(256) similarity_combine_kernel(const float* __
     const unsigned gmask = LPR == 32 ? 0xffffffffu : (((1u << LPR) - 1u) << gbase);
     simcore::run<float, D, SIM_RUN>(K + (size_t)u * S * D, sim + (size_t)u * S, j0, min(j0 + SIM_RUN, S), lane, gbase, gmask);
     grid_dependency_wait();                        // (always: this grid must not end before the column pass has)
-    if (part && lane < SIM_RUN && j0 + lane < S) combine_token(part, scores, plan, S, u, j0 + lane);
+    if (part && lane < SIM_RUN && j0 + lane < S) scores[(size_t)u * S + j0 + lane] = plan::column_sum(part, plan, S, u, j0 + lane);
 }
 
 // Bytes of the two passes' states and sums.
 size_t state_bytes(const Dims& d, const Plan& p) {
-    const size_t rows = (size_t)p.NH * d.S, keys = (size_t)p.U * d.S;
-    return p.split ? rows * p.pr * sizeof(float2) + keys * p.pc * sizeof(float) : rows * sizeof(float);
+    const size_t rows = (size_t)p.NH * d.S;
+    return p.split_row ? split_bytes(d, p) : rows * sizeof(float);
 }
 template <int KCH>
 cudaError_t launch_t(const Dims& d, const Plan& plan, const float* Q, const float* K, const float* lse_in, void* scratch,
@@ -575,14 +481,16 @@ cudaError_t launch_t(const Dims& d, const Plan& plan, const float* Q, const floa
             done[dev] = true;
         }
     }
-    const dim3 grid((plan.steps + plan.q - 1) / plan.q), block(NTHREADS);
+    const long long items = (long long)plan.NH * plan.T, citems = (long long)plan.U * plan.T;
+    const dim3 block(NTHREADS), rgrid(plan.split_row ? plan.grid_split() : (unsigned)(items < plan::CTAS ? items : plan::CTAS)),
+        cgrid(plan.split_col ? plan.grid_split() : (unsigned)(citems < plan::CTAS ? citems : plan::CTAS));
     const size_t rows = (size_t)plan.NH * d.S;
-    float2* states = plan.split ? (float2*)scratch : nullptr;
-    float* flat = plan.split ? nullptr : (float*)scratch;            // log2 units
-    float* part = plan.split ? (float*)((float2*)scratch + rows * plan.pr) : nullptr;
+    float2* states = plan.split_row ? (float2*)scratch : nullptr;
+    float* flat = plan.split_row ? nullptr : (float*)scratch;            // log2 units
+    float* part = plan.split_row ? (float*)((float2*)scratch + rows * plan.pr) : nullptr;
     const float scale2 = d.scale * LOG2E;
     if (!lse_in) {
-        e = launch_dependent(score_f32_kernel<KCH, 1>, grid, block, smem, st, Q, K, states, (const float*)nullptr,
+        e = launch_dependent(score_f32_kernel<KCH, 1>, rgrid, block, smem, st, Q, K, states, (const float*)nullptr,
                              1.f, flat, stats, plan, d.Hq, d.Hkv, d.S, scale2);
         if (e != cudaSuccess) return e;
     }
@@ -592,8 +500,8 @@ cudaError_t launch_t(const Dims& d, const Plan& plan, const float* Q, const floa
         if (e != cudaSuccess) return e;
     }
     if (!scores) return cudaSuccess;
-    e = launch_dependent(score_f32_kernel<KCH, 2>, grid, block, smem, st, Q, K, states,
-                         lse_in ? lse_in : (const float*)flat, lse_in ? LOG2E : 1.f, plan.split ? part : scores, stats, plan,
+    e = launch_dependent(score_f32_kernel<KCH, 2>, cgrid, block, smem, st, Q, K, states,
+                         lse_in ? lse_in : (const float*)flat, lse_in ? LOG2E : 1.f, plan.split_col ? part : scores, stats, plan,
                          d.Hq, d.Hkv, d.S, scale2);
     if (e != cudaSuccess) return e;
     if (sim_out) {
@@ -602,7 +510,7 @@ cudaError_t launch_t(const Dims& d, const Plan& plan, const float* Q, const floa
         return launch_dependent(similarity_combine_kernel<D>, dim3((unsigned)((threads + 255) / 256)), dim3(256), 0, st, K,
                                 sim_out, (const float*)part, scores, plan, d.S);
     }
-    if (!plan.split) return cudaSuccess;
+    if (!plan.split_col) return cudaSuccess;
     return launch_dependent(combine_kernel, dim3((d.S + 255) / 256, d.U), dim3(256), 0, st, (const float*)part, scores, plan, d.S);
 }
 

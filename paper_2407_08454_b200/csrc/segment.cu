@@ -20,9 +20,10 @@
 // rule (tokens re-read per phase, flags in shared memory, 8-bit radix digits),
 // and segment_unit_reg_kernel for the neighbour reading with at most four
 // tokens per thread (S <= 4096), which keeps a thread's tokens in registers.
+#include <float.h>
 #include <limits.h>
 
-#include "common.cuh"
+#include "score_plan.cuh"
 
 namespace kvm {
 namespace {
@@ -183,7 +184,8 @@ __device__ __forceinline__ void record_out_len(kvm_stats* stats, int n) {
     atomicAdd((unsigned long long*)&stats->sum_out_len, (unsigned long long)n);
 }
 
-__global__ void __launch_bounds__(NT) segment_unit_kernel(const float* __restrict__ scores,
+// (scores: where `parts` holds partial sums the kernel adds them up and writes the scores itself)
+__global__ void __launch_bounds__(NT, 1) segment_unit_kernel(float* __restrict__ scores, const ScorePart parts,
                                                           const float* __restrict__ sim, int32_t* __restrict__ set_id,
                                                           int32_t* __restrict__ set_start, int32_t* __restrict__ pivot,
                                                           int32_t* __restrict__ out_len, kvm_stats* stats, int S,
@@ -205,6 +207,8 @@ __global__ void __launch_bounds__(NT) segment_unit_kernel(const float* __restric
     const int nh = min(n_h, R);
 
     if (threadIdx.x < 4) sh.tot[threadIdx.x] = 0;   // (the barriers of step 1 come before their first use)
+    if (parts.part)                                 // (a thread reads the scores of its own tokens only)
+        for (int j = lo; j < hi; ++j) scores[(size_t)u * S + j] = plan::column_sum(parts.part, parts.plan, S, u, j);
 
     // ---- 1. conserved set: recent window + n_h largest scores (ties: lower index)
     uint32_t cut = 0;
@@ -379,8 +383,10 @@ __global__ void __launch_bounds__(NT) segment_unit_kernel(const float* __restric
     // the token index (last-index pivot of the average-weighted baseline) or the caller's key array.
     const float* pk = pivot_key ? pivot_key + (size_t)u * S : a;
     auto key_of = [&](int j) -> float {
-        return pivot_rule == KVM_PIVOT_LAST ? (float)j : (pivot_rule == KVM_PIVOT_KEY ? pk[j] : a[j]);
+        return pivot_rule == KVM_PIVOT_LAST ? (float)j : fmaxf(pivot_rule == KVM_PIVOT_KEY ? pk[j] : a[j], -FLT_MAX);
     };
+    // (A key that is NaN or -inf counts as the smallest number, so that every set has a pivot among its tokens whatever
+    // the inputs hold.)
     // Per thread: `head` = best of the tokens before the first cut in its range
     // (they belong to a set that started earlier), `run` = best since its last cut.
     Best head = {-INFINITY, INT_MAX}, run = {-INFINITY, INT_MAX};
@@ -543,7 +549,7 @@ __device__ __forceinline__ void radix_select_reg(const uint32_t (&key)[EM], unsi
 }
 
 template <int EM>
-__global__ void __launch_bounds__(NT) segment_unit_reg_kernel(const float* __restrict__ scores,
+__global__ void __launch_bounds__(NT, 1) segment_unit_reg_kernel(float* __restrict__ scores, const ScorePart parts,
                                                               const float* __restrict__ sim,
                                                               int32_t* __restrict__ set_id,
                                                               int32_t* __restrict__ set_start,
@@ -567,7 +573,14 @@ __global__ void __launch_bounds__(NT) segment_unit_reg_kernel(const float* __res
     uint32_t ka[EM];
     const size_t g0 = (size_t)u * S + lo;          // this thread's first token in the [U, S] arrays
     const bool vec = EM == 4 && n == 4 && (g0 & 3) == 0;   // four tokens on a 16-byte boundary: one access per array
-    if (vec) {
+    if (parts.part) {
+#pragma unroll
+        for (int t = 0; t < EM; ++t) {
+            a[t] = (t < n) ? plan::column_sum(parts.part, parts.plan, S, u, lo + t) : 0.f;
+            c[t] = (t < n) ? sim[g0 + t] : 0.f;
+            if (t < n) scores[g0 + t] = a[t];
+        }
+    } else if (vec) {
         const float4 av = *reinterpret_cast<const float4*>(scores + g0), cv = *reinterpret_cast<const float4*>(sim + g0);
         a[0] = av.x; a[1] = av.y; a[2] = av.z; a[3] = av.w;
         c[0] = cv.x; c[1] = cv.y; c[2] = cv.z; c[3] = cv.w;
@@ -712,6 +725,7 @@ __global__ void __launch_bounds__(NT) segment_unit_reg_kernel(const float* __res
         key[t] = a[t];
         if (pivot_rule == KVM_PIVOT_LAST) key[t] = (float)(lo + t);
         else if (pivot_rule == KVM_PIVOT_KEY && t < n) key[t] = pivot_key[g0 + t];
+        key[t] = fmaxf(key[t], -FLT_MAX);      // (NaN or -inf: the smallest number, see above)
     }
     Best head = {-INFINITY, INT_MAX}, run = {-INFINITY, INT_MAX};
     bool seen_cut = false;
@@ -801,7 +815,7 @@ cudaError_t launch_set_ratio(const Dims& d, const float* sim, float* ratio, cuda
     return cudaGetLastError();
 }
 
-cudaError_t launch_segment(const Dims& d, const float* scores, const float* sim, int32_t* set_id,
+cudaError_t launch_segment(const Dims& d, float* scores, const ScorePart& parts, const float* sim, int32_t* set_id,
                            int32_t* set_start, int32_t* pivot, int32_t* out_len, kvm_stats* stats, cudaStream_t st) {
     // flags [S] bytes; the anchor reading adds two uint16 jump arrays
     const size_t smem = d.set_rule == KVM_SETS_ANCHOR ? (size_t)((d.S + 15) & ~15) + 4 * (size_t)d.S : (size_t)d.S;
@@ -811,10 +825,10 @@ cudaError_t launch_segment(const Dims& d, const float* scores, const float* sim,
         if (e != cudaSuccess) return e;
     }
     if (d.set_rule == KVM_SETS_ADJACENT && d.S <= 4 * NT)
-        return launch_dependent(segment_unit_reg_kernel<4>, dim3(d.U), dim3(NT), 0, st, scores, sim, set_id, set_start,
+        return launch_dependent(segment_unit_reg_kernel<4>, dim3(d.U), dim3(NT), 0, st, scores, parts, sim, set_id, set_start,
                                 pivot, out_len, stats, d.S, d.cap, d.n_r, d.n_h, d.eps, d.enforce, d.pivot_rule,
                                 d.pivot_rule == KVM_PIVOT_KEY ? d.pivot_key : (const float*)nullptr);
-    return launch_dependent(segment_unit_kernel, dim3(d.U), dim3(NT), smem, st, scores, sim, set_id, set_start, pivot,
+    return launch_dependent(segment_unit_kernel, dim3(d.U), dim3(NT), smem, st, scores, parts, sim, set_id, set_start, pivot,
                             out_len, stats, d.S, d.cap, d.n_r, d.n_h, d.eps, d.enforce, d.pivot_rule,
                             d.pivot_rule == KVM_PIVOT_KEY ? d.pivot_key : (const float*)nullptr, d.set_rule);
 }
