@@ -507,24 +507,22 @@ cudaError_t launch_t(const Dims& d, const Plan& plan, const CUtensorMap& mq, con
                      const float* lse_in, char* scratch, float* scores, kvm_stats* stats, cudaStream_t st,
                      const __nv_bfloat16* Ksim, float* sim_out, float* lse_out, ScorePart* parts) {
     const size_t smem = 1024 + (size_t)(2 + NSTAGE) * KCH * TILE * 128 + (size_t)(NSTAGE + 1) * PTILE_BYTES + sizeof(Shared);
-    // the shared-memory opt-in and the SM count are looked up once per device and kernel instantiation
+    // the shared-memory opt-in is made once per device and kernel instantiation
     static std::mutex mu;
-    static int sms_of[KVM_MAX_DEVICES] = {};
+    static bool done[KVM_MAX_DEVICES] = {};
     cudaError_t e;
-    int dev = 0, sms = 0;
+    int dev = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if (dev < 0 || dev >= KVM_MAX_DEVICES) return cudaErrorInvalidDevice;
     {
         std::lock_guard<std::mutex> lock(mu);
-        if (!sms_of[dev]) {
+        if (!done[dev]) {
             e = cudaFuncSetAttribute(score_tc_kernel<KCH, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
             e = cudaFuncSetAttribute(score_tc_kernel<KCH, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
-            if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-            sms_of[dev] = sms;
+            done[dev] = true;
         }
-        sms = sms_of[dev];
     }
     const Scratch sc = layout(d, plan);
     __nv_bfloat16* side = reinterpret_cast<__nv_bfloat16*>(scratch);
@@ -535,7 +533,7 @@ cudaError_t launch_t(const Dims& d, const Plan& plan, const CUtensorMap& mq, con
     const dim3 row_blocks((unsigned)((rows + 255) / 256));
     auto grid = [&](int split, int heads) {
         const long long items = (long long)heads * plan.T;
-        return dim3(split ? plan.grid_split() : (unsigned)(items < sms ? items : sms));
+        return dim3(split ? plan.grid_split() : (unsigned)(items < plan::CTAS ? items : plan::CTAS));
     };
     if (!lse_in) {
         // (the kernels wait for what precedes them by themselves, so each is scheduled while that drains)
