@@ -102,14 +102,11 @@ __device__ __forceinline__ bool take_share(Work& w, Item& it, ShareSmem& sh) {
     return true;
 }
 
-// Piece end: the warps' states (sm_m, sm_l, sm_acc [warp][GH][D]) in a fixed order -> the piece's state of `heads` heads;
-// and, from the block that holds the item's first row, how many pieces it has.
+// Piece end: the warps' states (sm_m, sm_l, sm_acc [warp][GH][D]) in a fixed order -> the piece's state of `heads` heads at
+// dst: per head D weighted sums, the maximum and the sum.
 template <int D, int GH>
-__device__ __forceinline__ void store_piece(const Work& w, const Item& it, const float (*sm_m)[GH], const float (*sm_l)[GH],
-                                            const float* sm_acc, bool bad, float* part, int32_t* pieces, int max_pieces,
-                                            int heads, int stride) {
-    const int first = (int)(it.start / w.q);
-    float* dst = part + ((size_t)it.id * max_pieces + (blockIdx.x - first)) * stride * (D + 2);
+__device__ __forceinline__ void store_piece(const float (*sm_m)[GH], const float (*sm_l)[GH], const float* sm_acc, bool bad,
+                                            float* dst, int heads) {
     for (int i = threadIdx.x; i < heads * D; i += ATT_WARPS * 32) {
         const int h = i / D;
         float M = -INFINITY, L = 0.f, o = 0.f;
@@ -124,16 +121,70 @@ __device__ __forceinline__ void store_piece(const Work& w, const Item& it, const
         dst[h * (D + 2) + i % D] = bad ? NAN : o;
         if (i % D == 0) { dst[h * (D + 2) + D] = M; dst[h * (D + 2) + D + 1] = L; }
     }
+}
+// Where a piece's state goes; the block that holds the item's first row also tells how many pieces the item has.
+__device__ __forceinline__ float* piece_slot(const Work& w, const Item& it, float* part, int32_t* pieces, int max_pieces,
+                                             int state_floats) {
+    const int first = (int)(it.start / w.q);
     if (threadIdx.x == 0 && (int)blockIdx.x == first) pieces[it.id] = (int)((it.start + it.n - 1) / w.q) - first + 1;
+    return part + ((size_t)it.id * max_pieces + (blockIdx.x - first)) * state_floats;
+}
+
+// ------------------------------------------------------------------ short caches: a cluster per item
+// Where an item's rows divided over a few blocks take about as long as an equal share, the blocks of an item are a
+// thread-block cluster: each takes a slice of the item's rows and the states are joined through distributed shared
+// memory, without a second kernel (32 heads x 1536 rows on average: 12.0 us with one, of which its launch and three
+// dependent reads are 5).
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
+}
+__device__ __forceinline__ float peer_load(uint32_t addr, uint32_t rank) {
+    float v;
+    asm volatile("{\n\t.reg .b32 a;\n\tmapa.shared::cluster.u32 a, %1, %2;\n\tld.shared::cluster.f32 %0, [a];\n\t}"
+                 : "=f"(v) : "r"(addr), "r"(rank) : "memory");
+    return v;
+}
+// This block's slice as a share of its own, and an empty state to start from.
+template <int D, int GH>
+__device__ __forceinline__ void take_slice(Work& w, Item& it, int C, float* fin) {
+    for (int i = threadIdx.x; i < GH * (D + 2); i += ATT_NT) fin[i] = i % (D + 2) == D ? -INFINITY : 0.f;
+    it.start = 0;
+    it.id = blockIdx.x / C;
+    it.n = w.rows_of(it.id);
+    const int per = ((it.n + C - 1) / C + 15) & ~15, off = min(it.n, (int)(blockIdx.x % C) * per);
+    w.q = 1;
+    w.f = off;
+    w.f_end = min(it.n, off + per);
+    __syncthreads();
+}
+// Joins the cluster's states (fin, [head][D + 2]) in order of rank; every block stores a part of the item's heads.
+template <int D>
+__device__ __forceinline__ void join_cluster(const float* fin, int item, int HG, int GH, int G, int C, float* out) {
+    cluster_barrier();
+    const int u = item / HG, h0 = (item % HG) * GH, heads = min(G - h0, GH);
+    const uint32_t base = smem_u32(fin);
+    for (int i = (int)(blockIdx.x % C) * ATT_NT + threadIdx.x; i < heads * D; i += C * ATT_NT) {
+        const uint32_t at = base + (uint32_t)(i / D) * (D + 2) * 4u;
+        float M = -INFINITY, L = 0.f, o = 0.f;
+        for (int s = 0; s < C; ++s) {
+            const float ms = peer_load(at + D * 4u, s), ls = peer_load(at + (D + 1) * 4u, s), os = peer_load(at + (i % D) * 4u, s);
+            const float mn = fmaxf(M, ms), a = rescale(M, mn), c = rescale(ms, mn);
+            L = fmaf(ls, c, L * a);
+            o = fmaf(os, c, o * a);
+            M = mn;
+        }
+        out[((size_t)u * G + h0 + i / D) * D + i % D] = L > 0.f || L != L || o != o ? o / L : 0.f;   // (an empty cache attends to nothing)
+    }
+    cluster_barrier();          // (shared memory stays until every peer has read it)
 }
 
 // part: per item and piece, for each of the GH heads D weighted sums, the maximum and the sum (log2 units); pieces:
 // per item, how many there are.
-template <typename T, int D, int GH>
+template <typename T, int D, int GH, bool CL>
 __global__ void __launch_bounds__(ATT_NT, 1)
 attend_partial_fma_kernel(const T* __restrict__ q, const T* __restrict__ K, const T* __restrict__ V,
                       const int32_t* __restrict__ len, float* __restrict__ part, int32_t* __restrict__ pieces, int rows, int G,
-                      int U, int max_pieces, float scale_log2e) {
+                      int U, int max_pieces, float scale_log2e, int C, float* __restrict__ out) {
     constexpr int N = Vec<T>::N, LPR = D / N, GPW = 32 / LPR;      // elements per 16 bytes, lanes per row, groups per warp
     constexpr int SROWS = ATT_STAGE_BYTES / (D * (int)sizeof(T));  // rows per stage
     static_assert(SROWS == ATT_WARPS * GPW * RPI, "a stage is one round of every group");
@@ -143,6 +194,7 @@ attend_partial_fma_kernel(const T* __restrict__ q, const T* __restrict__ K, cons
     extern __shared__ __align__(128) uint8_t smem[];
     uint8_t* ring = smem;                                          // [stage][K | V][SROWS][D]
     float* sm_acc = reinterpret_cast<float*>(smem + ATT_STAGES * 2 * ATT_STAGE_BYTES);   // [warp][GH][D]
+    float* fin = sm_acc + ATT_WARPS * GH * D;                      // [GH][D + 2]: this block's state (clusters)
     __shared__ __align__(8) uint64_t full[ATT_STAGES], empty[ATT_STAGES];
     __shared__ float sm_m[ATT_WARPS][GH], sm_l[ATT_WARPS][GH];
     __shared__ ShareSmem sh;
@@ -161,7 +213,9 @@ attend_partial_fma_kernel(const T* __restrict__ q, const T* __restrict__ K, cons
     }
     grid_dependency_wait();
     Item it;
-    if (!take_share(w, it, sh)) return;
+    if (CL) take_slice<D, GH>(w, it, C, fin);
+    else if (!take_share(w, it, sh)) return;
+    const int item = it.id;
 
     if (warp == ATT_WARPS) {
         // ---- copies
@@ -185,7 +239,8 @@ attend_partial_fma_kernel(const T* __restrict__ q, const T* __restrict__ K, cons
                 w.f += it.cnt;
             }
         }
-        return;
+        if (!CL) return;
+        __syncwarp();
     }
     // ---- arithmetic
     const int lane = wl % LPR, g = wl / LPR;                       // lane within the row, group within the warp
@@ -193,7 +248,7 @@ attend_partial_fma_kernel(const T* __restrict__ q, const T* __restrict__ K, cons
     const int rl = (lane / REP) % RL;                              // ... for rows rl * CNT .. + CNT of the group's four
     const int lb = g * LPR;                                        // the group's first lane
     uint32_t k = 0;
-    while (w.settle(it)) {
+    while (warp != ATT_WARPS && w.settle(it)) {
         const int u = it.id / w.HG, h0 = (it.id % w.HG) * GH;
         uint64_t qp[GH][N / 2], acc[GH][N / 2];
 #pragma unroll
@@ -312,10 +367,11 @@ attend_partial_fma_kernel(const T* __restrict__ q, const T* __restrict__ K, cons
             }
         }
         named_bar(1, ATT_WARPS * 32);
-        store_piece<D, GH>(w, it, sm_m, sm_l, sm_acc, s_bad != 0, part, pieces, max_pieces, GH, GH);
+        store_piece<D, GH>(sm_m, sm_l, sm_acc, s_bad != 0, CL ? fin : piece_slot(w, it, part, pieces, max_pieces, GH * (D + 2)), GH);
         named_bar(1, ATT_WARPS * 32);
         w.f += it.cnt;
     }
+    if (CL) join_cluster<D>(fin, item, w.HG, GH, G, C, out);
 }
 
 // ------------------------------------------------------------------ bf16 caches: the same on warp-level matrix products
@@ -348,11 +404,11 @@ __device__ __forceinline__ uint32_t transpose8x8(uint32_t x) {
 
 constexpr int MMA_GH = 8;                   // query heads of a product
 
-template <int D>
+template <int D, bool CL>
 __global__ void __launch_bounds__(ATT_NT, 1)
 attend_partial_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                           const __nv_bfloat16* __restrict__ q, const int32_t* __restrict__ len, float* __restrict__ part,
-                          int32_t* __restrict__ pieces, int rows, int G, int U, int max_pieces, float scale_log2e) {
+                          int32_t* __restrict__ pieces, int rows, int G, int U, int max_pieces, float scale_log2e, int C, float* __restrict__ out) {
     constexpr int KCH = D / 64;                                    // 64-channel (128-byte) column chunks
     constexpr int SROWS = ATT_STAGE_BYTES / (D * 2);               // rows per stage (64 or 128)
     constexpr int CHUNK = SROWS * 128;                             // bytes of a column chunk of a stage
@@ -362,6 +418,7 @@ attend_partial_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* ring = smem_raw + (base - smem_u32(smem_raw));        // [stage][K | V][KCH][SROWS][128 B]
     float* sm_acc = reinterpret_cast<float*>(ring + ATT_STAGES * 2 * ATT_STAGE_BYTES);   // [warp][MMA_GH][D]
+    float* fin = sm_acc + ATT_WARPS * MMA_GH * D;                  // [MMA_GH][D + 2]: this block's state (clusters)
     __shared__ __align__(8) uint64_t full[ATT_STAGES], empty[ATT_STAGES];
     __shared__ float sm_m[ATT_WARPS][MMA_GH], sm_l[ATT_WARPS][MMA_GH];
     __shared__ ShareSmem sh;
@@ -381,7 +438,9 @@ attend_partial_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
     }
     grid_dependency_wait();
     Item it;
-    if (!take_share(w, it, sh)) return;
+    if (CL) take_slice<D, MMA_GH>(w, it, C, fin);
+    else if (!take_share(w, it, sh)) return;
+    const int item = it.id;
 
     if (warp == ATT_WARPS) {
         // ---- copies (a stage's rows past the piece are rows of the next pieces, or zeros past the tensor: masked)
@@ -405,7 +464,8 @@ attend_partial_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
                 w.f += it.cnt;
             }
         }
-        return;
+        if (!CL) return;
+        __syncwarp();
     }
     // ---- arithmetic.  gid, tig: row and column pair of this lane in the 8x8 fragments
     const int gid = wl >> 2, tig = wl & 3, blk = warp % NB;
@@ -414,7 +474,7 @@ attend_partial_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
     const int krow = blk * 16 + (wl & 15), kpc = wl >> 4;
     const int vrow = blk * 16 + (wl & 7) + ((wl >> 4) << 3), vpc = (wl >> 3) & 1;
     uint32_t k = 0;
-    while (w.settle(it)) {
+    while (warp != ATT_WARPS && w.settle(it)) {
         const int u = it.id / w.HG, h0 = (it.id % w.HG) * MMA_GH, heads = min(G - h0, MMA_GH);
         uint32_t qf[D / 16][2];                                    // q^T as B fragments: channels 2 tig.. (+8), head gid
 #pragma unroll
@@ -516,10 +576,12 @@ attend_partial_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
             for (int e = 0; e < 4; ++e)
                 if (2 * tig + (e & 1) < heads) sm_acc[(warp * MMA_GH + 2 * tig + (e & 1)) * D + dt * 16 + gid + (e >> 1) * 8] = o[dt][e];
         named_bar(1, ATT_WARPS * 32);
-        store_piece<D, MMA_GH>(w, it, sm_m, sm_l, sm_acc, s_bad != 0, part, pieces, max_pieces, heads, stride);
+        store_piece<D, MMA_GH>(sm_m, sm_l, sm_acc, s_bad != 0,
+                               CL ? fin : piece_slot(w, it, part, pieces, max_pieces, stride * (D + 2)), heads);
         named_bar(1, ATT_WARPS * 32);
         w.f += it.cnt;
     }
+    if (CL) join_cluster<D>(fin, item, w.HG, MMA_GH, G, C, out);
 }
 
 // One block per query head: its pieces' states in order.
@@ -602,39 +664,62 @@ cudaError_t prepare_kernel(void (*kernel)(KArgs...), int smem, int (&sms_of)[KVM
 struct Scratch {
     int items, gh, mp;
     int32_t* pieces;
-    float* states;
+    float *states, *out;
     unsigned grid(int sms, int rows) const {
         const long long most = ((long long)items * rows + ATT_MIN_SHARE - 1) / ATT_MIN_SHARE;
         return (unsigned)(most < sms ? most : sms);
     }
+    // Blocks of an item's cluster, 0: equal shares and a second kernel.  The estimates (us): a slice of the longest item
+    // through one SM at 65 bytes/ns, or at its part of 6.5 TB/s when many are at work; an equal share of the rows
+    // (lengths are three quarters of the capacity on average), 5 us of a second kernel and 0.2 us per piece it joins.
+    // Measured: 32 units x 1536 rows x 128 in bf16 8.4 (cluster) / 12.8 (shares), 4 x 16384 18.0 / 22.3, 64 x 16384
+    // 70.0 / 64.4, 1 x 32768 24.4 / 40.3.
+    int cluster(int sms, int rows, int row_bytes) const {
+        if (items > sms) return 0;
+        int C = 1;
+        while (C < 8 && items * C * 2 <= sms) C *= 2;
+        const double rate = 6500.0 / (items * C), slice = (double)((rows + C - 1) / C) * row_bytes / (rate < 65.0 ? rate : 65.0);
+        const double share = 0.75 * items * rows * row_bytes / 6500.0 + 5e3 + 2e2 * (1 + sms / items);
+        return slice <= share ? C : 0;
+    }
 };
+
+// One of a kernel's two forms on the stream.
+template <typename KC, typename KS, typename... Args>
+cudaError_t launch_form(KC clustered, KS shares, const Scratch& sc, int smem, int rows, int row_bytes, std::mutex& mu,
+                        int (&sms_of)[2][KVM_MAX_DEVICES], cudaStream_t st, bool& joined, Args... args) {
+    int sms = 0;
+    cudaError_t e = prepare_kernel(shares, smem, sms_of[0], mu, sms);
+    if (e == cudaSuccess) e = prepare_kernel(clustered, smem, sms_of[1], mu, sms);
+    if (e != cudaSuccess) return e;
+    const int C = sc.cluster(sms, rows, row_bytes);
+    joined = C > 0;
+    if (!joined) return launch_dependent(shares, dim3(sc.grid(sms, rows)), dim3(ATT_NT), smem, st, args..., 0, sc.out);
+    return launch_dependent_cluster(clustered, dim3(sc.items * C), dim3(ATT_NT), smem, C, st, args..., C, sc.out);
+}
 
 template <typename T, int D, int GH>
 cudaError_t launch_fma(const Dims& d, const void* q, const void* K, const void* V, int rows, const int32_t* len,
-                       const Scratch& sc, cudaStream_t st) {
-    constexpr int smem = ATT_STAGES * 2 * ATT_STAGE_BYTES + ATT_WARPS * GH * D * (int)sizeof(float);
+                       const Scratch& sc, cudaStream_t st, bool& joined) {
+    constexpr int smem = ATT_STAGES * 2 * ATT_STAGE_BYTES + (ATT_WARPS * D + D + 2) * GH * (int)sizeof(float);
     static std::mutex mu;
-    static int sms_of[KVM_MAX_DEVICES] = {};
-    int sms = 0;
-    const cudaError_t e = prepare_kernel(attend_partial_fma_kernel<T, D, GH>, smem, sms_of, mu, sms);
-    if (e != cudaSuccess) return e;
-    return launch_dependent(attend_partial_fma_kernel<T, D, GH>, dim3(sc.grid(sms, rows)), dim3(ATT_NT), smem, st, (const T*)q,
-                            (const T*)K, (const T*)V, len, sc.states, sc.pieces, rows, d.G, d.U, sc.mp, d.scale * LOG2E);
+    static int sms_of[2][KVM_MAX_DEVICES] = {};
+    return launch_form(attend_partial_fma_kernel<T, D, GH, true>, attend_partial_fma_kernel<T, D, GH, false>, sc, smem, rows,
+                       2 * D * (int)sizeof(T), mu, sms_of, st, joined, (const T*)q, (const T*)K, (const T*)V, len, sc.states,
+                       sc.pieces, rows, d.G, d.U, sc.mp, d.scale * LOG2E);
 }
 template <int D>
 cudaError_t launch_mma(const Dims& d, const void* q, const void* K, const void* V, int rows, const int32_t* len,
-                       const Scratch& sc, cudaStream_t st) {
-    constexpr int smem = 1024 + ATT_STAGES * 2 * ATT_STAGE_BYTES + ATT_WARPS * MMA_GH * D * (int)sizeof(float);
+                       const Scratch& sc, cudaStream_t st, bool& joined) {
+    constexpr int smem = 1024 + ATT_STAGES * 2 * ATT_STAGE_BYTES + (ATT_WARPS * D + D + 2) * MMA_GH * (int)sizeof(float);
     static std::mutex mu;
-    static int sms_of[KVM_MAX_DEVICES] = {};
-    int sms = 0;
-    const cudaError_t e = prepare_kernel(attend_partial_mma_kernel<D>, smem, sms_of, mu, sms);
-    if (e != cudaSuccess) return e;
+    static int sms_of[2][KVM_MAX_DEVICES] = {};
     CUtensorMap mk, mv;
     if (!make_map(&mk, K, d.U, rows, D, ATT_STAGE_BYTES / (2 * D)) || !make_map(&mv, V, d.U, rows, D, ATT_STAGE_BYTES / (2 * D)))
         return cudaErrorNotSupported;
-    return launch_dependent(attend_partial_mma_kernel<D>, dim3(sc.grid(sms, rows)), dim3(ATT_NT), smem, st, mk, mv,
-                            (const __nv_bfloat16*)q, len, sc.states, sc.pieces, rows, d.G, d.U, sc.mp, d.scale * LOG2E);
+    return launch_form(attend_partial_mma_kernel<D, true>, attend_partial_mma_kernel<D, false>, sc, smem, rows, 4 * D, mu, sms_of,
+                       st, joined, mk, mv, (const __nv_bfloat16*)q, len, sc.states, sc.pieces, rows, d.G, d.U, sc.mp,
+                       d.scale * LOG2E);
 }
 
 template <int D>
@@ -646,13 +731,15 @@ cudaError_t launch_t(const Dims& d, const void* q, const void* K, const void* V,
     sc.mp = most_pieces(rows);
     sc.pieces = reinterpret_cast<int32_t*>(part);
     sc.states = part + (sc.items + 3) / 4 * 4;
+    sc.out = out;
     auto fn = d.dtype == KVM_BF16 ? launch_mma<D>
               : sc.gh == 1        ? launch_fma<float, D, 1>
               : sc.gh == 2        ? launch_fma<float, D, 2>
               : sc.gh == 4        ? launch_fma<float, D, 4>
                                   : launch_fma<float, D, 8>;
-    const cudaError_t e = fn(d, q, K, V, rows, len, sc, st);
-    if (e != cudaSuccess) return e;
+    bool joined = false;
+    const cudaError_t e = fn(d, q, K, V, rows, len, sc, st, joined);
+    if (e != cudaSuccess || joined) return e;
     return launch_dependent(attend_combine_kernel<D>, dim3(d.B * d.Hq), dim3(D), 0, st, (const float*)sc.states,
                             (const int32_t*)sc.pieces, len, out, rows, d.G, sc.gh, sc.mp);
 }
