@@ -21,6 +21,24 @@ struct Dims {
     const float* pivot_key;                  // [U,S] when pivot_rule == KVM_PIVOT_KEY
 };
 
+// The tensors of up to MAX_LAYERS layers of one shape that go through the kernels together, as one problem of n times the
+// batch; everything between them (scores, similarities, sets) lies in the workspace, layer after layer.
+constexpr int MAX_LAYERS = 8;
+struct Layers {
+    int n, U, H;                                   // layers; units and query heads of one layer
+    const void *Q[MAX_LAYERS], *K[MAX_LAYERS], *V[MAX_LAYERS];
+    void *K_out[MAX_LAYERS], *V_out[MAX_LAYERS];
+    int32_t *out_len[MAX_LAYERS], *pivot[MAX_LAYERS];
+    float eps[MAX_LAYERS];
+};
+// The layer of unit u, which becomes the unit's index within the layer.
+__device__ __forceinline__ int layer_of(const Layers& L, long long& u) {
+    if (L.n == 1) return 0;
+    const int l = (int)u / L.U;
+    u -= (long long)l * L.U;
+    return l;
+}
+
 // 16-byte vector <-> fp32 lanes.  Vec<T>::N elements of T per 16 bytes.
 template <typename T> struct Vec;
 template <> struct Vec<float> {
@@ -104,25 +122,23 @@ cudaError_t launch_score_f32(const Dims& d, const void* Q, const void* K, const 
                              float* lse_out = nullptr);
 size_t score_f32_scratch_bytes(const Dims& d);
 struct ScorePart;             // partial column sums left for the segment kernel (score_plan.cuh)
-cudaError_t launch_score_tc(const Dims& d, const void* Q, const void* K, const float* lse_in, void* scratch,
+cudaError_t launch_score_tc(const Dims& d, const Layers& L, const float* lse_in, void* scratch,
                             float* scores, kvm_stats* stats, cudaStream_t st, float* sim_out = nullptr,
                             float* lse_out = nullptr, ScorePart* parts = nullptr);
 size_t score_tc_scratch_bytes(const Dims& d);
 cudaError_t launch_prefill_attend(const Dims& d, const void* Q, const void* K, const void* V, void* O, float* lse,
                                   kvm_stats* stats, cudaStream_t st);
 cudaError_t launch_similarity(const Dims& d, const void* K, float* sim, cudaStream_t st);
-cudaError_t launch_segment(const Dims& d, float* scores, const ScorePart& parts, const float* sim, int32_t* set_id,
-                           int32_t* set_start, int32_t* pivot, int32_t* out_len, kvm_stats* stats, cudaStream_t st);
+cudaError_t launch_segment(const Dims& d, const Layers& L, float* scores, const ScorePart& parts, const float* sim,
+                           int32_t* set_id, int32_t* set_start, kvm_stats* stats, cudaStream_t st);
 size_t segment_max_smem();
 cudaError_t launch_anchor_runs(const Dims& d, const void* K, float* run_out, float* inv_norm, cudaStream_t st);
 cudaError_t launch_set_ratio(const Dims& d, const float* sim, float* ratio, cudaStream_t st);
 size_t merge_scratch_floats(const Dims& d);
 cudaError_t launch_token_sets(const Dims& d, const int32_t* set_start, const int32_t* out_len, int32_t* set_id,
                               cudaStream_t st);
-cudaError_t launch_merge(const Dims& d, const void* K, const void* V, const int32_t* set_start,
-                         const int32_t* pivot, const int32_t* set_id, const int32_t* out_len, void* K_out,
-                         void* V_out, int32_t* out_size, float* scratch, float* set_coef, float* token_d2,
-                         kvm_stats* stats, cudaStream_t st);
+cudaError_t launch_merge(const Dims& d, const Layers& L, const int32_t* set_start, const int32_t* set_id, int32_t* out_size,
+                         float* scratch, float* set_coef, float* token_d2, kvm_stats* stats, cudaStream_t st);
 // Rows that are one input state each (pivot-only weights, eviction): a gather.
 cudaError_t launch_gather(const Dims& d, const void* K, const void* V, const int32_t* set_start,
                           const int32_t* pivot, const int32_t* out_len, void* K_out, void* V_out, int32_t* out_size,

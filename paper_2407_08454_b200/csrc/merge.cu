@@ -66,11 +66,9 @@ template <int D> struct Slots {
 enum : int { PIECE_COPY = 0, PIECE_WHOLE = 1, PIECE_HEAD = 2, PIECE_TAIL = 3 };
 
 template <typename T, int D, int TOK>
-__global__ void __launch_bounds__(2 * D) merge_tile_kernel(const T* __restrict__ K, const T* __restrict__ V,
+__global__ void __launch_bounds__(2 * D) merge_tile_kernel(const __grid_constant__ Layers L,
                                                            const int32_t* __restrict__ set_start,
-                                                           const int32_t* __restrict__ pivot,
                                                            const int32_t* __restrict__ set_id,
-                                                           T* __restrict__ K_out, T* __restrict__ V_out,
                                                            int32_t* __restrict__ out_size, Slots<D> slots, int S,
                                                            int cap, float neg_inv_2s2_log2e, int scale_v, int average,
                                                            const float* __restrict__ set_coef, kvm_stats* stats) {
@@ -92,8 +90,10 @@ __global__ void __launch_bounds__(2 * D) merge_tile_kernel(const T* __restrict__
     const int tok0 = tile * TOK;
     const int ntok = min(TOK, S - tok0);
     const int tile_end = tok0 + ntok;
-    const T* Ku = K + (size_t)u * S * D;
-    const T* Vu = V + (size_t)u * S * D;
+    long long lu = u;                                // the unit within its layer
+    const int layer = layer_of(L, lu);
+    const T* Ku = static_cast<const T*>(L.K[layer]) + (size_t)lu * S * D;
+    const T* Vu = static_cast<const T*>(L.V[layer]) + (size_t)lu * S * D;
     const int32_t* st = set_start + (size_t)u * (cap + 1);
     const uint32_t bytes = (uint32_t)ntok * D * sizeof(T);
 
@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(2 * D) merge_tile_kernel(const T* __restrict__
                 end = __ldcg(st + sid + 1);
                 s_sid[j] = sid;
                 s_len[j] = end - beg;
-                s_piv[j] = __ldcg(pivot + (size_t)u * cap + sid);
+                s_piv[j] = __ldcg(L.pivot[layer] + (size_t)lu * cap + sid);
                 s_coef[j] = set_coef ? __ldcg(set_coef + (size_t)u * cap + sid) : neg_inv_2s2_log2e;
             }
             if (j < 64) {                                     // warps 0 and 1: a piece starts where the set changes
@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(2 * D) merge_tile_kernel(const T* __restrict__
             const int which = (TPASS == 2) ? tp : gl / LPR;
             const int ch = (gl % LPR) * N;
             const uint4* sX4 = reinterpret_cast<const uint4*>(which ? sV : sK) + (gl % LPR);   // rows of LPR 16-byte pieces
-            uint4* out4 = reinterpret_cast<uint4*>((which ? V_out : K_out) + (size_t)u * cap * D) + (gl % LPR);
+            uint4* out4 = reinterpret_cast<uint4*>(static_cast<T*>(which ? L.V_out[layer] : L.K_out[layer]) + (size_t)lu * cap * D) + (gl % LPR);
             for (int k = wk; k < np; k += NWK) {
                 const int a = s_pbeg[k], b = s_pbeg[k + 1], kind = s_pkind[k], row = s_prow[k];
                 if (kind == PIECE_COPY) {
@@ -256,10 +256,9 @@ __global__ void __launch_bounds__(2 * D) merge_tile_kernel(const T* __restrict__
 
 // Sets that cross a tile boundary: the block of the LAST boundary a set crosses adds its slots in tile order.
 template <typename T, int D, int TOK>
-__global__ void __launch_bounds__(2 * D) merge_fixup_kernel(const int32_t* __restrict__ set_start,
-                                                            const int32_t* __restrict__ set_id,
-                                                            T* __restrict__ K_out, T* __restrict__ V_out,
-                                                            int32_t* __restrict__ out_size, Slots<D> slots, int S,
+__global__ void __launch_bounds__(2 * D) merge_fixup_kernel(const __grid_constant__ Layers L,
+                                                            const int32_t* __restrict__ set_start,
+                                                            const int32_t* __restrict__ set_id, int32_t* __restrict__ out_size, Slots<D> slots, int S,
                                                             int cap, int Tn, int scale_v) {
     // The sets were written before the tile kernel began (it triggers this launch only after it has waited for
     // them), so they can be looked up while that kernel's last blocks still run; they are read through L2.
@@ -284,8 +283,10 @@ __global__ void __launch_bounds__(2 * D) merge_fixup_kernel(const int32_t* __res
     }
     const int which = threadIdx.x / D, ch = threadIdx.x % D;
     const int n = end - beg;
-    T* out = which ? V_out : K_out;
-    out[((size_t)u * cap + sid) * D + ch] = f32_to_elem<T>(which && scale_v ? acc * ((float)n / gs) : acc / gs);
+    long long lu = u;
+    const int layer = layer_of(L, lu);
+    T* out = static_cast<T*>(which ? L.V_out[layer] : L.K_out[layer]);
+    out[((size_t)lu * cap + sid) * D + ch] = f32_to_elem<T>(which && scale_v ? acc * ((float)n / gs) : acc / gs);
     if (out_size && threadIdx.x == 0) out_size[(size_t)u * cap + sid] = n;
 }
 
@@ -379,8 +380,7 @@ cudaError_t launch_gather_t(const Dims& d, const void* K, const void* V, const i
 }
 
 template <typename T, int D, int TOK>
-cudaError_t launch_t(const Dims& d, const void* K, const void* V, const int32_t* set_start, const int32_t* pivot,
-                     const int32_t* set_id, const int32_t* out_len, void* K_out, void* V_out, int32_t* out_size,
+cudaError_t launch_t(const Dims& d, const Layers& L, const int32_t* set_start, const int32_t* set_id, int32_t* out_size,
                      float* scratch, float* set_coef, float* token_d2, kvm_stats* stats, cudaStream_t st) {
     const int Tn = (d.S + TOK - 1) / TOK;
     Slots<D> slots;
@@ -390,24 +390,23 @@ cudaError_t launch_t(const Dims& d, const void* K, const void* V, const int32_t*
     cudaError_t e = cudaSuccess;
     const float c = -LOG2E / (2.f * d.sigma * d.sigma);
     const bool per_set = d.weight_rule == KVM_WEIGHT_SET_SIGMA;
-    if (per_set) {
+    if (per_set) {                                   // (one layer at a time)
         const long long rows = (long long)d.U * d.S;
         const unsigned blocks = (unsigned)((rows * (D / Vec<T>::N) + 255) / 256);
-        e = launch_dependent(token_dist_kernel<T, D>, dim3(blocks), dim3(256), 0, st, (const T*)K, set_id, pivot,
-                             token_d2, d.S, d.cap, rows);
+        e = launch_dependent(token_dist_kernel<T, D>, dim3(blocks), dim3(256), 0, st, (const T*)L.K[0], set_id,
+                             (const int32_t*)L.pivot[0], token_d2, d.S, d.cap, rows);
         if (e != cudaSuccess) return e;
         e = launch_dependent(set_coef_kernel, dim3((d.cap + 7) / 8, d.U), dim3(256), 0, st, (const float*)token_d2,
-                             set_start, out_len, set_coef, d.S, d.cap);
+                             set_start, (const int32_t*)L.out_len[0], set_coef, d.S, d.cap);
         if (e != cudaSuccess) return e;
     }
-    e = launch_dependent(merge_tile_kernel<T, D, TOK>, dim3(Tn, d.U), dim3(2 * D), smem, st, (const T*)K,
-                         (const T*)V, set_start, pivot, set_id, (T*)K_out, (T*)V_out, out_size, slots, d.S, d.cap, c,
-                         d.scale_v, d.weight_rule == KVM_WEIGHT_AVERAGE ? 1 : 0,
+    e = launch_dependent(merge_tile_kernel<T, D, TOK>, dim3(Tn, d.U), dim3(2 * D), smem, st, L, set_start, set_id, out_size,
+                         slots, d.S, d.cap, c, d.scale_v, d.weight_rule == KVM_WEIGHT_AVERAGE ? 1 : 0,
                          per_set ? (const float*)set_coef : (const float*)nullptr, stats);
     if (e != cudaSuccess) return e;
     if (Tn > 1)
-        e = launch_dependent(merge_fixup_kernel<T, D, TOK>, dim3(Tn - 1, d.U), dim3(2 * D), 0, st, set_start, set_id,
-                             (T*)K_out, (T*)V_out, out_size, slots, d.S, d.cap, Tn, d.scale_v);
+        e = launch_dependent(merge_fixup_kernel<T, D, TOK>, dim3(Tn - 1, d.U), dim3(2 * D), 0, st, L, set_start, set_id,
+                             out_size, slots, d.S, d.cap, Tn, d.scale_v);
     return e;
 }
 
@@ -443,21 +442,13 @@ cudaError_t launch_gather(const Dims& d, const void* K, const void* V, const int
                       : launch_gather_t<float, 64>(d, K, V, set_start, pivot, out_len, K_out, V_out, out_size, st);
 }
 
-// set_coef [U, cap] and token_d2 [U, S]: fp32 scratch, used only by the per-set bandwidth rule; out_len: device [U].
-cudaError_t launch_merge(const Dims& d, const void* K, const void* V, const int32_t* set_start,
-                         const int32_t* pivot, const int32_t* set_id, const int32_t* out_len, void* K_out,
-                         void* V_out, int32_t* out_size, float* scratch, float* set_coef, float* token_d2,
-                         kvm_stats* stats, cudaStream_t st) {
-    if (d.dtype == KVM_BF16) {
-        return d.D == 128 ? launch_t<__nv_bfloat16, 128, KVM_MERGE_TOK_BF16>(d, K, V, set_start, pivot, set_id, out_len,
-                                                                          K_out, V_out, out_size, scratch, set_coef, token_d2, stats, st)
-                          : launch_t<__nv_bfloat16, 64, KVM_MERGE_TOK_BF16>(d, K, V, set_start, pivot, set_id, out_len,
-                                                                         K_out, V_out, out_size, scratch, set_coef, token_d2, stats, st);
-    }
-    return d.D == 128 ? launch_t<float, 128, 32>(d, K, V, set_start, pivot, set_id, out_len, K_out, V_out, out_size,
-                                                 scratch, set_coef, token_d2, stats, st)
-                      : launch_t<float, 64, 32>(d, K, V, set_start, pivot, set_id, out_len, K_out, V_out, out_size,
-                                                scratch, set_coef, token_d2, stats, st);
+// set_coef [U, cap] and token_d2 [U, S]: fp32 scratch, used only by the per-set bandwidth rule.
+cudaError_t launch_merge(const Dims& d, const Layers& L, const int32_t* set_start, const int32_t* set_id, int32_t* out_size,
+                         float* scratch, float* set_coef, float* token_d2, kvm_stats* stats, cudaStream_t st) {
+    auto fn = d.dtype == KVM_BF16
+                  ? (d.D == 128 ? launch_t<__nv_bfloat16, 128, KVM_MERGE_TOK_BF16> : launch_t<__nv_bfloat16, 64, KVM_MERGE_TOK_BF16>)
+                  : (d.D == 128 ? launch_t<float, 128, 32> : launch_t<float, 64, 32>);
+    return fn(d, L, set_start, set_id, out_size, scratch, set_coef, token_d2, stats, st);
 }
 
 }  // namespace kvm

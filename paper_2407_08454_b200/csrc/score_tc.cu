@@ -144,14 +144,21 @@ __device__ __forceinline__ void store_side(__nv_bfloat16* dst_row, float e) {
     dst[1] = make_uint4(0u, 0u, 0u, 0u);
 }
 
+// Tensor maps of the layers' queries and keys, the keys themselves, and the map of the side tensor (which lies in the
+// workspace: one for all layers); units and query heads of a layer.
+struct Maps {
+    CUtensorMap q[MAX_LAYERS], k[MAX_LAYERS], side;
+    const __nv_bfloat16* keys[MAX_LAYERS];
+    int n, U, H;
+};
+
 // out: the column pass's scores [U,S], or its partial sums [piece][U,S] when items are cut; states: the row pass's
 // partial (maximum, sum) per piece and row when items are cut, else it writes the side tensor.
 template <int KCH, int PASS>
 __global__ void __launch_bounds__(NTHREADS, 1)
-score_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
-                const __grid_constant__ CUtensorMap map_p, __nv_bfloat16* __restrict__ lsep_out, float2* __restrict__ states,
+score_tc_kernel(const __grid_constant__ Maps maps, __nv_bfloat16* __restrict__ lsep_out, float2* __restrict__ states,
                 float* __restrict__ out, kvm_stats* stats, const Plan plan, int Hq, int Hkv, int S, float scale2,
-                const __nv_bfloat16* __restrict__ Ksim, float* __restrict__ sim_out) {
+                float* __restrict__ sim_out) {
     constexpr int pass = PASS;
     extern __shared__ uint8_t smem_raw[];
     constexpr uint32_t CHUNK_BYTES = TILE * 128;            // one [128 rows x 64 bf16] TMA box
@@ -198,8 +205,6 @@ score_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     if (warp == NEPI_WARPS) {
         // ============================== producer ==============================
         if (lane == 0) {
-            const CUtensorMap* mapA = (pass == 1) ? &map_q : &map_k;
-            const CUtensorMap* mapB = (pass == 1) ? &map_k : &map_q;
             uint32_t cnt = 0;
             bool ok = true;
             int last_a[2] = {-1, -1}, last_b[NSTAGE];      // parity of the last load issued per buffer (-1: none)
@@ -209,12 +214,16 @@ score_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                 ok = mbar_wait(&sh.bar.empty_a[ab], ((n >> 1) & 1) ^ 1, abort_flag);
                 if (!ok) break;
                 last_a[ab] = (n >> 1) & 1;
+                const int per_layer = (pass == 1) ? maps.H : maps.U, layer = maps.n > 1 ? w.head / per_layer : 0;
+                const int head = w.head - layer * per_layer;             // within its layer
+                const CUtensorMap* mapA = (pass == 1) ? &maps.q[layer] : &maps.k[layer];
+                const CUtensorMap* mapB = (pass == 1) ? &maps.k[layer] : &maps.q[layer];
                 mbar_expect_tx(&sh.bar.full_a[ab], TILE_BYTES);
 #pragma unroll
                 for (int kc = 0; kc < KCH; ++kc)
                     tma_load_3d(sA + ab * TILE_BYTES + kc * CHUNK_BYTES, mapA, &sh.bar.full_a[ab], kc * KCHUNK,
-                                w.tile * TILE, w.head);
-                const int b = w.head / (pass == 1 ? Hq : Hkv), hh = w.head % (pass == 1 ? Hq : Hkv), per = T - w.tile;
+                                w.tile * TILE, head);
+                const int b = head / (pass == 1 ? Hq : Hkv), hh = head % (pass == 1 ? Hq : Hkv), per = T - w.tile;
                 int bhead = (pass == 1) ? b * Hkv + hh / G : b * Hq + hh * G + w.i0 / per;   // B tile cursor, advanced incrementally
                 int btile = (pass == 1) ? w.i0 : w.tile + w.i0 % per;
                 for (int t = 0; t < w.n; ++t, ++cnt) {
@@ -229,7 +238,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
 #pragma unroll
                     for (int kc = 0; kc < KCH; ++kc)
                         tma_load_3d(sB + s * TILE_BYTES + kc * CHUNK_BYTES, mapB, &sh.bar.full_b[s], kc * KCHUNK, btile * TILE, bhead);
-                    if (pass == 2) tma_load_3d(sP + s * PTILE_BYTES, &map_p, &sh.bar.full_b[s], 0, btile * TILE, bhead);
+                    if (pass == 2) tma_load_3d(sP + s * PTILE_BYTES, &maps.side, &sh.bar.full_b[s], 0, btile * TILE, layer * maps.H + bhead);
                     if (++btile == T && pass == 2) { btile = w.tile; ++bhead; }   // next query head of the group
                 }
             }
@@ -295,9 +304,9 @@ score_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             const unsigned stride = gridDim.x * NSIM_WARPS * GPW;
             for (unsigned g = (blockIdx.x * NSIM_WARPS + (warp - NEPI_WARPS - 2)) * GPW + lane / LPR;
                  g < n_runs; g += stride) {
-                const unsigned u = g / (unsigned)runs;
+                const unsigned u = g / (unsigned)runs, layer = maps.n > 1 ? u / (unsigned)maps.U : 0u;
                 const int j0 = (int)(g - u * (unsigned)runs) * SIM_RUN;
-                simcore::run<__nv_bfloat16, D, SIM_RUN>(Ksim + (size_t)u * S * D, sim_out + (size_t)u * S, j0,
+                simcore::run<__nv_bfloat16, D, SIM_RUN>(maps.keys[layer] + (size_t)(u - layer * maps.U) * S * D, sim_out + (size_t)u * S, j0,
                                                         min(j0 + SIM_RUN, S), gl, gbase, gmask);
             }
         }
@@ -503,9 +512,8 @@ Scratch layout(const Dims& d, const Plan& p) {
 }
 
 template <int KCH>
-cudaError_t launch_t(const Dims& d, const Plan& plan, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mp,
-                     const float* lse_in, char* scratch, float* scores, kvm_stats* stats, cudaStream_t st,
-                     const __nv_bfloat16* Ksim, float* sim_out, float* lse_out, ScorePart* parts) {
+cudaError_t launch_t(const Dims& d, const Plan& plan, const Maps& maps, const float* lse_in, char* scratch, float* scores,
+                     kvm_stats* stats, cudaStream_t st, float* sim_out, float* lse_out, ScorePart* parts) {
     const size_t smem = 1024 + (size_t)(2 + NSTAGE) * KCH * TILE * 128 + (size_t)(NSTAGE + 1) * PTILE_BYTES + sizeof(Shared);
     // the shared-memory opt-in is made once per device and kernel instantiation
     static std::mutex mu;
@@ -537,8 +545,8 @@ cudaError_t launch_t(const Dims& d, const Plan& plan, const CUtensorMap& mq, con
     };
     if (!lse_in) {
         // (the kernels wait for what precedes them by themselves, so each is scheduled while that drains)
-        e = launch_dependent(score_tc_kernel<KCH, 1>, grid(plan.split_row, plan.NH), dim3(NTHREADS), smem, st, mq, mk, mp, side,
-                             states, (float*)nullptr, stats, plan, d.Hq, d.Hkv, d.S, scale2, Ksim,
+        e = launch_dependent(score_tc_kernel<KCH, 1>, grid(plan.split_row, plan.NH), dim3(NTHREADS), smem, st, maps, side,
+                             states, (float*)nullptr, stats, plan, d.Hq, d.Hkv, d.S, scale2,
                              scores ? (float*)nullptr : sim_out);
         if (e == cudaSuccess && plan.split_row)
             e = launch_dependent(join_rows_kernel, row_blocks, dim3(256), 0, st, (const float2*)states, side, lse_out, plan, d.S, scale2);
@@ -549,9 +557,9 @@ cudaError_t launch_t(const Dims& d, const Plan& plan, const CUtensorMap& mq, con
         e = launch_dependent(lse_split_kernel, row_blocks, dim3(256), 0, st, lse_in, side, rows, -LOG2E / scale2);
     }
     if (e != cudaSuccess || !scores) return e;        // (row pass only)
-    e = launch_dependent(score_tc_kernel<KCH, 2>, grid(plan.split_col, plan.U), dim3(NTHREADS), smem, st, mq, mk, mp,
+    e = launch_dependent(score_tc_kernel<KCH, 2>, grid(plan.split_col, plan.U), dim3(NTHREADS), smem, st, maps,
                          (__nv_bfloat16*)nullptr, (float2*)nullptr, plan.split_col ? part : scores, stats, plan, d.Hq, d.Hkv,
-                         d.S, scale2, Ksim, sim_out);
+                         d.S, scale2, sim_out);
     if (e != cudaSuccess || !plan.split_col) return e;
     if (parts) {                                      // the caller's next kernel adds the pieces up
         parts->part = part;
@@ -576,18 +584,20 @@ size_t score_tc_scratch_bytes(const Dims& d) {
 // TMEM lane quarters, which then lag the others, and an accumulator goes back when its slowest warp is done.)
 // scores may be NULL (row pass only); lse_out (nullable) receives the natural-log row log-sum-exp [B,Hq,S].
 // parts (nullable): lets the column pass leave partial sums (parts->part set) for the caller's next kernel to add.
-cudaError_t launch_score_tc(const Dims& d, const void* Q, const void* K, const float* lse_in, void* scratch,
-                            float* scores, kvm_stats* stats, cudaStream_t st, float* sim_out, float* lse_out,
-                            ScorePart* parts) {
-    CUtensorMap mq, mk, mp;
+// d: the layers together (a batch of n times a layer's).
+cudaError_t launch_score_tc(const Dims& d, const Layers& L, const float* lse_in, void* scratch, float* scores, kvm_stats* stats,
+                            cudaStream_t st, float* sim_out, float* lse_out, ScorePart* parts) {
+    Maps maps;
     Plan plan;
     if (!make_plan(d, plan)) return cudaErrorInvalidValue;
-    if (!make_map(&mq, Q, d.B * d.Hq, d.S, d.D) || !make_map(&mk, K, d.B * d.Hkv, d.S, d.D) ||
-        !make_map_side(&mp, scratch, d.B * d.Hq, d.S))
-        return cudaErrorNotSupported;
-    const __nv_bfloat16* Ks = reinterpret_cast<const __nv_bfloat16*>(K);
+    maps.n = L.n; maps.U = L.U; maps.H = L.H;
+    for (int l = 0; l < L.n; ++l) {
+        if (!make_map(&maps.q[l], L.Q[l], L.H, d.S, d.D) || !make_map(&maps.k[l], L.K[l], L.U, d.S, d.D)) return cudaErrorNotSupported;
+        maps.keys[l] = reinterpret_cast<const __nv_bfloat16*>(L.K[l]);
+    }
+    if (!make_map_side(&maps.side, scratch, d.B * d.Hq, d.S)) return cudaErrorNotSupported;
     auto fn = d.D == 128 ? launch_t<2> : launch_t<1>;
-    return fn(d, plan, mq, mk, mp, lse_in, (char*)scratch, scores, stats, st, Ks, sim_out, lse_out, parts);
+    return fn(d, plan, maps, lse_in, (char*)scratch, scores, stats, st, sim_out, lse_out, parts);
 }
 
 }  // namespace kvm

@@ -187,10 +187,9 @@ __device__ __forceinline__ void record_out_len(kvm_stats* stats, int n) {
 // (scores: where `parts` holds partial sums the kernel adds them up and writes the scores itself)
 __global__ void __launch_bounds__(NT, 1) segment_unit_kernel(float* __restrict__ scores, const ScorePart parts,
                                                           const float* __restrict__ sim, int32_t* __restrict__ set_id,
-                                                          int32_t* __restrict__ set_start, int32_t* __restrict__ pivot,
-                                                          int32_t* __restrict__ out_len, kvm_stats* stats, int S,
-                                                          int cap, int n_r, int n_h, float eps, int enforce,
-                                                          int pivot_rule, const float* __restrict__ pivot_key,
+                                                          int32_t* __restrict__ set_start,
+                                                          const __grid_constant__ Layers L, kvm_stats* stats, int S,
+                                                          int cap, int n_r, int n_h, int enforce, int pivot_rule, const float* __restrict__ pivot_key,
                                                           int set_rule) {
     extern __shared__ __align__(16) uint8_t flags[];  // [S] (+ jump arrays for the anchor reading)
     __shared__ Shared sh;
@@ -199,6 +198,10 @@ __global__ void __launch_bounds__(NT, 1) segment_unit_kernel(float* __restrict__
     grid_launch_dependents();
     grid_dependency_wait();     // scores and similarities come from the kernels before this one
     const int u = blockIdx.x;
+    long long lu = u;                              // the unit within its layer
+    const int layer = layer_of(L, lu);
+    const float eps = L.eps[layer];
+    int32_t* pv = L.pivot[layer] + (size_t)lu * cap;
     const float* a = scores + (size_t)u * S;
     const float* c = sim + (size_t)u * S;
     const int E = (S + NT - 1) / NT;               // tokens per thread, contiguous
@@ -241,7 +244,6 @@ __global__ void __launch_bounds__(NT, 1) segment_unit_kernel(float* __restrict__
     __syncthreads();
 
     int32_t* st = set_start + (size_t)u * (cap + 1);
-    int32_t* pv = pivot + (size_t)u * cap;
 
     // ---- eviction (Section 2.2): the conserved tokens are the output, one state each
     if (set_rule == KVM_SETS_CONSERVED_ONLY) {
@@ -257,7 +259,7 @@ __global__ void __launch_bounds__(NT, 1) segment_unit_kernel(float* __restrict__
         }
         if (threadIdx.x == 0) {
             if (n_keep <= cap) st[n_keep] = S;
-            out_len[u] = n_keep;
+            L.out_len[layer][lu] = n_keep;
             if (stats) {
                 record_out_len(stats, n_keep);
             }
@@ -371,7 +373,7 @@ __global__ void __launch_bounds__(NT, 1) segment_unit_kernel(float* __restrict__
     }
     if (threadIdx.x == 0) {
         if (n_sets <= cap) st[n_sets] = S;
-        out_len[u] = n_sets;
+        L.out_len[layer][lu] = n_sets;
         if (stats) {
             if (fire) atomicAdd(&stats->units_budget_rule, 1);
             if (tot_near) atomicAdd(&stats->near_threshold, tot_near);
@@ -381,7 +383,7 @@ __global__ void __launch_bounds__(NT, 1) segment_unit_kernel(float* __restrict__
 
     // ---- 5. segmented arg-max: pivot of each set (ties: lowest index).  The key is the score (Eq. 6),
     // the token index (last-index pivot of the average-weighted baseline) or the caller's key array.
-    const float* pk = pivot_key ? pivot_key + (size_t)u * S : a;
+    const float* pk = pivot_key ? pivot_key + (size_t)lu * S : a;
     auto key_of = [&](int j) -> float {
         return pivot_rule == KVM_PIVOT_LAST ? (float)j : fmaxf(pivot_rule == KVM_PIVOT_KEY ? pk[j] : a[j], -FLT_MAX);
     };
@@ -553,14 +555,17 @@ __global__ void __launch_bounds__(NT, 1) segment_unit_reg_kernel(float* __restri
                                                               const float* __restrict__ sim,
                                                               int32_t* __restrict__ set_id,
                                                               int32_t* __restrict__ set_start,
-                                                              int32_t* __restrict__ pivot, int32_t* __restrict__ out_len,
-                                                              kvm_stats* stats, int S, int cap, int n_r, int n_h,
-                                                              float eps, int enforce, int pivot_rule,
+                                                              const __grid_constant__ Layers L, kvm_stats* stats, int S,
+                                                              int cap, int n_r, int n_h, int enforce, int pivot_rule,
                                                               const float* __restrict__ pivot_key) {
     __shared__ SharedReg sh;
     grid_launch_dependents();   // (as in segment_unit_kernel)
     grid_dependency_wait();
     const int u = blockIdx.x;
+    long long lu = u;                              // the unit within its layer
+    const int layer = layer_of(L, lu);
+    const float eps = L.eps[layer];
+    int32_t* pv = L.pivot[layer] + (size_t)lu * cap;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int E = (S + NT - 1) / NT;               // tokens per thread, contiguous; E <= EM
     const int lo = min(S, (int)threadIdx.x * E);
@@ -685,7 +690,6 @@ __global__ void __launch_bounds__(NT, 1) segment_unit_reg_kernel(float* __restri
 
     // ---- 4. scan of the cut flags -> set ids and starts
     int32_t* st = set_start + (size_t)u * (cap + 1);
-    int32_t* pv = pivot + (size_t)u * cap;
     int n_sets;
     const int before = block_exscan(__popc(cutm), n_sets, sh, 0);
     {
@@ -710,7 +714,7 @@ __global__ void __launch_bounds__(NT, 1) segment_unit_reg_kernel(float* __restri
     }
     if (threadIdx.x == 0) {
         if (n_sets <= cap) st[n_sets] = S;
-        out_len[u] = n_sets;
+        L.out_len[layer][lu] = n_sets;
         if (stats) {
             if (fire) atomicAdd(&stats->units_budget_rule, 1);
             if (tot_near) atomicAdd(&stats->near_threshold, tot_near);
@@ -724,7 +728,7 @@ __global__ void __launch_bounds__(NT, 1) segment_unit_reg_kernel(float* __restri
     for (int t = 0; t < EM; ++t) {
         key[t] = a[t];
         if (pivot_rule == KVM_PIVOT_LAST) key[t] = (float)(lo + t);
-        else if (pivot_rule == KVM_PIVOT_KEY && t < n) key[t] = pivot_key[g0 + t];
+        else if (pivot_rule == KVM_PIVOT_KEY && t < n) key[t] = pivot_key[(size_t)lu * S + lo + t];
         key[t] = fmaxf(key[t], -FLT_MAX);      // (NaN or -inf: the smallest number, see above)
     }
     Best head = {-INFINITY, INT_MAX}, run = {-INFINITY, INT_MAX};
@@ -815,8 +819,8 @@ cudaError_t launch_set_ratio(const Dims& d, const float* sim, float* ratio, cuda
     return cudaGetLastError();
 }
 
-cudaError_t launch_segment(const Dims& d, float* scores, const ScorePart& parts, const float* sim, int32_t* set_id,
-                           int32_t* set_start, int32_t* pivot, int32_t* out_len, kvm_stats* stats, cudaStream_t st) {
+cudaError_t launch_segment(const Dims& d, const Layers& L, float* scores, const ScorePart& parts, const float* sim,
+                           int32_t* set_id, int32_t* set_start, kvm_stats* stats, cudaStream_t st) {
     // flags [S] bytes; the anchor reading adds two uint16 jump arrays
     const size_t smem = d.set_rule == KVM_SETS_ANCHOR ? (size_t)((d.S + 15) & ~15) + 4 * (size_t)d.S : (size_t)d.S;
     if (smem > 40 * 1024) {   // more dynamic shared memory than the default limit: opt in (cheap, idempotent)
@@ -825,11 +829,11 @@ cudaError_t launch_segment(const Dims& d, float* scores, const ScorePart& parts,
         if (e != cudaSuccess) return e;
     }
     if (d.set_rule == KVM_SETS_ADJACENT && d.S <= 4 * NT)
-        return launch_dependent(segment_unit_reg_kernel<4>, dim3(d.U), dim3(NT), 0, st, scores, parts, sim, set_id, set_start,
-                                pivot, out_len, stats, d.S, d.cap, d.n_r, d.n_h, d.eps, d.enforce, d.pivot_rule,
+        return launch_dependent(segment_unit_reg_kernel<4>, dim3(d.U), dim3(NT), 0, st, scores, parts, sim, set_id, set_start, L,
+                                stats, d.S, d.cap, d.n_r, d.n_h, d.enforce, d.pivot_rule,
                                 d.pivot_rule == KVM_PIVOT_KEY ? d.pivot_key : (const float*)nullptr);
-    return launch_dependent(segment_unit_kernel, dim3(d.U), dim3(NT), smem, st, scores, parts, sim, set_id, set_start, pivot,
-                            out_len, stats, d.S, d.cap, d.n_r, d.n_h, d.eps, d.enforce, d.pivot_rule,
+    return launch_dependent(segment_unit_kernel, dim3(d.U), dim3(NT), smem, st, scores, parts, sim, set_id, set_start, L, stats, d.S,
+                            d.cap, d.n_r, d.n_h, d.enforce, d.pivot_rule,
                             d.pivot_rule == KVM_PIVOT_KEY ? d.pivot_key : (const float*)nullptr, d.set_rule);
 }
 
