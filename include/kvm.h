@@ -250,7 +250,9 @@ int kvm_layer_ratio(const kvm_params* p, const void* K, float* ratio, float* sim
  * A stack of layers with one similarity threshold each (Section 3.2: the layer-wise compression ratios can be set
  * by adjusting the threshold layer by layer): n_layers calls of kvm_compress, layer l with sim_threshold =
  * sim_thresholds[l] (p->sim_threshold for all layers when sim_thresholds is NULL), enqueued one after the other on
- * the stream; the workspace is shared, the layers' tensors are not.
+ * the stream; the workspace is shared, the layers' tensors are not.  Short layers go through the kernels several at a
+ * time where the workspace has room for it: kvm_layers_workspace_bytes tells how much lets them (the size for one layer
+ * is always enough).
  *   Q, K, V, K_out, V_out, out_len, out_pos: HOST arrays of n_layers device pointers, each as in kvm_compress
  *   sim_thresholds: NULL or a HOST array of n_layers floats (read before the call returns)
  *   stats: NULL or one device kvm_stats that accumulates over the layers
@@ -260,6 +262,7 @@ int kvm_compress_layers(const kvm_params* p, int32_t n_layers, const float* sim_
                         const void* const* K, const void* const* V, void* const* K_out, void* const* V_out,
                         int32_t* const* out_len, int32_t* const* out_pos, kvm_stats* stats, void* ws,
                         size_t ws_bytes, void* cuda_stream);
+int kvm_layers_workspace_bytes(const kvm_params* p, int32_t n_layers, size_t* bytes);   /* Host only. */
 
 /*
  * Causal attention over the whole prompt (Eq. 1 for every position: O_i = softmax_{j<=i}(q_i K^T * scale) V), the

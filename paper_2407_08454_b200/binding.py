@@ -24,7 +24,7 @@ KVM_WEIGHT_GAUSSIAN, KVM_WEIGHT_AVERAGE, KVM_WEIGHT_PIVOT_ONLY, KVM_WEIGHT_SET_S
 KVM_SETS_ADJACENT, KVM_SETS_CONSERVED_ONLY, KVM_SETS_ANCHOR = 0, 1, 2
 EXPORTS = (
     "kvm_sizes", "kvm_workspace_bytes", "kvm_score", "kvm_row_lse", "kvm_segment", "kvm_merge_compact", "kvm_compress",
-    "kvm_compress_with_lse", "kvm_compress_layers",
+    "kvm_compress_with_lse", "kvm_compress_layers", "kvm_layers_workspace_bytes",
     "kvm_host_staging_bytes", "kvm_compress_host", "kvm_score_static", "kvm_layer_ratio", "kvm_attend",
     "kvm_output_perturbation", "kvm_prefill_attend", "kvm_status_string",
     "kvm_version",
@@ -83,6 +83,7 @@ _ARGTYPES = {
     "kvm_compress": (_PARAMS,) + (_P,) * 10 + (_Z, _P),
     "kvm_compress_with_lse": (_PARAMS,) + (_P,) * 11 + (_Z, _P),
     "kvm_compress_layers": (_PARAMS, _I) + (_P,) * 10 + (_Z, _P),
+    "kvm_layers_workspace_bytes": (_PARAMS, _I, ctypes.POINTER(_Z)),
     "kvm_compress_host": (_PARAMS,) + (_P,) * 8 + (_Z, _P),
 }
 
@@ -172,6 +173,12 @@ def kvm_sizes(p: KvmParams):
 def kvm_workspace_bytes(p: KvmParams) -> int:
     n = ctypes.c_size_t()
     _call("kvm_workspace_bytes", p, n)
+    return n.value
+
+
+def kvm_layers_workspace_bytes(p: KvmParams, n_layers: int) -> int:
+    n = ctypes.c_size_t()
+    _call("kvm_layers_workspace_bytes", p, n_layers, n)
     return n.value
 
 
@@ -293,7 +300,7 @@ def compress_layers(p: KvmParams, layers, sim_thresholds=None, device="cuda", st
     B, H, cap, D = p.batch, p.n_kv_heads, kvm_sizes(p)[0], p.head_dim
     dt = torch.bfloat16 if p.dtype == KVM_BF16 else torch.float32
     # one allocation per kind for the whole stack (each layer's tensors are views of it) and one zero fill
-    ws = torch.empty(kvm_workspace_bytes(p), dtype=torch.uint8, device=device)
+    ws = torch.empty(kvm_layers_workspace_bytes(p, n), dtype=torch.uint8, device=device)
     kv = torch.zeros(2, n, B, H, cap, D, dtype=dt, device=device)
     ints = torch.zeros(n * B * H * (cap + 1), dtype=torch.int32, device=device)
     out_len, out_pos = ints[:n * B * H].view(n, B, H), ints[n * B * H:].view(n, B, H, cap)

@@ -103,14 +103,59 @@ int check_ws(const Dims& d, void* ws, size_t ws_bytes, Workspace& w) {
     return KVM_OK;
 }
 
+// One layer's tensors as the kernels take them.
+Layers one_layer(const Dims& d, const void* Q, const void* K, const void* V = nullptr, void* K_out = nullptr,
+                 void* V_out = nullptr, int32_t* out_len = nullptr, int32_t* pivot = nullptr) {
+    Layers L = {};
+    L.n = 1; L.U = d.U; L.H = d.B * d.Hq;
+    L.Q[0] = Q; L.K[0] = K; L.V[0] = V; L.K_out[0] = K_out; L.V_out[0] = V_out;
+    L.out_len[0] = out_len; L.pivot[0] = pivot; L.eps[0] = d.eps;
+    return L;
+}
+
 // sim_out (nullable): where the neighbour-key similarities are wanted, which the score step produces on the side.
-cudaError_t run_score(const Dims& d, const void* Q, const void* K, const float* lse_in, float* scores,
-                      const Workspace& w, kvm_stats* stats, cudaStream_t st, float* sim_out = nullptr,
-                      ScorePart* parts = nullptr) {
+cudaError_t run_score(const Dims& d, const Layers& L, const float* lse_in, float* scores, const Workspace& w,
+                      kvm_stats* stats, cudaStream_t st, float* sim_out = nullptr, ScorePart* parts = nullptr) {
     // fp32 tensors enter the tensor cores as exact sums of three bf16 planes: rounding them would not hold the
     // score tolerance
-    return d.dtype == KVM_BF16 ? launch_score_tc(d, Q, K, lse_in, w.lse, scores, stats, st, sim_out, nullptr, parts)
-                               : launch_score_f32(d, Q, K, lse_in, w.lse, scores, stats, st, sim_out);
+    return d.dtype == KVM_BF16 ? launch_score_tc(d, L, lse_in, w.lse, scores, stats, st, sim_out, nullptr, parts)
+                               : launch_score_f32(d, L.Q[0], L.K[0], lse_in, w.lse, scores, stats, st, sim_out);
+}
+
+// The whole chain over the layers in L (d: the layers together, a batch of n times a layer's).
+int run_chain(const Dims& d, const Layers& L, const float* lse_in, float* scores, const Workspace& w, kvm_stats* stats,
+              cudaStream_t st) {
+    const bool want_sim = d.set_rule == KVM_SETS_ADJACENT;
+    ScorePart parts;
+    if (run_score(d, L, lse_in, scores, w, stats, st, want_sim ? w.sim : nullptr, &parts) != cudaSuccess) return KVM_E_CUDA;
+    if (d.set_rule == KVM_SETS_ANCHOR)
+        if (launch_anchor_runs(d, L.K[0], w.sim, (float*)w.set_id, st) != cudaSuccess) return KVM_E_CUDA;
+    if (launch_segment(d, L, scores, parts, w.sim, w.set_id, w.set_start, stats, st) != cudaSuccess) return KVM_E_CUDA;
+    const cudaError_t e =
+        d.weight_rule == KVM_WEIGHT_PIVOT_ONLY
+            ? launch_gather(d, L.K[0], L.V[0], w.set_start, L.pivot[0], L.out_len[0], L.K_out[0], L.V_out[0], nullptr, st)
+            : launch_merge(d, L, w.set_start, w.set_id, nullptr, w.merge_part, w.sim, w.scores, stats, st);
+    return e == cudaSuccess ? KVM_OK : KVM_E_CUDA;
+}
+
+// How many layers of a stack go through the kernels together.  A layer whose score pass gives a CTA few steps loses most
+// of its time to the launches, the passes' start and drain and the last, half-empty round (32 query / 8 KV heads x 2048
+// tokens, about 30 steps per CTA: 78 us a layer); together the layers share them.  From about 300 steps on there is
+// nothing left to share.  The variants beside the method, and fp32 tensors, run layer by layer.
+int layers_together(const Dims& d, int n_layers) {
+    if (d.dtype != KVM_BF16 || d.set_rule != KVM_SETS_ADJACENT ||
+        (d.weight_rule != KVM_WEIGHT_GAUSSIAN && d.weight_rule != KVM_WEIGHT_AVERAGE))
+        return 1;
+    const long long T = (d.S + 127) / 128, steps = (long long)d.B * d.Hq * T * (T + 1) / 2 / 148 + 1;
+    long long n = 300 / steps;
+    if (n > (long long)(65535 / (d.B * d.Hq))) n = 65535 / (d.B * d.Hq);      // (grid dimensions)
+    if (n > n_layers) n = n_layers;
+    return (int)(n < 1 ? 1 : n > MAX_LAYERS ? MAX_LAYERS : n);
+}
+Dims times_batch(Dims d, int n) {
+    d.B *= n;
+    d.U *= n;
+    return d;
 }
 
 }  // namespace
@@ -168,7 +213,7 @@ int kvm_score(const kvm_params* p, const void* Q, const void* K, const float* ls
     if (misaligned(Q) || misaligned(K) || misaligned(scores) || (lse_in && misaligned(lse_in))) return KVM_E_ALIGN;
     Workspace w;
     if ((rc = check_ws(d, ws, ws_bytes, w)) != KVM_OK) return rc;
-    return run_score(d, Q, K, lse_in, scores, w, nullptr, (cudaStream_t)cuda_stream) == cudaSuccess ? KVM_OK
+    return run_score(d, one_layer(d, Q, K), lse_in, scores, w, nullptr, (cudaStream_t)cuda_stream) == cudaSuccess ? KVM_OK
                                                                                                     : KVM_E_CUDA;
 }
 
@@ -183,7 +228,7 @@ int kvm_row_lse(const kvm_params* p, const void* Q, const void* K, float* lse_ou
     if ((rc = check_ws(d, ws, ws_bytes, w)) != KVM_OK) return rc;
     cudaStream_t st = (cudaStream_t)cuda_stream;
     const cudaError_t e = d.dtype == KVM_BF16
-                              ? launch_score_tc(d, Q, K, nullptr, w.lse, nullptr, nullptr, st, nullptr, lse_out)
+                              ? launch_score_tc(d, one_layer(d, Q, K), nullptr, w.lse, nullptr, nullptr, st, nullptr, lse_out)
                               : launch_score_f32(d, Q, K, nullptr, w.lse, nullptr, nullptr, st, nullptr, lse_out);
     return e == cudaSuccess ? KVM_OK : KVM_E_CUDA;
 }
@@ -206,7 +251,8 @@ int kvm_segment(const kvm_params* p, const void* K, const float* scores, int32_t
     } else if (d.set_rule == KVM_SETS_ADJACENT || sim_out) {
         if (launch_similarity(d, K, sim, st) != cudaSuccess) return KVM_E_CUDA;
     }
-    if (launch_segment(d, const_cast<float*>(scores), ScorePart{}, sim, set_id, set_start, pivot, out_len, stats, st) != cudaSuccess)
+    if (launch_segment(d, one_layer(d, nullptr, K, nullptr, nullptr, nullptr, out_len, pivot), const_cast<float*>(scores), ScorePart{},
+                       sim, set_id, set_start, stats, st) != cudaSuccess)
         return KVM_E_CUDA;
     return KVM_OK;
 }
@@ -288,9 +334,8 @@ int kvm_merge_compact(const kvm_params* p, const void* K, const void* V, const i
                    : KVM_E_CUDA;
     if (launch_token_sets(d, set_start, out_len, w.set_id, st) != cudaSuccess) return KVM_E_CUDA;
     // (the similarity and score regions of the workspace are free here: scratch for the per-set bandwidths)
-    return launch_merge(d, K, V, set_start, pivot, w.set_id, out_len, K_out, V_out, out_size, w.merge_part, w.sim,
-                        w.scores, nullptr, st) ==
-                   cudaSuccess
+    const Layers L = one_layer(d, nullptr, K, V, K_out, V_out, const_cast<int32_t*>(out_len), const_cast<int32_t*>(pivot));
+    return launch_merge(d, L, set_start, w.set_id, out_size, w.merge_part, w.sim, w.scores, nullptr, st) == cudaSuccess
                ? KVM_OK
                : KVM_E_CUDA;
 }
@@ -315,22 +360,21 @@ int kvm_compress_with_lse(const kvm_params* p, const void* Q, const void* K, con
     Workspace w;
     if ((rc = check_ws(d, ws, ws_bytes, w)) != KVM_OK) return rc;
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    float* scores = scores_out ? scores_out : w.scores;
-    const bool want_sim = d.set_rule == KVM_SETS_ADJACENT;
-    ScorePart parts;
-    if (run_score(d, Q, K, lse_in, scores, w, stats, st, want_sim ? w.sim : nullptr, &parts) != cudaSuccess) return KVM_E_CUDA;
-    if (d.set_rule == KVM_SETS_ANCHOR)
-        if (launch_anchor_runs(d, K, w.sim, (float*)w.set_id, st) != cudaSuccess) return KVM_E_CUDA;
-    if (launch_segment(d, scores, parts, w.sim, w.set_id, w.set_start, out_pos, out_len, stats, st) != cudaSuccess)
-        return KVM_E_CUDA;
-    if (d.weight_rule == KVM_WEIGHT_PIVOT_ONLY)
-        return launch_gather(d, K, V, w.set_start, out_pos, out_len, K_out, V_out, nullptr, st) == cudaSuccess
-                   ? KVM_OK
-                   : KVM_E_CUDA;
-    if (launch_merge(d, K, V, w.set_start, out_pos, w.set_id, out_len, K_out, V_out, nullptr, w.merge_part, w.sim,
-                     w.scores, stats, st) !=
-        cudaSuccess)
-        return KVM_E_CUDA;
+    return run_chain(d, one_layer(d, Q, K, V, K_out, V_out, out_len, out_pos), lse_in, scores_out ? scores_out : w.scores, w,
+                     stats, st);
+}
+
+int kvm_layers_workspace_bytes(const kvm_params* p, int32_t n_layers, size_t* bytes) {
+    Dims d;
+    const int rc = derive(p, d);
+    if (rc != KVM_OK) return rc;
+    if (!bytes) return KVM_E_NULL;
+    if (n_layers < 1) return KVM_E_SHAPE;
+    *bytes = 0;
+    for (int n = 1; n <= layers_together(d, n_layers); ++n) {      // (a smaller last group may be split differently)
+        const size_t b = carve(times_batch(d, n), nullptr).bytes;
+        if (b > *bytes) *bytes = b;
+    }
     return KVM_OK;
 }
 
@@ -351,12 +395,23 @@ int kvm_compress_layers(const kvm_params* p, int32_t n_layers, const float* sim_
             return KVM_E_ALIGN;
         if (sim_thresholds && !isfinite(sim_thresholds[l])) return KVM_E_PARAM;
     }
-    for (int32_t l = 0; l < n_layers; ++l) {
-        kvm_params pl = *p;
-        if (sim_thresholds) pl.sim_threshold = sim_thresholds[l];
-        rc = kvm_compress(&pl, Q[l], K[l], V[l], K_out[l], V_out[l], out_len[l], out_pos[l], nullptr, stats, ws,
-                          ws_bytes, cuda_stream);
+    const int together = layers_together(d, n_layers);
+    for (int32_t l0 = 0; l0 < n_layers;) {
+        int n = n_layers - l0 < together ? n_layers - l0 : together;
+        while (n > 1 && carve(times_batch(d, n), nullptr).bytes > ws_bytes) --n;
+        Layers L = one_layer(d, nullptr, nullptr);
+        L.n = n;
+        for (int i = 0; i < n; ++i) {
+            L.Q[i] = Q[l0 + i]; L.K[i] = K[l0 + i]; L.V[i] = V[l0 + i];
+            L.K_out[i] = K_out[l0 + i]; L.V_out[i] = V_out[l0 + i];
+            L.out_len[i] = out_len[l0 + i]; L.pivot[i] = out_pos[l0 + i];
+            L.eps[i] = sim_thresholds ? sim_thresholds[l0 + i] : d.eps;
+        }
+        const Dims dn = times_batch(d, n);
+        const Workspace wn = carve(dn, ws);
+        rc = run_chain(dn, L, nullptr, wn.scores, wn, stats, (cudaStream_t)cuda_stream);
         if (rc != KVM_OK) return rc;
+        l0 += n;
     }
     return KVM_OK;
 }
@@ -552,7 +607,7 @@ int kvm_score_static(const kvm_params* p, const void* Q, const void* K, float* s
     w.merge_part = nullptr;
     w.attend_part = nullptr;
     w.bytes = sizeof(g_static_score_scratch);
-    return run_score(d, Q, K, nullptr, scores, w, nullptr, st) == cudaSuccess ? KVM_OK : KVM_E_CUDA;
+    return run_score(d, one_layer(d, Q, K), nullptr, scores, w, nullptr, st) == cudaSuccess ? KVM_OK : KVM_E_CUDA;
 }
 
 }  // extern "C"
