@@ -53,7 +53,7 @@ struct __align__(8) Bars {
     uint64_t q_full, q_empty;
     uint64_t k_full[NKV], k_empty[NKV], v_full[NKV], v_empty[NKV];
     uint64_t s_full[NGRP], s_empty[NGRP];
-    uint64_t p_full[NGRP], pv_done[NGRP], o_empty[NGRP];
+    uint64_t p_full[NGRP][2], pv_half[NGRP], pv_done[NGRP], o_empty[NGRP];   // P by halves of the key tile
     uint64_t part_full, part_empty;     // the handing group's row state at item end: written / read
 };
 struct alignas(16) Shared {
@@ -108,7 +108,8 @@ prefill_attend_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
         }
         for (int i = 0; i < NGRP; ++i) {
             mbar_init(&sh.bar.s_full[i], 1); mbar_init(&sh.bar.s_empty[i], 4);
-            mbar_init(&sh.bar.p_full[i], 4); mbar_init(&sh.bar.pv_done[i], 1);
+            for (int h = 0; h < 2; ++h) mbar_init(&sh.bar.p_full[i][h], 4);
+            mbar_init(&sh.bar.pv_half[i], 1); mbar_init(&sh.bar.pv_done[i], 1);
         }
         for (int i = 0; i < NGRP; ++i) mbar_init(&sh.bar.o_empty[i], 4);
         mbar_init(&sh.bar.part_full, 4); mbar_init(&sh.bar.part_empty, 4);
@@ -192,7 +193,7 @@ prefill_attend_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
             const uint64_t desc_q = smem_desc(base);
             const uint64_t desc_k0 = smem_desc(base + TILE_BYTES);
             uint32_t ks_cnt = 0;                             // K tiles consumed so far
-            uint32_t s_cnt[NGRP] = {0, 0};                   // per group: S tiles produced
+            uint32_t s_ph = 0;                               // bit g: parity of the S tiles produced for group g
             bool ok = true;
             int head, tile;
             for (int n = 0; ok && sc.item(n, head, tile); ++n) {
@@ -201,19 +202,20 @@ prefill_attend_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
                     const int g = (j + n) & 1;
                     const int s = ks_cnt % NKV;
                     ok = mbar_wait(&sh.bar.k_full[s], (ks_cnt / NKV) & 1, abort_flag) &&
-                         mbar_wait(&sh.bar.s_empty[g], (s_cnt[g] & 1) ^ 1, abort_flag);
+                         mbar_wait(&sh.bar.s_empty[g], ((s_ph >> g) & 1) ^ 1, abort_flag);
                     if (!ok) break;
                     tc_fence_after();
-                    const uint64_t dk = desc_k0 + (uint64_t)s * (TILE_BYTES >> 4);
+                    const uint32_t dk = (uint32_t)desc_k0 + s * (TILE_BYTES >> 4);
 #pragma unroll
                     for (int kc = 0; kc < KCH; ++kc)
 #pragma unroll
                         for (int ks = 0; ks < KCHUNK / 16; ++ks)
-                            umma_bf16(tmem_base + g * S_COLS, desc_q + ((kc * CHUNK_BYTES + ks * 32) >> 4),
-                                      dk + ((kc * CHUNK_BYTES + ks * 32) >> 4), IDESC_S, (kc | ks) ? 1u : 0u);
+                            umma_bf16_lo(tmem_base + g * S_COLS, (uint32_t)desc_q + ((kc * CHUNK_BYTES + ks * 32) >> 4),
+                                         (uint32_t)(desc_q >> 32), dk + ((kc * CHUNK_BYTES + ks * 32) >> 4),
+                                         (uint32_t)(desc_k0 >> 32), IDESC_S, (kc | ks) ? 1u : 0u);
                     umma_commit(&sh.bar.k_empty[s]);
                     umma_commit(&sh.bar.s_full[g]);
-                    ++ks_cnt; ++s_cnt[g];
+                    ++ks_cnt; s_ph ^= 1u << g;
                 }
                 if (ok) umma_commit(&sh.bar.q_empty);        // every product that reads this Q tile has been issued
             }
@@ -224,8 +226,10 @@ prefill_attend_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
             constexpr uint32_t IDESC_O = idesc_bf16(D, true);
             const uint32_t v_addr0 = base + TILE_BYTES + NKV * TILE_BYTES;
             const uint64_t desc_p0 = smem_desc(v_addr0 + NKV * TILE_BYTES);
+            const uint64_t desc_v0 = smem_desc_mn(v_addr0, CHUNK_BYTES);
+            const uint32_t dv_base = (uint32_t)desc_v0, v_hi = (uint32_t)(desc_v0 >> 32), p_hi = (uint32_t)(desc_p0 >> 32);
             uint32_t vs_cnt = 0;                             // V tiles consumed so far
-            uint32_t pv_cnt[NGRP] = {0, 0};                  // per group: P V products issued
+            uint32_t pv_ph = 0;                              // bit g: parity of the P V products issued for group g
             bool ok = true;
             int head, tile;
             for (int n = 0; ok && sc.item(n, head, tile); ++n) {
@@ -233,19 +237,26 @@ prefill_attend_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
                     const int g = (j + n) & 1;
                     if (j < 2) ok = mbar_wait(&sh.bar.o_empty[g], (n & 1) ^ 1, abort_flag);   // the last item's O of this group has been read
                     const int s = vs_cnt % NKV;
-                    ok = ok && mbar_wait(&sh.bar.p_full[g], pv_cnt[g] & 1, abort_flag) &&
-                         mbar_wait(&sh.bar.v_full[s], (vs_cnt / NKV) & 1, abort_flag);
-                    if (!ok) break;
-                    tc_fence_after();
-                    const uint64_t dv0 = smem_desc_mn(v_addr0 + s * TILE_BYTES, CHUNK_BYTES);   // 16 keys further: + 2 KB
-                    const uint64_t dp = desc_p0 + (uint64_t)g * (P_BYTES >> 4);
+                    ok = ok && mbar_wait(&sh.bar.v_full[s], (vs_cnt / NKV) & 1, abort_flag);
+                    const uint32_t dv0 = dv_base + s * (TILE_BYTES >> 4);                          // 16 keys further: + 2 KB
+                    const uint32_t dp = (uint32_t)desc_p0 + g * (P_BYTES >> 4);
 #pragma unroll
-                    for (int kk = 0; kk < TILE / 16; ++kk)          // 16 keys per MMA
-                        umma_bf16(tmem_base + O_COL0 + g * S_COLS, dp + (((kk / 4) * CHUNK_BYTES + (kk % 4) * 32) >> 4),
-                                  dv0 + (uint64_t)((kk * 16 * 128) >> 4), IDESC_O, ((j >> 1) | kk) ? 1u : 0u);
+                    for (int h = 0; h < 2; ++h) {                   // the first half's products run while the second is made
+                        ok = ok && mbar_wait(&sh.bar.p_full[g][h], (pv_ph >> g) & 1, abort_flag);
+                        if (!ok) break;
+                        tc_fence_after();
+#pragma unroll
+                        for (int k4 = 0; k4 < 4; ++k4) {            // 16 keys per MMA
+                            const int kk = h * 4 + k4;
+                            umma_bf16_lo(tmem_base + O_COL0 + g * S_COLS, dp + ((h * CHUNK_BYTES + k4 * 32) >> 4), p_hi,
+                                         dv0 + ((kk * 16 * 128) >> 4), v_hi, IDESC_O, ((j >> 1) | kk) ? 1u : 0u);
+                        }
+                        if (h == 0) umma_commit(&sh.bar.pv_half[g]);
+                    }
+                    if (!ok) break;
                     umma_commit(&sh.bar.v_empty[s]);
                     umma_commit(&sh.bar.pv_done[g]);         // the group's P may be overwritten, its O read or rescaled
-                    ++vs_cnt; ++pv_cnt[g];
+                    ++vs_cnt; pv_ph ^= 1u << g;
                 }
             }
         }
@@ -300,24 +311,11 @@ prefill_attend_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
                 if (first) m = mx;
                 else if (grow) { alpha = ex2(m - mx); m = mx; }
                 const bool rescale = !first && __any_sync(0xffffffffu, grow);
-                // p = 2^(x - m), summed in fp32, rounded to bf16 for the tensor core
-                const uint64_t sc2 = pack2(scale2, scale2), nm2 = pack2(-m, -m);
-                float sum[4] = {0.f, 0.f, 0.f, 0.f};
-                uint32_t pk[TILE / 2];
-#pragma unroll
-                for (int c = 0; c < TILE; c += 2) {
-                    float x0, x1;
-                    unpack2(ffma2(pack2(v[c], v[c + 1]), sc2, nm2), x0, x1);
-                    const float e0 = ex2(x0), e1 = ex2(x1);
-                    sum[(c >> 1) & 3] += e0 + e1;
-                    pk[c >> 1] = Vec<__nv_bfloat16>::pack2(e0, e1);
-                }
-                l = l * alpha + ((sum[0] + sum[1]) + (sum[2] + sum[3]));
-                // the group's previous P V has to be done before its P is overwritten or its O rescaled
-                ok = mbar_wait(&sh.bar.pv_done[grp], (pv_cnt & 1) ^ 1, abort_flag);
-                ok = __all_sync(0xffffffffu, ok);
-                if (!ok) break;
                 if (rescale) {
+                    // (the group's previous P V has to be done before its O is touched)
+                    ok = mbar_wait(&sh.bar.pv_done[grp], (pv_cnt & 1) ^ 1, abort_flag);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
                     tc_fence_after();
 #pragma unroll
                     for (int q = 0; q < D / 32; ++q) {
@@ -331,17 +329,37 @@ prefill_attend_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
                     }
                     tmem_st_wait();
                 }
-                // P row: 16-byte piece c of key chunk kc sits at piece c ^ (row & 7) of the row's 128 bytes
+                // p = 2^(x - m), summed in fp32, rounded to bf16 for the tensor core, in two halves of 64 keys: the
+                // products with the first half run while the second is computed, and a half of the P tile may be
+                // overwritten as soon as the last step's products with that half are done
+                const uint64_t sc2 = pack2(scale2, scale2), nm2 = pack2(-m, -m);
+                float sum[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-                for (int c = 0; c < 16; ++c) {
-                    const int kc = c >> 3, piece = c & 7;
-                    *reinterpret_cast<uint4*>(prow + kc * CHUNK_BYTES + ((piece ^ (row & 7)) << 4)) =
-                        make_uint4(pk[4 * c], pk[4 * c + 1], pk[4 * c + 2], pk[4 * c + 3]);
+                for (int h = 0; h < 2; ++h) {
+                    uint32_t pk[TILE / 4];
+#pragma unroll
+                    for (int c = 0; c < TILE / 2; c += 2) {
+                        float x0, x1;
+                        unpack2(ffma2(pack2(v[h * 64 + c], v[h * 64 + c + 1]), sc2, nm2), x0, x1);
+                        const float e0 = ex2(x0), e1 = ex2(x1);
+                        sum[(c >> 1) & 3] += e0 + e1;
+                        pk[c >> 1] = Vec<__nv_bfloat16>::pack2(e0, e1);
+                    }
+                    ok = mbar_wait(h ? &sh.bar.pv_done[grp] : &sh.bar.pv_half[grp], (pv_cnt & 1) ^ 1, abort_flag);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                    // P row: 16-byte piece c of key chunk h sits at piece c ^ (row & 7) of the row's 128 bytes
+#pragma unroll
+                    for (int c = 0; c < 8; ++c)
+                        *reinterpret_cast<uint4*>(prow + h * CHUNK_BYTES + ((c ^ (row & 7)) << 4)) =
+                            make_uint4(pk[4 * c], pk[4 * c + 1], pk[4 * c + 2], pk[4 * c + 3]);
+                    fence_proxy_async();
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&sh.bar.p_full[grp][h]);
                 }
-                fence_proxy_async();
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&sh.bar.p_full[grp]);
+                if (!ok) break;
+                l = l * alpha + ((sum[0] + sum[1]) + (sum[2] + sum[3]));
                 ++pv_cnt;
             }
             const int n_own = tile >= j_first ? (tile - j_first) / 2 + 1 : 0;
