@@ -437,7 +437,12 @@ int kvm_host_staging_bytes(const kvm_params* p, size_t* bytes) {
 // kept until the process exits.
 namespace {
 
-constexpr int kHostChunksMax = 4;     // measured on a C1 layer: 2 groups 2.34 ms, 3 2.25, 4 2.23, 6 2.24, 8 2.29
+constexpr int kHostChunksMax = 6;
+// (us a call for a Llama2-7B-shaped layer of 4096 tokens, 101 MB in: equal quarters 2223; ratio 0.7 2242, 0.6 2201, 0.5 2136,
+// 0.4 2166, 0.3 2236.  15 heads x 2 x 488 x 64, 5.6 MB in: quarters 387; ratio 0.5 with groups of at least 3 MB 285, 2 MB
+// 209, 1 MB 226)
+constexpr double kHostRatio = 0.5;
+constexpr long long kHostMinBytes = 2ll << 20;
 constexpr int kPipeDevices = 64;
 
 struct HostPipe {
@@ -447,6 +452,33 @@ struct HostPipe {
 };
 HostPipe g_pipe[kPipeDevices];
 std::mutex g_pipe_mu;      // held while a call enqueues: calls on one device share the events
+
+// Cuts U units of `unit_bytes` input each into groups: group c is units [first[c], first[c + 1]).  What the pipeline's end
+// costs is the last group's kernels and copy out, with nothing left to overlap them, so every group is kHostRatio of the one
+// before it; none is copied in with less than kHostMinBytes (shorter copies do not reach the link's rate, and a group
+// costs a dozen launches and copies).
+int host_groups(int U, size_t unit_bytes, int* first) {
+    const long long total = (long long)U * (long long)unit_bytes;
+    int n = 1;
+    double w = 1.0, sum = 1.0;                 // weights 1, r, r^2, ...
+    while (n < kHostChunksMax && n < U) {
+        const double w2 = w * kHostRatio;
+        if ((double)total * w2 / (sum + w2) < (double)kHostMinBytes) break;
+        w = w2;
+        sum += w;
+        ++n;
+    }
+    double acc = 0.0, wi = 1.0;
+    first[0] = 0;
+    for (int c = 0; c < n; ++c, wi *= kHostRatio) {
+        acc += wi;
+        int e = (int)(acc / sum * U + 0.5);
+        const int lo = first[c] + 1, hi = U - (n - 1 - c);
+        e = e < lo ? lo : e > hi ? hi : e;
+        first[c + 1] = c + 1 == n ? U : e;
+    }
+    return n;
+}
 
 HostPipe* host_pipe_for_current_device() {
     int dev = -1;
@@ -496,8 +528,8 @@ int kvm_compress_host(const kvm_params* p, const void* Q, const void* K, const v
     std::lock_guard<std::mutex> lock(g_pipe_mu);
     HostPipe* hp = host_pipe_for_current_device();
     if (!hp) return KVM_E_CUDA;
-    const int nch = d.U < kHostChunksMax ? d.U : kHostChunksMax;
-    const int per = (d.U + nch - 1) / nch;
+    int first[kHostChunksMax + 1];
+    const int nch = host_groups(d.U, rowQ + 2 * rowK, first);
     auto ok = [](cudaError_t err) { return err == cudaSuccess; };
     // a group of units as a layer of its own: one batch entry, nu KV heads
     auto group_params = [&](int u0, int nu) {
@@ -509,8 +541,8 @@ int kvm_compress_host(const kvm_params* p, const void* Q, const void* K, const v
         return pc;
     };
     // every group is validated before anything is enqueued, so a refusal leaves no copy in flight
-    for (int u0 = 0; u0 < d.U; u0 += per) {
-        const kvm_params pc = group_params(u0, (d.U - u0 < per) ? d.U - u0 : per);
+    for (int c = 0; c < nch; ++c) {
+        const kvm_params pc = group_params(first[c], first[c + 1] - first[c]);
         Dims dc;
         size_t need_c = 0;
         if ((rc = derive(&pc, dc)) != KVM_OK) return rc;
@@ -524,8 +556,8 @@ int kvm_compress_host(const kvm_params* p, const void* Q, const void* K, const v
     // to wait for all of it before the call returns, so that an error return never leaves copies writing the
     // caller's buffers behind its back.
     int status = KVM_OK;
-    for (int c = 0, u0 = 0; u0 < d.U && status == KVM_OK; ++c, u0 += per) {
-        const int nu = (d.U - u0 < per) ? d.U - u0 : per;
+    for (int c = 0; c < nch && status == KVM_OK; ++c) {
+        const int u0 = first[c], nu = first[c + 1] - u0;
         const kvm_params pc = group_params(u0, nu);
         if (!ok(cudaMemcpyAsync(dQ + rowQ * u0, (const char*)Q + rowQ * u0, rowQ * nu, cudaMemcpyHostToDevice, st)) ||
             !ok(cudaMemcpyAsync(dK + rowK * u0, (const char*)K + rowK * u0, rowK * nu, cudaMemcpyHostToDevice, st)) ||
