@@ -296,26 +296,33 @@ def compress_layers(p: KvmParams, layers, sim_thresholds=None, device="cuda", st
     """Compress a stack of layers, each an (Q, K, V) triple of CUDA tensors of the shape `p` describes, with one
     similarity threshold per layer (Section 3.2: thresholds chosen layer by layer), through kvm_compress_layers.
     Returns, per layer, a `Compressed` holding the outputs, and the layer's compression ratio mean(out_len) / S."""
+    # (the GPU waits for this function: whatever its results do not need is left until the kernels are enqueued, and the
+    # addresses are worked out from the bases)
     n = len(layers)
     B, H, cap, D = p.batch, p.n_kv_heads, kvm_sizes(p)[0], p.head_dim
-    dt = torch.bfloat16 if p.dtype == KVM_BF16 else torch.float32
-    # one allocation per kind for the whole stack (each layer's tensors are views of it) and one zero fill
+    units, size = B * H, 2 if p.dtype == KVM_BF16 else 4
+    # one allocation per kind for the whole stack (each layer's tensors are views of it), zero-filled
+    kv = torch.zeros(2 * n * units * cap * D, dtype=torch.bfloat16 if size == 2 else torch.float32, device=device)
+    ints = torch.zeros(n * units * (cap + 1), dtype=torch.int32, device=device)
     ws = torch.empty(kvm_layers_workspace_bytes(p, n), dtype=torch.uint8, device=device)
-    kv = torch.zeros(2, n, B, H, cap, D, dtype=dt, device=device)
-    ints = torch.zeros(n * B * H * (cap + 1), dtype=torch.int32, device=device)
-    out_len, out_pos = ints[:n * B * H].view(n, B, H), ints[n * B * H:].view(n, B, H, cap)
+    array = ctypes.c_void_p * n
 
-    def rows(t):            # the layers' addresses within a stacked tensor
-        step = t[0].numel() * t.element_size()
-        return (ctypes.c_void_p * n)(*range(t.data_ptr(), t.data_ptr() + n * step, step))
+    def rows(base, step):            # the layers' addresses within a stacked tensor
+        return array(*range(base, base + n * step, step))
 
-    ptrs = lambda i: (ctypes.c_void_p * n)(*[_ptr(l[i]) for l in layers])
+    for layer in layers:
+        assert len(layer) == 3 and all([t.is_contiguous() for t in layer]), "tensors must be contiguous"
+    q, k, v = (array(*[layer[i].data_ptr() for layer in layers]) for i in range(3))
     eps = None
     if sim_thresholds is not None:
         assert len(sim_thresholds) == n
         eps = (ctypes.c_float * n)(*[float(e) for e in sim_thresholds])
-    _call("kvm_compress_layers", p, n, eps, ptrs(0), ptrs(1), ptrs(2), rows(kv[0]), rows(kv[1]), rows(out_len),
-          rows(out_pos), None, ws.data_ptr(), ws.nbytes, _stream(stream))
-    out = [Compressed(kv[0, l], kv[1, l], out_len[l], out_pos[l], None, cap) for l in range(n)]
+    kv_base, kv_step, ints_base = kv.data_ptr(), units * cap * D * size, ints.data_ptr()
+    _call("kvm_compress_layers", p, n, eps, q, k, v, rows(kv_base, kv_step), rows(kv_base + n * kv_step, kv_step),
+          rows(ints_base, 4 * units), rows(ints_base + 4 * n * units, 4 * units * cap), None, ws.data_ptr(), ws.nbytes,
+          _stream(stream))
+    K_out, V_out = kv.view(2, n, B, H, cap, D).unbind(0)
+    out_len, out_pos = ints[:n * units].view(n, B, H), ints[n * units:].view(n, B, H, cap)
+    out = [Compressed(*ts, None, cap) for ts in zip(K_out.unbind(0), V_out.unbind(0), out_len.unbind(0), out_pos.unbind(0))]
     ratios = (out_len.cpu().float().mean((1, 2)) / p.seq).tolist()      # the one read-back of the call
     return out, ratios
