@@ -23,17 +23,23 @@ struct Dims {
 
 // The tensors of up to MAX_LAYERS layers of one shape that go through the kernels together, as one problem of n times the
 // batch; everything between them (scores, similarities, sets) lies in the workspace, layer after layer.
+// (Kernels take the tables by value, sized for one layer or for MAX_LAYERS: the larger parameters cost a call of five
+// launches 0.6 us of 30.)
 constexpr int MAX_LAYERS = 8;
-struct Layers {
+template <int NL> struct LayersOf {
     int n, U, H;                                   // layers; units and query heads of one layer
-    const void *Q[MAX_LAYERS], *K[MAX_LAYERS], *V[MAX_LAYERS];
-    void *K_out[MAX_LAYERS], *V_out[MAX_LAYERS];
-    int32_t *out_len[MAX_LAYERS], *pivot[MAX_LAYERS];
-    float eps[MAX_LAYERS];
+    const void *Q[NL], *K[NL], *V[NL];
+    void *K_out[NL], *V_out[NL];
+    int32_t *out_len[NL], *pivot[NL];
+    float eps[NL];
 };
+using Layers = LayersOf<MAX_LAYERS>;
+inline LayersOf<1> first_of(const Layers& L) {
+    return {1, L.U, L.H, {L.Q[0]}, {L.K[0]}, {L.V[0]}, {L.K_out[0]}, {L.V_out[0]}, {L.out_len[0]}, {L.pivot[0]}, {L.eps[0]}};
+}
 // The layer of unit u, which becomes the unit's index within the layer.
-__device__ __forceinline__ int layer_of(const Layers& L, long long& u) {
-    if (L.n == 1) return 0;
+template <int NL> __device__ __forceinline__ int layer_of(const LayersOf<NL>& L, long long& u) {
+    if (NL == 1) return 0;
     const int l = (int)u / L.U;
     u -= (long long)l * L.U;
     return l;

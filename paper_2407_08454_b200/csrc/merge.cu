@@ -65,8 +65,8 @@ template <int D> struct Slots {
 // Piece kinds of the walk.
 enum : int { PIECE_COPY = 0, PIECE_WHOLE = 1, PIECE_HEAD = 2, PIECE_TAIL = 3 };
 
-template <typename T, int D, int TOK>
-__global__ void __launch_bounds__(2 * D) merge_tile_kernel(const __grid_constant__ Layers L,
+template <typename T, int D, int TOK, int NL>
+__global__ void __launch_bounds__(2 * D) merge_tile_kernel(const __grid_constant__ LayersOf<NL> L,
                                                            const int32_t* __restrict__ set_start,
                                                            const int32_t* __restrict__ set_id,
                                                            int32_t* __restrict__ out_size, Slots<D> slots, int S,
@@ -255,8 +255,8 @@ __global__ void __launch_bounds__(2 * D) merge_tile_kernel(const __grid_constant
 }
 
 // Sets that cross a tile boundary: the block of the LAST boundary a set crosses adds its slots in tile order.
-template <typename T, int D, int TOK>
-__global__ void __launch_bounds__(2 * D) merge_fixup_kernel(const __grid_constant__ Layers L,
+template <typename T, int D, int TOK, int NL>
+__global__ void __launch_bounds__(2 * D) merge_fixup_kernel(const __grid_constant__ LayersOf<NL> L,
                                                             const int32_t* __restrict__ set_start,
                                                             const int32_t* __restrict__ set_id, int32_t* __restrict__ out_size, Slots<D> slots, int S,
                                                             int cap, int Tn, int scale_v) {
@@ -379,8 +379,8 @@ cudaError_t launch_gather_t(const Dims& d, const void* K, const void* V, const i
                             d.cap, d.scale_v, d.set_rule == KVM_SETS_CONSERVED_ONLY ? 1 : 0);
 }
 
-template <typename T, int D, int TOK>
-cudaError_t launch_t(const Dims& d, const Layers& L, const int32_t* set_start, const int32_t* set_id, int32_t* out_size,
+template <typename T, int D, int TOK, int NL>
+cudaError_t launch_n(const Dims& d, const LayersOf<NL>& L, const int32_t* set_start, const int32_t* set_id, int32_t* out_size,
                      float* scratch, float* set_coef, float* token_d2, kvm_stats* stats, cudaStream_t st) {
     const int Tn = (d.S + TOK - 1) / TOK;
     Slots<D> slots;
@@ -400,14 +400,20 @@ cudaError_t launch_t(const Dims& d, const Layers& L, const int32_t* set_start, c
                              set_start, (const int32_t*)L.out_len[0], set_coef, d.S, d.cap);
         if (e != cudaSuccess) return e;
     }
-    e = launch_dependent(merge_tile_kernel<T, D, TOK>, dim3(Tn, d.U), dim3(2 * D), smem, st, L, set_start, set_id, out_size,
+    e = launch_dependent(merge_tile_kernel<T, D, TOK, NL>, dim3(Tn, d.U), dim3(2 * D), smem, st, L, set_start, set_id, out_size,
                          slots, d.S, d.cap, c, d.scale_v, d.weight_rule == KVM_WEIGHT_AVERAGE ? 1 : 0,
                          per_set ? (const float*)set_coef : (const float*)nullptr, stats);
     if (e != cudaSuccess) return e;
     if (Tn > 1)
-        e = launch_dependent(merge_fixup_kernel<T, D, TOK>, dim3(Tn - 1, d.U), dim3(2 * D), 0, st, L, set_start, set_id,
+        e = launch_dependent(merge_fixup_kernel<T, D, TOK, NL>, dim3(Tn - 1, d.U), dim3(2 * D), 0, st, L, set_start, set_id,
                              out_size, slots, d.S, d.cap, Tn, d.scale_v);
     return e;
+}
+template <typename T, int D, int TOK>
+cudaError_t launch_t(const Dims& d, const Layers& L, const int32_t* set_start, const int32_t* set_id, int32_t* out_size,
+                     float* scratch, float* set_coef, float* token_d2, kvm_stats* stats, cudaStream_t st) {
+    return L.n == 1 ? launch_n<T, D, TOK>(d, first_of(L), set_start, set_id, out_size, scratch, set_coef, token_d2, stats, st)
+                    : launch_n<T, D, TOK>(d, L, set_start, set_id, out_size, scratch, set_coef, token_d2, stats, st);
 }
 
 }  // namespace

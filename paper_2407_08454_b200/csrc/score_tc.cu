@@ -146,17 +146,17 @@ __device__ __forceinline__ void store_side(__nv_bfloat16* dst_row, float e) {
 
 // Tensor maps of the layers' queries and keys, the keys themselves, and the map of the side tensor (which lies in the
 // workspace: one for all layers); units and query heads of a layer.
-struct Maps {
-    CUtensorMap q[MAX_LAYERS], k[MAX_LAYERS], side;
-    const __nv_bfloat16* keys[MAX_LAYERS];
-    int n, U, H;
+template <int NL> struct Maps {
+    CUtensorMap q[NL], k[NL], side;
+    const __nv_bfloat16* keys[NL];
+    int U, H;
 };
 
 // out: the column pass's scores [U,S], or its partial sums [piece][U,S] when items are cut; states: the row pass's
 // partial (maximum, sum) per piece and row when items are cut, else it writes the side tensor.
-template <int KCH, int PASS>
+template <int KCH, int PASS, int NL>
 __global__ void __launch_bounds__(NTHREADS, 1)
-score_tc_kernel(const __grid_constant__ Maps maps, __nv_bfloat16* __restrict__ lsep_out, float2* __restrict__ states,
+score_tc_kernel(const __grid_constant__ Maps<NL> maps, __nv_bfloat16* __restrict__ lsep_out, float2* __restrict__ states,
                 float* __restrict__ out, kvm_stats* stats, const Plan plan, int Hq, int Hkv, int S, float scale2,
                 float* __restrict__ sim_out) {
     constexpr int pass = PASS;
@@ -214,7 +214,7 @@ score_tc_kernel(const __grid_constant__ Maps maps, __nv_bfloat16* __restrict__ l
                 ok = mbar_wait(&sh.bar.empty_a[ab], ((n >> 1) & 1) ^ 1, abort_flag);
                 if (!ok) break;
                 last_a[ab] = (n >> 1) & 1;
-                const int per_layer = (pass == 1) ? maps.H : maps.U, layer = maps.n > 1 ? w.head / per_layer : 0;
+                const int per_layer = (pass == 1) ? maps.H : maps.U, layer = NL > 1 ? w.head / per_layer : 0;
                 const int head = w.head - layer * per_layer;             // within its layer
                 const CUtensorMap* mapA = (pass == 1) ? &maps.q[layer] : &maps.k[layer];
                 const CUtensorMap* mapB = (pass == 1) ? &maps.k[layer] : &maps.q[layer];
@@ -304,7 +304,7 @@ score_tc_kernel(const __grid_constant__ Maps maps, __nv_bfloat16* __restrict__ l
             const unsigned stride = gridDim.x * NSIM_WARPS * GPW;
             for (unsigned g = (blockIdx.x * NSIM_WARPS + (warp - NEPI_WARPS - 2)) * GPW + lane / LPR;
                  g < n_runs; g += stride) {
-                const unsigned u = g / (unsigned)runs, layer = maps.n > 1 ? u / (unsigned)maps.U : 0u;
+                const unsigned u = g / (unsigned)runs, layer = NL > 1 ? u / (unsigned)maps.U : 0u;
                 const int j0 = (int)(g - u * (unsigned)runs) * SIM_RUN;
                 simcore::run<__nv_bfloat16, D, SIM_RUN>(maps.keys[layer] + (size_t)(u - layer * maps.U) * S * D, sim_out + (size_t)u * S, j0,
                                                         min(j0 + SIM_RUN, S), gl, gbase, gmask);
@@ -485,15 +485,15 @@ __global__ void __launch_bounds__(256) combine_kernel(const float* __restrict__ 
     if (j < S) scores[(size_t)blockIdx.y * S + j] = plan::column_sum(part, plan, S, blockIdx.y, j);
 }
 
-// How the passes are dealt.  Rows: cutting costs a launch (join_rows_kernel, about as long as four steps), so it is done
-// where the longest item exceeds a CTA's equal share by more.  Columns: cutting costs a few additions in the kernel that
-// reads the scores, so it is done unless a CTA gets several of even the longest items and whole ones balance by
-// themselves (at 32 heads x 4096 tokens the share is 115 steps and the longest item 32: whole).
+// How the passes are dealt: items are cut where the longest one exceeds a CTA's equal share by more than cutting costs.
+// Rows: a launch (join_rows_kernel, about as long as four steps).  Columns: the additions in the kernel that reads the
+// scores, about as long as three (32 heads x 389 tokens, 3 steps per CTA and items of up to 4: cut 30.0 us a call,
+// whole 29.2; 32 query / 8 KV heads x 2048 tokens, 30 and up to 64: column pass 28.3 us cut, 49.9 whole).
 bool make_plan(const Dims& d, Plan& p) {
     if (!plan::make(d, p)) return false;
     if ((long long)d.B * d.Hkv * ((d.S + SIM_RUN - 1) / SIM_RUN) + plan::CTAS * 64 >= (1ll << 31)) return false;   // (the similarity warps' runs)
     p.split_row = p.T > (int)p.q + 4;
-    p.split_col = 3ll * p.G * p.T > (long long)p.q;
+    p.split_col = p.G * p.T > (int)p.q + 3;
     if (p.split_row) p.pr = p.pieces(p.T);
     if (p.split_col) p.pc = p.pieces(p.G * p.T);
     return true;
@@ -511,8 +511,8 @@ Scratch layout(const Dims& d, const Plan& p) {
     return s;
 }
 
-template <int KCH>
-cudaError_t launch_t(const Dims& d, const Plan& plan, const Maps& maps, const float* lse_in, char* scratch, float* scores,
+template <int KCH, int NL>
+cudaError_t launch_t(const Dims& d, const Plan& plan, const Maps<NL>& maps, const float* lse_in, char* scratch, float* scores,
                      kvm_stats* stats, cudaStream_t st, float* sim_out, float* lse_out, ScorePart* parts) {
     const size_t smem = 1024 + (size_t)(2 + NSTAGE) * KCH * TILE * 128 + (size_t)(NSTAGE + 1) * PTILE_BYTES + sizeof(Shared);
     // the shared-memory opt-in is made once per device and kernel instantiation
@@ -525,9 +525,9 @@ cudaError_t launch_t(const Dims& d, const Plan& plan, const Maps& maps, const fl
     {
         std::lock_guard<std::mutex> lock(mu);
         if (!done[dev]) {
-            e = cudaFuncSetAttribute(score_tc_kernel<KCH, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            e = cudaFuncSetAttribute(score_tc_kernel<KCH, 1, NL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
-            e = cudaFuncSetAttribute(score_tc_kernel<KCH, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            e = cudaFuncSetAttribute(score_tc_kernel<KCH, 2, NL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
             done[dev] = true;
         }
@@ -545,7 +545,7 @@ cudaError_t launch_t(const Dims& d, const Plan& plan, const Maps& maps, const fl
     };
     if (!lse_in) {
         // (the kernels wait for what precedes them by themselves, so each is scheduled while that drains)
-        e = launch_dependent(score_tc_kernel<KCH, 1>, grid(plan.split_row, plan.NH), dim3(NTHREADS), smem, st, maps, side,
+        e = launch_dependent(score_tc_kernel<KCH, 1, NL>, grid(plan.split_row, plan.NH), dim3(NTHREADS), smem, st, maps, side,
                              states, (float*)nullptr, stats, plan, d.Hq, d.Hkv, d.S, scale2,
                              scores ? (float*)nullptr : sim_out);
         if (e == cudaSuccess && plan.split_row)
@@ -557,7 +557,7 @@ cudaError_t launch_t(const Dims& d, const Plan& plan, const Maps& maps, const fl
         e = launch_dependent(lse_split_kernel, row_blocks, dim3(256), 0, st, lse_in, side, rows, -LOG2E / scale2);
     }
     if (e != cudaSuccess || !scores) return e;        // (row pass only)
-    e = launch_dependent(score_tc_kernel<KCH, 2>, grid(plan.split_col, plan.U), dim3(NTHREADS), smem, st, maps,
+    e = launch_dependent(score_tc_kernel<KCH, 2, NL>, grid(plan.split_col, plan.U), dim3(NTHREADS), smem, st, maps,
                          (__nv_bfloat16*)nullptr, (float2*)nullptr, plan.split_col ? part : scores, stats, plan, d.Hq, d.Hkv,
                          d.S, scale2, sim_out);
     if (e != cudaSuccess || !plan.split_col) return e;
@@ -584,20 +584,26 @@ size_t score_tc_scratch_bytes(const Dims& d) {
 // TMEM lane quarters, which then lag the others, and an accumulator goes back when its slowest warp is done.)
 // scores may be NULL (row pass only); lse_out (nullable) receives the natural-log row log-sum-exp [B,Hq,S].
 // parts (nullable): lets the column pass leave partial sums (parts->part set) for the caller's next kernel to add.
-// d: the layers together (a batch of n times a layer's).
-cudaError_t launch_score_tc(const Dims& d, const Layers& L, const float* lse_in, void* scratch, float* scores, kvm_stats* stats,
-                            cudaStream_t st, float* sim_out, float* lse_out, ScorePart* parts) {
-    Maps maps;
+template <int NL>
+static cudaError_t launch_score_n(const Dims& d, const Layers& L, const float* lse_in, void* scratch, float* scores,
+                                  kvm_stats* stats, cudaStream_t st, float* sim_out, float* lse_out, ScorePart* parts) {
+    Maps<NL> maps;
     Plan plan;
     if (!make_plan(d, plan)) return cudaErrorInvalidValue;
-    maps.n = L.n; maps.U = L.U; maps.H = L.H;
+    maps.U = L.U; maps.H = L.H;
     for (int l = 0; l < L.n; ++l) {
         if (!make_map(&maps.q[l], L.Q[l], L.H, d.S, d.D) || !make_map(&maps.k[l], L.K[l], L.U, d.S, d.D)) return cudaErrorNotSupported;
         maps.keys[l] = reinterpret_cast<const __nv_bfloat16*>(L.K[l]);
     }
     if (!make_map_side(&maps.side, scratch, d.B * d.Hq, d.S)) return cudaErrorNotSupported;
-    auto fn = d.D == 128 ? launch_t<2> : launch_t<1>;
+    auto fn = d.D == 128 ? launch_t<2, NL> : launch_t<1, NL>;
     return fn(d, plan, maps, lse_in, (char*)scratch, scores, stats, st, sim_out, lse_out, parts);
+}
+// d: the layers together (a batch of n times a layer's).
+cudaError_t launch_score_tc(const Dims& d, const Layers& L, const float* lse_in, void* scratch, float* scores, kvm_stats* stats,
+                            cudaStream_t st, float* sim_out, float* lse_out, ScorePart* parts) {
+    auto fn = L.n == 1 ? launch_score_n<1> : launch_score_n<MAX_LAYERS>;
+    return fn(d, L, lse_in, scratch, scores, stats, st, sim_out, lse_out, parts);
 }
 
 }  // namespace kvm

@@ -185,10 +185,11 @@ __device__ __forceinline__ void record_out_len(kvm_stats* stats, int n) {
 }
 
 // (scores: where `parts` holds partial sums the kernel adds them up and writes the scores itself)
+template <int NL>
 __global__ void __launch_bounds__(NT, 1) segment_unit_kernel(float* __restrict__ scores, const ScorePart parts,
                                                           const float* __restrict__ sim, int32_t* __restrict__ set_id,
                                                           int32_t* __restrict__ set_start,
-                                                          const __grid_constant__ Layers L, kvm_stats* stats, int S,
+                                                          const __grid_constant__ LayersOf<NL> L, kvm_stats* stats, int S,
                                                           int cap, int n_r, int n_h, int enforce, int pivot_rule, const float* __restrict__ pivot_key,
                                                           int set_rule) {
     extern __shared__ __align__(16) uint8_t flags[];  // [S] (+ jump arrays for the anchor reading)
@@ -550,12 +551,12 @@ __device__ __forceinline__ void radix_select_reg(const uint32_t (&key)[EM], unsi
     n_eq = cnt;
 }
 
-template <int EM>
+template <int EM, int NL>
 __global__ void __launch_bounds__(NT, 1) segment_unit_reg_kernel(float* __restrict__ scores, const ScorePart parts,
                                                               const float* __restrict__ sim,
                                                               int32_t* __restrict__ set_id,
                                                               int32_t* __restrict__ set_start,
-                                                              const __grid_constant__ Layers L, kvm_stats* stats, int S,
+                                                              const __grid_constant__ LayersOf<NL> L, kvm_stats* stats, int S,
                                                               int cap, int n_r, int n_h, int enforce, int pivot_rule,
                                                               const float* __restrict__ pivot_key) {
     __shared__ SharedReg sh;
@@ -819,22 +820,29 @@ cudaError_t launch_set_ratio(const Dims& d, const float* sim, float* ratio, cuda
     return cudaGetLastError();
 }
 
-cudaError_t launch_segment(const Dims& d, const Layers& L, float* scores, const ScorePart& parts, const float* sim,
+template <int NL>
+static cudaError_t launch_segment_n(const Dims& d, const LayersOf<NL>& L, float* scores, const ScorePart& parts, const float* sim,
                            int32_t* set_id, int32_t* set_start, kvm_stats* stats, cudaStream_t st) {
     // flags [S] bytes; the anchor reading adds two uint16 jump arrays
     const size_t smem = d.set_rule == KVM_SETS_ANCHOR ? (size_t)((d.S + 15) & ~15) + 4 * (size_t)d.S : (size_t)d.S;
     if (smem > 40 * 1024) {   // more dynamic shared memory than the default limit: opt in (cheap, idempotent)
-        cudaError_t e = cudaFuncSetAttribute(segment_unit_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t e = cudaFuncSetAttribute(segment_unit_kernel<NL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)segment_max_smem());
         if (e != cudaSuccess) return e;
     }
     if (d.set_rule == KVM_SETS_ADJACENT && d.S <= 4 * NT)
-        return launch_dependent(segment_unit_reg_kernel<4>, dim3(d.U), dim3(NT), 0, st, scores, parts, sim, set_id, set_start, L,
+        return launch_dependent(segment_unit_reg_kernel<4, NL>, dim3(d.U), dim3(NT), 0, st, scores, parts, sim, set_id, set_start, L,
                                 stats, d.S, d.cap, d.n_r, d.n_h, d.enforce, d.pivot_rule,
                                 d.pivot_rule == KVM_PIVOT_KEY ? d.pivot_key : (const float*)nullptr);
-    return launch_dependent(segment_unit_kernel, dim3(d.U), dim3(NT), smem, st, scores, parts, sim, set_id, set_start, L, stats, d.S,
+    return launch_dependent(segment_unit_kernel<NL>, dim3(d.U), dim3(NT), smem, st, scores, parts, sim, set_id, set_start, L, stats, d.S,
                             d.cap, d.n_r, d.n_h, d.enforce, d.pivot_rule,
                             d.pivot_rule == KVM_PIVOT_KEY ? d.pivot_key : (const float*)nullptr, d.set_rule);
+}
+
+cudaError_t launch_segment(const Dims& d, const Layers& L, float* scores, const ScorePart& parts, const float* sim,
+                           int32_t* set_id, int32_t* set_start, kvm_stats* stats, cudaStream_t st) {
+    return L.n == 1 ? launch_segment_n(d, first_of(L), scores, parts, sim, set_id, set_start, stats, st)
+                    : launch_segment_n(d, L, scores, parts, sim, set_id, set_start, stats, st);
 }
 
 }  // namespace kvm
