@@ -119,7 +119,7 @@ cudaError_t run_score(const Dims& d, const Layers& L, const float* lse_in, float
     // fp32 tensors enter the tensor cores as exact sums of three bf16 planes: rounding them would not hold the
     // score tolerance
     return d.dtype == KVM_BF16 ? launch_score_tc(d, L, lse_in, w.lse, scores, stats, st, sim_out, nullptr, parts)
-                               : launch_score_f32(d, L.Q[0], L.K[0], lse_in, w.lse, scores, stats, st, sim_out);
+                               : launch_score_f32(d, L.Q[0], L.K[0], lse_in, w.lse, scores, stats, st, sim_out, nullptr, parts);
 }
 
 // The whole chain over the layers in L (d: the layers together, a batch of n times a layer's).

@@ -123,11 +123,11 @@ cudaError_t launch_dependent_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 b
 }
 
 // Launchers (each enqueues on the stream and returns the launch status).
+struct ScorePart;             // partial column sums left for the segment kernel (score_plan.cuh)
 cudaError_t launch_score_f32(const Dims& d, const void* Q, const void* K, const float* lse_in, void* scratch,
                              float* scores, kvm_stats* stats, cudaStream_t st, float* sim_out = nullptr,
-                             float* lse_out = nullptr);
+                             float* lse_out = nullptr, ScorePart* parts = nullptr);
 size_t score_f32_scratch_bytes(const Dims& d);
-struct ScorePart;             // partial column sums left for the segment kernel (score_plan.cuh)
 cudaError_t launch_score_tc(const Dims& d, const Layers& L, const float* lse_in, void* scratch,
                             float* scores, kvm_stats* stats, cudaStream_t st, float* sim_out = nullptr,
                             float* lse_out = nullptr, ScorePart* parts = nullptr);

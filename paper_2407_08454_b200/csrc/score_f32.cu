@@ -22,7 +22,7 @@
 // fp32 layers come in (40 for 4 heads x 512 tokens, 4800 for 16 x 2999), so items are not dealt whole: the steps of all
 // items form one list and every CTA takes q = ceil(steps / 148) consecutive ones, which is balanced to one step.  An
 // item that is cut leaves one partial state per piece: (max, sum) per query row, combined by whoever reads it, or a
-// partial column sum per key, added in piece order by combine_kernel (or by the similarity kernel that follows in a
+// partial column sum per key, added in piece order by combine_kernel (or by the segment kernel that follows in a
 // compress call).  Where the pieces' states would not fit 4 MiB (large problems, where whole items balance well
 // anyway) items stay whole and the states are final.  The rule depends on the shape only: results are reproducible.
 //
@@ -59,6 +59,7 @@ constexpr int NSTAGE = 2;                          // ring of B chunks (three pl
 constexpr int NACC = 2;                            // accumulator pairs: 2 x (128 + 128) columns = all of TMEM
 constexpr int NEPI = 8, NCONV = 7;                // warps; with the MMA warp sixteen, i.e. 128 registers a thread
 constexpr int NTHREADS = (NEPI + NCONV + 1) * 32;
+constexpr int SIM_RUN = 8;                         // consecutive tokens per lane group (similarities)
 constexpr int NSLOT = 8;                           // piece-end buffers in rotation
 constexpr size_t SPLIT_BYTES_MAX = (size_t)KVM_STATIC_SCORE_ROWS * sizeof(float);
 constexpr float LOG2E = 1.4426950408889634f, LN2 = 0.6931471805599453f;
@@ -158,7 +159,7 @@ template <int KCH, int PASS>
 __global__ void __launch_bounds__(NTHREADS, 1)
 score_f32_kernel(const float* __restrict__ Q, const float* __restrict__ K, float2* __restrict__ states,
                  const float* __restrict__ flat, float flat_mul, float* __restrict__ out, kvm_stats* stats,
-                 const Plan plan, int Hq, int Hkv, int S, float scale2) {
+                 const Plan plan, int Hq, int Hkv, int S, float scale2, float* __restrict__ sim_out) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* sA = smem_raw + (base - smem_u32(smem_raw));     // [KCH][plane][128 rows][128 B]
@@ -223,6 +224,19 @@ score_f32_kernel(const float* __restrict__ Q, const float* __restrict__ K, float
             fence_proxy_async();
             __syncwarp();
             if (lane == 0) mbar_arrive(fa ? &sh.full_a[ac] : &sh.full_b[s]);
+        }
+        // The neighbour similarities (Eq. 2, which need K alone), while the last products and exponentials drain: the key
+        // rows are dealt to the converter warps of all CTAs in runs of SIM_RUN tokens.
+        if (PASS == 2 && sim_out) {
+            constexpr int D = KCH * KCHUNK, LPR = D / Vec<float>::N, GPW = 32 / LPR;
+            const unsigned runs = (unsigned)(S + SIM_RUN - 1) / SIM_RUN, n_runs = (unsigned)plan.U * runs;
+            const int gl = lane % LPR, gbase = lane / LPR * LPR;
+            const unsigned gmask = LPR == 32 ? 0xffffffffu : (((1u << LPR) - 1u) << gbase);
+            for (unsigned g = (blockIdx.x * NCONV + (warp - NEPI)) * GPW + lane / LPR; g < n_runs; g += gridDim.x * NCONV * GPW) {
+                const unsigned u = g / runs;
+                const int j0 = (int)(g - u * runs) * SIM_RUN;
+                simcore::run<float, D, SIM_RUN>(K + (size_t)u * S * D, sim_out + (size_t)u * S, j0, min(j0 + SIM_RUN, S), gl, gbase, gmask);
+            }
         }
     } else if (warp == NEPI + NCONV) {
         // ============================== MMA issue ==============================
@@ -437,25 +451,6 @@ __global__ void __launch_bounds__(256) combine_kernel(const float* __restrict__ 
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j < S) scores[(size_t)blockIdx.y * S + j] = plan::column_sum(part, plan, S, blockIdx.y, j);
 }
-// The same beside the neighbour similarities (Eq. 2, which need K alone and run while the column pass drains).
-constexpr int SIM_RUN = 8;                         // consecutive tokens per lane group
-template <int D>
-__global__ void __launch_bounds__(256) similarity_combine_kernel(const float* __restrict__ K, float* __restrict__ sim,
-                                                                 const float* __restrict__ part,
-                                                                 float* __restrict__ scores, const Plan plan, int S) {
-    constexpr int LPR = D / Vec<float>::N;
-    static_assert(LPR >= SIM_RUN, "a lane per token of the run");
-    const int runs = (S + SIM_RUN - 1) / SIM_RUN;
-    const unsigned g = (blockIdx.x * 256u + threadIdx.x) / LPR;
-    const int lane = threadIdx.x % LPR, u = (int)(g / (unsigned)runs);
-    if (u >= plan.U) return;                       // whole groups leave together
-    const int gbase = (threadIdx.x % 32) / LPR * LPR, j0 = (int)(g - (unsigned)u * runs) * SIM_RUN;
-    const unsigned gmask = LPR == 32 ? 0xffffffffu : (((1u << LPR) - 1u) << gbase);
-    simcore::run<float, D, SIM_RUN>(K + (size_t)u * S * D, sim + (size_t)u * S, j0, min(j0 + SIM_RUN, S), lane, gbase, gmask);
-    grid_dependency_wait();                        // (always: this grid must not end before the column pass has)
-    if (part && lane < SIM_RUN && j0 + lane < S) scores[(size_t)u * S + j0 + lane] = plan::column_sum(part, plan, S, u, j0 + lane);
-}
-
 // Bytes of the two passes' states and sums.
 size_t state_bytes(const Dims& d, const Plan& p) {
     const size_t rows = (size_t)p.NH * d.S;
@@ -463,7 +458,7 @@ size_t state_bytes(const Dims& d, const Plan& p) {
 }
 template <int KCH>
 cudaError_t launch_t(const Dims& d, const Plan& plan, const float* Q, const float* K, const float* lse_in, void* scratch,
-                     float* scores, kvm_stats* stats, cudaStream_t st, float* sim_out, float* lse_out) {
+                     float* scores, kvm_stats* stats, cudaStream_t st, float* sim_out, float* lse_out, ScorePart* parts) {
     const size_t smem = 1024 + (size_t)(KCH + NSTAGE) * CHUNK_BYTES + sizeof(Shared);
     static std::mutex mu;
     static bool done[KVM_MAX_DEVICES] = {};
@@ -491,7 +486,7 @@ cudaError_t launch_t(const Dims& d, const Plan& plan, const float* Q, const floa
     const float scale2 = d.scale * LOG2E;
     if (!lse_in) {
         e = launch_dependent(score_f32_kernel<KCH, 1>, rgrid, block, smem, st, Q, K, states, (const float*)nullptr,
-                             1.f, flat, stats, plan, d.Hq, d.Hkv, d.S, scale2);
+                             1.f, flat, stats, plan, d.Hq, d.Hkv, d.S, scale2, (float*)nullptr);
         if (e != cudaSuccess) return e;
     }
     if (lse_out) {
@@ -502,15 +497,13 @@ cudaError_t launch_t(const Dims& d, const Plan& plan, const float* Q, const floa
     if (!scores) return cudaSuccess;
     e = launch_dependent(score_f32_kernel<KCH, 2>, cgrid, block, smem, st, Q, K, states,
                          lse_in ? lse_in : (const float*)flat, lse_in ? LOG2E : 1.f, plan.split_col ? part : scores, stats, plan,
-                         d.Hq, d.Hkv, d.S, scale2);
-    if (e != cudaSuccess) return e;
-    if (sim_out) {
-        constexpr int D = KCH * KCHUNK;
-        const long long threads = (long long)d.U * ((d.S + SIM_RUN - 1) / SIM_RUN) * (D / Vec<float>::N);
-        return launch_dependent(similarity_combine_kernel<D>, dim3((unsigned)((threads + 255) / 256)), dim3(256), 0, st, K,
-                                sim_out, (const float*)part, scores, plan, d.S);
+                         d.Hq, d.Hkv, d.S, scale2, sim_out);
+    if (e != cudaSuccess || !plan.split_col) return e;
+    if (parts) {                                      // the caller's next kernel adds the pieces up
+        parts->part = part;
+        parts->plan = plan;
+        return cudaSuccess;
     }
-    if (!plan.split_col) return cudaSuccess;
     return launch_dependent(combine_kernel, dim3((d.S + 255) / 256, d.U), dim3(256), 0, st, (const float*)part, scores, plan, d.S);
 }
 
@@ -524,13 +517,15 @@ size_t score_f32_scratch_bytes(const Dims& d) {
 }
 
 // lse_in (nullable): natural-log row log-sum-exp, skips the row pass.  scores may be NULL (row pass only); lse_out
-// (nullable) receives the natural-log row log-sum-exp; sim_out (nullable, with scores) the neighbour similarities [U,S].
+// (nullable) receives the natural-log row log-sum-exp; sim_out (nullable, with scores) the neighbour similarities [U,S];
+// parts (nullable): lets the column pass leave partial sums (parts->part set) for the caller's next kernel to add.
 cudaError_t launch_score_f32(const Dims& d, const void* Q, const void* K, const float* lse_in, void* scratch,
-                             float* scores, kvm_stats* stats, cudaStream_t st, float* sim_out, float* lse_out) {
+                             float* scores, kvm_stats* stats, cudaStream_t st, float* sim_out, float* lse_out,
+                             ScorePart* parts) {
     Plan plan;
     if (!make_plan(d, plan)) return cudaErrorInvalidValue;
     auto fn = d.D == 128 ? launch_t<2> : launch_t<1>;
-    return fn(d, plan, (const float*)Q, (const float*)K, lse_in, scratch, scores, stats, st, sim_out, lse_out);
+    return fn(d, plan, (const float*)Q, (const float*)K, lse_in, scratch, scores, stats, st, sim_out, lse_out, parts);
 }
 
 }  // namespace kvm
