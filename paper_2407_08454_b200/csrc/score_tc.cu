@@ -46,6 +46,7 @@
 #include <cuda.h>
 
 #include <mutex>
+#include <type_traits>
 
 #include "score_plan.cuh"
 #include "similarity_core.cuh"
@@ -317,8 +318,8 @@ score_tc_kernel(const __grid_constant__ Maps<NL> maps, __nv_bfloat16* __restrict
         // Four groups of four warps take the steps in turn, each with an accumulator of its own, so that one group's
         // waits, TMEM loads and bookkeeping run beside the other three groups' exponentials.  Within a group a warp
         // owns a TMEM lane quarter and takes the step's 128 columns 32 at a time; the accumulator is handed back as
-        // soon as the last load has landed.  One rolled-up loop serves masked and unmasked columns: two copies of it,
-        // unrolled, leave the instruction cache (see the fp32 kernel).
+        // soon as the last load has landed.  The loops are kept short: unrolled whole, with a copy for each mask, they leave
+        // the instruction cache (see the fp32 kernel).
         const int lq = warp & 3, grp = warp >> 2;
         const int row = lq * 32 + lane;                      // A row = TMEM lane
         const uint32_t t_lane = tmem_base + ((uint32_t)(lq * 32) << 16) + grp * TILE;
@@ -339,14 +340,12 @@ score_tc_kernel(const __grid_constant__ Maps<NL> maps, __nv_bfloat16* __restrict
                 if (ok) tc_fence_after();
                 const bool diag = (pass == 1) ? w.i0 + t == w.tile : bt == 0;
                 const int left = (pass == 2) ? S - (w.tile + bt) * TILE : TILE;      // live columns (queries < S)
-                // On the diagonal tile whole 32-column quarters are masked (left out) or valid, one is mixed.
-                const int q0 = (pass == 2 && diag) ? lq : 0, q1 = (pass == 1 && diag) ? lq + 1 : 4;
-#pragma unroll 1
-                for (int cq = q0; ok && cq < q1; ++cq) {
+                // 32 columns; the last ones of the accumulator release it once they have landed
+                auto quarter = [&](int cq, bool last, auto masked) {
                     uint32_t vr[QCOLS];
                     tmem_ld32_issue(t_lane + cq * QCOLS, vr);
                     tmem_ld_wait();
-                    if (cq == q1 - 1) {                       // last read of this accumulator: release it
+                    if (last) {
                         tc_fence_before();
                         __syncwarp();
                         if (lane == 0) mbar_arrive(&sh.bar.acc_empty[grp]);
@@ -356,7 +355,7 @@ score_tc_kernel(const __grid_constant__ Maps<NL> maps, __nv_bfloat16* __restrict
 #pragma unroll
                     for (int c = 0; c < QCOLS; ++c) v[c] = __uint_as_float(vr[c]);
                     const int ncol = left - cq * QCOLS;
-                    if ((diag && cq == lq) || ncol < QCOLS) {
+                    if (decltype(masked)::value && ((diag && cq == lq) || ncol < QCOLS)) {
                         const int lo = (pass == 2 && diag && cq == lq) ? lane : 0;                 // query before key
                         const int hi = (pass == 1) ? lane + 1 : ncol;                              // key after query; past the end
 #pragma unroll
@@ -365,6 +364,16 @@ score_tc_kernel(const __grid_constant__ Maps<NL> maps, __nv_bfloat16* __restrict
                     }
                     if (pass == 1) chunk_row_pass(v, m, l, scale2, sc2);
                     else chunk_col_pass(v, acc, sc2);
+                };
+                if (ok && !diag && left >= TILE) {
+                    // (two quarters per round: 1 % less time than one on 32768 tokens, four the same)
+#pragma unroll 2
+                    for (int cq = 0; cq < 4; ++cq) quarter(cq, cq == 3, std::false_type{});
+                } else {
+                    // On the diagonal tile whole 32-column quarters are masked (left out) or valid, one is mixed.
+                    const int q0 = (pass == 2 && diag) ? lq : 0, q1 = (pass == 1 && diag) ? lq + 1 : 4;
+#pragma unroll 1
+                    for (int cq = q0; ok && cq < q1; ++cq) quarter(cq, cq == q1 - 1, std::true_type{});
                 }
                 if (pass == 2) { bt += NGRP; while (bt >= per) bt -= per; }
             }
