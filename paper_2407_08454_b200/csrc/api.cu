@@ -416,25 +416,7 @@ int kvm_compress_layers(const kvm_params* p, int32_t n_layers, const float* sim_
     return KVM_OK;
 }
 
-int kvm_host_staging_bytes(const kvm_params* p, size_t* bytes) {
-    Dims d;
-    const int rc = derive(p, d);
-    if (rc != KVM_OK) return rc;
-    if (!bytes) return KVM_E_NULL;
-    const size_t e = d.dtype == KVM_BF16 ? 2 : 4;
-    size_t off = 0;
-    off += align_up((size_t)d.B * d.Hq * d.S * d.D * e);        // Q
-    off += 2 * align_up((size_t)d.U * d.S * d.D * e);           // K, V
-    off += 2 * align_up((size_t)d.U * d.cap * d.D * e);         // K_out, V_out
-    off += align_up((size_t)d.U * sizeof(int32_t));             // out_len
-    off += align_up((size_t)d.U * d.cap * sizeof(int32_t));     // out_pos
-    off += carve(d, nullptr).bytes;
-    *bytes = off;
-    return KVM_OK;
-}
-
-// Streams and events of kvm_compress_host's copy/compute pipeline: created once per device on first use,
-// kept until the process exits.
+// The groups of units that kvm_compress_host's pipeline takes one after the other.
 namespace {
 
 constexpr int kHostChunksMax = 6;
@@ -443,15 +425,6 @@ constexpr int kHostChunksMax = 6;
 // 209, 1 MB 226)
 constexpr double kHostRatio = 0.5;
 constexpr long long kHostMinBytes = 2ll << 20;
-constexpr int kPipeDevices = 64;
-
-struct HostPipe {
-    bool ready = false;
-    cudaStream_t compute = nullptr, d2h = nullptr;
-    cudaEvent_t start = nullptr, end = nullptr, h2d[kHostChunksMax] = {}, done[kHostChunksMax] = {};
-};
-HostPipe g_pipe[kPipeDevices];
-std::mutex g_pipe_mu;      // held while a call enqueues: calls on one device share the events
 
 // Cuts U units of `unit_bytes` input each into groups: group c is units [first[c], first[c + 1]).  What the pipeline's end
 // costs is the last group's kernels and copy out, with nothing left to overlap them, so every group is kHostRatio of the one
@@ -479,6 +452,61 @@ int host_groups(int U, size_t unit_bytes, int* first) {
     }
     return n;
 }
+
+// A group of units as a layer of its own: one batch entry, nu KV heads.
+kvm_params group_params(const kvm_params* p, const Dims& d, int u0, int nu) {
+    kvm_params pc = *p;
+    pc.batch = 1;
+    pc.n_kv_heads = nu;
+    pc.n_q_heads = nu * d.G;
+    if (pc.pivot_key) pc.pivot_key += (size_t)u0 * d.S;
+    return pc;
+}
+size_t host_unit_bytes(const Dims& d) { return (size_t)(d.G + 2) * d.S * d.D * (d.dtype == KVM_BF16 ? 2 : 4); }
+
+}  // namespace
+
+int kvm_host_staging_bytes(const kvm_params* p, size_t* bytes) {
+    Dims d;
+    int rc = derive(p, d);
+    if (rc != KVM_OK) return rc;
+    if (!bytes) return KVM_E_NULL;
+    const size_t e = d.dtype == KVM_BF16 ? 2 : 4;
+    size_t off = 0;
+    off += align_up((size_t)d.B * d.Hq * d.S * d.D * e);        // Q
+    off += 2 * align_up((size_t)d.U * d.S * d.D * e);           // K, V
+    off += 2 * align_up((size_t)d.U * d.cap * d.D * e);         // K_out, V_out
+    off += align_up((size_t)d.U * sizeof(int32_t));             // out_len
+    off += align_up((size_t)d.U * d.cap * sizeof(int32_t));     // out_pos
+    // The groups' kernels run one after the other in one workspace.  A group can need more than the whole layer: its score
+    // passes may be cut where the layer's are not, and then leave partial results.
+    size_t ws = carve(d, nullptr).bytes;
+    int first[kHostChunksMax + 1];
+    const int n = host_groups(d.U, host_unit_bytes(d), first);
+    for (int c = 0; c < n; ++c) {
+        const kvm_params pc = group_params(p, d, first[c], first[c + 1] - first[c]);
+        Dims dc;
+        if ((rc = derive(&pc, dc)) != KVM_OK) return rc;
+        const size_t b = carve(dc, nullptr).bytes;
+        if (b > ws) ws = b;
+    }
+    *bytes = off + ws;
+    return KVM_OK;
+}
+
+// Streams and events of kvm_compress_host's copy/compute pipeline: created once per device on first use,
+// kept until the process exits.
+namespace {
+
+constexpr int kPipeDevices = 64;
+
+struct HostPipe {
+    bool ready = false;
+    cudaStream_t compute = nullptr, d2h = nullptr;
+    cudaEvent_t start = nullptr, end = nullptr, h2d[kHostChunksMax] = {}, done[kHostChunksMax] = {};
+};
+HostPipe g_pipe[kPipeDevices];
+std::mutex g_pipe_mu;      // held while a call enqueues: calls on one device share the events
 
 HostPipe* host_pipe_for_current_device() {
     int dev = -1;
@@ -529,20 +557,11 @@ int kvm_compress_host(const kvm_params* p, const void* Q, const void* K, const v
     HostPipe* hp = host_pipe_for_current_device();
     if (!hp) return KVM_E_CUDA;
     int first[kHostChunksMax + 1];
-    const int nch = host_groups(d.U, rowQ + 2 * rowK, first);
+    const int nch = host_groups(d.U, host_unit_bytes(d), first);
     auto ok = [](cudaError_t err) { return err == cudaSuccess; };
-    // a group of units as a layer of its own: one batch entry, nu KV heads
-    auto group_params = [&](int u0, int nu) {
-        kvm_params pc = *p;
-        pc.batch = 1;
-        pc.n_kv_heads = nu;
-        pc.n_q_heads = nu * d.G;
-        if (pc.pivot_key) pc.pivot_key += (size_t)u0 * d.S;
-        return pc;
-    };
     // every group is validated before anything is enqueued, so a refusal leaves no copy in flight
     for (int c = 0; c < nch; ++c) {
-        const kvm_params pc = group_params(first[c], first[c + 1] - first[c]);
+        const kvm_params pc = group_params(p, d, first[c], first[c + 1] - first[c]);
         Dims dc;
         size_t need_c = 0;
         if ((rc = derive(&pc, dc)) != KVM_OK) return rc;
@@ -558,7 +577,7 @@ int kvm_compress_host(const kvm_params* p, const void* Q, const void* K, const v
     int status = KVM_OK;
     for (int c = 0; c < nch && status == KVM_OK; ++c) {
         const int u0 = first[c], nu = first[c + 1] - u0;
-        const kvm_params pc = group_params(u0, nu);
+        const kvm_params pc = group_params(p, d, u0, nu);
         if (!ok(cudaMemcpyAsync(dQ + rowQ * u0, (const char*)Q + rowQ * u0, rowQ * nu, cudaMemcpyHostToDevice, st)) ||
             !ok(cudaMemcpyAsync(dK + rowK * u0, (const char*)K + rowK * u0, rowK * nu, cudaMemcpyHostToDevice, st)) ||
             !ok(cudaMemcpyAsync(dV + rowK * u0, (const char*)V + rowK * u0, rowK * nu, cudaMemcpyHostToDevice, st)) ||

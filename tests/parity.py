@@ -374,3 +374,19 @@ def check_evict_case(case: Case, g: Optional[GpuOut] = None) -> Report:
             rep.units_near_tie += 1
     assert np.array_equal(g.c_out_len.reshape(U), g_len)
     return rep
+
+
+def host_groups(units, unit_bytes):
+    """The sizes of the groups of units that kvm_compress_host makes: each half of the one before it, at most six, none
+    copied in with less than 2 MiB."""
+    n, w, total = 1, 1.0, 1.0
+    while n < 6 and n < units and units * unit_bytes * (w / 2) / (total + w / 2) >= 2 << 20:
+        w /= 2
+        total += w
+        n += 1
+    first, acc = [0], 0.0
+    for c in range(n):
+        acc += 0.5 ** c
+        e = int(acc / total * units + 0.5)
+        first.append(units if c + 1 == n else min(max(e, first[c] + 1), units - (n - 1 - c)))
+    return [b - a for a, b in zip(first, first[1:])]

@@ -159,3 +159,30 @@ int main(void) {
     assert int(ws) == kvm.kvm_workspace_bytes(kvm.make_params(1, 32, 8, 32768, 128, kvm.KVM_BF16))
     assert int(host) > int(ws) and int(ver) == kvm.kvm_version()
     assert "shape" in out.stdout
+
+
+def test_host_staging_holds_the_workspace_of_every_group(lib):
+    """A group of units may need more workspace than the whole layer (its score passes are cut where the layer's are not):
+    the staging buffer of the documented size has to hold every group's."""
+    from parity import host_groups
+    align = lambda n: (n + 255) // 256 * 256
+    shapes = [(1, 16, 4, 1024, 128, kvm.KVM_BF16), (1, 18, 18, 1024, 64, kvm.KVM_BF16), (1, 72, 9, 3584, 64, kvm.KVM_F32),
+              (1, 16, 4, 1724, 128, kvm.KVM_BF16), (1, 8, 4, 4712, 64, kvm.KVM_BF16), (1, 18, 18, 999, 64, kvm.KVM_BF16),
+              (1, 72, 9, 3582, 64, kvm.KVM_F32)]
+    for heads, kv in ((16, 4), (16, 16), (12, 12), (8, 8), (32, 32), (5, 5), (64, 8)):
+        for S in range(256, 8193, 163):
+            shapes += [(1, heads, kv, S, 64 + 64 * (S % 2), kvm.KVM_BF16), (2, heads, kv, S, 128, kvm.KVM_F32)]
+    groups_seen = set()
+    for B, Hq, Hkv, S, D, dtype in shapes:
+        p = kvm.make_params(B, Hq, Hkv, S, D, dtype, budget=0.5)
+        cap, e, U, G = kvm.kvm_sizes(p)[0], 2 if dtype == kvm.KVM_BF16 else 4, B * Hkv, Hq // Hkv
+        tensors = (align(U * G * S * D * e) + 2 * align(U * S * D * e) + 2 * align(U * cap * D * e) + align(4 * U)
+                   + align(4 * U * cap))
+        room = kvm.kvm_host_staging_bytes(p) - tensors
+        assert room >= kvm.kvm_workspace_bytes(p)
+        groups = host_groups(U, (G + 2) * S * D * e)
+        groups_seen.add(len(groups))
+        for n in groups:
+            need = kvm.kvm_workspace_bytes(kvm.make_params(1, n * G, n, S, D, dtype, budget=0.5))
+            assert need <= room, (B, Hq, Hkv, S, D, dtype, groups)
+    assert {1, 2, 3, 4} <= groups_seen

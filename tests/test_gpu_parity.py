@@ -6,7 +6,7 @@ import torch
 
 import paper_2407_08454_b200 as kvm
 from paper_2407_08454_b200 import synth_inputs as si
-from parity import Case, check_case, check_invariants_all_units, run_gpu
+from parity import Case, check_case, check_invariants_all_units, host_groups, run_gpu
 
 pytestmark = pytest.mark.gpu
 
@@ -258,10 +258,15 @@ def test_compress_is_reproducible_bit_for_bit():
 
 @pytest.mark.parametrize("B,Hq,Hkv,S,D,dtype", [
     (1, 4, 4, 512, 64, torch.float32),
-    (2, 6, 3, 700, 128, torch.bfloat16),      # 6 units: one per group
-    (5, 4, 2, 300, 128, torch.bfloat16),      # 10 units: groups of 2, GQA
+    (2, 6, 3, 700, 128, torch.bfloat16),
+    (5, 4, 2, 300, 128, torch.bfloat16),
     (1, 2, 1, 256, 64, torch.bfloat16),       # a single unit
-    (3, 3, 3, 1001, 64, torch.bfloat16),      # 9 units in groups of 2: a group's pivot keys start 4004 bytes apart
+    (3, 3, 3, 1001, 64, torch.bfloat16),
+    # (the above are copied in with less than 6 MiB and go through as one group; from here on several)
+    (1, 16, 4, 1024, 128, torch.bfloat16),    # groups of 3 and 1 units; the first needs more workspace than the layer
+    (2, 8, 4, 2001, 64, torch.bfloat16),      # 5 and 3: pivot keys of the second start 5 * 8004 bytes on
+    (1, 30, 15, 1300, 128, torch.bfloat16),   # 9, 4 and 2
+    (1, 40, 40, 999, 64, torch.float32),      # 23, 11 and 6
 ])
 def test_host_entry_point_equals_the_device_path(B, Hq, Hkv, S, D, dtype):
     cfg = si.CONFIGS["C1"].scaled(seq=S, head_dim=D, n_q_heads=Hq, n_kv_heads=Hkv, batch=B,
@@ -270,10 +275,21 @@ def test_host_entry_point_equals_the_device_path(B, Hq, Hkv, S, D, dtype):
     key = torch.rand(B, Hkv, S)
     for rules in (dict(), dict(pivot_rule=kvm.KVM_PIVOT_KEY, pivot_key=key.cuda())):
         p = kvm.make_params(B, Hq, Hkv, S, D, dtype, budget=0.5, **rules)
-        comp = kvm.Compressor(p)
-        r = comp(d["Q"].cuda(), d["K"].cuda(), d["V"].cuda())
+        # the device path: on the whole layer where it goes through as one group, else on each group by itself (whose score
+        # passes may be cut otherwise than the whole layer's)
+        G, units, u0, ref = Hq // Hkv, B * Hkv, 0, []
+        groups = host_groups(units, (G + 2) * S * D * d["K"].element_size())
+        for n in groups:
+            b = B if len(groups) == 1 else 1
+            pick = lambda x, h: x.reshape(units, h // Hkv, *x.shape[2:])[u0:u0 + n].reshape(b, n * h // (Hkv * b), *x.shape[2:]).cuda()
+            group_rules = {**rules, "pivot_key": pick(key, Hkv)} if rules else rules
+            comp = kvm.Compressor(kvm.make_params(b, n * G // b, n // b, S, D, dtype, budget=0.5, **group_rules))
+            ref.append(comp(pick(d["Q"], Hq), pick(d["K"], Hkv), pick(d["V"], Hkv)))
+            u0 += n
         torch.cuda.synchronize()
         cap = comp.cap
+        r_len, r_pos, r_K, r_V = (torch.cat([getattr(r, k).flatten(0, 1) for r in ref]).cpu()
+                                  for k in ("out_len", "out_pos", "K_out", "V_out"))
         pin = {k: v.pin_memory() for k, v in d.items()}
         hK = torch.full((B, Hkv, cap, D), 768.0, dtype=dtype).pin_memory()
         hV = torch.full_like(hK, 768.0).pin_memory()
@@ -286,12 +302,12 @@ def test_host_entry_point_equals_the_device_path(B, Hq, Hkv, S, D, dtype):
             with torch.cuda.stream(side if stream is not None else torch.cuda.current_stream()):
                 kvm.kvm_compress_host(p, pin["Q"], pin["K"], pin["V"], hK, hV, hlen, hpos, stage, stream)
             (stream or torch.cuda.current_stream()).synchronize()
-            assert torch.equal(hlen, r.out_len.cpu().view(-1))
+            assert torch.equal(hlen, r_len)
             for u in range(B * Hkv):
                 n = int(hlen[u])
-                assert torch.equal(hpos[u, :n], r.out_pos.cpu().view(B * Hkv, cap)[u, :n])
-                assert torch.equal(hK.view(B * Hkv, cap, D)[u, :n], r.K_out.cpu().view(B * Hkv, cap, D)[u, :n])
-                assert torch.equal(hV.view(B * Hkv, cap, D)[u, :n], r.V_out.cpu().view(B * Hkv, cap, D)[u, :n])
+                assert torch.equal(hpos[u, :n], r_pos[u, :n])
+                assert torch.equal(hK.view(B * Hkv, cap, D)[u, :n], r_K[u, :n])
+                assert torch.equal(hV.view(B * Hkv, cap, D)[u, :n], r_V[u, :n])
 
 
 def test_seeded_sweep_of_shapes_and_parameters():
