@@ -262,6 +262,9 @@ __global__ void __launch_bounds__(2 * D) merge_fixup_kernel(const __grid_constan
                                                             int cap, int Tn, int scale_v) {
     // The sets were written before the tile kernel began (it triggers this launch only after it has waited for
     // them), so they can be looked up while that kernel's last blocks still run; they are read through L2.
+    // One block waits for the tile kernel whatever its boundary holds: were there no set that crosses one, this grid could
+    // complete before the tile kernel does, and a kernel that is launched to depend on this one waits for this grid only.
+    if (blockIdx.x == 0 && blockIdx.y == 0) grid_dependency_wait();
     const int c = blockIdx.x + 1;                 // boundary between tiles c-1 and c
     const long long u = blockIdx.y;
     const int b = c * TOK;

@@ -101,3 +101,25 @@ def test_no_merging_gives_zero_perturbation():
     cfg = si.CONFIGS["C1"].scaled(seq=640, n_q_heads=4, n_kv_heads=2, seed=32)
     mean, worst = _perturb(cfg, sim_threshold=1.5, enforce_budget=0, recent_ratio=0.0, heavy_ratio=0.0)
     assert mean == 0.0 and worst == 0.0
+
+
+@pytest.mark.parametrize("Hq,Hkv,S,D,dtype", [(4, 4, 200, 64, torch.bfloat16), (64, 64, 640, 128, torch.bfloat16),
+                                              (32, 16, 500, 128, torch.float32)])
+def test_attention_enqueued_right_behind_a_compression_sees_every_row(Hq, Hkv, S, D, dtype):
+    """No set crosses a tile here (no similarity exceeds the threshold), so no block of the merge's second kernel has a slot
+    to wait for; the attention that is enqueued behind it still has to wait for the first one's rows."""
+    g = torch.Generator().manual_seed(S)
+    Q, K, V, q = (torch.randn(1, h, n, D, generator=g).to(dtype).cuda() for h, n in ((Hq, S), (Hkv, S), (Hkv, S), (Hq, 1)))
+    p = kvm.make_params(1, Hq, Hkv, S, D, dtype, budget=1.0, recent_ratio=0.0, heavy_ratio=0.0, sim_threshold=2.0)
+    comp = kvm.Compressor(p)
+    q = q.squeeze(2).contiguous()
+    ws = torch.empty_like(comp.ws)
+    ref, out = torch.empty(1, Hq, D, device="cuda"), torch.empty(1, Hq, D, device="cuda")
+    kvm.kvm_attend(p, q, K, V, S, None, ref, ws)                  # every token is a set of its own: the cache is K, V
+    for _ in range(20):
+        comp.K_out.fill_(float("nan"))
+        comp.V_out.fill_(float("nan"))
+        r = comp(Q, K, V)
+        kvm.kvm_attend(p, q, r.K_out, r.V_out, S, r.out_len, out, ws)
+        assert torch.equal(out, ref)
+    assert torch.equal(r.K_out, K) and torch.equal(r.V_out, V)
