@@ -21,11 +21,12 @@ def sources():
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
 
-# A second library for the test of the give-up path of the bounded device waits: the same sources with a short
-# wait limit and a producer that leaves out one stage, so that a wait runs out, the kernel returns and reports
-# it.  It is never loaded by the package itself.
+# A second library for the tests of the give-up paths of the bounded device waits: the same sources with a short
+# wait limit and producers that leave out one stage (the prefill attention's in every block, the score passes' in one),
+# so that a wait runs out, the kernel returns and reports it.  It is never loaded by the package itself.
 WAITTEST_LIB = os.path.join(_PKG, "libkvm_waittest.so")
-WAITTEST_FLAGS = ("-DKVM_TEST_WAIT_LIMIT_CLOCKS=4000000ll", "-DKVM_TEST_DROP_B_STAGE=3", "-DKVM_TEST_DROP_SCORE_STEP=0")
+WAITTEST_FLAGS = ("-DKVM_TEST_WAIT_LIMIT_CLOCKS=4000000ll", "-DKVM_TEST_DROP_B_STAGE=3", "-DKVM_TEST_DROP_SCORE_STEP=0",
+                  "-DKVM_TEST_DROP_CTA=1")
 
 
 def _stale(lib: str = LIB) -> bool:

@@ -41,8 +41,8 @@
 //
 // Two compile-time switches exist for the test of that give-up path and are never set in the
 // library that ships: KVM_TEST_WAIT_LIMIT_CLOCKS shortens the limit of every wait, and
-// KVM_TEST_DROP_SCORE_STEP = k makes the producer leave out its k-th B stage (barrier not armed,
-// copies not issued), so that the MMA warp's wait for it runs out.
+// KVM_TEST_DROP_SCORE_STEP = k makes the producer of block KVM_TEST_DROP_CTA leave out its k-th B stage (barrier not
+// armed, copies not issued), so that the MMA warp's wait for it runs out.
 #include <cuda.h>
 
 #include <mutex>
@@ -234,7 +234,7 @@ score_tc_kernel(const __grid_constant__ Maps<NL> maps, __nv_bfloat16* __restrict
                     ok = mbar_wait(&sh.bar.empty_b[s], ((cnt / NSTAGE) & 1) ^ 1, abort_flag);
                     if (!ok) break;
 #ifdef KVM_TEST_DROP_SCORE_STEP
-                    if (cnt == (uint32_t)(KVM_TEST_DROP_SCORE_STEP)) continue;   // test build only: this stage never arrives
+                    if (blockIdx.x == KVM_TEST_DROP_CTA && cnt == (uint32_t)(KVM_TEST_DROP_SCORE_STEP)) continue;   // test build only: this stage never arrives
 #endif
                     last_b[s] = (cnt / NSTAGE) & 1;
                     mbar_expect_tx(&sh.bar.full_b[s], TILE_BYTES + (pass == 2 ? PTILE_BYTES : 0u));

@@ -4,8 +4,8 @@ Every wait on an mbarrier in the tensor-core score kernel has a limit; when one 
 touching tensor memory, writes NaN for the work items it could not finish, reports KVM_E_DEVICE_TIMEOUT through
 kvm_stats, frees its tensor memory and returns.  Nothing in the shipped library can make a wait run out, so
 this test uses a second build of the same sources (never loaded by the package) in which the limit is two
-milliseconds of SM clocks and the TMA producer leaves out its fourth stage: the barrier of that stage is never
-armed, the MMA warp's wait for it gives up, and the kernel must come back by itself.  No trap, no unbounded
+milliseconds of SM clocks and the TMA producer of one block leaves out its first stage: the barrier of that stage is
+never armed, the MMA warp's wait for it gives up, and the kernel must come back by itself.  No trap, no unbounded
 loop, no bad address is involved.  The eviction rule is used so that what runs after the score step (the
 conserved tokens are gathered by index) does not depend on the values of the scores.
 """
@@ -55,6 +55,35 @@ def test_a_wait_that_runs_out_is_reported_and_the_next_call_is_correct():
     ref = kvmo.scores(d["Q"].double().numpy(), d["K"].double().numpy(), f32(1.0 / np.sqrt(np.float32(cfg.head_dim))))
     g = good.cpu().numpy().astype(np.float64)
     assert np.all(np.abs(g - ref) <= SCORE_RTOL * np.abs(ref) + SCORE_ATOL)
+
+
+def _ptrs(*tensors):
+    return [ctypes.c_void_p(0 if t is None else t.data_ptr()) for t in tensors]
+
+
+def test_a_piece_that_gave_up_marks_every_row_and_score_that_depends_on_it():
+    """Every step is a piece of its own here (4 heads x 8 tiles, 144 steps) and block 1 gives up its only one: in the row
+    pass the first of the two pieces of query tile 1, in the column pass the first piece of key tile 6.  The row's other
+    piece is good; joined, the row is still NaN, and with it the scores of every key that its queries see."""
+    lib = ctypes.CDLL(build.build_waittest())
+    g = torch.Generator().manual_seed(5)
+    Q, K = ((torch.randn(1, 4, 1024, 128, generator=g) * s).bfloat16().cuda() for s in (2, 1))
+    p = kvm.make_params(1, 4, 4, 1024, 128, torch.bfloat16)
+    ws = torch.zeros(kvm.kvm_workspace_bytes(p), dtype=torch.uint8, device="cuda")
+    scores, lse, good_scores, good_lse = (torch.zeros(1, 4, 1024, device="cuda") for _ in range(4))
+    size, st = ctypes.c_size_t(ws.numel()), ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    assert lib.kvm_score(ctypes.byref(p), *_ptrs(Q, K, None, scores, ws), size, st) == 0
+    assert lib.kvm_row_lse(ctypes.byref(p), *_ptrs(Q, K, lse, ws), size, st) == 0
+    torch.cuda.synchronize()
+    kvm.kvm_score(p, Q, K, None, good_scores, ws)
+    kvm.kvm_row_lse(p, Q, K, good_lse, ws)
+    bad_lse, bad_scores = torch.zeros_like(lse, dtype=torch.bool), torch.zeros_like(scores, dtype=torch.bool)
+    bad_lse[0, 0, 128:256] = True
+    bad_scores[0, 0, :256] = True
+    bad_scores[0, 0, 768:896] = True
+    for got, good, bad in ((lse, good_lse, bad_lse), (scores, good_scores, bad_scores)):
+        assert torch.equal(torch.isnan(got), bad)
+        assert torch.equal(got[~bad], good[~bad])
 
 
 def test_the_prefill_attention_kernel_also_comes_back_and_reports():
