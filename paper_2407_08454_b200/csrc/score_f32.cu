@@ -204,11 +204,13 @@ score_f32_kernel(const float* __restrict__ Q, const float* __restrict__ K, float
         }
         while (more) {
             const bool fa = f.is_a();
-            const int ac = f.a, s = f.bcnt % NSTAGE;
+            const int ac = f.a;
+            const uint32_t bc = f.bcnt;
+            const int s = bc % NSTAGE;
             if (fa) {
                 if (ac == 0) ok = mbar_wait(&sh.empty_a, (f.n & 1) ^ 1, abort_flag);
             } else {
-                ok = mbar_wait(&sh.empty_b[s], ((f.bcnt / NSTAGE) & 1) ^ 1, abort_flag);
+                ok = mbar_wait(&sh.empty_b[s], ((bc / NSTAGE) & 1) ^ 1, abort_flag);
             }
             if (!__all_sync(0xffffffffu, ok)) break;
             uint8_t* dst = fa ? sA + ac * CHUNK_BYTES : sB + s * CHUNK_BYTES;
@@ -223,6 +225,9 @@ score_f32_kernel(const float* __restrict__ Q, const float* __restrict__ K, float
             }
             fence_proxy_async();
             __syncwarp();
+#ifdef KVM_TEST_DROP_SCORE_STEP
+            if (blockIdx.x == KVM_TEST_DROP_CTA && !fa && bc == (uint32_t)(KVM_TEST_DROP_SCORE_STEP)) continue;   // test build only (see the bf16 kernel)
+#endif
             if (lane == 0) mbar_arrive(fa ? &sh.full_a[ac] : &sh.full_b[s]);
         }
         // The neighbour similarities (Eq. 2, which need K alone), while the last products and exponentials drain: the key
@@ -382,26 +387,31 @@ score_f32_kernel(const float* __restrict__ Q, const float* __restrict__ K, float
             // With one-step pieces the warp then delivers piece k, and piece k + 1 in which it has no step: five
             // pieces are open at most.)
             const int slot = n % NSLOT;
-            sh.part_m[slot][grp][row] = m;
-            sh.part_l[slot][grp][row] = (l[0] + l[1]) + (l[2] + l[3]);
-            __syncwarp();
-            int before = 0;
-            if (lane == 0) {
-                __threadfence_block();
-                before = atomicAdd(&sh.arrived[slot][lq], 1);
+            // (After a give-up nothing keeps the groups within a few steps of one another, and a piece's buffer could be
+            // taken for a later one's: every warp marks the rows of its pieces by itself then.)
+            bool bad = __any_sync(0xffffffffu, *abort_flag != 0);
+            int before = 1;
+            if (!bad) {
+                sh.part_m[slot][grp][row] = m;
+                sh.part_l[slot][grp][row] = (l[0] + l[1]) + (l[2] + l[3]);
+                __syncwarp();
+                if (lane == 0) {
+                    __threadfence_block();
+                    before = atomicAdd(&sh.arrived[slot][lq], 1);
+                }
+                before = __shfl_sync(0xffffffffu, before, 0);
             }
-            before = __shfl_sync(0xffffffffu, before, 0);
             if (before == 1) {
                 __threadfence_block();
-                if (lane == 0) sh.arrived[slot][lq] = 0;
-                const bool bad = *abort_flag != 0;
+                if (!bad && lane == 0) sh.arrived[slot][lq] = 0;
+                bad = bad || *abort_flag != 0;   // (read again: the other group may have given up before it came here)
                 const int gi = w.tile * TILE + row;
                 const float m0 = sh.part_m[slot][0][row], m1 = sh.part_m[slot][1][row];
                 const float l0 = sh.part_l[slot][0][row], l1 = sh.part_l[slot][1][row];
                 if (gi < S) {
                     const size_t at = (size_t)w.head * S + gi;
                     if (PASS == 1) {
-                        const float M = fmaxf(m0, m1);
+                        const float M = bad ? 0.f : fmaxf(m0, m1);
                         const float L = bad ? NAN : (m0 > -INFINITY ? l0 * exp2f(m0 - M) : 0.f) + (m1 > -INFINITY ? l1 * exp2f(m1 - M) : 0.f);
                         if (plan.split_row) {
                             states[(size_t)w.piece(plan) * rows + at] = make_float2(M, L);

@@ -152,12 +152,11 @@ struct Walk {
     }
 };
 
-// Folds a partial (maximum, sum) of a query row into (M, L); log2 units.  A sum that is NaN (a piece whose wait ran out,
-// perhaps before it had a maximum) stays NaN whatever comes after it.
+// Folds a partial (maximum, sum) of a query row into (M, L); log2 units.  (A piece whose wait ran out leaves the state
+// (0, NaN), whatever maximum it had by then: with -inf the sum would be passed over here.)
 __device__ __forceinline__ void add_state(float& M, float& L, float2 st) {
     const float mn = fmaxf(M, st.x);
     if (mn > -INFINITY) L = L * exp2f(M - mn) + st.y * exp2f(st.x - mn);
-    if (st.y != st.y) L = st.y;
     M = mn;
 }
 

@@ -390,34 +390,39 @@ score_tc_kernel(const __grid_constant__ Maps<NL> maps, __nv_bfloat16* __restrict
             const int gi = w.tile * TILE + row;
             const float mine = (pass == 1) ? l : ((acc[0] + acc[1]) + (acc[2] + acc[3])) + ((acc[4] + acc[5]) + (acc[6] + acc[7]));
             float M = m, L = mine;
+            // (After a give-up nothing keeps the groups within a few steps of one another, and an item's buffer could be
+            // taken for a later one's: every warp marks the rows of its items by itself then.)
+            bool bad = __any_sync(0xffffffffu, *abort_flag != 0);
             if (w.n > 1) {
                 const int slot = multi % NSLOT;
                 ++multi;
-                float* pm = part_m + slot * NGRP * TILE + row;       // + q * TILE: the group with the item's step q
-                float* pl = part_l + slot * NGRP * TILE + row;
-                if (pass == 1) pm[first * TILE] = m;
-                pl[first * TILE] = mine;
-                __syncwarp();
-                int before = 0;
-                if (lane == 0) {
+                if (!bad) {
+                    float* pm = part_m + slot * NGRP * TILE + row;       // + q * TILE: the group with the item's step q
+                    float* pl = part_l + slot * NGRP * TILE + row;
+                    if (pass == 1) pm[first * TILE] = m;
+                    pl[first * TILE] = mine;
+                    __syncwarp();
+                    int before = 0;
+                    if (lane == 0) {
+                        __threadfence_block();
+                        before = atomicAdd(&sh.arrived[slot][lq], 1);
+                    }
+                    before = __shfl_sync(0xffffffffu, before, 0);
+                    if (before != nstep - 1) continue;
                     __threadfence_block();
-                    before = atomicAdd(&sh.arrived[slot][lq], 1);
-                }
-                before = __shfl_sync(0xffffffffu, before, 0);
-                if (before != nstep - 1) continue;
-                __threadfence_block();
-                if (lane == 0) sh.arrived[slot][lq] = 0;
-                L = 0.f;
-                if (pass == 1) {
-                    M = pm[0];
-                    for (int q = 1; q < nstep; ++q) M = fmaxf(M, pm[q * TILE]);
-                    for (int q = 0; q < nstep; ++q) L += pl[q * TILE] * ex2(pm[q * TILE] - M);
-                } else {
-                    for (int q = 0; q < nstep; ++q) L += pl[q * TILE];
+                    if (lane == 0) sh.arrived[slot][lq] = 0;
+                    L = 0.f;
+                    if (pass == 1) {
+                        M = pm[0];
+                        for (int q = 1; q < nstep; ++q) M = fmaxf(M, pm[q * TILE]);
+                        for (int q = 0; q < nstep; ++q) L += pl[q * TILE] * ex2(pm[q * TILE] - M);
+                    } else {
+                        for (int q = 0; q < nstep; ++q) L += pl[q * TILE];
+                    }
+                    bad = *abort_flag != 0;      // (read again: another group may have given up before it came here)
                 }
             }
-            // (read after all have delivered: a warp whose wait ran out raised the flag before it came here)
-            if (*abort_flag != 0) L = NAN;
+            if (bad) { M = 0.f; L = NAN; }
             if (gi < S) {
                 const size_t at = (size_t)w.head * S + gi;
                 if (pass == 1) {

@@ -86,6 +86,49 @@ def test_a_piece_that_gave_up_marks_every_row_and_score_that_depends_on_it():
         assert torch.equal(got[~bad], good[~bad])
 
 
+@pytest.mark.parametrize("H,S,dtype", [(300, 500, torch.bfloat16), (750, 200, torch.float32)])
+def test_after_a_give_up_every_item_of_the_block_is_marked(H, S, dtype):
+    """More items per block than the passes have buffers to join an item's parts in.  Block 1 gives up at its first step:
+    every row (key) of every item it has a step of is NaN, none keeps what was in memory before, and the other blocks'
+    are those of the library.  bf16: items stay whole here and are dealt back and forth, longest first; fp32: block c takes
+    the steps from c q on."""
+    lib = ctypes.CDLL(build.build_waittest())
+    D, T, P = 64, (S + 127) // 128, 148
+    g = torch.Generator(device="cuda").manual_seed(S)
+    Q, K = ((torch.randn(1, H, S, D, generator=g, device="cuda") * s).to(dtype) for s in (2, 1))
+    p = kvm.make_params(1, H, H, S, D, dtype)
+    ws = torch.zeros(kvm.kvm_workspace_bytes(p), dtype=torch.uint8, device="cuda")
+    scores, lse = (torch.full((1, H, S), 5.0, device="cuda") for _ in range(2))
+    good_scores, good_lse = torch.empty_like(scores), torch.empty_like(lse)
+    kvm.kvm_row_lse(p, Q, K, good_lse, ws)
+    kvm.kvm_score(p, Q, K, good_lse, good_scores, ws)
+    kvm.kvm_row_lse(p, Q, K, good_lse, ws)                        # (finite states in the workspace)
+    size, st = ctypes.c_size_t(ws.numel()), ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    assert lib.kvm_row_lse(ctypes.byref(p), *_ptrs(Q, K, lse, ws), size, st) == 0
+    assert lib.kvm_score(ctypes.byref(p), *_ptrs(Q, K, good_lse, scores, ws), size, st) == 0
+    torch.cuda.synchronize()
+    bad_rows, bad_keys = (torch.zeros(H, T * 128, dtype=torch.bool) for _ in range(2))
+    if dtype == torch.bfloat16:
+        for f in range(H * T // P + 1):
+            k = f * P + (P - 2 if f & 1 else 1)
+            if k < H * T:
+                bad_rows[k % H, (T - 1 - k // H) * 128:(T - k // H) * 128] = True
+                bad_keys[k % H, k // H * 128:(k // H + 1) * 128] = True
+    else:
+        tri = T * (T + 1) // 2
+        q = -(-H * tri // P)
+        for h in range(H):
+            for n in range(T):                                    # an item of n + 1 steps that starts at step s of the pass
+                s = h * tri + n * (n + 1) // 2
+                if s < 2 * q and s + n + 1 > q:
+                    bad_rows[h, n * 128:(n + 1) * 128] = True
+                    bad_keys[h, (T - 1 - n) * 128:(T - n) * 128] = True
+    for got, good, bad in ((lse, good_lse, bad_rows), (scores, good_scores, bad_keys)):
+        bad = bad[None, :, :S].cuda()
+        assert bad.any() and torch.equal(torch.isnan(got), bad)
+        assert torch.equal(got[~bad], good[~bad])
+
+
 def test_the_prefill_attention_kernel_also_comes_back_and_reports():
     """Same build, the attention kernel: its producer leaves out the fourth V tile of every work item that has one,
     the MMA thread's wait for it runs out, the kernel returns, the status is set, the rows that were in hand are NaN
