@@ -22,11 +22,11 @@ def sources():
 
 
 # A second library for the tests of the give-up paths of the bounded device waits: the same sources with a short
-# wait limit and producers that leave out one stage (the prefill attention's in every block, the score passes' in one),
+# wait limit and producers that leave out one stage (the prefill attention's in every block, the score passes' and the decode attention's in one),
 # so that a wait runs out, the kernel returns and reports it.  It is never loaded by the package itself.
 WAITTEST_LIB = os.path.join(_PKG, "libkvm_waittest.so")
 WAITTEST_FLAGS = ("-DKVM_TEST_WAIT_LIMIT_CLOCKS=4000000ll", "-DKVM_TEST_DROP_B_STAGE=3", "-DKVM_TEST_DROP_SCORE_STEP=0",
-                  "-DKVM_TEST_DROP_CTA=1")
+                  "-DKVM_TEST_DROP_ATTEND_STAGE=0", "-DKVM_TEST_DROP_CTA=1")
 
 
 def _stale(lib: str = LIB) -> bool:

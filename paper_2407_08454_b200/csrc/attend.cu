@@ -102,6 +102,17 @@ __device__ __forceinline__ bool take_share(Work& w, Item& it, ShareSmem& sh) {
     return true;
 }
 
+// Copies complete on their own; the copying thread, which has issued k stages, stays until its last ones have landed (the
+// wait is bounded like the others), so that a block whose other warps gave up does not hand its shared memory back under a
+// copy in flight.
+__device__ __forceinline__ void drain(uint64_t* full, uint32_t k) {
+    for (uint32_t s = 0; s < ATT_STAGES && s < k; ++s) {
+        const uint32_t parity = ((k - 1 - s) / ATT_STAGES) & 1;
+        const long long t0 = clock64();
+        while (!mbar_try(&full[s], parity) && clock64() - t0 <= WAIT_LIMIT_CLOCKS) {}
+    }
+}
+
 // Piece end: the warps' states (sm_m, sm_l, sm_acc [warp][GH][D]) in a fixed order -> the piece's state of `heads` heads at
 // dst: per head D weighted sums, the maximum and the sum.
 template <int D, int GH>
@@ -228,6 +239,9 @@ attend_partial_fma_kernel(const T* __restrict__ q, const T* __restrict__ K, cons
                     const int s = k % ATT_STAGES;
                     ok = mbar_wait(&empty[s], ((k / ATT_STAGES) & 1) ^ 1, &s_bad);
                     if (!ok) break;
+#ifdef KVM_TEST_DROP_ATTEND_STAGE
+                    if (blockIdx.x == KVM_TEST_DROP_CTA && k == (uint32_t)(KVM_TEST_DROP_ATTEND_STAGE)) continue;   // test build only: this stage never arrives
+#endif
                     const uint32_t bytes = (uint32_t)min(SROWS, it.cnt - r) * D * sizeof(T);
                     const uint32_t dst = smem_u32(ring + s * 2 * ATT_STAGE_BYTES), bar = smem_u32(&full[s]);
                     mbar_expect_tx(&full[s], 2 * bytes);
@@ -238,6 +252,7 @@ attend_partial_fma_kernel(const T* __restrict__ q, const T* __restrict__ K, cons
                 }
                 w.f += it.cnt;
             }
+            drain(full, k);
         }
         if (!CL) return;
         __syncwarp();
@@ -453,6 +468,9 @@ attend_partial_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
                     const int s = k % ATT_STAGES;
                     ok = mbar_wait(&empty[s], ((k / ATT_STAGES) & 1) ^ 1, &s_bad);
                     if (!ok) break;
+#ifdef KVM_TEST_DROP_ATTEND_STAGE
+                    if (blockIdx.x == KVM_TEST_DROP_CTA && k == (uint32_t)(KVM_TEST_DROP_ATTEND_STAGE)) continue;   // test build only: this stage never arrives
+#endif
                     mbar_expect_tx(&full[s], 2 * ATT_STAGE_BYTES);
                     uint8_t* st = ring + s * 2 * ATT_STAGE_BYTES;
 #pragma unroll
@@ -463,6 +481,7 @@ attend_partial_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
                 }
                 w.f += it.cnt;
             }
+            drain(full, k);
         }
         if (!CL) return;
         __syncwarp();

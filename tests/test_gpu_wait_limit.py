@@ -129,6 +129,27 @@ def test_after_a_give_up_every_item_of_the_block_is_marked(H, S, dtype):
         assert torch.equal(got[~bad], good[~bad])
 
 
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("U,G,rows,bad", [
+    (4, 4, 512, [0]),              # clusters: block 1 holds rows of unit 0
+])
+def test_the_decode_attention_kernels_also_come_back_and_mark_their_units(U, G, rows, bad, dtype):
+    """Block 1 leaves out its first stage: the units that it holds rows of are NaN, the others are the library's."""
+    lib = ctypes.CDLL(build.build_waittest())
+    g = torch.Generator().manual_seed(U)
+    q, K, V = (torch.randn(1, h, n, 64, generator=g).to(dtype).cuda() for h, n in ((U * G, 1), (U, rows), (U, rows)))
+    p = kvm.make_params(1, U * G, U, rows, 64, dtype, budget=1.0, recent_ratio=0.0, heavy_ratio=0.0)
+    ws = torch.zeros(kvm.kvm_workspace_bytes(p), dtype=torch.uint8, device="cuda")
+    out, good = (torch.full((U, G, 64), 5.0, device="cuda") for _ in range(2))
+    size, st = ctypes.c_size_t(ws.numel()), ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    assert lib.kvm_attend(ctypes.byref(p), *_ptrs(q, K, V), ctypes.c_int32(rows), *_ptrs(None, out, ws), size, st) == 0
+    torch.cuda.synchronize()                        # the kernels came back by themselves
+    kvm.kvm_attend(p, q.squeeze(2).contiguous(), K, V, rows, None, good, ws)
+    assert torch.isfinite(good).all() and torch.isnan(out[bad]).all()
+    rest = [u for u in range(U) if u not in bad]
+    assert torch.equal(out[rest], good[rest])
+
+
 def test_the_prefill_attention_kernel_also_comes_back_and_reports():
     """Same build, the attention kernel: its producer leaves out the fourth V tile of every work item that has one,
     the MMA thread's wait for it runs out, the kernel returns, the status is set, the rows that were in hand are NaN
