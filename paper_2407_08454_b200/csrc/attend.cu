@@ -627,7 +627,7 @@ __global__ void __launch_bounds__(D) attend_combine_kernel(const float* __restri
             M = mn;
         }
     }
-    out[(size_t)blockIdx.x * D + threadIdx.x] = L > 0.f || L != L ? o / L : 0.f;
+    out[(size_t)blockIdx.x * D + threadIdx.x] = L > 0.f || L != L || o != o ? o / L : 0.f;   // (o alone is NaN where every piece gave up)
 }
 
 // err = |O - O*|_2 and ref = |O|_2 per (batch, query head).
