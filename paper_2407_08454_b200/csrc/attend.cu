@@ -397,7 +397,8 @@ attend_partial_fma_kernel(const T* __restrict__ q, const T* __restrict__ K, cons
 //   S = K q^T   16 rows x 8 heads per product chain (K rows as they lie, q as the constant operand)
 //   O^T += V^T P  16 channels x 8 heads per product; P enters as three bf16 terms (24 bits, exact), V is bf16 already,
 //               and every 16 rows' products start from zero and are added in fp32, so that nothing is rounded earlier
-//               than in fp32 arithmetic
+//               than in fp32 arithmetic.  The terms are all positive, so that an infinite V times any weight is infinite
+//               as in fp32 arithmetic (a term that is zero or negative would make it NaN)
 // Rows come by TMA with the 128-byte swizzle (ldmatrix without bank conflicts).
 __device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t addr) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
@@ -415,6 +416,14 @@ __device__ __forceinline__ uint32_t transpose8x8(uint32_t x) {
     uint32_t r;
     asm("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(r) : "r"(x));
     return r;
+}
+
+// Takes the largest bf16 number below x out of x (8 bits; what is left is exact), but at least `least`.  Three of these
+// use up a positive fp32 number without ever leaving zero: 1 = 255/256 + 255/65536 + 1/65536.  (x = 0 with least = 0: 0.)
+__device__ __forceinline__ uint32_t take_bf16(float& x, float least) {
+    const float t = fmaxf(__uint_as_float((__float_as_uint(x) - 1u) & 0xffff0000u), least);
+    x -= t;
+    return __float_as_uint(t);
 }
 
 constexpr int MMA_GH = 8;                   // query heads of a product
@@ -544,21 +553,20 @@ attend_partial_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
                         for (int e = 0; e < 4; ++e) o[dt][e] *= alpha[e & 1];
                 }
                 // weights, as three bf16 terms each, in the B operand's layout (rows 2 tig.. of head gid)
-                float p[4];
+                float p[4], least[4];                              // (least: the smallest bf16 number, 0 for a weight of 0)
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     p[e] = rescale(x[e], m[e & 1]);
                     l[e & 1] += p[e];
+                    least[e] = p[e] > 0.f ? __uint_as_float(0x00010000u) : 0.f;
                 }
                 uint32_t pb[3][2];
 #pragma unroll
                 for (int t = 0; t < 3; ++t)
 #pragma unroll
                     for (int y = 0; y < 2; ++y) {
-                        const uint32_t pk = Vec<__nv_bfloat16>::pack2(p[2 * y], p[2 * y + 1]);
-                        p[2 * y] -= __uint_as_float(pk << 16);     // exact
-                        p[2 * y + 1] -= __uint_as_float(pk & 0xffff0000u);
-                        pb[t][y] = transpose8x8(pk);
+                        const uint32_t lo = take_bf16(p[2 * y], least[2 * y]), hi = take_bf16(p[2 * y + 1], least[2 * y + 1]);
+                        pb[t][y] = transpose8x8(__byte_perm(lo, hi, 0x7632));
                     }
                 // rows that do not exist may hold anything: their V becomes zero (masks of the operand's rows 2 tig.. + 8)
                 uint32_t mask[2] = {0xffffffffu, 0xffffffffu};

@@ -40,3 +40,25 @@ def test_attend_against_fp64(B, G, Hkv, rows, D, dtype):
         qk = (q.double().norm(dim=-1).max() * K.double().norm(dim=-1).max() / D ** 0.5).item()
         tol = (2 * (D / 16 + 4) * 2.0 ** -23 * qk + 2.0 ** -20) * V.double().abs().max().item()
         assert (out.double().view_as(ref) - ref).abs().max().item() <= tol
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("G,Hkv,rows,D", [(1, 2, 300, 64), (4, 3, 2000, 128), (2, 200, 333, 64), (8, 150, 400, 128)])
+def test_attend_with_infinite_values(G, Hkv, rows, D, dtype):
+    """An infinite value in a row that has any weight makes its channel infinite, and no other."""
+    g = torch.Generator().manual_seed(rows + G)
+    q = torch.randn(1, Hkv * G, D, generator=g).to(dtype).cuda()
+    K = torch.randn(1, Hkv, rows, D, generator=g).to(dtype).cuda()
+    V = torch.randn(1, Hkv, rows, D, generator=g).to(dtype).cuda()
+    V[0, 0, 0, 3], V[0, 1, rows - 1, 5], V[0, -1, rows // 2, D - 1] = float("inf"), float("-inf"), float("inf")
+    V[0, -1, 7, D - 1], V[0, -1, rows // 3, 0], V[0, -1, rows // 3 + 1, 0] = float("inf"), float("inf"), float("-inf")
+    p = kvm.make_params(1, Hkv * G, Hkv, rows, D, dtype, budget=1.0, recent_ratio=0.0, heavy_ratio=0.0)
+    ws = torch.empty(kvm.kvm_workspace_bytes(p), dtype=torch.uint8, device="cuda")
+    out = torch.empty(1, Hkv * G, D, device="cuda")
+    kvm.kvm_attend(p, q, K, V, rows, None, out, ws)
+    L = (q.double().view(1, Hkv, G, D) @ K.double().transpose(-1, -2)) / D ** 0.5
+    ref = (torch.softmax(L, -1) @ V.double()).view_as(out)
+    for test in (torch.isposinf, torch.isneginf, torch.isnan):
+        assert torch.equal(test(out), test(ref)) and test(ref).any()
+    fine = torch.isfinite(ref)
+    assert (out.double() - ref)[fine].abs().max().item() <= 1e-4      # |V| is below 5: fp32 sums, logits off by ~1e-5
