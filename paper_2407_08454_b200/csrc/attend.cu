@@ -12,7 +12,8 @@
 //     its own; eight warps compute.
 // A group of LPR lanes owns four rows of a stage.  Its products (rows x heads) are summed across the lanes by a
 // transposing butterfly that leaves each lane one (row, head) to exponentiate; the weights come back by shuffle for
-// the second product.  The reference maximum moves only when it has been outgrown by 8 (log2 units).
+// the second product.  The weights' reference is never below a logit (no weight exceeds 1, as with the plain running maximum)
+// and moves only when it is: to 8 above the new maximum (log2 units), so that a slowly growing maximum moves it seldom.
 // A unit's rows that fall into several blocks' shares leave partial states (weighted V sum, maximum, sum), combined in a
 // fixed order by a second kernel: results are reproducible.
 #include <mutex>
@@ -31,7 +32,7 @@ constexpr int ATT_STAGE_BYTES = 16384;      // of K, and as much of V
 constexpr int ATT_MIN_SHARE = 64;           // fewest rows a block is given (bounds the number of pieces)
 constexpr int RPI = 4;                      // rows of a stage per lane group
 constexpr float LOG2E = 1.4426950408889634f;
-constexpr float REF_STEP = 8.f;             // the reference maximum follows in steps of at least this (log2 units)
+constexpr float REF_STEP = 8.f;             // room above the maximum that the reference is set with (log2 units)
 
 // Weight of a partial state with maximum m when the overall maximum is M (an empty state has m = -inf).
 __device__ __forceinline__ float rescale(float m, float M) { return m == -INFINITY ? 0.f : exp2f(m - M); }
@@ -319,10 +320,10 @@ attend_partial_fma_kernel(const T* __restrict__ q, const T* __restrict__ K, cons
             }
 #pragma unroll
             for (int o = REP; o < REP * RL; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-            const bool grow = mx > m + REF_STEP || (m == -INFINITY && mx > -INFINITY);
+            const bool grow = mx > m;
             if (__any_sync(0xffffffffu, grow)) {
-                const float alpha = grow ? exp2f(m - mx) : 1.f;
-                if (grow) m = mx;
+                const float mn = grow ? mx + REF_STEP : m, alpha = grow ? exp2f(m - mn) : 1.f;
+                m = mn;
                 l *= alpha;
 #pragma unroll
                 for (int h = 0; h < GH; ++h) {
@@ -535,14 +536,14 @@ attend_partial_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
 #pragma unroll
                 for (int e = 0; e < 4; ++e) x[e] = gid + (e >> 1) * 8 < live ? (c0[e] + c1[e]) * scale_log2e : -INFINITY;
                 const float mx[2] = {fmaxf(x[0], x[2]), fmaxf(x[1], x[3])};
-                if (__any_sync(0xffffffffu, mx[0] > m[0] + REF_STEP || mx[1] > m[1] + REF_STEP)) {
+                if (__any_sync(0xffffffffu, mx[0] > m[0] || mx[1] > m[1])) {
                     float alpha[2];
 #pragma unroll
                     for (int y = 0; y < 2; ++y) {
                         float t = mx[y];
 #pragma unroll
                         for (int z = 4; z < 32; z <<= 1) t = fmaxf(t, __shfl_xor_sync(0xffffffffu, t, z));
-                        const float mn = t > m[y] + REF_STEP ? t : m[y];
+                        const float mn = t > m[y] ? t + REF_STEP : m[y];
                         alpha[y] = rescale(m[y], mn);
                         m[y] = mn;
                         l[y] *= alpha[y];

@@ -62,3 +62,21 @@ def test_attend_with_infinite_values(G, Hkv, rows, D, dtype):
         assert torch.equal(test(out), test(ref)) and test(ref).any()
     fine = torch.isfinite(ref)
     assert (out.double() - ref)[fine].abs().max().item() <= 1e-4      # |V| is below 5: fp32 sums, logits off by ~1e-5
+
+
+@pytest.mark.parametrize("dtype,step", [(torch.bfloat16, 128), (torch.float32, 64)])
+def test_attend_at_the_end_of_the_value_range(dtype, step):
+    """Two rows of a unit have weight, a stage of rows apart in the same lanes' hands, the later one 2^7.5 times the
+    earlier one's: weights are taken relative to a reference that is not below any logit, so that values near the largest
+    number do not overflow on the way."""
+    q = torch.zeros(1, 1, 64, dtype=dtype, device="cuda")
+    q[..., 0] = 8.0
+    K = torch.zeros(1, 1, 2048, 64, dtype=dtype, device="cuda")
+    K[..., 0] = -1000.0
+    K[0, 0, 0, 0], K[0, 0, step, 0] = 0.0, 5.1875
+    V = torch.full_like(K, 3e38)
+    p = kvm.make_params(1, 1, 1, 2048, 64, dtype, budget=1.0, recent_ratio=0.0, heavy_ratio=0.0)
+    ws = torch.empty(kvm.kvm_workspace_bytes(p), dtype=torch.uint8, device="cuda")
+    out = torch.empty(1, 1, 64, device="cuda")
+    kvm.kvm_attend(p, q, K, V, 2048, None, out, ws)
+    assert ((out.double() / V[0, 0, 0].double() - 1).abs() <= 2.0 ** -18).all()
