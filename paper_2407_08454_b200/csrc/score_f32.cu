@@ -101,13 +101,23 @@ __device__ __forceinline__ void load_unit(float4 (&v)[2], const Chunk& c, int u,
     v[0] = in ? __ldg(p) : make_float4(0.f, 0.f, 0.f, 0.f);
     v[1] = in ? __ldg(p + 1) : make_float4(0.f, 0.f, 0.f, 0.f);
 }
+// Eight numbers rounded to bf16, those that would round to infinity to the largest finite number (the residual of fp32's
+// lowest value, say, is then a number).
+__device__ __forceinline__ uint32_t pack2_finite(float lo, float hi) {
+    uint32_t r;
+    asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+    return r;
+}
+__device__ __forceinline__ uint4 pack_finite(const float* f) {
+    return make_uint4(pack2_finite(f[0], f[1]), pack2_finite(f[2], f[3]), pack2_finite(f[4], f[5]), pack2_finite(f[6], f[7]));
+}
 __device__ __forceinline__ void split_unit(const float4 (&v)[2], uint8_t* dst, int u) {
     const int r = u >> 3, piece = u & 7;
     float x[8] = {v[0].x, v[0].y, v[0].z, v[0].w, v[1].x, v[1].y, v[1].z, v[1].w};
     uint8_t* at = dst + r * 128 + ((piece ^ (r & 7)) << 4);
 #pragma unroll
     for (int pl = 0; pl < NPLANE; ++pl) {
-        const uint4 w = Vec<__nv_bfloat16>::pack(x);
+        const uint4 w = pl == 0 ? pack_finite(x) : Vec<__nv_bfloat16>::pack(x);
         *reinterpret_cast<uint4*>(at + (NPLANE - 1 - pl) * PLANE_BYTES) = w;
         if (pl + 1 < NPLANE) {
             float y[8];
@@ -322,7 +332,7 @@ score_f32_kernel(const float* __restrict__ Q, const float* __restrict__ K, float
                     }
                     __syncwarp();                                   // the last step's values have been read
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) nl[e * 32 + lane] = -v[e];
+                    for (int e = 0; e < 4; ++e) nl[e * 32 + lane] = v[e] > -INFINITY || v[e] != v[e] ? -v[e] : -INFINITY;   // (a query with no key to see weighs nothing)
                     __syncwarp();
                 }
                 ok = mbar_wait(&sh.acc_full[grp], own & 1, abort_flag);
@@ -353,6 +363,16 @@ score_f32_kernel(const float* __restrict__ Q, const float* __restrict__ K, float
                     float v[32];
 #pragma unroll
                     for (int c = 0; c < 32; ++c) v[c] = __uint_as_float(hi[c]) + __uint_as_float(lo[c]);
+                    if (PASS == 2) {
+#pragma unroll
+                        for (int c = 0; c < 32; c += 4) {
+                            const float4 x = *reinterpret_cast<const float4*>(nl + cq * 32 + c);
+                            v[c] = fmaf(v[c], scale2, x.x);
+                            v[c + 1] = fmaf(v[c + 1], scale2, x.y);
+                            v[c + 2] = fmaf(v[c + 2], scale2, x.z);
+                            v[c + 3] = fmaf(v[c + 3], scale2, x.w);
+                        }
+                    }
                     if (mask) {
 #pragma unroll
                         for (int c = 0; c < 32; ++c)
@@ -362,22 +382,16 @@ score_f32_kernel(const float* __restrict__ Q, const float* __restrict__ K, float
                         float mx = v[0];
 #pragma unroll
                         for (int c = 1; c + 1 < 32; c += 2) mx = fmax3(mx, v[c], v[c + 1]);
-                        const float mn = fmaxf(m, fmaxf(mx, v[31]) * scale2);
-                        const float f = exp2f(m - mn);
+                        const float mn = fmaxf(m, fmaxf(mx, v[31]) * scale2), ref = mn == -INFINITY ? 0.f : mn;
+                        const float f = exp2f(m - ref);
 #pragma unroll
                         for (int e = 0; e < 4; ++e) l[e] *= f;
 #pragma unroll
-                        for (int c = 0; c < 32; ++c) l[c & 3] += exp2f(fmaf(v[c], scale2, -mn));
+                        for (int c = 0; c < 32; ++c) l[c & 3] += exp2f(fmaf(v[c], scale2, -ref));
                         m = mn;
                     } else {
 #pragma unroll
-                        for (int c = 0; c < 32; c += 4) {
-                            const float4 x = *reinterpret_cast<const float4*>(nl + cq * 32 + c);
-                            l[0] += exp2f(fmaf(v[c], scale2, x.x));
-                            l[1] += exp2f(fmaf(v[c + 1], scale2, x.y));
-                            l[2] += exp2f(fmaf(v[c + 2], scale2, x.z));
-                            l[3] += exp2f(fmaf(v[c + 3], scale2, x.w));
-                        }
+                        for (int c = 0; c < 32; ++c) l[c & 3] += exp2f(v[c]);
                     }
                 }
             }

@@ -47,3 +47,46 @@ def test_scores_and_row_lse_against_fp64(B, Hq, Hkv, S, D):
             for got in (scores, with_lse):
                 # every term of a column sum is off by at most exp(2 delta) - 1; fp32 sums of positive terms add 2^-17
                 assert ((got[b, u].double() - ref).abs() / ref).max().item() <= 2.1 * delta + 2.0 ** -17
+
+
+def _reference(Q, K, allowed):
+    L = (Q.double() @ K.double().transpose(-1, -2) / math.sqrt(Q.shape[-1])).masked_fill(~allowed, float("-inf"))
+    return torch.nan_to_num(torch.softmax(L, -1)).sum(-2)          # (rows without any key weigh nothing)
+
+
+@pytest.mark.parametrize("S,D", [(300, 64), (1000, 128)])
+def test_keys_at_the_lowest_value_get_no_weight(S, D):
+    """Key rows filled with the type's lowest value, as masks are: their logits overflow to -inf, their weight is zero and
+    the other keys' scores are what they are without them, also where a query's first keys are all masked."""
+    g = torch.Generator().manual_seed(S)
+    Q = torch.randn(1, 4, S, D, generator=g).abs().cuda() + 0.1
+    K = torch.randn(1, 4, S, D, generator=g).cuda()
+    masked = torch.zeros(4, S, dtype=torch.bool, device="cuda")
+    masked[0, 3], masked[1, 40:170], masked[2, :40], masked[3, :200] = True, True, True, True
+    K[0][masked] = torch.finfo(torch.float32).min
+    p = kvm.make_params(1, 4, 4, S, D, torch.float32, budget=1.0, recent_ratio=0.0, heavy_ratio=0.0)
+    ws = torch.empty(kvm.kvm_workspace_bytes(p), dtype=torch.uint8, device="cuda")
+    scores, lse, with_lse = (torch.empty(1, 4, S, device="cuda") for _ in range(3))
+    kvm.kvm_score(p, Q, K, None, scores, ws)
+    kvm.kvm_row_lse(p, Q, K, lse, ws)
+    kvm.kvm_score(p, Q, K, lse, with_lse, ws)
+    causal = torch.ones(S, S, dtype=torch.bool, device="cuda").tril()
+    for u in range(4):
+        ref = _reference(Q[0, u], K[0, u].masked_fill(masked[u, :, None], 0.0), causal & ~masked[u])
+        dead = masked[u] & (torch.arange(S, device="cuda") >= masked[u].logical_not().nonzero()[0])
+        for got in (scores[0, u], with_lse[0, u]):
+            assert (got[dead] == 0).all()
+            live = ~masked[u]
+            assert ((got[live].double() - ref[live]).abs() <= 1e-4 * ref[live]).all()
+
+
+def test_a_nan_query_reaches_only_the_keys_before_it():
+    Q, K = (torch.randn(1, 1, 700, 64, generator=torch.Generator().manual_seed(s)).cuda() for s in (1, 2))
+    Q[0, 0, 333, 5] = float("nan")
+    p = kvm.make_params(1, 1, 1, 700, 64, torch.float32, budget=1.0, recent_ratio=0.0, heavy_ratio=0.0)
+    ws = torch.empty(kvm.kvm_workspace_bytes(p), dtype=torch.uint8, device="cuda")
+    scores = torch.empty(1, 1, 700, device="cuda")
+    kvm.kvm_score(p, Q, K, None, scores, ws)
+    assert torch.isnan(scores[0, 0, :334]).all()
+    ref = _reference(torch.nan_to_num(Q[0, 0]), K[0, 0], torch.ones(700, 700, dtype=torch.bool, device="cuda").tril())
+    assert ((scores[0, 0, 334:].double() - ref[334:]).abs() <= 1e-4 * ref[334:]).all()
