@@ -7,7 +7,8 @@
 //   - the query heads of a KV head share a row's one way through shared memory (up to eight at a time; one block per
 //     query head read everything G times through L2: 206 us against 72 us on 8 x 32/8 heads x 12288 rows on average);
 //   - one persistent block per SM takes an equal share of all the rows there are (lengths differ; the shares are cut by
-//     a prefix sum over the units' lengths, so that no SM idles while another finishes a long unit);
+//     a prefix sum over the units' lengths, so that no SM idles while another finishes a long unit; a unit counts as
+//     many rows more as a block could take in the time that starting and joining it costs);
 //   - the rows come by bulk copies into a ring of 16 KB + 16 KB stages, 128 KB in flight per SM, issued by a warp of
 //     its own; eight warps compute.
 // A group of LPR lanes owns four rows of a stage.  Its products (rows x heads) are summed across the lanes by a
@@ -30,33 +31,41 @@ constexpr int ATT_NT = (ATT_WARPS + 1) * 32;
 constexpr int ATT_STAGES = 4;
 constexpr int ATT_STAGE_BYTES = 16384;      // of K, and as much of V
 constexpr int ATT_MIN_SHARE = 64;           // fewest rows a block is given (bounds the number of pieces)
+// What an item costs a block beside its rows, about 3 us, in rows at a block's part of the bandwidth.  (Counted by rows
+// alone, 160 units of up to 3 rows fell to 4 blocks, 40 each: 64 us, 12 so.)
+constexpr int ATT_ITEM_BYTES = 131072;
+__host__ __device__ constexpr int item_rows(int D, int elem) { return ATT_ITEM_BYTES / (2 * D * elem); }
 constexpr int RPI = 4;                      // rows of a stage per lane group
 constexpr float LOG2E = 1.4426950408889634f;
 constexpr float REF_STEP = 8.f;             // room above the maximum that the reference is set with (log2 units)
 
 // Weight of a partial state with maximum m when the overall maximum is M (an empty state has m = -inf).
 __device__ __forceinline__ float rescale(float m, float M) { return m == -INFINITY ? 0.f : exp2f(m - M); }
-// The block's walk over the items of its share.  Item = (unit, group of GH query heads), in that order; `start` counts
-// rows over all items.
+// The block's walk over the items of its share.  Item = (unit, group of GH query heads), in that order.  Shares are cut in
+// a list in which an item with rows is `pad` entries for itself, then one for each of its rows.
 struct Item {
-    unsigned long long start;    // rows of all items before this one
+    unsigned long long start;    // entries of all items before this one
     int id, n;                   // item, rows of its unit
     int off, cnt;                // this block's part: rows [off, off + cnt)
 };
 struct Work {
     const int32_t* len;
-    int rows, HG, items;
-    unsigned long long q, f, f_end;      // rows per block; this block's share [f, f_end)
+    int rows, HG, items, pad;
+    unsigned long long q, f, f_end;      // entries per block; what is left of this block's share: [f, f_end)
     __device__ __forceinline__ int rows_of(int item) const { return len ? max(0, min(__ldg(len + item / HG), rows)) : rows; }
-    // moves to the part of item `it` that belongs to the share (skipping empty items); false when the share is done
-    __device__ __forceinline__ bool settle(Item& it) const {
+    __device__ __forceinline__ int entries(int n) const { return n > 0 ? n + pad : 0; }
+    // moves to the rows of item `it` that belong to the share (skipping items without any); false when the share is done
+    __device__ __forceinline__ bool settle(Item& it) {
         while (f < f_end && it.id < items) {
-            if (it.start + it.n > f) {
-                it.off = (int)(f - it.start);
-                it.cnt = (int)min((unsigned long long)(it.n - it.off), f_end - f);
+            const unsigned long long r0 = it.start + pad, end = it.start + entries(it.n);
+            if (end > f) {
+                if (f < r0) f = r0;
+                if (f >= f_end) return false;
+                it.off = (int)(f - r0);
+                it.cnt = (int)(min(end, f_end) - f);
                 return true;
             }
-            it.start += it.n;
+            it.start = end;
             if (++it.id < items) it.n = rows_of(it.id);
         }
         return false;
@@ -72,7 +81,7 @@ __device__ __forceinline__ bool take_share(Work& w, Item& it, ShareSmem& sh) {
     const int warp = threadIdx.x >> 5, wl = threadIdx.x & 31;
     const int E = (w.items + ATT_NT - 1) / ATT_NT, i0 = min(w.items, (int)threadIdx.x * E), i1 = min(w.items, i0 + E);
     unsigned long long mine = 0;
-    for (int i = i0; i < i1; ++i) mine += w.rows_of(i);
+    for (int i = i0; i < i1; ++i) mine += w.entries(w.rows_of(i));
     unsigned long long inc = mine;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -93,8 +102,8 @@ __device__ __forceinline__ bool take_share(Work& w, Item& it, ShareSmem& sh) {
     if (w.f == w.f_end) return false;
     if (before <= w.f && w.f < before + mine) {                    // true in exactly one thread
         unsigned long long st = before;
-        int id = i0, n = w.rows_of(id);
-        while (st + n <= w.f) { st += n; n = w.rows_of(++id); }
+        int id = i0, n = w.entries(w.rows_of(id));
+        while (st + n <= w.f) { st += n; n = w.entries(w.rows_of(++id)); }
         sh.start = st;
         sh.id = id;
     }
@@ -137,8 +146,9 @@ __device__ __forceinline__ void store_piece(const float (*sm_m)[GH], const float
 // Where a piece's state goes; the block that holds the item's first row also tells how many pieces the item has.
 __device__ __forceinline__ float* piece_slot(const Work& w, const Item& it, float* part, int32_t* pieces, int max_pieces,
                                              int state_floats) {
-    const int first = (int)(it.start / w.q);
-    if (threadIdx.x == 0 && (int)blockIdx.x == first) pieces[it.id] = (int)((it.start + it.n - 1) / w.q) - first + 1;
+    const unsigned long long r0 = it.start + w.pad;
+    const int first = (int)(r0 / w.q);
+    if (threadIdx.x == 0 && (int)blockIdx.x == first) pieces[it.id] = (int)((r0 + it.n - 1) / w.q) - first + 1;
     return part + ((size_t)it.id * max_pieces + (blockIdx.x - first)) * state_floats;
 }
 
@@ -214,7 +224,7 @@ attend_partial_fma_kernel(const T* __restrict__ q, const T* __restrict__ K, cons
 
     const int warp = threadIdx.x >> 5, wl = threadIdx.x & 31;
     Work w;
-    w.len = len; w.rows = rows; w.HG = (G + GH - 1) / GH; w.items = U * w.HG;
+    w.len = len; w.rows = rows; w.HG = (G + GH - 1) / GH; w.items = U * w.HG; w.pad = CL ? 0 : item_rows(D, sizeof(T));
     if (threadIdx.x == 0) {
         for (int i = 0; i < ATT_STAGES; ++i) {
             mbar_init(&full[i], 1);
@@ -452,7 +462,7 @@ attend_partial_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
     const int warp = threadIdx.x >> 5, wl = threadIdx.x & 31;
     const int stride = min(G, MMA_GH);                             // heads a piece's state is laid out for
     Work w;
-    w.len = len; w.rows = rows; w.HG = (G + MMA_GH - 1) / MMA_GH; w.items = U * w.HG;
+    w.len = len; w.rows = rows; w.HG = (G + MMA_GH - 1) / MMA_GH; w.items = U * w.HG; w.pad = CL ? 0 : item_rows(D, 2);
     if (threadIdx.x == 0) {
         for (int i = 0; i < ATT_STAGES; ++i) {
             mbar_init(&full[i], 1);
@@ -693,8 +703,8 @@ struct Scratch {
     int items, gh, mp;
     int32_t* pieces;
     float *states, *out;
-    unsigned grid(int sms, int rows) const {
-        const long long most = ((long long)items * rows + ATT_MIN_SHARE - 1) / ATT_MIN_SHARE;
+    unsigned grid(int sms, int rows, int row_bytes) const {
+        const long long most = ((long long)items * (rows + ATT_ITEM_BYTES / row_bytes) + ATT_MIN_SHARE - 1) / ATT_MIN_SHARE;
         return (unsigned)(most < sms ? most : sms);
     }
     // Blocks of an item's cluster, 0: equal shares and a second kernel.  The estimates (us): a slice of the longest item
@@ -722,7 +732,7 @@ cudaError_t launch_form(KC clustered, KS shares, const Scratch& sc, int smem, in
     if (e != cudaSuccess) return e;
     const int C = sc.cluster(sms, rows, row_bytes);
     joined = C > 0;
-    if (!joined) return launch_dependent(shares, dim3(sc.grid(sms, rows)), dim3(ATT_NT), smem, st, args..., 0, sc.out);
+    if (!joined) return launch_dependent(shares, dim3(sc.grid(sms, rows, row_bytes)), dim3(ATT_NT), smem, st, args..., 0, sc.out);
     return launch_dependent_cluster(clustered, dim3(sc.items * C), dim3(ATT_NT), smem, C, st, args..., C, sc.out);
 }
 

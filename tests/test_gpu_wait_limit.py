@@ -132,7 +132,8 @@ def test_after_a_give_up_every_item_of_the_block_is_marked(H, S, dtype):
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
 @pytest.mark.parametrize("U,G,rows,bad", [
     (4, 4, 512, [0]),              # clusters: block 1 holds rows of unit 0
-    (300, 4, 600, [2, 3, 4]),      # equal shares of 1217 rows: block 1 holds the end of unit 2, all of 3, the start of 4
+    (300, 4, 600, [2, 3]),         # equal shares: block 1 holds all rows of units 2 and 3
+    (200, 4, 3000, [1, 2]),        # ... the end of unit 1 and the beginning of unit 2
 ])
 def test_the_decode_attention_kernels_also_come_back_and_mark_their_units(U, G, rows, bad, dtype):
     """Block 1 leaves out its first stage: the units that it holds rows of are NaN, the others are the library's."""
