@@ -703,20 +703,40 @@ inline int head_group(const Dims& d) {
 // Pieces an item can fall into: shares are at least ATT_MIN_SHARE rows.
 inline int most_pieces(int rows) { return (rows + ATT_MIN_SHARE - 2) / ATT_MIN_SHARE + 1; }
 
-// SM count of the current device; the kernel's shared-memory opt-in, once per device.
-template <typename... KArgs>
-cudaError_t prepare_kernel(void (*kernel)(KArgs...), int smem, int (&sms_of)[KVM_MAX_DEVICES], std::mutex& mu, int& sms) {
+// What the current device holds of a kernel's two forms at a time: SMs, and clusters of 1, 2, 4 and 8 blocks (a cluster
+// lies within a GPC, whose SMs eight rarely divides: 15 clusters of eight, 33 of four on 148 SMs).
+struct Room {
+    int sms = 0, clusters[4] = {};
+};
+// Finds it out once per device, together with the shared-memory opt-in.
+template <typename KC, typename KS>
+cudaError_t prepare_forms(KC clustered, KS shares, int smem, Room (&room_of)[KVM_MAX_DEVICES], std::mutex& mu, Room& room) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= KVM_MAX_DEVICES) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lock(mu);
-    if (!sms_of[dev]) {
-        if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
-        if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-        sms_of[dev] = sms;
+    if (!room_of[dev].sms) {
+        Room r;
+        if ((e = cudaFuncSetAttribute(shares, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
+        if ((e = cudaFuncSetAttribute(clustered, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
+        if ((e = cudaDeviceGetAttribute(&r.sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+        for (int i = 0; i < 4; ++i) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3((unsigned)(r.sms << i));
+            cfg.blockDim = dim3(ATT_NT);
+            cfg.dynamicSmemBytes = smem;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = 1u << i;
+            attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            if ((e = cudaOccupancyMaxActiveClusters(&r.clusters[i], clustered, &cfg)) != cudaSuccess) return e;
+        }
+        room_of[dev] = r;
     }
-    sms = sms_of[dev];
+    room = room_of[dev];
     return cudaSuccess;
 }
 
@@ -732,11 +752,14 @@ struct Scratch {
     // through one SM at 65 bytes/ns, or at its part of 6.5 TB/s when many are at work; an equal share of the rows
     // (lengths are three quarters of the capacity on average), 5 us of a second kernel and 0.2 us per piece it joins.
     // Measured: 32 units x 1536 rows x 128 in bf16 8.4 (cluster) / 12.8 (shares), 4 x 16384 18.0 / 22.3, 64 x 16384
-    // 70.0 / 64.4, 1 x 32768 24.4 / 40.3.
-    int cluster(int sms, int rows, int row_bytes) const {
+    // 70.0 / 64.4, 1 x 32768 24.4 / 40.3.  All clusters have to be at work at the same time: 16 units x 8192 rows take 25.9
+    // us in clusters of eight, of which 15 fit, and 20.3 in clusters of four.
+    int cluster(const Room& room, int rows, int row_bytes) const {
+        const int sms = room.sms;
         if (items > sms) return 0;
-        int C = 1;
-        while (C < 8 && items * C * 2 <= sms) C *= 2;
+        int i = 3;
+        while (i > 0 && items > room.clusters[i]) --i;
+        const int C = 1 << i;
         const double rate = 6500.0 / (items * C), slice = (double)((rows + C - 1) / C) * row_bytes / (rate < 65.0 ? rate : 65.0);
         const double share = 0.75 * items * rows * row_bytes / 6500.0 + 5e3 + 2e2 * (1 + sms / items);
         return slice <= share ? C : 0;
@@ -746,14 +769,13 @@ struct Scratch {
 // One of a kernel's two forms on the stream.
 template <typename KC, typename KS, typename... Args>
 cudaError_t launch_form(KC clustered, KS shares, const Scratch& sc, int smem, int rows, int row_bytes, std::mutex& mu,
-                        int (&sms_of)[2][KVM_MAX_DEVICES], cudaStream_t st, bool& joined, Args... args) {
-    int sms = 0;
-    cudaError_t e = prepare_kernel(shares, smem, sms_of[0], mu, sms);
-    if (e == cudaSuccess) e = prepare_kernel(clustered, smem, sms_of[1], mu, sms);
+                        Room (&room_of)[KVM_MAX_DEVICES], cudaStream_t st, bool& joined, Args... args) {
+    Room room;
+    const cudaError_t e = prepare_forms(clustered, shares, smem, room_of, mu, room);
     if (e != cudaSuccess) return e;
-    const int C = sc.cluster(sms, rows, row_bytes);
+    const int C = sc.cluster(room, rows, row_bytes);
     joined = C > 0;
-    if (!joined) return launch_dependent(shares, dim3(sc.grid(sms, rows, row_bytes)), dim3(ATT_NT), smem, st, args..., 0, sc.out);
+    if (!joined) return launch_dependent(shares, dim3(sc.grid(room.sms, rows, row_bytes)), dim3(ATT_NT), smem, st, args..., 0, sc.out);
     return launch_dependent_cluster(clustered, dim3(sc.items * C), dim3(ATT_NT), smem, C, st, args..., C, sc.out);
 }
 
@@ -762,9 +784,9 @@ cudaError_t launch_fma(const Dims& d, const void* q, const void* K, const void* 
                        const Scratch& sc, cudaStream_t st, bool& joined) {
     constexpr int smem = ATT_STAGES * 2 * ATT_STAGE_BYTES + (ATT_WARPS * D + D + 2) * GH * (int)sizeof(float);
     static std::mutex mu;
-    static int sms_of[2][KVM_MAX_DEVICES] = {};
+    static Room room_of[KVM_MAX_DEVICES];
     return launch_form(attend_partial_fma_kernel<T, D, GH, true>, attend_partial_fma_kernel<T, D, GH, false>, sc, smem, rows,
-                       2 * D * (int)sizeof(T), mu, sms_of, st, joined, (const T*)q, (const T*)K, (const T*)V, len, sc.states,
+                       2 * D * (int)sizeof(T), mu, room_of, st, joined, (const T*)q, (const T*)K, (const T*)V, len, sc.states,
                        sc.pieces, rows, d.G, d.U, sc.mp, d.scale * LOG2E);
 }
 template <int D>
@@ -772,11 +794,11 @@ cudaError_t launch_mma(const Dims& d, const void* q, const void* K, const void* 
                        const Scratch& sc, cudaStream_t st, bool& joined) {
     constexpr int smem = 1024 + ATT_STAGES * 2 * ATT_STAGE_BYTES + (ATT_WARPS * D + D + 2) * MMA_GH * (int)sizeof(float);
     static std::mutex mu;
-    static int sms_of[2][KVM_MAX_DEVICES] = {};
+    static Room room_of[KVM_MAX_DEVICES];
     CUtensorMap mk, mv;
     if (!make_map(&mk, K, d.U, rows, D, ATT_STAGE_BYTES / (2 * D)) || !make_map(&mv, V, d.U, rows, D, ATT_STAGE_BYTES / (2 * D)))
         return cudaErrorNotSupported;
-    return launch_form(attend_partial_mma_kernel<D, true>, attend_partial_mma_kernel<D, false>, sc, smem, rows, 4 * D, mu, sms_of,
+    return launch_form(attend_partial_mma_kernel<D, true>, attend_partial_mma_kernel<D, false>, sc, smem, rows, 4 * D, mu, room_of,
                        st, joined, mk, mv, (const __nv_bfloat16*)q, len, sc.states, sc.pieces, rows, d.G, d.U, sc.mp,
                        d.scale * LOG2E);
 }
