@@ -17,6 +17,7 @@
 // and moves only when it is: to 8 above the new maximum (log2 units), so that a slowly growing maximum moves it seldom.
 // A unit's rows that fall into several blocks' shares leave partial states (weighted V sum, maximum, sum), combined in a
 // fixed order by a second kernel: results are reproducible.
+// Two more forms, for few units (clusters) and for many short ones (small blocks), below; Scratch::choose says which is when.
 #include <mutex>
 #include <type_traits>
 
@@ -623,6 +624,100 @@ attend_partial_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
     if (CL) join_cluster<D>(fin, item, w.HG, MMA_GH, G, C, out);
 }
 
+// ------------------------------------------------------------------ short units in numbers: small blocks, several per SM
+// An item costs a persistent block about 3 us beside its rows (lengths, queries, the joining of its warps, one after the
+// other), which nothing hides where the items are short and many.  Here every (query head, chunk of rows) is a block of its
+// own, four to an SM: a group of LPR lanes takes four rows at a time from memory straight into registers.  The query heads
+// of a KV head read its rows one by one (through L2), which is why this form is for few of them.
+constexpr int ROW_NT = 256, ROW_BLOCKS_PER_SM = 4;
+constexpr int ROW_MIN_CHUNK = 64;           // fewest rows of a chunk (bounds the number of pieces)
+template <typename T, int D>
+__global__ void __launch_bounds__(ROW_NT) attend_partial_rows_kernel(const T* __restrict__ q, const T* __restrict__ K,
+                                                                     const T* __restrict__ V, const int32_t* __restrict__ len,
+                                                                     float* __restrict__ part, int32_t* __restrict__ pieces,
+                                                                     int rows, int chunk, int G, float scale_log2e) {
+    constexpr int N = Vec<T>::N, LPR = D / N, NGRP = ROW_NT / LPR;
+    __shared__ float sm_m[NGRP], sm_l[NGRP];
+    __shared__ __align__(16) float sm_acc[NGRP][D];
+    const int split = blockIdx.x, bh = blockIdx.y, u = bh / G;     // b * Hq + h = unit * G + head of the group
+    grid_dependency_wait();
+    const int n = len ? max(0, min(len[u], rows)) : rows;
+    const int r0 = split * chunk, r1 = min(r0 + chunk, n);
+    const int grp = threadIdx.x / LPR, lane = threadIdx.x % LPR;
+    const unsigned gmask = (LPR == 32) ? 0xffffffffu : (((1u << LPR) - 1u) << ((threadIdx.x % 32) / LPR * LPR));
+    const T* Ku = K + (size_t)u * rows * D;
+    const T* Vu = V + (size_t)u * rows * D;
+    float qf[N];
+    Vec<T>::unpack(ldg16(q + (size_t)bh * D + lane * N), qf);
+    float m = -INFINITY, l = 0.f, acc[N];
+#pragma unroll
+    for (int e = 0; e < N; ++e) acc[e] = 0.f;
+    for (int r = r0 + grp * RPI; r < r1; r += NGRP * RPI) {
+        uint4 kraw[RPI], vraw[RPI];
+#pragma unroll
+        for (int i = 0; i < RPI; ++i) {
+            const int ri = min(r + i, r1 - 1);                     // clamped rows are loaded but given no weight
+            kraw[i] = ldg16(Ku + (size_t)ri * D + lane * N);
+            vraw[i] = ldg16(Vu + (size_t)ri * D + lane * N);
+        }
+        float s[RPI];
+#pragma unroll
+        for (int i = 0; i < RPI; ++i) {
+            float kf[N];
+            Vec<T>::unpack(kraw[i], kf);
+            s[i] = 0.f;
+#pragma unroll
+            for (int e = 0; e < N; ++e) s[i] = fmaf(qf[e], kf[e], s[i]);
+        }
+#pragma unroll
+        for (int off = 1; off < LPR; off <<= 1)
+#pragma unroll
+            for (int i = 0; i < RPI; ++i) s[i] += __shfl_xor_sync(gmask, s[i], off);
+        float mn = m;
+#pragma unroll
+        for (int i = 0; i < RPI; ++i) {
+            s[i] = r + i < r1 ? s[i] * scale_log2e : -INFINITY;
+            mn = fmaxf(mn, s[i]);
+        }
+        const float corr = rescale(m, mn);
+        l *= corr;
+#pragma unroll
+        for (int e = 0; e < N; ++e) acc[e] *= corr;
+#pragma unroll
+        for (int i = 0; i < RPI; ++i) {
+            const float p = rescale(s[i], mn);                     // 0 for a clamped row
+            float vf[N];
+            if (r + i >= r1) vraw[i] = make_uint4(0, 0, 0, 0);
+            Vec<T>::unpack(vraw[i], vf);
+            l += p;
+#pragma unroll
+            for (int e = 0; e < N; ++e) acc[e] = fmaf(p, vf[e], acc[e]);
+        }
+        m = mn;
+    }
+    if (lane == 0) { sm_m[grp] = m; sm_l[grp] = l; }
+#pragma unroll
+    for (int e = 0; e < N; ++e) sm_acc[grp][lane * N + e] = acc[e];
+    __syncthreads();
+    if (threadIdx.x < D) {
+        float M = -INFINITY, L = 0.f, o = 0.f;
+#pragma unroll
+        for (int g = 0; g < NGRP; ++g) M = fmaxf(M, sm_m[g]);
+#pragma unroll
+        for (int g = 0; g < NGRP; ++g) {
+            const float w = rescale(sm_m[g], M);
+            L = fmaf(sm_l[g], w, L);
+            o = fmaf(sm_acc[g][threadIdx.x], w, o);
+        }
+        float* dst = part + ((size_t)bh * gridDim.x + split) * (D + 2);
+        dst[threadIdx.x] = o;
+        if (threadIdx.x == 0) {
+            dst[D] = M; dst[D + 1] = L;
+            if (split == 0) pieces[bh] = gridDim.x;
+        }
+    }
+}
+
 // One block per query head: its pieces' states in order.
 template <int D>
 __global__ void __launch_bounds__(D) attend_combine_kernel(const float* __restrict__ part, const int32_t* __restrict__ pieces,
@@ -740,67 +835,125 @@ cudaError_t prepare_forms(KC clustered, KS shares, int smem, Room (&room_of)[KVM
     return cudaSuccess;
 }
 
+// The small blocks: as many chunks per query head as keep every SM's blocks busy in one wave.
+template <typename T, int D>
+cudaError_t launch_rows(const Dims& d, const void* q, const void* K, const void* V, int rows, const int32_t* len, float* out,
+                        float* part, int sms, cudaStream_t st) {
+    const int heads = d.B * d.Hq, most = (rows + ROW_MIN_CHUNK - 1) / ROW_MIN_CHUNK;
+    int want = ROW_BLOCKS_PER_SM * sms / heads;
+    want = want < 1 ? 1 : want > most ? most : want;
+    const int chunk = (rows + want - 1) / want, n = (rows + chunk - 1) / chunk;
+    int32_t* pieces = reinterpret_cast<int32_t*>(part);
+    float* states = part + (heads + 3) / 4 * 4;
+    const cudaError_t e = launch_dependent(attend_partial_rows_kernel<T, D>, dim3(n, heads), dim3(ROW_NT), 0, st, (const T*)q,
+                                           (const T*)K, (const T*)V, len, states, pieces, rows, chunk, d.G, d.scale * LOG2E);
+    if (e != cudaSuccess) return e;
+    return launch_dependent(attend_combine_kernel<D>, dim3(heads), dim3(D), 0, st, (const float*)states, (const int32_t*)pieces,
+                            len, out, rows, d.G, 1, n);
+}
+
+// How a call is dealt: clusters of `cluster` blocks per item, small blocks per query head and chunk (`rows`), or, with
+// neither, equal shares.
+struct Form {
+    int cluster = 0;
+    bool rows = false;
+};
+
 struct Scratch {
     int items, gh, mp;
+    float* part;            // the scratch; laid out for the two large forms:
     int32_t* pieces;
     float *states, *out;
     unsigned grid(int sms, int rows, int row_bytes) const {
         const long long most = ((long long)items * (rows + ATT_ITEM_BYTES / row_bytes) + ATT_MIN_SHARE - 1) / ATT_MIN_SHARE;
         return (unsigned)(most < sms ? most : sms);
     }
-    // Blocks of an item's cluster, 0: equal shares and a second kernel.  The estimates (us): a slice of the longest item
-    // through one SM at 65 bytes/ns, or at its part of 6.5 TB/s when many are at work; an equal share of the rows
-    // (lengths are three quarters of the capacity on average), 5 us of a second kernel and 0.2 us per piece it joins.
-    // Measured: 32 units x 1536 rows x 128 in bf16 8.4 (cluster) / 12.8 (shares), 4 x 16384 18.0 / 22.3, 64 x 16384
-    // 70.0 / 64.4, 1 x 32768 24.4 / 40.3.  All clusters have to be at work at the same time: 16 units x 8192 rows take 25.9
-    // us in clusters of eight, of which 15 fit, and 20.3 in clusters of four.
-    int cluster(const Room& room, int rows, int row_bytes) const {
-        const int sms = room.sms;
-        if (items > sms) return 0;
+    // The form that is fastest for full units (lengths are on the device), shares where it is close: they follow the lengths.
+    // Measured in us, bf16, D = 128 unless said otherwise; clusters / shares / small blocks.
+    //   No more items than blocks: by estimates (`block`: bytes/ns that a block of the two large forms gets through, 6.5 TB/s
+    // together): a slice of an item, all clusters being at work at the same time; all rows, a second kernel and the pieces
+    // of an item; every query head's rows through L2, a second kernel and the pieces of a head.  1 unit x 8192 rows 11.6 /
+    // 14.6 / 13.1, 1 x 32768 32 / 20 / 44, 16 x 8192 20.3 (clusters of four) and 25.9 (of eight, of which 15 fit) / 19.0 / 21,
+    // 32 x 2048 10.5 / 12.2 / 11.6, 64 x 16384 half full 72 / 65 / -, one unit of eight fp32 heads x 8192 32 / 18 / 16.
+    //   More items: small blocks while what they save, the items' cost, exceeds their way through L2 per query head.  One
+    // head: - / 107 / 77 (4096 x 200), 50.5 / 49.0 (1024 x 512), 33 / 34 (320 x 1024), 57 / 61 (320 x 2048); in fp32 42 / 41
+    // (1024 x 200), 85 / 93 (1024 x 512).  Two heads: 35.5 / 34.5 (1024 x 200), 54 / 64 (1024 x 512).  Four: 10.1 / 8.2 (160 x
+    // 48), 12.1 / 15.2 (160 x 200), 107 / 110 (4096 x 48).
+    Form choose(const Room& room, const Dims& d, int rows, int row_bytes, double block) const {
+        Form f;
+        const int heads = d.B * d.Hq, sms = room.sms;
+        const double unit = rows * (double)row_bytes;
+        if (items > sms) {
+            f.rows = (d.G * unit <= 208.0 * 1024 && (d.G <= 2 || heads <= 9 * sms)) ||
+                     (d.dtype == KVM_BF16 && d.G == 1 && unit <= 512.0 * 1024);
+            return f;
+        }
+        const double most = (rows + ATT_MIN_SHARE - 1) / ATT_MIN_SHARE;
+        auto pieces = [&](double n) { return n < most ? n : most; };
+        const double all = sms * block < 6500.0 ? sms * block : 6500.0, l2 = d.G == 1 ? 5800.0 : d.G == 2 ? 7700.0 : 9000.0;
+        const double shares = 7.0 + items * unit / 1e3 / all + 0.055 * pieces((double)sms / items);
+        const double small = 6.8 + heads * unit / 1e3 / l2 + 0.06 * pieces((double)ROW_BLOCKS_PER_SM * sms / heads);
         int i = 3;
         while (i > 0 && items > room.clusters[i]) --i;
         const int C = 1 << i;
-        const double rate = 6500.0 / (items * C), slice = (double)((rows + C - 1) / C) * row_bytes / (rate < 65.0 ? rate : 65.0);
-        const double share = 0.75 * items * rows * row_bytes / 6500.0 + 5e3 + 2e2 * (1 + sms / items);
-        return slice <= share ? C : 0;
+        const double part = 6500.0 / (items * C);
+        const double cluster = 4.8 + (rows + C - 1) / C * (double)row_bytes / 1e3 / (part < block ? part : block);
+        if (cluster * 1.06 < shares && cluster < small) f.cluster = C;
+        else f.rows = small < shares;
+        return f;
     }
 };
 
 // One of a kernel's two forms on the stream.
-template <typename KC, typename KS, typename... Args>
-cudaError_t launch_form(KC clustered, KS shares, const Scratch& sc, int smem, int rows, int row_bytes, std::mutex& mu,
-                        Room (&room_of)[KVM_MAX_DEVICES], cudaStream_t st, bool& joined, Args... args) {
-    Room room;
-    const cudaError_t e = prepare_forms(clustered, shares, smem, room_of, mu, room);
+template <int D, typename KC, typename KS, typename... Args>
+cudaError_t launch_form(KC clustered, KS shares, const Dims& d, const Scratch& sc, const Room& room, const Form& f, int smem, int rows,
+                        int row_bytes, const int32_t* len, cudaStream_t st, Args... args) {
+    if (f.cluster)
+        return launch_dependent_cluster(clustered, dim3(sc.items * f.cluster), dim3(ATT_NT), smem, f.cluster, st, args..., f.cluster, sc.out);
+    const cudaError_t e = launch_dependent(shares, dim3(sc.grid(room.sms, rows, row_bytes)), dim3(ATT_NT), smem, st, args..., 0, sc.out);
     if (e != cudaSuccess) return e;
-    const int C = sc.cluster(room, rows, row_bytes);
-    joined = C > 0;
-    if (!joined) return launch_dependent(shares, dim3(sc.grid(room.sms, rows, row_bytes)), dim3(ATT_NT), smem, st, args..., 0, sc.out);
-    return launch_dependent_cluster(clustered, dim3(sc.items * C), dim3(ATT_NT), smem, C, st, args..., C, sc.out);
+    return launch_dependent(attend_combine_kernel<D>, dim3(d.B * d.Hq), dim3(D), 0, st, (const float*)sc.states,
+                            (const int32_t*)sc.pieces, len, sc.out, rows, d.G, sc.gh, sc.mp);
 }
 
 template <typename T, int D, int GH>
 cudaError_t launch_fma(const Dims& d, const void* q, const void* K, const void* V, int rows, const int32_t* len,
-                       const Scratch& sc, cudaStream_t st, bool& joined) {
+                       const Scratch& sc, cudaStream_t st) {
     constexpr int smem = ATT_STAGES * 2 * ATT_STAGE_BYTES + (ATT_WARPS * D + D + 2) * GH * (int)sizeof(float);
+    constexpr int row_bytes = 2 * D * (int)sizeof(T);
+    constexpr double block = GH == 1 ? 80.0 : GH == 2 ? 72.0 : GH == 4 ? 56.0 : 40.0;
+    const auto clustered = attend_partial_fma_kernel<T, D, GH, true>;
+    const auto shares = attend_partial_fma_kernel<T, D, GH, false>;
     static std::mutex mu;
     static Room room_of[KVM_MAX_DEVICES];
-    return launch_form(attend_partial_fma_kernel<T, D, GH, true>, attend_partial_fma_kernel<T, D, GH, false>, sc, smem, rows,
-                       2 * D * (int)sizeof(T), mu, room_of, st, joined, (const T*)q, (const T*)K, (const T*)V, len, sc.states,
-                       sc.pieces, rows, d.G, d.U, sc.mp, d.scale * LOG2E);
+    Room room;
+    const cudaError_t e = prepare_forms(clustered, shares, smem, room_of, mu, room);
+    if (e != cudaSuccess) return e;
+    const Form f = sc.choose(room, d, rows, row_bytes, block);
+    if (f.rows) return launch_rows<T, D>(d, q, K, V, rows, len, sc.out, sc.part, room.sms, st);
+    return launch_form<D>(clustered, shares, d, sc, room, f, smem, rows, row_bytes, len, st, (const T*)q, (const T*)K, (const T*)V,
+                          len, sc.states, sc.pieces, rows, d.G, d.U, sc.mp, d.scale * LOG2E);
 }
 template <int D>
 cudaError_t launch_mma(const Dims& d, const void* q, const void* K, const void* V, int rows, const int32_t* len,
-                       const Scratch& sc, cudaStream_t st, bool& joined) {
+                       const Scratch& sc, cudaStream_t st) {
     constexpr int smem = 1024 + ATT_STAGES * 2 * ATT_STAGE_BYTES + (ATT_WARPS * D + D + 2) * MMA_GH * (int)sizeof(float);
+    constexpr int row_bytes = 4 * D;
+    constexpr double block = D == 128 ? 72.0 : 56.0;
+    const auto clustered = attend_partial_mma_kernel<D, true>;
+    const auto shares = attend_partial_mma_kernel<D, false>;
     static std::mutex mu;
     static Room room_of[KVM_MAX_DEVICES];
+    Room room;
+    const cudaError_t e = prepare_forms(clustered, shares, smem, room_of, mu, room);
+    if (e != cudaSuccess) return e;
+    const Form f = sc.choose(room, d, rows, row_bytes, block);
+    if (f.rows) return launch_rows<__nv_bfloat16, D>(d, q, K, V, rows, len, sc.out, sc.part, room.sms, st);
     CUtensorMap mk, mv;
     if (!make_map(&mk, K, d.U, rows, D, ATT_STAGE_BYTES / (2 * D)) || !make_map(&mv, V, d.U, rows, D, ATT_STAGE_BYTES / (2 * D)))
         return cudaErrorNotSupported;
-    return launch_form(attend_partial_mma_kernel<D, true>, attend_partial_mma_kernel<D, false>, sc, smem, rows, 4 * D, mu, room_of,
-                       st, joined, mk, mv, (const __nv_bfloat16*)q, len, sc.states, sc.pieces, rows, d.G, d.U, sc.mp,
-                       d.scale * LOG2E);
+    return launch_form<D>(clustered, shares, d, sc, room, f, smem, rows, row_bytes, len, st, mk, mv, (const __nv_bfloat16*)q, len,
+                          sc.states, sc.pieces, rows, d.G, d.U, sc.mp, d.scale * LOG2E);
 }
 
 template <int D>
@@ -810,6 +963,7 @@ cudaError_t launch_t(const Dims& d, const void* q, const void* K, const void* V,
     sc.gh = head_group(d);
     sc.items = d.U * ((d.G + sc.gh - 1) / sc.gh);
     sc.mp = most_pieces(rows);
+    sc.part = part;
     sc.pieces = reinterpret_cast<int32_t*>(part);
     sc.states = part + (sc.items + 3) / 4 * 4;
     sc.out = out;
@@ -818,20 +972,18 @@ cudaError_t launch_t(const Dims& d, const void* q, const void* K, const void* V,
               : sc.gh == 2        ? launch_fma<float, D, 2>
               : sc.gh == 4        ? launch_fma<float, D, 4>
                                   : launch_fma<float, D, 8>;
-    bool joined = false;
-    const cudaError_t e = fn(d, q, K, V, rows, len, sc, st, joined);
-    if (e != cudaSuccess || joined) return e;
-    return launch_dependent(attend_combine_kernel<D>, dim3(d.B * d.Hq), dim3(D), 0, st, (const float*)sc.states,
-                            (const int32_t*)sc.pieces, len, out, rows, d.G, sc.gh, sc.mp);
+    return fn(d, q, K, V, rows, len, sc, st);
 }
 
 }  // namespace
 
-// States of every item's pieces and the items' piece counts.
+// The pieces' states and their counts, in the form that needs more.
 size_t attend_scratch_floats(const Dims& d) {
     const int gh = head_group(d);
     const size_t items = (size_t)d.U * ((d.G + gh - 1) / gh);
-    return (items + 3) / 4 * 4 + items * most_pieces(d.S) * gh * (d.D + 2);
+    const size_t shares = (items + 3) / 4 * 4 + items * most_pieces(d.S) * gh * (d.D + 2), heads = (size_t)d.B * d.Hq;
+    const size_t small = (heads + 3) / 4 * 4 + heads * ((d.S + ROW_MIN_CHUNK - 1) / ROW_MIN_CHUNK) * (d.D + 2);
+    return shares > small ? shares : small;
 }
 
 cudaError_t launch_attend(const Dims& d, const void* q, const void* K, const void* V, int rows, const int32_t* len,

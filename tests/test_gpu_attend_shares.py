@@ -17,6 +17,9 @@ pytestmark = pytest.mark.gpu
     (1, 9, 3, 333, 128),       # more query heads than one pass takes
     (3, 2, 37, 97, 64),        # more units than blocks need, shares cut in the middle of units
     (1, 1, 300, 70, 128),      # more units than SMs
+    (1, 1, 600, 129, 64),      # many short units: small blocks, one row past two groups' rounds
+    (3, 2, 70, 200, 128),      # ... for two query heads
+    (1, 8, 200, 150, 64),      # as many units for eight: equal shares
     (4, 4, 100, 3, 64),        # many units of a row or two: shares whose ends fall between units' rows
     (1, 2, 1100, 30, 128),     # several units per share, most of each for the unit itself
 ])
