@@ -300,15 +300,15 @@ def compress_layers(p: KvmParams, layers, sim_thresholds=None, device="cuda", st
     # addresses are worked out from the bases)
     n = len(layers)
     B, H, cap, D = p.batch, p.n_kv_heads, kvm_sizes(p)[0], p.head_dim
-    units, size = B * H, 2 if p.dtype == KVM_BF16 else 4
-    # one allocation per kind for the whole stack (each layer's tensors are views of it), zero-filled
-    kv = torch.zeros(2 * n * units * cap * D, dtype=torch.bfloat16 if size == 2 else torch.float32, device=device)
-    ints = torch.zeros(n * units * (cap + 1), dtype=torch.int32, device=device)
+    units, dtype = B * H, torch.bfloat16 if p.dtype == KVM_BF16 else torch.float32
+    # A layer's rows and positions are one allocation (a layer that the caller drops is freed), zero-filled by one kernel for
+    # the stack; the lengths of all layers are read back together.
+    kv_bytes = units * cap * D * (2 if p.dtype == KVM_BF16 else 4)
+    blobs = [torch.empty(2 * kv_bytes + 4 * units * cap, dtype=torch.uint8, device=device) for _ in range(n)]
+    torch._foreach_zero_(blobs)
+    out_len = torch.zeros((n, B, H), dtype=torch.int32, device=device)
     ws = torch.empty(kvm_layers_workspace_bytes(p, n), dtype=torch.uint8, device=device)
     array = ctypes.c_void_p * n
-
-    def rows(base, step):            # the layers' addresses within a stacked tensor
-        return array(*range(base, base + n * step, step))
 
     for layer in layers:
         assert len(layer) == 3 and all([t.is_contiguous() for t in layer]), "tensors must be contiguous"
@@ -317,12 +317,13 @@ def compress_layers(p: KvmParams, layers, sim_thresholds=None, device="cuda", st
     if sim_thresholds is not None:
         assert len(sim_thresholds) == n
         eps = (ctypes.c_float * n)(*[float(e) for e in sim_thresholds])
-    kv_base, kv_step, ints_base = kv.data_ptr(), units * cap * D * size, ints.data_ptr()
-    _call("kvm_compress_layers", p, n, eps, q, k, v, rows(kv_base, kv_step), rows(kv_base + n * kv_step, kv_step),
-          rows(ints_base, 4 * units), rows(ints_base + 4 * n * units, 4 * units * cap), None, ws.data_ptr(), ws.nbytes,
-          _stream(stream))
-    K_out, V_out = kv.view(2, n, B, H, cap, D).unbind(0)
-    out_len, out_pos = ints[:n * units].view(n, B, H), ints[n * units:].view(n, B, H, cap)
-    out = [Compressed(*ts, None, cap) for ts in zip(K_out.unbind(0), V_out.unbind(0), out_len.unbind(0), out_pos.unbind(0))]
+    bases, len_base = [b.data_ptr() for b in blobs], out_len.data_ptr()
+    _call("kvm_compress_layers", p, n, eps, q, k, v, array(*bases), array(*[b + kv_bytes for b in bases]),
+          array(*range(len_base, len_base + 4 * n * units, 4 * units)), array(*[b + 2 * kv_bytes for b in bases]), None,
+          ws.data_ptr(), ws.nbytes, _stream(stream))
+    out = []
+    for blob, lengths in zip(blobs, out_len.unbind(0)):
+        K_out, V_out = blob[:2 * kv_bytes].view(dtype).view(2, B, H, cap, D).unbind(0)
+        out.append(Compressed(K_out, V_out, lengths, blob[2 * kv_bytes:].view(torch.int32).view(B, H, cap), None, cap))
     ratios = (out_len.cpu().float().mean((1, 2)) / p.seq).tolist()      # the one read-back of the call
     return out, ratios

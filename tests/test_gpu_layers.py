@@ -36,3 +36,14 @@ def test_layers_together_match_layers_alone(n, S, Hq, Hkv, D, dtype, monkeypatch
         assert same >= 0.99
         if torch.equal(together[l].out_pos, ref.out_pos):
             assert torch.equal(together[l].K_out, ref.K_out) and torch.equal(together[l].V_out, ref.V_out)
+
+
+def test_a_layer_that_is_dropped_is_freed():
+    p = kvm.make_params(1, 4, 4, 1024, 128, torch.bfloat16)
+    layers = [tuple(torch.randn(1, 4, 1024, 128, device="cuda").bfloat16() for _ in "QKV") for _ in range(4)]
+    out, _ = kvm.compress_layers(p, layers)
+    size = sum(t.nbytes for t in (out[0].K_out, out[0].V_out, out[0].out_pos))
+    kept, before = out[2].K_out.clone(), torch.cuda.memory_allocated()
+    del out[0]
+    assert before - torch.cuda.memory_allocated() >= size
+    assert torch.equal(out[1].K_out, kept)
