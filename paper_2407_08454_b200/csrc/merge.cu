@@ -23,6 +23,8 @@
 // Sets of one token are copied bit for bit.
 // Variants: average-weighted merging (Section 4.2) is the same kernel with every
 // g_j = 1; pivot-only weights and eviction write single input rows (gather_rows_kernel).
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace kvm {
@@ -415,8 +417,9 @@ cudaError_t launch_n(const Dims& d, const LayersOf<NL>& L, const int32_t* set_st
 template <typename T, int D, int TOK>
 cudaError_t launch_t(const Dims& d, const Layers& L, const int32_t* set_start, const int32_t* set_id, int32_t* out_size,
                      float* scratch, float* set_coef, float* token_d2, kvm_stats* stats, cudaStream_t st) {
-    return L.n == 1 ? launch_n<T, D, TOK>(d, first_of(L), set_start, set_id, out_size, scratch, set_coef, token_d2, stats, st)
-                    : launch_n<T, D, TOK>(d, L, set_start, set_id, out_size, scratch, set_coef, token_d2, stats, st);
+    if constexpr (!std::is_same<T, float>::value)      // (fp32 layers go one by one)
+        if (L.n > 1) return launch_n<T, D, TOK>(d, L, set_start, set_id, out_size, scratch, set_coef, token_d2, stats, st);
+    return launch_n<T, D, TOK>(d, first_of(L), set_start, set_id, out_size, scratch, set_coef, token_d2, stats, st);
 }
 
 }  // namespace

@@ -4,7 +4,7 @@
 // (bounded) for the mbarrier; clock64() before the first issue, after the last issue and after the wait.
 // Every access stays inside the 100 KB of dynamic shared memory and the 512 TMEM columns the block allocates.
 //   nvcc -gencode arch=compute_100a,code=sm_100a -O3 -std=c++17 --expt-relaxed-constexpr \
-//        -I paper_2407_08454_b200/csrc -I include paper_2407_08454_b200/csrc/microbench/mma_rate.cu -o mma_rate -lcuda
+//        -I paper_2407_08454_b200/csrc -I include profiles/mma_rate.cu -o mma_rate -lcuda
 #include <cstdio>
 #include <cuda.h>
 #include <cuda_runtime.h>
