@@ -141,7 +141,8 @@ int kvm_workspace_bytes(const kvm_params* p, size_t* bytes);
  *           the scaled causal logits (e.g. from the prefill attention kernel);
  *           when given, the row pass is skipped.
  *   scores: [batch, n_kv_heads, S] fp32, written.
- * bf16 runs on tensor cores with fp32 accumulation and fp32 softmax; fp32 runs in fp32 FMA.
+ * Both run on tensor cores with fp32 accumulation and fp32 softmax; fp32 rows as exact sums of three bf16 numbers, of whose
+ * products those below 2^-26 of |q||k| are left out.
  */
 int kvm_score(const kvm_params* p, const void* Q, const void* K, const float* lse_in,
               float* scores, void* ws, size_t ws_bytes, void* cuda_stream);
@@ -225,7 +226,8 @@ int kvm_compress_with_lse(const kvm_params* p, const void* Q, const void* K, con
  * on `cuda_stream`, kernels and copy out on two streams of the library's own), so
  * that the copies in both directions overlap each other and the kernels;
  * `cuda_stream` waits for the last copy out, and the caller synchronises it before
- * reading.  The first call on a device creates the two streams and a handful of
+ * reading.  A group's scores may differ in their last bits from those of kvm_compress on
+ * the whole layer (see kvm_compress_layers).  The first call on a device creates the two streams and a handful of
  * events, which live until the process exits (the one piece of state the library
  * keeps); calls are serialised by a host mutex while they enqueue.
  */
@@ -253,6 +255,10 @@ int kvm_layer_ratio(const kvm_params* p, const void* K, float* ratio, float* sim
  * the stream; the workspace is shared, the layers' tensors are not.  Short layers go through the kernels several at a
  * time where the workspace has room for it: kvm_layers_workspace_bytes tells how much lets them (the size for one layer
  * is always enough).
+ * How many go together decides in how many pieces a column of the attention map is added up, so a layer's scores may differ
+ * in their last bits from those of kvm_compress on that layer alone (and with another workspace size, or as part of a
+ * smaller last group): where scores tie to fp32 rounding another token may be conserved or become a pivot.  The same call
+ * with the same workspace size gives the same bits.
  *   Q, K, V, K_out, V_out, out_len, out_pos: HOST arrays of n_layers device pointers, each as in kvm_compress
  *   sim_thresholds: NULL or a HOST array of n_layers floats (read before the call returns)
  *   stats: NULL or one device kvm_stats that accumulates over the layers
@@ -289,8 +295,9 @@ int kvm_prefill_attend(const kvm_params* p, const void* Q, const void* K, const 
  *   q    [batch, n_q_heads, D] in p->dtype
  *   K, V [batch, n_kv_heads, rows, D] in p->dtype, 1 <= rows <= S
  *   len  NULL (every unit holds `rows` rows) or device [U] i32: rows of each unit that are valid
- *   out  [batch, n_q_heads, D] fp32, written; a unit with no rows gives zeros
- * fp32 arithmetic.  Only the shape, dtype and softmax_scale of p are used.
+ *   out  [batch, n_q_heads, D] fp32, written; a unit with no rows gives zeros; NaN where a bounded wait inside the kernel
+ *        gave up
+ * fp32 arithmetic (bf16 rows: exact products, weights of 24 bits, fp32 sums).  Only the shape, dtype and softmax_scale of p are used.
  */
 int kvm_attend(const kvm_params* p, const void* q, const void* K, const void* V, int32_t rows, const int32_t* len,
                float* out, void* ws, size_t ws_bytes, void* cuda_stream);

@@ -62,7 +62,7 @@ int derive(const kvm_params* p, Dims& d) {
     return KVM_OK;
 }
 
-// scratch of the score step: the bf16 path's side tensor, or the fp32 path's states, partial sums and split planes
+// scratch of the score step: the bf16 path's side tensor, and what cut items leave (row states, partial column sums)
 inline size_t score_bytes(const Dims& d) {
     return d.dtype == KVM_BF16 ? score_tc_scratch_bytes(d) : score_f32_scratch_bytes(d);
 }

@@ -19,7 +19,7 @@ namespace plan {
 constexpr int TILE = 128;
 constexpr long long GROUP_BYTES = 40ll << 20;
 constexpr int MIN_ROUNDS = 6;
-constexpr int CTAS = 148;       // (the split is a function of the shape alone, so that results are)
+constexpr int CTAS = 148;       // (the split is a function of the shape alone, that of all layers that go together, so that results are)
 
 struct Plan {
     int NH, U, G, T;            // query heads and units in total, query heads per unit, tiles per head

@@ -30,13 +30,19 @@ def test_layers_together_match_layers_alone(n, S, Hq, Hkv, D, dtype, monkeypatch
     for l, (Q, K, V) in enumerate(layers):
         ref = kvm.Compressor(kvm.make_params(1, Hq, Hkv, S, D, cfg.torch_dtype, sim_threshold=eps[l], **kw))(Q, K, V)
         assert all(torch.equal(getattr(alone[l], k), getattr(ref, k)) for k in ("out_len", "out_pos", "K_out", "V_out"))
-        # together the column sums may be added in other pieces: scores that tie to fp32 rounding may change places
-        assert torch.equal(together[l].out_len, ref.out_len) or (together[l].out_len - ref.out_len).abs().max() <= 2
-        same = (together[l].out_pos == ref.out_pos).float().mean().item()
-        assert same >= 0.99
-        if torch.equal(together[l].out_pos, ref.out_pos):
-            assert torch.equal(together[l].K_out, ref.K_out) and torch.equal(together[l].V_out, ref.V_out)
-
+        # together the column sums may be added in other pieces: scores that tie to fp32 rounding may change places, and
+        # with them a token be conserved or not.  A row that has the same pivot in both results, as its two neighbours
+        # have, is the same set (the similarities are the same) and has to be the same bits.
+        got, rows, same = together[l], 0, 0
+        assert (got.out_len - ref.out_len).abs().max() <= 2
+        for h in range(Hkv):
+            a, b = (c.out_pos[0, h, :int(c.out_len[0, h])].tolist() for c in (got, ref))
+            triples = {t: i for i, t in enumerate(zip([-1] + b, b, b[1:] + [S]))}
+            pairs = [(i, triples[t]) for i, t in enumerate(zip([-1] + a, a, a[1:] + [S])) if t in triples]
+            rows, same = rows + len(b), same + len(pairs)
+            x, y = (torch.tensor(ix, device="cuda") for ix in zip(*pairs))
+            assert torch.equal(got.K_out[0, h, x], ref.K_out[0, h, y]) and torch.equal(got.V_out[0, h, x], ref.V_out[0, h, y])
+        assert same >= 0.97 * rows
 
 def test_a_layer_that_is_dropped_is_freed():
     p = kvm.make_params(1, 4, 4, 1024, 128, torch.bfloat16)

@@ -1,6 +1,6 @@
 """The give-up path of the bounded device waits (failure detection without a fault).
 
-Every wait on an mbarrier in the tensor-core score kernel has a limit; when one runs out the kernel stops
+Every wait on an mbarrier has a limit; in the score kernels, when one runs out the kernel stops
 touching tensor memory, writes NaN for the work items it could not finish, reports KVM_E_DEVICE_TIMEOUT through
 kvm_stats, frees its tensor memory and returns.  Nothing in the shipped library can make a wait run out, so
 this test uses a second build of the same sources (never loaded by the package) in which the limit is two
