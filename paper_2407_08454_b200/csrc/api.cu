@@ -420,9 +420,9 @@ int kvm_compress_layers(const kvm_params* p, int32_t n_layers, const float* sim_
 namespace {
 
 constexpr int kHostChunksMax = 6;
-// (us a call for a Llama2-7B-shaped layer of 4096 tokens, 101 MB in: equal quarters 2223; ratio 0.7 2242, 0.6 2201, 0.5 2136,
-// 0.4 2166, 0.3 2236.  15 heads x 2 x 488 x 64, 5.6 MB in: quarters 387; ratio 0.5 with groups of at least 3 MB 285, 2 MB
-// 209, 1 MB 226)
+// (us a call for a Llama2-7B-shaped layer of 4096 tokens, 101 MB in, in one run: equal quarters 2223; ratio 0.7 2242, 0.6 2201,
+// 0.5 2136, 0.4 2166, 0.3 2236; over several boxes quarters 2203-2225, ratio 0.5 2124-2190.  15 heads x 2 x 488 x 64, 5.6 MB
+// in: quarters 387; ratio 0.5 with groups of at least 3 MB 285, 2 MB 209, 1 MB 226)
 constexpr double kHostRatio = 0.5;
 constexpr long long kHostMinBytes = 2ll << 20;
 

@@ -26,11 +26,12 @@
 // compress call).  Where the pieces' states would not fit 4 MiB (large problems, where whole items balance well
 // anyway) items stay whole and the states are final.  The rule depends on the shape only: results are reproducible.
 //
-// Measured on a B200 (us, row / column pass; FMA tiles before): 16 / 8 heads x 2999 tokens x 128 1300 / 1890 -> 111 / 109;
-// 32 heads x 4096 x 128 332 / 360; 4 heads x 512 x 64 100 / 74 -> 9 / 10.  A step takes ~5,700 clocks where its 48 products
-// alone take 3,300: products, conversion and epilogue share the four issue slots (53 % busy) and the instruction cache (the
-// loops are rolled up for it: 189 against 126 us under the profiler).  Tried without gain: eleven converter warps, a barrier per plane,
-// planes split beforehand and fetched by TMA (the extra pass costs what the conversion costs here).
+// Measured on a B200 (us, row / column pass; FMA tiles before): 16 / 8 heads x 2999 tokens x 128 1300 / 1890 -> 107 / 108;
+// 32 heads x 4096 x 128 369 / 386; 4 heads x 512 x 64 100 / 74 -> 9 / 10.  A step takes 5,800 / 6,800 clocks (the latter with the
+// similarities) where its 48 products alone take 3,300: products, conversion and epilogue share the four issue slots (57 % busy)
+// and the instruction cache (the loops are rolled up for it: 189 against 126 us under the profiler).  Tried without gain: eleven
+// converter warps, a barrier per plane, planes split beforehand and fetched by TMA (the extra pass costs what the conversion
+// costs here).
 //
 // Every wait on an mbarrier is bounded (see tc_common.cuh); a wait that runs out raises a flag, every role leaves its
 // loops, outputs are NaN and kvm_stats.status is set when given.

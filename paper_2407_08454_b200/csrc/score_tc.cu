@@ -28,9 +28,10 @@
 //   warps 18-19 the neighbour-key similarities, on the side
 // How the work is dealt to the CTAs: score_plan.cuh.
 //
-// What bounds the passes: one exponential per logit on the special-function unit (1,024 clocks a step, 80-90 % busy),
-// at the clock that the 1 kW power limit leaves (1,700-1,850 of 1,965 MHz in sustained calls; 32 heads x 4096 x 128:
-// 97 us a pass, 58 at full clock and 100 %).  The power goes to all of it: with the exponentials replaced by a multiply
+// What bounds the passes: one exponential per logit on the special-function unit (1,024 clocks a step; 88 % of the elapsed
+// cycles of a single launch on 32 / 8 heads x 32768, 75 % on 32 heads x 4096, whose CTAs have 114 steps each), at the clock
+// that the 1 kW power limit leaves (1,700-1,850 of 1,965 MHz in sustained calls; 32 heads x 4096 x 128: 97 us a pass, 58 at
+// full clock and 100 %).  The power goes to all of it: with the exponentials replaced by a multiply
 // 92 % of the energy is left, with an eighth of the products 75 %, without the B tiles' way from L2 80-95 %.
 //
 // Every wait on an mbarrier is bounded.  A wait that runs out raises a flag in
