@@ -140,8 +140,10 @@ int run_chain(const Dims& d, const Layers& L, const float* lse_in, float* scores
 
 // How many layers of a stack go through the kernels together.  A layer whose score pass gives a CTA few steps loses most
 // of its time to the launches, the passes' start and drain and the last, half-empty round (32 query / 8 KV heads x 2048
-// tokens, about 30 steps per CTA: 78 us a layer); together the layers share them.  From about 300 steps on there is
-// nothing left to share.  The variants beside the method, and fp32 tensors, run layer by layer.
+// tokens, about 30 steps per CTA: 78 us a layer); together the layers share them.  As many go together as give a CTA about
+// 300 steps (us a layer of 8, alone / together: 3 steps 31.9 / 12.8, 8 42.5 / 25.9 and 38.7 / 16.0, 30 71.0 / 47.1, 46 96 / 73,
+// 65 124 / 99; what is shared, about 25 us, stays the same while the rest grows).  The variants beside the method, and fp32
+// tensors, run layer by layer.
 int layers_together(const Dims& d, int n_layers) {
     if (d.dtype != KVM_BF16 || d.set_rule != KVM_SETS_ADJACENT ||
         (d.weight_rule != KVM_WEIGHT_GAUSSIAN && d.weight_rule != KVM_WEIGHT_AVERAGE))
