@@ -121,6 +121,7 @@ prefill_attend_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = sh.tmem_base;
+    grid_dependency_wait();
 
     if (warp >= NSOFT) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_OTHER));
@@ -455,10 +456,367 @@ prefill_attend_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
     }
 }
 
+// ------------------------------------------------------------------ two query tiles per CTA
+// The same attention with two query tiles in hand that read the same keys and values: two query heads of a group with one
+// tile each, or (one head per group, or an odd number) two neighbouring tiles of a head.  Softmax group g owns tile g:
+//   S_g = Q_g K_j^T  ->  P_g = exp(S_g - reference), written over S_g in tensor memory  ->  O_g += P_g V_j,
+// and while one tile's products run the other's exponentials do.  What bounds the kernel above is shared memory: a step of
+// 128 x 128 x 128 reads two operands for each product (128 KB), writes P (32 KB) and receives K and V (64 KB), 1,750 clocks at
+// 128 bytes a clock.  Here P is read from tensor memory and K and V serve two tiles: 64 + 32 + 32 KB.  Two steps, one of each
+// tile, take 2,950 clocks (head dimension 64: 2,680): 1,720 of a tile's softmax (1,024 of them exponentials at the unit's full
+// rate), the rest until its next logits are there; the tensor pipe is busy 2,180 (1,300) of them.
+// O is divided by the sum of the rounded weights, so that what rounding them did to a row's largest weight cancels (the
+// kernel above has two references a row, whose weights are exactly 1): error of O against 64 bits 1.984e-3 against 2.081e-3
+// of the kernel above (32 heads x 4096), 1.983e-3 against 1.992e-3 (10007 x 64), 2.08e-3 without, for 3 % (5 %) of the time.
+// A tile's products are issued in the order P V (j), Q K^T (j + 1) by one thread, so an S that is there says that the last
+// P V is done: O may be rescaled, and P written, without another barrier.
+constexpr int NST = 2;                  // iterations in the rings of K and V tiles
+constexpr int REGS_PAIR_OTHER = 88;     // (2 x 128 x 208 + 128 x 88 = 384 x 168, what the block is launched with)
+constexpr int P_FIRST = 96;             // keys of a step whose P is handed over first
+
+struct __align__(8) PairBars {
+    uint64_t q_full[2], q_empty[2], k0_full, k0_done;   // an item's Q tiles; its first K tile, loaded and used
+    uint64_t kv_full[NST], kv_empty[NST];   // iteration j: V tile j and K tile j + 1
+    uint64_t s_full[2], p_full[2][2], o_full[2];
+};
+struct alignas(16) PairShared {
+    PairBars bar;
+    uint32_t tmem_base;
+    int abort_flag;
+};
+
+// Item i of a CTA: tile[g] of query head[g] (n[g] key tiles; 0: none), longest first, boustrophedon.
+struct PairSched {
+    int P, c, NH, T, by_head;
+    __device__ __forceinline__ bool item(int i, int (&head)[2], int (&tile)[2], int (&n)[2]) const {
+        const unsigned k = (unsigned)i * (unsigned)P + (unsigned)((i & 1) ? (P - 1 - c) : c);
+        const unsigned per = (unsigned)(by_head ? NH / 2 : NH), rows = (unsigned)(by_head ? T : (T + 1) / 2);
+        if (k >= per * rows) return false;
+        const unsigned r = k / per, h = k - r * per, t = rows - 1 - r;
+        for (int g = 0; g < 2; ++g) {
+            head[g] = (int)(by_head ? 2 * h + g : h);
+            tile[g] = (int)(by_head ? t : 2 * t + g);
+            n[g] = tile[g] < T ? tile[g] + 1 : 0;
+        }
+        return true;
+    }
+};
+
 template <int KCH>
-cudaError_t launch_t(const Dims& d, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
+__global__ void __launch_bounds__(NTHREADS, 1)
+prefill_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
+                    const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_o, __nv_bfloat16* __restrict__ O,
+                    float* __restrict__ lse, kvm_stats* stats, int NH, int G, int S, float scale2) {
+    constexpr int D = KCH * KCHUNK;
+    constexpr uint32_t TILE_BYTES = KCH * CHUNK_BYTES;
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    uint8_t* sQ = smem_raw + (base - smem_u32(smem_raw));  // two Q tiles
+    uint8_t* sK = sQ + 2 * TILE_BYTES;
+    uint8_t* sV = sK + NST * TILE_BYTES;
+    uint8_t* sO = sV + NST * TILE_BYTES;                   // 32 rows of 64 channels per softmax warp
+    PairShared& sh = *reinterpret_cast<PairShared*>(sO + NSOFT * 4096);
+    volatile int* abort_flag = &sh.abort_flag;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int T = (S + TILE - 1) / TILE;
+    const PairSched sc{(int)gridDim.x, (int)blockIdx.x, NH, T, G % 2 == 0};
+    int head[2], tile[2], n[2];
+
+    if (threadIdx.x == 0) {
+        mbar_init(&sh.bar.k0_full, 1); mbar_init(&sh.bar.k0_done, 1);
+        for (int i = 0; i < NST; ++i) { mbar_init(&sh.bar.kv_full[i], 1); mbar_init(&sh.bar.kv_empty[i], 1); }
+        for (int g = 0; g < 2; ++g) {
+            mbar_init(&sh.bar.q_full[g], 1); mbar_init(&sh.bar.q_empty[g], 1);
+            mbar_init(&sh.bar.s_full[g], 1); mbar_init(&sh.bar.o_full[g], 1);
+            for (int h = 0; h < 2; ++h) mbar_init(&sh.bar.p_full[g][h], 4);
+        }
+        sh.abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == NSOFT + 1) tmem_alloc(&sh.tmem_base, 512);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = sh.tmem_base;
+    grid_dependency_wait();
+
+    if (warp >= NSOFT) {
+      asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_PAIR_OTHER));
+      if (warp == NSOFT) {
+        // ============================== producer ==============================
+        if (lane == 0) {
+            uint32_t kv = 0;                                  // K tiles (= V tiles = iterations) before this item
+            uint32_t q_ph = 0;                                // bit g: phase of Q tile g
+            bool ok = true;
+            auto load = [&](uint8_t* dst, const CUtensorMap* map, uint64_t* bar, int t, int h) {
+#pragma unroll
+                for (int kc = 0; kc < KCH; ++kc) tma_load_3d(dst + kc * CHUNK_BYTES, map, bar, kc * KCHUNK, t * TILE, h);
+            };
+            for (int i = 0; ok && sc.item(i, head, tile, n); ++i) {
+                const int kvhead = head[0] / G, len = max(n[0], n[1]);
+                // The first K tile's place is free (the last item's third iteration from the end has been waited for, or it was
+                // that item's first tile), and a Q tile's as soon as its own last Q K^T is done.
+                if (i > 0) ok = mbar_wait(&sh.bar.k0_done, (i & 1) ^ 1, abort_flag);
+                if (!ok) break;
+                mbar_expect_tx(&sh.bar.k0_full, TILE_BYTES);
+                load(sK + (kv % NST) * TILE_BYTES, &map_k, &sh.bar.k0_full, 0, kvhead);
+                for (int g = 0; ok && g < 2; ++g) {
+                    if (n[g] == 0) continue;
+                    ok = mbar_wait(&sh.bar.q_empty[g], ((q_ph >> g) & 1) ^ 1, abort_flag);
+                    if (!ok) break;
+                    q_ph ^= 1u << g;
+                    mbar_expect_tx(&sh.bar.q_full[g], TILE_BYTES);
+                    load(sQ + g * TILE_BYTES, &map_q, &sh.bar.q_full[g], tile[g], head[g]);
+                }
+                for (int j = 0; ok && j < len; ++j) {
+                    const uint32_t x = kv + (uint32_t)j, s = x % NST;
+                    ok = mbar_wait(&sh.bar.kv_empty[s], ((x / NST) & 1) ^ 1, abort_flag);
+                    if (j == 1) ok = ok && mbar_wait(&sh.bar.k0_done, i & 1, abort_flag);   // K tile 2 takes the first one's place
+                    if (!ok) break;
+#ifdef KVM_TEST_DROP_B_STAGE
+                    if (x == (uint32_t)(KVM_TEST_DROP_B_STAGE)) continue;   // test build only: these tiles never arrive
+#endif
+                    mbar_expect_tx(&sh.bar.kv_full[s], TILE_BYTES * (1u + (j + 1 < len)));
+                    if (j + 1 < len) load(sK + ((x + 1) % NST) * TILE_BYTES, &map_k, &sh.bar.kv_full[s], j + 1, kvhead);
+                    load(sV + s * TILE_BYTES, &map_v, &sh.bar.kv_full[s], j, kvhead);
+                }
+                kv += (uint32_t)len;
+            }
+            if (*abort_flag)                                  // copies already issued land (bounded)
+                for (uint32_t it = 0; it < (1u << 14); ++it) mbar_try(&sh.bar.k0_full, 0);
+        }
+      } else if (warp == NSOFT + 1) {
+        // ============================== MMA issue ==============================
+        // (One warp for both tiles, a tile's two products together: issued by two threads they share the tensor pipe evenly, both
+        // tiles' logits arrive at the same time, and the exponentials of both run together and wait together: 4,280 clocks for
+        // two steps against 3,070.)
+        constexpr uint32_t IDESC_S = idesc_bf16(TILE), IDESC_O = idesc_bf16(D, true);
+        const uint64_t dq = smem_desc(base), dk = smem_desc(base + 2 * TILE_BYTES);
+        const uint64_t dv = smem_desc_mn(base + (2 + NST) * TILE_BYTES, CHUNK_BYTES);
+        const uint32_t q_lo = (uint32_t)dq, k_lo = (uint32_t)dk, hi = (uint32_t)(dk >> 32), v_lo = (uint32_t)dv, v_hi = (uint32_t)(dv >> 32);
+        uint32_t kv = 0, p_ph = 0, q_ph = 0;                 // iterations before this item; phases of P and Q (bit g)
+        bool ok = true;
+        auto logits = [&](int g, uint32_t x, bool last) {    // S_g = Q_g K^T with K tile number x; the item's last one
+            if (elect_one()) {
+#pragma unroll
+                for (int kc = 0; kc < KCH; ++kc)
+#pragma unroll
+                    for (int ks = 0; ks < KCHUNK / 16; ++ks)
+                        umma_bf16_lo(tmem_base + g * S_COLS, q_lo + ((g * TILE_BYTES + kc * CHUNK_BYTES + ks * 32) >> 4), hi,
+                                     k_lo + (x % NST) * (TILE_BYTES >> 4) + ((kc * CHUNK_BYTES + ks * 32) >> 4), hi, IDESC_S, (kc | ks) ? 1u : 0u);
+                umma_commit(&sh.bar.s_full[g]);
+                if (last) umma_commit(&sh.bar.q_empty[g]);
+            }
+        };
+        // An item's first logits of a tile come right after the tile's last P V of the item before.
+        int nn[2] = {0, 0};
+        auto first_logits = [&](int g, int i, uint32_t x) {
+            if (nn[g] == 0) return;
+            ok = ok && mbar_wait_warp(&sh.bar.k0_full, i & 1, abort_flag) && mbar_wait_warp(&sh.bar.q_full[g], (q_ph >> g) & 1, abort_flag);
+            if (!ok) return;
+            q_ph ^= 1u << g;
+            tc_fence_after();
+            logits(g, x, nn[g] == 1);
+        };
+        bool valid = sc.item(0, head, tile, nn);
+        for (int i = 0; ok && valid; ++i) {
+            n[0] = nn[0]; n[1] = nn[1];
+            const int len = max(n[0], n[1]);
+            if (i == 0) {
+#pragma unroll
+                for (int g = 0; g < 2; ++g) first_logits(g, 0, 0u);
+                if (ok && elect_one()) umma_commit(&sh.bar.k0_done);
+            }
+            valid = sc.item(i + 1, head, tile, nn);
+            for (int j = 0; ok && j < len; ++j) {
+                const uint32_t x = kv + (uint32_t)j, s = x % NST;
+                ok = mbar_wait_warp(&sh.bar.kv_full[s], (x / NST) & 1, abort_flag);
+#pragma unroll
+                for (int g = 0; g < 2; ++g) {
+                    if (!ok || j >= n[g]) continue;
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {            // the first keys' products run while the last ones' P is made
+                        ok = ok && mbar_wait_warp(&sh.bar.p_full[g][h], (p_ph >> g) & 1, abort_flag);
+                        if (!ok) break;
+                        tc_fence_after();
+                        if (elect_one()) {
+#pragma unroll
+                            for (int kk = h ? P_FIRST / 16 : 0; kk < (h ? TILE / 16 : P_FIRST / 16); ++kk)   // 16 keys per MMA: 8 columns of P, 2 KB of V
+                                umma_bf16_ts(tmem_base + O_COL0 + g * D, tmem_base + g * S_COLS + kk * 8,
+                                             v_lo + s * (TILE_BYTES >> 4) + ((kk * 16 * 128) >> 4), v_hi, IDESC_O, (j | kk) ? 1u : 0u);
+                            if (h && j == n[g] - 1) umma_commit(&sh.bar.o_full[g]);
+                        }
+                    }
+                    if (!ok) break;
+                    p_ph ^= 1u << g;
+                    if (j + 1 < n[g]) logits(g, x + 1, j + 2 == n[g]);
+                    else if (valid) first_logits(g, i + 1, kv + (uint32_t)len);
+                }
+                if (ok && elect_one()) umma_commit(&sh.bar.kv_empty[s]);
+            }
+#pragma unroll
+            for (int g = 0; g < 2; ++g)
+                if (ok && valid && n[g] == 0) first_logits(g, i + 1, kv + (uint32_t)len);
+            if (ok && valid && elect_one()) umma_commit(&sh.bar.k0_done);
+            kv += (uint32_t)len;
+        }
+      }
+    } else {
+        // ============================== softmax of tile g ==============================
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_SOFTMAX));
+        const int g = warp >> 2, lq = warp & 3;
+        const int row = lq * 32 + lane;                      // query row of the tile = TMEM lane
+        const uint32_t t_lane = tmem_base + ((uint32_t)(lq * 32) << 16);
+        const uint32_t t_s = t_lane + g * S_COLS, t_o = t_lane + O_COL0 + g * D;
+        const uint64_t sc2 = pack2(scale2, scale2);
+        uint32_t s_ph = 0, o_ph = 0;
+        bool ok = true;
+        for (int i = 0; sc.item(i, head, tile, n); ++i) {
+            const int mine = g ? n[1] : n[0], my_tile = g ? tile[1] : tile[0], my_head = g ? head[1] : head[0];
+            if (mine == 0) continue;
+            float m = -INFINITY, l = 0.f, lr = 0.f;          // reference maximum (log2 units); sums relative to it: exact, of the rounded weights
+#pragma unroll 1
+            for (int j = 0; j < mine; ++j) {
+                ok = ok && mbar_wait(&sh.bar.s_full[g], s_ph, abort_flag);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                s_ph ^= 1;
+                tc_fence_after();
+                uint32_t vr[TILE];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) tmem_ld32_issue(t_s + q * 32, vr + q * 32);
+                tmem_ld_wait();
+#pragma unroll
+                for (int q = 0; q < 4; ++q) tmem_ld_fence(vr + q * 32);
+                float v[TILE];
+#pragma unroll
+                for (int c = 0; c < TILE; ++c) v[c] = __uint_as_float(vr[c]);
+                if (j == my_tile) {                          // diagonal tile: keys after the query do not exist for it
+#pragma unroll
+                    for (int c = 0; c < TILE; ++c)
+                        if (c > row) v[c] = -INFINITY;
+                }
+                // p = 2^(x - m), summed in fp32, rounded to bf16 for the tensor core.  The first 32 keys are tried with the
+                // reference as it is, beside the search for the step's maximum (which alone takes 300 of 1,700 clocks): the
+                // reference moves only when the maximum has outgrown it by RESCALE_STEP, seldom after the first step.
+                uint64_t sum[2] = {0ull, 0ull};
+                float rsum[4] = {0.f, 0.f, 0.f, 0.f};
+                float pk[16];                                // (two bf16 each)
+                auto exponentials = [&](int q) {
+                    const uint64_t nm2 = pack2(-m, -m);
+#pragma unroll
+                    for (int c = 0; c < 32; c += 2) {
+                        float x0, x1;
+                        unpack2(ffma2(pack2(v[q * 32 + c], v[q * 32 + c + 1]), sc2, nm2), x0, x1);
+                        const float e0 = ex2(x0), e1 = ex2(x1);
+                        sum[(c >> 1) & 1] = fadd2(sum[(c >> 1) & 1], pack2(e0, e1));
+                        const uint32_t r = Vec<__nv_bfloat16>::pack2(e0, e1);
+                        add_bf16x2(rsum[c & 2], rsum[(c & 2) + 1], r);
+                        pk[c >> 1] = __uint_as_float(r);
+                    }
+                };
+                exponentials(0);
+                float mx4[4] = {v[0], v[1], v[2], v[3]};
+#pragma unroll
+                for (int c = 4; c + 7 < TILE; c += 8)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) mx4[e] = fmax3(mx4[e], v[c + e], v[c + 4 + e]);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) mx4[e] = fmaxf(mx4[e], v[TILE - 4 + e]);
+                const float mx = fmaxf(fmax3(mx4[0], mx4[1], mx4[2]), mx4[3]) * scale2;
+                float alpha = 1.f;
+                const bool grow = mx > m + RESCALE_STEP;
+                if (__any_sync(0xffffffffu, grow)) {
+                    if (grow) { alpha = ex2(m - mx); m = mx; }
+                    sum[0] = sum[1] = 0ull;
+                    rsum[0] = rsum[1] = rsum[2] = rsum[3] = 0.f;
+                    exponentials(0);
+                    if (j > 0) {                             // (an S that is there says that the last P V is done)
+#pragma unroll
+                        for (int q = 0; q < D / 16; ++q) {
+                            float o[16];
+                            tmem_ld16(t_o + q * 16, o);
+#pragma unroll
+                            for (int c = 0; c < 16; ++c) o[c] *= alpha;
+                            tmem_st16(t_o + q * 16, o);
+                        }
+                    }
+                }
+                // (96 keys are handed over first: their products run while the last ones' P is made)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (q > 0) exponentials(q);
+                    tmem_st16(t_s + q * 16, pk);
+                    if (q == P_FIRST / 32 - 1 || q == 3) {
+                        tmem_st_wait();
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&sh.bar.p_full[g][q == 3]);
+                    }
+                }
+                float s0, s1;
+                unpack2(fadd2(sum[0], sum[1]), s0, s1);
+                l = l * alpha + (s0 + s1);
+                lr = lr * alpha + ((rsum[0] + rsum[1]) + (rsum[2] + rsum[3]));
+            }
+            // ---- item end: O / l, 64 channels of the warp's 32 rows at a time through shared memory (stored by the threads that
+            // own the rows, 16 bytes each: 3,000 clocks)
+            const int gi = my_tile * TILE + row;
+            ok = ok && mbar_wait(&sh.bar.o_full[g], o_ph, abort_flag);
+            ok = __all_sync(0xffffffffu, ok);
+            if (ok) {
+                o_ph ^= 1;
+                tc_fence_after();
+                const float f = 1.f / lr;
+                uint8_t* buf = sO + warp * 4096;
+#pragma unroll
+                for (int kc = 0; kc < KCH; ++kc) {
+                    uint32_t o[64];
+                    tmem_ld32_issue(t_o + kc * 64, o);
+                    tmem_ld32_issue(t_o + kc * 64 + 32, o + 32);
+                    tmem_ld_wait();
+                    tmem_ld_fence(o);
+                    tmem_ld_fence(o + 32);
+                    if (lane == 0) bulk_wait_read();
+                    __syncwarp();
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) {
+                        float y[8];
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) y[e] = __uint_as_float(o[c * 8 + e]) * f;
+                        *reinterpret_cast<uint4*>(buf + lane * 128 + ((c ^ (lane & 7)) << 4)) = Vec<__nv_bfloat16>::pack(y);
+                    }
+                    fence_proxy_async();
+                    __syncwarp();
+                    if (lane == 0 && my_tile * TILE + lq * 32 < S)
+                        tma_store_3d(&map_o, buf, kc * KCHUNK, my_tile * TILE + lq * 32, my_head);
+                }
+                tc_fence_before();                           // (the next item's first P says that O has been read)
+                if (gi < S) lse[(size_t)my_head * S + gi] = (m + log2f(l)) * LN2;
+            } else if (gi < S) {
+                // a wait gave up: what this row, and those of the items after it, would have received is marked, not made up
+                __nv_bfloat16* orow = O + ((size_t)my_head * S + gi) * D;
+                for (int c = 0; c < D; c += 8)
+                    *reinterpret_cast<uint4*>(orow + c) = make_uint4(0x7FC07FC0u, 0x7FC07FC0u, 0x7FC07FC0u, 0x7FC07FC0u);
+                lse[(size_t)my_head * S + gi] = NAN;
+            }
+        }
+        if (lane == 0) bulk_wait();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && sh.abort_flag && stats) stats->status = KVM_E_DEVICE_TIMEOUT;
+    if (warp == NSOFT + 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem_base, 512);
+    }
+}
+
+template <int KCH>
+cudaError_t launch_t(const Dims& d, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mo,
                      __nv_bfloat16* O, float* lse, kvm_stats* stats, cudaStream_t st) {
     const size_t smem = 1024 + (size_t)(1 + 2 * NKV) * KCH * CHUNK_BYTES + NGRP * 2 * CHUNK_BYTES + sizeof(Shared);
+    const size_t pair_smem = 1024 + (size_t)(2 + 2 * NST) * KCH * CHUNK_BYTES + NSOFT * 4096 + sizeof(PairShared);
     static std::mutex mu;
     static int sms_of[KVM_MAX_DEVICES] = {};
     cudaError_t e;
@@ -470,6 +828,8 @@ cudaError_t launch_t(const Dims& d, const CUtensorMap& mq, const CUtensorMap& mk
         if (!sms_of[dev]) {
             e = cudaFuncSetAttribute(prefill_attend_kernel<KCH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
+            e = cudaFuncSetAttribute(prefill_pair_kernel<KCH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pair_smem);
+            if (e != cudaSuccess) return e;
             if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
             sms_of[dev] = sms;
         }
@@ -478,22 +838,30 @@ cudaError_t launch_t(const Dims& d, const CUtensorMap& mq, const CUtensorMap& mk
     const int T = (d.S + TILE - 1) / TILE;
     const long long items = (long long)d.B * d.Hq * T;
     if (items + sms >= (1ll << 31)) return cudaErrorInvalidValue;   // the schedule counts items in 32 bits
+    const int G = d.Hq / d.Hkv;
+    const long long pairs = G % 2 == 0 ? items / 2 : (long long)d.B * d.Hq * ((T + 1) / 2);
+    // Two tiles at a time where the longest pair is not what a CTA's share is made of: its two tiles take turns where single ones
+    // would run beside one another.  (us, single tiles / pairs, steps over T x 148 beside them; D = 128: 8 heads x 4096 tokens 0.9
+    // 40.9 / 57.8, 10 heads 1.1 52.3 / 58.7, 12 heads 1.3 62.2 / 59.0, 14 heads 1.6 69.6 / 59.5, 32 heads 3.6 147.6 / 127; 32 x 1024 1.0
+    // 24.7 / 23.4, 48 x 1024 1.5 25.8 / 19.9; D = 64: 100 x 500 1.7 16.5 / 16.2, 32 / 8 x 10007 8.6 703 / 558.)
+    if ((long long)d.B * d.Hq * T * (T + 1) >= 3ll * sms * T)
+        return launch_dependent(prefill_pair_kernel<KCH>, dim3((unsigned)(pairs < sms ? pairs : sms)), dim3(NTHREADS), pair_smem, st, mq, mk,
+                                mv, mo, O, lse, stats, d.B * d.Hq, G, d.S, d.scale * LOG2E);
     const int grid = (int)(items < sms ? items : sms);
-    prefill_attend_kernel<KCH><<<grid, NTHREADS, smem, st>>>(mq, mk, mv, O, lse, stats, d.B, d.Hq, d.Hkv, d.S,
-                                                            d.scale * LOG2E);
-    return cudaGetLastError();
+    return launch_dependent(prefill_attend_kernel<KCH>, dim3((unsigned)grid), dim3(NTHREADS), smem, st, mq, mk, mv, O, lse, stats, d.B,
+                            d.Hq, d.Hkv, d.S, d.scale * LOG2E);
 }
 
 }  // namespace
 
 cudaError_t launch_prefill_attend(const Dims& d, const void* Q, const void* K, const void* V, void* O, float* lse,
                                   kvm_stats* stats, cudaStream_t st) {
-    CUtensorMap mq, mk, mv;
+    CUtensorMap mq, mk, mv, mo;
     if (!make_map(&mq, Q, d.B * d.Hq, d.S, d.D) || !make_map(&mk, K, d.B * d.Hkv, d.S, d.D) ||
-        !make_map(&mv, V, d.B * d.Hkv, d.S, d.D))
+        !make_map(&mv, V, d.B * d.Hkv, d.S, d.D) || !make_map(&mo, O, d.B * d.Hq, d.S, d.D, 32))
         return cudaErrorNotSupported;
     __nv_bfloat16* Ob = reinterpret_cast<__nv_bfloat16*>(O);
-    return d.D == 128 ? launch_t<2>(d, mq, mk, mv, Ob, lse, stats, st) : launch_t<1>(d, mq, mk, mv, Ob, lse, stats, st);
+    return d.D == 128 ? launch_t<2>(d, mq, mk, mv, mo, Ob, lse, stats, st) : launch_t<1>(d, mq, mk, mv, mo, Ob, lse, stats, st);
 }
 
 }  // namespace kvm

@@ -54,6 +54,30 @@ def test_prefill_attention_matches_the_checker_elementwise(S, D, Hq, Hkv, B):
     _check(O, lse, refO, ref_lse, d["V"], Hq // Hkv)
 
 
+@pytest.mark.parametrize("S,D,Hq,Hkv,B,logit_std", [
+    (300, 128, 150, 150, 1, 4.0),     # neighbouring tiles of a head, an odd number of them, the last one ragged
+    (513, 64, 57, 19, 2, 4.0),        # ... of groups of three; one row in the last tile
+    (257, 64, 160, 20, 1, 4.0),       # two heads of a group
+    (128, 128, 240, 120, 1, 4.0),     # one key tile per item
+    (1700, 128, 32, 8, 1, 4.0),       # items of 28 steps, several per CTA
+    (640, 128, 80, 80, 1, -1.0),      # nearly one-hot rows: the reference moves often
+])
+def test_two_query_tiles_at_a_time_match_the_checker_elementwise(S, D, Hq, Hkv, B, logit_std):
+    from oracle import kvmo
+    T = (S + 127) // 128
+    assert B * Hq * (T + 1) >= 3 * 148                        # (the sizes from which on tiles go in pairs)
+    cfg = si.CONFIGS["C1"].scaled(seq=S, head_dim=D, n_q_heads=Hq, n_kv_heads=Hkv, batch=B, seed=33, logit_std=logit_std)
+    d = si.make_layer(cfg)
+    _, _, _, _, O, lse = _run(cfg, d)
+    refO, ref_lse = kvmo.prefill_attend(d["Q"], d["K"], d["V"])
+    if logit_std > 0:
+        _check(O, lse, refO, ref_lse, d["V"], Hq // Hkv)
+    else:                                                     # (logits of magnitude 100s: lse relative to them, as below)
+        assert np.abs(lse.cpu().numpy() - ref_lse).max() <= 1e-5 * np.abs(ref_lse).max() + LSE_ATOL
+        tol = 1e-2 * np.abs(refO) + 2.0 ** -8 * np.abs(d["V"].float().numpy()).max()
+        assert (np.abs(O.float().cpu().numpy() - refO) <= tol).all()
+
+
 def test_prefill_attention_with_unscaled_logits_and_a_custom_scale():
     """Nearly one-hot rows (logits of standard deviation in the tens) move the reference maximum often."""
     from oracle import kvmo

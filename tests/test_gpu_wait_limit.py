@@ -181,3 +181,23 @@ def test_the_prefill_attention_kernel_also_comes_back_and_reports():
     torch.cuda.synchronize()
     refO, ref_lse = kvmo.prefill_attend(d["Q"], d["K"], d["V"])
     assert torch.isfinite(lse).all() and np.abs(lse.cpu().numpy() - ref_lse).max() <= 2e-4
+
+
+def test_after_a_give_up_of_the_two_tile_attention_every_row_of_the_block_is_marked():
+    """450 pairs of tiles: every block's first one is the longest (tiles 4 and 5 of a head), whose fourth V tile never comes, so
+    that every row of every block's items is marked and none keeps what was in memory before."""
+    lib = ctypes.CDLL(build.build_waittest())
+    H, S, D = 150, 700, 64
+    g = torch.Generator(device="cuda").manual_seed(79)
+    Q, K, V = (torch.randn(1, H, S, D, generator=g, device="cuda").bfloat16() for _ in range(3))
+    p = kvm.make_params(1, H, H, S, D, torch.bfloat16)
+    O, lse, stats = torch.zeros_like(Q), torch.zeros(1, H, S, device="cuda"), kvm.new_stats("cuda")
+    st = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    assert lib.kvm_prefill_attend(ctypes.byref(p), *_ptrs(Q, K, V, O, lse, stats), st) == 0
+    torch.cuda.synchronize()                        # the kernel came back by itself
+    assert kvm.read_stats(stats).status == -9       # KVM_E_DEVICE_TIMEOUT
+    # (a block's first pair: the rows of tile 4 too, whose group had its four steps' logits but not the fourth product)
+    assert torch.isnan(lse).all() and torch.isnan(O).all()
+    kvm.kvm_prefill_attend(p, Q, K, V, O, lse)      # the context is intact
+    torch.cuda.synchronize()
+    assert torch.isfinite(lse).all() and torch.isfinite(O).all()
