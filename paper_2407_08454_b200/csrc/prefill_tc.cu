@@ -472,6 +472,10 @@ prefill_attend_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
 // P V is done: O may be rescaled, and P written, without another barrier.
 constexpr int NST = 2;                  // iterations in the rings of K and V tiles
 constexpr int REGS_PAIR_OTHER = 88;     // (2 x 128 x 208 + 128 x 88 = 384 x 168, what the block is launched with)
+// How far (log2) a maximum may outgrow its row's reference.  Keys of one neighbourhood are alike, so a row's maximum grows by
+// several steps' worth now and then: 32 heads x 4096 129 / 127 / 124 / 123 us for 8 / 12 / 16 / 24, 10007 x 64 579 / 570 / 564 / 560; error of
+// O against 64 bits 1.97e-3 / 2.01e-3 / 2.03e-3 / 2.05e-3 (the reference's own weight is exact; of the kernel above 2.03e-3).
+constexpr float PAIR_RESCALE_STEP = 12.f;
 constexpr int P_FIRST = 96;             // keys of a step whose P is handed over first
 
 struct __align__(8) PairBars {
@@ -699,7 +703,7 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                 }
                 // p = 2^(x - m), summed in fp32, rounded to bf16 for the tensor core.  The first 32 keys are tried with the
                 // reference as it is, beside the search for the step's maximum (which alone takes 300 of 1,700 clocks): the
-                // reference moves only when the maximum has outgrown it by RESCALE_STEP, seldom after the first step.
+                // reference moves only when the maximum has outgrown it by PAIR_RESCALE_STEP, seldom after the first step.
                 uint64_t sum[2] = {0ull, 0ull};
                 float rsum[4] = {0.f, 0.f, 0.f, 0.f};
                 float pk[16];                                // (two bf16 each)
@@ -726,7 +730,7 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                 for (int e = 0; e < 4; ++e) mx4[e] = fmaxf(mx4[e], v[TILE - 4 + e]);
                 const float mx = fmaxf(fmax3(mx4[0], mx4[1], mx4[2]), mx4[3]) * scale2;
                 float alpha = 1.f;
-                const bool grow = mx > m + RESCALE_STEP;
+                const bool grow = mx > m + PAIR_RESCALE_STEP;
                 if (__any_sync(0xffffffffu, grow)) {
                     if (grow) { alpha = ex2(m - mx); m = mx; }
                     sum[0] = sum[1] = 0ull;
