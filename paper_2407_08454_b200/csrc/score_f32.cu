@@ -26,12 +26,13 @@
 // compress call).  Where the pieces' states would not fit 4 MiB (large problems, where whole items balance well
 // anyway) items stay whole and the states are final.  The rule depends on the shape only: results are reproducible.
 //
-// Measured on a B200 (us, row / column pass; FMA tiles before): 16 / 8 heads x 2999 tokens x 128 1300 / 1890 -> 107 / 108;
-// 32 heads x 4096 x 128 369 / 386; 4 heads x 512 x 64 100 / 74 -> 9 / 10.  A step takes 5,800 / 6,800 clocks (the latter with the
-// similarities) where its 48 products alone take 3,300: products, conversion and epilogue share the four issue slots (57 % busy)
-// and the instruction cache (the loops are rolled up for it: 189 against 126 us under the profiler).  Tried without gain: eleven
-// converter warps, a barrier per plane, planes split beforehand and fetched by TMA (the extra pass costs what the conversion
-// costs here).
+// Measured on a B200 (us, row / column pass; FMA tiles before): 16 / 8 heads x 2999 tokens x 128 1300 / 1890 -> 105 / 107;
+// 32 heads x 4096 x 128 351 / 377; 4 heads x 512 x 64 100 / 74 -> 9 / 9.  What bounds a step now is its 48 products: 3,340 of
+// 3,960 clocks, at the clock that so busy a tensor pipe is left by the power limit.  Before, the epilogue did (two steps in
+// 10,900 clocks, 5,000 of a step's 10,000 spent on joining the row pass's states): now those are joined by a kernel between
+// the passes where a CTA has several steps, asked for a step ahead, and the exponentials are single instructions.
+// Tried without gain: eleven converter warps, a barrier per plane, planes split beforehand and fetched by TMA (the extra pass
+// costs what the conversion costs here).
 //
 // Every wait on an mbarrier is bounded (see tc_common.cuh); a wait that runs out raises a flag, every role leaves its
 // loops, outputs are NaN and kvm_stats.status is set when given.
@@ -62,6 +63,9 @@ constexpr int NEPI = 8, NCONV = 7;                // warps; with the MMA warp si
 constexpr int NTHREADS = (NEPI + NCONV + 1) * 32;
 constexpr int SIM_RUN = 8;                         // consecutive tokens per lane group (similarities)
 constexpr int NSLOT = 8;                           // piece-end buffers in rotation
+// Steps per CTA from which on the row states are joined between the passes (a launch, about 3 us) and not by every step that
+// reads them: 18 heads x 1000 x 64, 5 steps, 41.2 us a call with the latter, 38.2 joined; 4 heads x 512, one step, 19.5 / 22.
+constexpr unsigned JOIN_STEPS = 4;
 constexpr size_t SPLIT_BYTES_MAX = (size_t)KVM_STATIC_SCORE_ROWS * sizeof(float);
 constexpr float LOG2E = 1.4426950408889634f, LN2 = 0.6931471805599453f;
 
@@ -170,7 +174,7 @@ template <int KCH, int PASS>
 __global__ void __launch_bounds__(NTHREADS, 1)
 score_f32_kernel(const float* __restrict__ Q, const float* __restrict__ K, float2* __restrict__ states,
                  const float* __restrict__ flat, float flat_mul, float* __restrict__ out, kvm_stats* stats,
-                 const Plan plan, int Hq, int Hkv, int S, float scale2, float* __restrict__ sim_out) {
+                 const Plan plan, int Hq, int Hkv, int S, float scale2, int joined, float* __restrict__ sim_out) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* sA = smem_raw + (base - smem_u32(smem_raw));     // [KCH][plane][128 rows][128 B]
@@ -256,7 +260,9 @@ score_f32_kernel(const float* __restrict__ Q, const float* __restrict__ K, float
         }
     } else if (warp == NEPI + NCONV) {
         // ============================== MMA issue ==============================
-        if (lane == 0) {
+        {
+            // (The whole warp walks and waits, one elected lane issues: descriptors stay in uniform registers.  250 -> 244 us on
+            // 16 / 8 heads x 2999 x 128.)
             constexpr uint32_t IDESC = idesc_bf16(TILE);
             // (planes lie in the order l, m, h)
             const uint32_t da0 = (uint32_t)smem_desc(base), db0 = (uint32_t)smem_desc(base + KCH * CHUNK_BYTES);
@@ -265,30 +271,32 @@ score_f32_kernel(const float* __restrict__ Q, const float* __restrict__ K, float
             for (int n = 0; ok && w.valid(); ++n, w.next(plan)) {
                 for (int i = 0; ok && i < w.n; ++i, ++cnt) {
                     const int as = cnt & 1;
-                    ok = mbar_wait(&sh.acc_empty[as], ((cnt >> 1) & 1) ^ 1, abort_flag);
+                    ok = mbar_wait_warp(&sh.acc_empty[as], ((cnt >> 1) & 1) ^ 1, abort_flag);
                     const uint32_t d_hi = tmem_base + as * (2 * TILE), d_lo = d_hi + TILE;
 #pragma unroll
                     for (int kc = 0; kc < KCH; ++kc, ++bcnt) {
                         const int s = bcnt % NSTAGE;
-                        if (i == 0) ok = ok && mbar_wait(&sh.full_a[kc], n & 1, abort_flag);
-                        ok = ok && mbar_wait(&sh.full_b[s], (bcnt / NSTAGE) & 1, abort_flag);
+                        if (i == 0) ok = ok && mbar_wait_warp(&sh.full_a[kc], n & 1, abort_flag);
+                        ok = ok && mbar_wait_warp(&sh.full_b[s], (bcnt / NSTAGE) & 1, abort_flag);
                         if (!ok) break;
                         tc_fence_after();
-                        const uint32_t da = da0 + ((kc * CHUNK_BYTES) >> 4), db = db0 + s * (CHUNK_BYTES >> 4);
+                        if (elect_one()) {
+                            const uint32_t da = da0 + ((kc * CHUNK_BYTES) >> 4), db = db0 + s * (CHUNK_BYTES >> 4);
 #pragma unroll
-                        for (int ks = 0; ks < KCHUNK / 16; ++ks)
+                            for (int ks = 0; ks < KCHUNK / 16; ++ks)
 #pragma unroll
-                            for (int z = 0; z < 6; ++z) {
-                                constexpr int PX[6] = {2, 1, 2, 0, 1, 2}, PY[6] = {0, 1, 1, 2, 2, 2};
-                                umma_bf16_lo(z == 5 ? d_hi : d_lo, da + ((PX[z] * PLANE_BYTES + ks * 32) >> 4), dhi,
-                                             db + ((PY[z] * PLANE_BYTES + ks * 32) >> 4), dhi, IDESC,
-                                             z == 5 ? (kc | ks) != 0 : (kc | ks | z) != 0);
-                            }
-                        umma_commit(&sh.empty_b[s]);
+                                for (int z = 0; z < 6; ++z) {
+                                    constexpr int PX[6] = {2, 1, 2, 0, 1, 2}, PY[6] = {0, 1, 1, 2, 2, 2};
+                                    umma_bf16_lo(z == 5 ? d_hi : d_lo, da + ((PX[z] * PLANE_BYTES + ks * 32) >> 4), dhi,
+                                                 db + ((PY[z] * PLANE_BYTES + ks * 32) >> 4), dhi, IDESC,
+                                                 z == 5 ? (kc | ks) != 0 : (kc | ks | z) != 0);
+                                }
+                            umma_commit(&sh.empty_b[s]);
+                        }
                     }
-                    if (ok) umma_commit(&sh.acc_full[as]);
+                    if (ok && elect_one()) umma_commit(&sh.acc_full[as]);
                 }
-                if (ok) umma_commit(&sh.empty_a);
+                if (ok && elect_one()) umma_commit(&sh.empty_a);
             }
         }
     } else {
@@ -296,41 +304,58 @@ score_f32_kernel(const float* __restrict__ Q, const float* __restrict__ K, float
         const int lq = warp & 3, grp = warp >> 2, row = lq * 32 + lane;
         const uint32_t t_lane = tmem_base + ((uint32_t)(lq * 32) << 16) + grp * (2 * TILE);
         float* nl = sh.nl[warp];
+        const uint64_t sc2 = pack2(scale2, scale2);
         uint32_t cnt = 0, own = 0;
         const size_t rows = (size_t)plan.NH * S;
+        // The log-sum-exp (log2 units) of four of the 128 queries of tile t of the group's query head h: the caller's, one
+        // that join_states_kernel left, or made of the row pass's states here.  Queries past the end weigh nothing.
+        auto ask = [&](float (&v)[4], int h, int t) {
+            const int qh = (w.head / Hkv) * Hq + (w.head % Hkv) * plan.G + h;
+            const size_t r = (size_t)qh * S + t * TILE + lane;
+            const int left = S - t * TILE - lane;
+            if (flat) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) v[e] = e * 32 < left ? flat[r + e * 32] * flat_mul : INFINITY;
+            } else if (joined) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) v[e] = e * 32 < left ? __ldcg(&states[r + e * 32].x) : INFINITY;
+            } else {
+                const int np = plan.row_pieces(qh, t);
+                float M[4], L[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) { M[e] = -INFINITY; L[e] = 0.f; }
+#pragma unroll 2
+                for (int x = 0; x < np; ++x) {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        if (e * 32 >= left) continue;
+                        const float2 st = __ldcg(states + (size_t)x * rows + r + e * 32);
+                        add_state(M[e], L[e], st);
+                    }
+                }
+#pragma unroll
+                for (int e = 0; e < 4; ++e) v[e] = e * 32 < left ? M[e] + log2f(L[e]) : INFINITY;
+            }
+        };
+        float ahead[4] = {0.f, 0.f, 0.f, 0.f};
         for (int n = 0; w.valid(); ++n, w.next(plan)) {
-            float m = -INFINITY, l[4] = {0.f, 0.f, 0.f, 0.f};
+            float m = -INFINITY;
+            uint64_t l2[2] = {0ull, 0ull};                   // four sums, of every fourth column
             const int per = plan.T - w.tile;
+            bool asked = false;
             int g = PASS == 1 ? 0 : w.i0 / per, bt = PASS == 1 ? w.i0 : w.tile + w.i0 % per;
             for (int i = 0; i < w.n; ++i, ++cnt) {
                 const int cur = bt, cg = g;
                 if (++bt == plan.T && PASS == 2) { bt = w.tile; ++g; }
                 if ((int)(cnt & 1) != grp) continue;
                 if (PASS == 2) {
-                    // the step's 128 queries, four per lane; queries past the end weigh nothing
-                    const int qh = (w.head / Hkv) * Hq + (w.head % Hkv) * plan.G + cg;
-                    const size_t r = (size_t)qh * S + cur * TILE + lane;
+                    // minus the log-sum-exp of the step's 128 queries, four per lane (asked for during this group's step
+                    // before where that belongs to the same piece)
                     float v[4];
-                    if (flat) {
+                    if (!asked) ask(v, cg, cur);
+                    else
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) v[e] = cur * TILE + e * 32 + lane < S ? flat[r + e * 32] * flat_mul : INFINITY;
-                    } else {
-                        const int np = plan.row_pieces(qh, cur);
-                        float M[4], L[4];
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) { M[e] = -INFINITY; L[e] = 0.f; }
-#pragma unroll 2
-                        for (int x = 0; x < np; ++x) {
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                if (cur * TILE + e * 32 + lane >= S) continue;
-                                const float2 st = __ldcg(states + (size_t)x * rows + r + e * 32);
-                                add_state(M[e], L[e], st);
-                            }
-                        }
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) v[e] = cur * TILE + e * 32 + lane < S ? M[e] + log2f(L[e]) : INFINITY;
-                    }
+                        for (int e = 0; e < 4; ++e) v[e] = ahead[e];
                     __syncwarp();                                   // the last step's values have been read
 #pragma unroll
                     for (int e = 0; e < 4; ++e) nl[e * 32 + lane] = v[e] > -INFINITY || v[e] != v[e] ? -v[e] : -INFINITY;   // (a query with no key to see weighs nothing)
@@ -340,6 +365,13 @@ score_f32_kernel(const float* __restrict__ Q, const float* __restrict__ K, float
                 ok = __all_sync(0xffffffffu, ok);
                 ++own;
                 if (ok) tc_fence_after();
+                if (PASS == 2) {
+                    asked = joined && i + 2 < w.n;
+                    if (asked) {
+                        const int bn = bt + 1 == plan.T ? w.tile : bt + 1, gn = bt + 1 == plan.T ? g + 1 : g;
+                        ask(ahead, gn, bn);
+                    }
+                }
                 const bool diag = cur == w.tile;
                 // (rolled up: with every role's loops unrolled the instruction cache is what the kernel waits for)
 #pragma unroll 1
@@ -363,16 +395,11 @@ score_f32_kernel(const float* __restrict__ Q, const float* __restrict__ K, float
                     tmem_ld_fence(lo);
                     float v[32];
 #pragma unroll
-                    for (int c = 0; c < 32; ++c) v[c] = __uint_as_float(hi[c]) + __uint_as_float(lo[c]);
-                    if (PASS == 2) {
-#pragma unroll
-                        for (int c = 0; c < 32; c += 4) {
-                            const float4 x = *reinterpret_cast<const float4*>(nl + cq * 32 + c);
-                            v[c] = fmaf(v[c], scale2, x.x);
-                            v[c + 1] = fmaf(v[c + 1], scale2, x.y);
-                            v[c + 2] = fmaf(v[c + 2], scale2, x.z);
-                            v[c + 3] = fmaf(v[c + 3], scale2, x.w);
-                        }
+                    for (int c = 0; c < 32; c += 2) {
+                        uint64_t x = fadd2(pack2(__uint_as_float(hi[c]), __uint_as_float(hi[c + 1])),
+                                           pack2(__uint_as_float(lo[c]), __uint_as_float(lo[c + 1])));
+                        if (PASS == 2) x = ffma2(x, sc2, *reinterpret_cast<const uint64_t*>(nl + cq * 32 + c));
+                        unpack2(x, v[c], v[c + 1]);
                     }
                     if (mask) {
 #pragma unroll
@@ -384,18 +411,37 @@ score_f32_kernel(const float* __restrict__ Q, const float* __restrict__ K, float
 #pragma unroll
                         for (int c = 1; c + 1 < 32; c += 2) mx = fmax3(mx, v[c], v[c + 1]);
                         const float mn = fmaxf(m, fmaxf(mx, v[31]) * scale2), ref = mn == -INFINITY ? 0.f : mn;
-                        const float f = exp2f(m - ref);
+                        // (what is flushed to zero below 2^-126 would not change a sum that holds the maximum's 1)
+                        const float f = ex2(m - ref);
+                        const uint64_t f2 = pack2(f, f), nref2 = pack2(-ref, -ref);
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) l[e] *= f;
+                        for (int e = 0; e < 2; ++e) l2[e] = fmul2(l2[e], f2);
 #pragma unroll
-                        for (int c = 0; c < 32; ++c) l[c & 3] += exp2f(fmaf(v[c], scale2, -ref));
+                        for (int c = 0; c < 32; c += 2) {
+                            float x0, x1;
+                            unpack2(ffma2(pack2(v[c], v[c + 1]), sc2, nref2), x0, x1);
+                            l2[(c >> 1) & 1] = fadd2(l2[(c >> 1) & 1], pack2(ex2(x0), ex2(x1)));
+                        }
                         m = mn;
                     } else {
+                        // A key whose every weight is below 2^-126 keeps a score: the slow exponential, which does not flush,
+                        // where one could be (four instructions for one).
+                        float low = v[0];
 #pragma unroll
-                        for (int c = 0; c < 32; ++c) l[c & 3] += exp2f(v[c]);
+                        for (int c = 1; c + 1 < 32; c += 2) low = fmin3(low, v[c], v[c + 1]);
+                        if (__any_sync(0xffffffffu, !(fminf(low, v[31]) >= -126.f))) {
+#pragma unroll
+                            for (int c = 0; c < 32; c += 2) l2[(c >> 1) & 1] = fadd2(l2[(c >> 1) & 1], pack2(exp2f(v[c]), exp2f(v[c + 1])));
+                        } else {
+#pragma unroll
+                            for (int c = 0; c < 32; c += 2) l2[(c >> 1) & 1] = fadd2(l2[(c >> 1) & 1], pack2(ex2(v[c]), ex2(v[c + 1])));
+                        }
                     }
                 }
             }
+            float l[4];
+            unpack2(l2[0], l[0], l[1]);
+            unpack2(l2[1], l[2], l[3]);
             // ---- piece end: the two warps that own a row leave their sums in shared memory; whichever comes
             // last adds them in a fixed order and stores.  Nobody waits.  (Buffers: when a warp finishes step k the MMA
             // thread has issued step k - 1, so the other group has handed step k - 3 back but may not have delivered it.
@@ -476,6 +522,17 @@ __global__ void __launch_bounds__(256) combine_kernel(const float* __restrict__ 
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j < S) scores[(size_t)blockIdx.y * S + j] = plan::column_sum(part, plan, S, blockIdx.y, j);
 }
+// The row pass's states of cut items -> the rows' log-sum-exp (log2 units), in the place of their first states.
+__global__ void __launch_bounds__(256) join_states_kernel(float2* __restrict__ states, const Plan plan, int S) {
+    grid_dependency_wait();
+    const size_t rows = (size_t)plan.NH * S, r = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= rows) return;
+    const int head = (int)(r / S), np = plan.row_pieces(head, (int)(r - (size_t)head * S) / TILE);
+    float M = -INFINITY, L = 0.f;
+#pragma unroll 2
+    for (int x = 0; x < np; ++x) add_state(M, L, __ldcg(states + (size_t)x * rows + r));
+    states[r].x = M + log2f(L);
+}
 // Bytes of the two passes' states and sums.
 size_t state_bytes(const Dims& d, const Plan& p) {
     const size_t rows = (size_t)p.NH * d.S;
@@ -511,7 +568,7 @@ cudaError_t launch_t(const Dims& d, const Plan& plan, const float* Q, const floa
     const float scale2 = d.scale * LOG2E;
     if (!lse_in) {
         e = launch_dependent(score_f32_kernel<KCH, 1>, rgrid, block, smem, st, Q, K, states, (const float*)nullptr,
-                             1.f, flat, stats, plan, d.Hq, d.Hkv, d.S, scale2, (float*)nullptr);
+                             1.f, flat, stats, plan, d.Hq, d.Hkv, d.S, scale2, 0, (float*)nullptr);
         if (e != cudaSuccess) return e;
     }
     if (lse_out) {
@@ -520,9 +577,14 @@ cudaError_t launch_t(const Dims& d, const Plan& plan, const float* Q, const floa
         if (e != cudaSuccess) return e;
     }
     if (!scores) return cudaSuccess;
+    const bool join = !lse_in && plan.split_row && plan.q >= JOIN_STEPS;
+    if (join) {
+        e = launch_dependent(join_states_kernel, dim3((unsigned)((rows + 255) / 256)), dim3(256), 0, st, states, plan, d.S);
+        if (e != cudaSuccess) return e;
+    }
     e = launch_dependent(score_f32_kernel<KCH, 2>, cgrid, block, smem, st, Q, K, states,
                          lse_in ? lse_in : (const float*)flat, lse_in ? LOG2E : 1.f, plan.split_col ? part : scores, stats, plan,
-                         d.Hq, d.Hkv, d.S, scale2, sim_out);
+                         d.Hq, d.Hkv, d.S, scale2, (int)join, sim_out);
     if (e != cudaSuccess || !plan.split_col) return e;
     if (parts) {                                      // the caller's next kernel adds the pieces up
         parts->part = part;
