@@ -268,6 +268,12 @@ int kvm_compress_layers(const kvm_params* p, int32_t n_layers, const float* sim_
                         const void* const* K, const void* const* V, void* const* K_out, void* const* V_out,
                         int32_t* const* out_len, int32_t* const* out_pos, kvm_stats* stats, void* ws,
                         size_t ws_bytes, void* cuda_stream);
+
+/* The same, and every output row and position past a unit's length (up to cap) is set to zero. */
+int kvm_compress_layers_filled(const kvm_params* p, int32_t n_layers, const float* sim_thresholds, const void* const* Q,
+                        const void* const* K, const void* const* V, void* const* K_out, void* const* V_out,
+                        int32_t* const* out_len, int32_t* const* out_pos, kvm_stats* stats, void* ws,
+                        size_t ws_bytes, void* cuda_stream);
 int kvm_layers_workspace_bytes(const kvm_params* p, int32_t n_layers, size_t* bytes);   /* Host only. */
 
 /*

@@ -24,7 +24,7 @@ KVM_WEIGHT_GAUSSIAN, KVM_WEIGHT_AVERAGE, KVM_WEIGHT_PIVOT_ONLY, KVM_WEIGHT_SET_S
 KVM_SETS_ADJACENT, KVM_SETS_CONSERVED_ONLY, KVM_SETS_ANCHOR = 0, 1, 2
 EXPORTS = (
     "kvm_sizes", "kvm_workspace_bytes", "kvm_score", "kvm_row_lse", "kvm_segment", "kvm_merge_compact", "kvm_compress",
-    "kvm_compress_with_lse", "kvm_compress_layers", "kvm_layers_workspace_bytes",
+    "kvm_compress_with_lse", "kvm_compress_layers", "kvm_compress_layers_filled", "kvm_layers_workspace_bytes",
     "kvm_host_staging_bytes", "kvm_compress_host", "kvm_score_static", "kvm_layer_ratio", "kvm_attend",
     "kvm_output_perturbation", "kvm_prefill_attend", "kvm_status_string",
     "kvm_version",
@@ -83,6 +83,7 @@ _ARGTYPES = {
     "kvm_compress": (_PARAMS,) + (_P,) * 10 + (_Z, _P),
     "kvm_compress_with_lse": (_PARAMS,) + (_P,) * 11 + (_Z, _P),
     "kvm_compress_layers": (_PARAMS, _I) + (_P,) * 10 + (_Z, _P),
+    "kvm_compress_layers_filled": (_PARAMS, _I) + (_P,) * 10 + (_Z, _P),
     "kvm_layers_workspace_bytes": (_PARAMS, _I, ctypes.POINTER(_Z)),
     "kvm_compress_host": (_PARAMS,) + (_P,) * 8 + (_Z, _P),
 }
@@ -294,19 +295,18 @@ class Compressor:
 
 def compress_layers(p: KvmParams, layers, sim_thresholds=None, device="cuda", stream=None):
     """Compress a stack of layers, each an (Q, K, V) triple of CUDA tensors of the shape `p` describes, with one
-    similarity threshold per layer (Section 3.2: thresholds chosen layer by layer), through kvm_compress_layers.
+    similarity threshold per layer (Section 3.2: thresholds chosen layer by layer), through kvm_compress_layers_filled.
     Returns, per layer, a `Compressed` holding the outputs, and the layer's compression ratio mean(out_len) / S."""
     # (the GPU waits for this function: whatever its results do not need is left until the kernels are enqueued, and the
     # addresses are worked out from the bases)
     n = len(layers)
     B, H, cap, D = p.batch, p.n_kv_heads, kvm_sizes(p)[0], p.head_dim
     units, dtype = B * H, torch.bfloat16 if p.dtype == KVM_BF16 else torch.float32
-    # A layer's rows and positions are one allocation (a layer that the caller drops is freed), zero-filled by one kernel for
-    # the stack; the lengths of all layers are read back together.
+    # A layer's rows and positions are one allocation (a layer that the caller drops is freed); what lies past the lengths is
+    # zeroed by the merge; the lengths of all layers are read back together.
     kv_bytes = units * cap * D * (2 if p.dtype == KVM_BF16 else 4)
     blobs = [torch.empty(2 * kv_bytes + 4 * units * cap, dtype=torch.uint8, device=device) for _ in range(n)]
-    torch._foreach_zero_(blobs)
-    out_len = torch.zeros((n, B, H), dtype=torch.int32, device=device)
+    out_len = torch.empty((n, B, H), dtype=torch.int32, device=device)
     ws = torch.empty(kvm_layers_workspace_bytes(p, n), dtype=torch.uint8, device=device)
     array = ctypes.c_void_p * n
 
@@ -318,7 +318,7 @@ def compress_layers(p: KvmParams, layers, sim_thresholds=None, device="cuda", st
         assert len(sim_thresholds) == n
         eps = (ctypes.c_float * n)(*[float(e) for e in sim_thresholds])
     bases, len_base = [b.data_ptr() for b in blobs], out_len.data_ptr()
-    _call("kvm_compress_layers", p, n, eps, q, k, v, array(*bases), array(*[b + kv_bytes for b in bases]),
+    _call("kvm_compress_layers_filled", p, n, eps, q, k, v, array(*bases), array(*[b + kv_bytes for b in bases]),
           array(*range(len_base, len_base + 4 * n * units, 4 * units)), array(*[b + 2 * kv_bytes for b in bases]), None,
           ws.data_ptr(), ws.nbytes, _stream(stream))
     out = []

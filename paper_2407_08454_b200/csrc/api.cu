@@ -380,7 +380,7 @@ int kvm_layers_workspace_bytes(const kvm_params* p, int32_t n_layers, size_t* by
     return KVM_OK;
 }
 
-int kvm_compress_layers(const kvm_params* p, int32_t n_layers, const float* sim_thresholds, const void* const* Q,
+static int compress_layers(int zero_rest, const kvm_params* p, int32_t n_layers, const float* sim_thresholds, const void* const* Q,
                         const void* const* K, const void* const* V, void* const* K_out, void* const* V_out,
                         int32_t* const* out_len, int32_t* const* out_pos, kvm_stats* stats, void* ws,
                         size_t ws_bytes, void* cuda_stream) {
@@ -403,6 +403,7 @@ int kvm_compress_layers(const kvm_params* p, int32_t n_layers, const float* sim_
         while (n > 1 && carve(times_batch(d, n), nullptr).bytes > ws_bytes) --n;
         Layers L = one_layer(d, nullptr, nullptr);
         L.n = n;
+        L.zero_rest = zero_rest;
         for (int i = 0; i < n; ++i) {
             L.Q[i] = Q[l0 + i]; L.K[i] = K[l0 + i]; L.V[i] = V[l0 + i];
             L.K_out[i] = K_out[l0 + i]; L.V_out[i] = V_out[l0 + i];
@@ -411,11 +412,31 @@ int kvm_compress_layers(const kvm_params* p, int32_t n_layers, const float* sim_
         }
         const Dims dn = times_batch(d, n);
         const Workspace wn = carve(dn, ws);
+        if (zero_rest && d.weight_rule == KVM_WEIGHT_PIVOT_ONLY) {       // (a gather, no merge: one layer at a time)
+            const size_t kv = (size_t)d.U * d.cap * d.D * (d.dtype == KVM_BF16 ? 2 : 4);
+            cudaStream_t st = (cudaStream_t)cuda_stream;
+            if (cudaMemsetAsync(L.K_out[0], 0, kv, st) != cudaSuccess || cudaMemsetAsync(L.V_out[0], 0, kv, st) != cudaSuccess ||
+                cudaMemsetAsync(L.pivot[0], 0, (size_t)d.U * d.cap * sizeof(int32_t), st) != cudaSuccess)
+                return KVM_E_CUDA;
+        }
         rc = run_chain(dn, L, nullptr, wn.scores, wn, stats, (cudaStream_t)cuda_stream);
         if (rc != KVM_OK) return rc;
         l0 += n;
     }
     return KVM_OK;
+}
+
+int kvm_compress_layers(const kvm_params* p, int32_t n_layers, const float* sim_thresholds, const void* const* Q,
+                        const void* const* K, const void* const* V, void* const* K_out, void* const* V_out,
+                        int32_t* const* out_len, int32_t* const* out_pos, kvm_stats* stats, void* ws,
+                        size_t ws_bytes, void* cuda_stream) {
+    return compress_layers(0, p, n_layers, sim_thresholds, Q, K, V, K_out, V_out, out_len, out_pos, stats, ws, ws_bytes, cuda_stream);
+}
+int kvm_compress_layers_filled(const kvm_params* p, int32_t n_layers, const float* sim_thresholds, const void* const* Q,
+                        const void* const* K, const void* const* V, void* const* K_out, void* const* V_out,
+                        int32_t* const* out_len, int32_t* const* out_pos, kvm_stats* stats, void* ws,
+                        size_t ws_bytes, void* cuda_stream) {
+    return compress_layers(1, p, n_layers, sim_thresholds, Q, K, V, K_out, V_out, out_len, out_pos, stats, ws, ws_bytes, cuda_stream);
 }
 
 // The groups of units that kvm_compress_host's pipeline takes one after the other.

@@ -32,10 +32,11 @@ template <int NL> struct LayersOf {
     void *K_out[NL], *V_out[NL];
     int32_t *out_len[NL], *pivot[NL];
     float eps[NL];
+    int zero_rest;                                 // the merge also zero-fills the rows and positions past a unit's length
 };
 using Layers = LayersOf<MAX_LAYERS>;
 inline LayersOf<1> first_of(const Layers& L) {
-    return {1, L.U, L.H, {L.Q[0]}, {L.K[0]}, {L.V[0]}, {L.K_out[0]}, {L.V_out[0]}, {L.out_len[0]}, {L.pivot[0]}, {L.eps[0]}};
+    return {1, L.U, L.H, {L.Q[0]}, {L.K[0]}, {L.V[0]}, {L.K_out[0]}, {L.V_out[0]}, {L.out_len[0]}, {L.pivot[0]}, {L.eps[0]}, L.zero_rest};
 }
 // The layer of unit u, which becomes the unit's index within the layer.
 template <int NL> __device__ __forceinline__ int layer_of(const LayersOf<NL>& L, long long& u) {

@@ -44,6 +44,29 @@ def test_layers_together_match_layers_alone(n, S, Hq, Hkv, D, dtype, monkeypatch
             assert torch.equal(got.K_out[0, h, x], ref.K_out[0, h, y]) and torch.equal(got.V_out[0, h, x], ref.V_out[0, h, y])
         assert same >= 0.97 * rows
 
+
+@pytest.mark.parametrize("n,S,Hkv,D,dtype,rules", [
+    (3, 389, 4, 128, "bf16", {}),                     # layers together; the last tile's share of the rows is cut
+    (2, 33, 3, 64, "f32", {}),                        # two tiles, capacity 16
+    (2, 700, 2, 64, "bf16", {"set_rule": kvm.KVM_SETS_CONSERVED_ONLY}),     # a gather instead of the merge
+    (2, 640, 2, 128, "bf16", {"weight_rule": kvm.KVM_WEIGHT_SET_SIGMA}),
+])
+def test_rows_past_a_units_length_are_zero(n, S, Hkv, D, dtype, rules):
+    cfg = si.CONFIGS["C1"].scaled(seq=S, head_dim=D, n_q_heads=Hkv, n_kv_heads=Hkv, dtype=dtype, seed=S)
+    layers = [tuple(si.make_layer(cfg, l)[k].cuda() for k in "QKV") for l in range(n)]
+    p = kvm.make_params(1, Hkv, Hkv, S, D, cfg.torch_dtype, **rules)
+    dirty = [torch.full((1 << 20,), -1, dtype=torch.int32, device="cuda") for _ in range(8)]
+    del dirty                                         # (what the results are allocated from is not zero)
+    out, _ = kvm.compress_layers(p, layers)
+    for c, (Q, K, V) in zip(out, layers):
+        ref = kvm.Compressor(p)(Q, K, V)              # (its buffers start at zero)
+        assert int(c.out_len.min()) < c.cap and torch.equal(c.out_len, ref.out_len)
+        rest = torch.arange(c.cap, device="cuda") >= c.out_len[..., None]
+        for t in (c.K_out, c.V_out, c.out_pos):
+            assert not t[rest].any()
+        if n == 2:                                    # (alone: the same bits)
+            assert all(torch.equal(getattr(c, k), getattr(ref, k)) for k in ("K_out", "V_out", "out_pos"))
+
 def test_a_layer_that_is_dropped_is_freed():
     p = kvm.make_params(1, 4, 4, 1024, 128, torch.bfloat16)
     layers = [tuple(torch.randn(1, 4, 1024, 128, device="cuda").bfloat16() for _ in "QKV") for _ in range(4)]
