@@ -468,8 +468,9 @@ prefill_attend_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
 // O is divided by the sum of the rounded weights, so that what rounding them did to a row's largest weight cancels (the
 // kernel above has two references a row, whose weights are exactly 1): error of O against 64 bits 1.984e-3 against 2.081e-3
 // of the kernel above (32 heads x 4096), 1.983e-3 against 1.992e-3 (10007 x 64), 2.08e-3 without, for 3 % (5 %) of the time.
-// A tile's products are issued in the order P V (j), Q K^T (j + 1) by one thread, so an S that is there says that the last
-// P V is done: O may be rescaled, and P written, without another barrier.
+// A tile's products are issued in the order P V (j), Q K^T (j + 1) by one thread and run in that order (a CTA's products pass
+// the tensor pipe one after the other), so S may take P's place, and an S that is there says that the last P V is done (a
+// commit covers all that its thread issued before): O may be rescaled, and P written, without another barrier.
 constexpr int NST = 2;                  // iterations in the rings of K and V tiles
 constexpr int REGS_PAIR_OTHER = 88;     // (2 x 128 x 208 + 128 x 88 = 384 x 168, what the block is launched with)
 // How far (log2) a maximum may outgrow its row's reference.  Keys of one neighbourhood are alike, so a row's maximum grows by
