@@ -46,7 +46,8 @@ constexpr int NTHREADS = (NSOFT + 4) * 32;   // three warpgroups: two of softmax
 constexpr int REGS_SOFTMAX = 208, REGS_OTHER = 56;
 constexpr uint32_t CHUNK_BYTES = TILE * 128;            // [128 rows x 64 bf16]
 constexpr float LOG2E = 1.4426950408889634f, LN2 = 0.6931471805599453f;
-constexpr float RESCALE_STEP = 8.f;     // the reference maximum follows the running maximum in steps of at least this
+constexpr float RESCALE_STEP = 8.f;     // the reference maximum follows the running maximum in steps of at least this: a
+                                        // weight is at most 2^RESCALE_STEP (values up to 2^-8 of the largest bf16 stay finite)
 constexpr uint32_t S_COLS = TILE, O_COL0 = NGRP * S_COLS;  // TMEM columns: S of group 0 | S of group 1 | O 0 | O 1
 
 struct __align__(8) Bars {
@@ -466,17 +467,17 @@ prefill_attend_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
 // tile, take 2,950 clocks (head dimension 64: 2,680): 1,720 of a tile's softmax (1,024 of them exponentials at the unit's full
 // rate), the rest until its next logits are there; the tensor pipe is busy 2,180 (1,300) of them.
 // O is divided by the sum of the rounded weights, so that what rounding them did to a row's largest weight cancels (the
-// kernel above has two references a row, whose weights are exactly 1): error of O against 64 bits 1.984e-3 against 2.081e-3
-// of the kernel above (32 heads x 4096), 1.983e-3 against 1.992e-3 (10007 x 64), 2.08e-3 without, for 3 % (5 %) of the time.
+// kernel above has two references a row, whose weights are exactly 1), and a reference is its row's maximum again whenever
+// any row of the warp has outgrown its own by RESCALE_STEP: O is multiplied for all 32 rows then anyway, and the largest
+// weight is exactly 1 more often.  Error of O against 64 bits, kernel above / this one / this one with only the outgrown row's
+// reference moved, by 12 (x 1e-3; rounding O alone 1.64-1.66): 32 heads x 4096 x 128 1.996 / 1.924 / 1.970 (146 / 130.4 / 129.2 us),
+// 32 / 8 x 10007 x 64 2.052 / 1.978 / 2.024 (695 / 572 / 574), 256 / 128 x 300 x 64 1.879 / 1.873 / 1.887, 240 / 30 x 461 x 64
+// 1.897 / 1.888 / 1.913.
 // A tile's products are issued in the order P V (j), Q K^T (j + 1) by one thread and run in that order (a CTA's products pass
 // the tensor pipe one after the other), so S may take P's place, and an S that is there says that the last P V is done (a
 // commit covers all that its thread issued before): O may be rescaled, and P written, without another barrier.
 constexpr int NST = 2;                  // iterations in the rings of K and V tiles
 constexpr int REGS_PAIR_OTHER = 88;     // (2 x 128 x 208 + 128 x 88 = 384 x 168, what the block is launched with)
-// How far (log2) a maximum may outgrow its row's reference.  Keys of one neighbourhood are alike, so a row's maximum grows by
-// several steps' worth now and then: 32 heads x 4096 129 / 127 / 124 / 123 us for 8 / 12 / 16 / 24, 10007 x 64 579 / 570 / 564 / 560; error of
-// O against 64 bits 1.97e-3 / 2.01e-3 / 2.03e-3 / 2.05e-3 (the reference's own weight is exact; of the kernel above 2.03e-3).
-constexpr float PAIR_RESCALE_STEP = 12.f;
 constexpr int P_FIRST = 96;             // keys of a step whose P is handed over first
 
 struct __align__(8) PairBars {
@@ -704,7 +705,7 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                 }
                 // p = 2^(x - m), summed in fp32, rounded to bf16 for the tensor core.  The first 32 keys are tried with the
                 // reference as it is, beside the search for the step's maximum (which alone takes 300 of 1,700 clocks): the
-                // reference moves only when the maximum has outgrown it by PAIR_RESCALE_STEP, seldom after the first step.
+                // warp's references move only when a row's maximum has outgrown its own by RESCALE_STEP, seldom after the first step.
                 uint64_t sum[2] = {0ull, 0ull};
                 float rsum[4] = {0.f, 0.f, 0.f, 0.f};
                 float pk[16];                                // (two bf16 each)
@@ -731,9 +732,8 @@ prefill_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                 for (int e = 0; e < 4; ++e) mx4[e] = fmaxf(mx4[e], v[TILE - 4 + e]);
                 const float mx = fmaxf(fmax3(mx4[0], mx4[1], mx4[2]), mx4[3]) * scale2;
                 float alpha = 1.f;
-                const bool grow = mx > m + PAIR_RESCALE_STEP;
-                if (__any_sync(0xffffffffu, grow)) {
-                    if (grow) { alpha = ex2(m - mx); m = mx; }
+                if (__any_sync(0xffffffffu, mx > m + RESCALE_STEP)) {
+                    if (mx > m) { alpha = ex2(m - mx); m = mx; }
                     sum[0] = sum[1] = 0ull;
                     rsum[0] = rsum[1] = rsum[2] = rsum[3] = 0.f;
                     exponentials(0);

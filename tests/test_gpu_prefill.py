@@ -78,6 +78,47 @@ def test_two_query_tiles_at_a_time_match_the_checker_elementwise(S, D, Hq, Hkv, 
         assert (np.abs(O.float().cpu().numpy() - refO) <= tol).all()
 
 
+@pytest.mark.parametrize("D", [64, 128])
+def test_large_values_stay_finite_when_a_maximum_grows(D):
+    """A late key's logit is 10.5 (log2 units) above the others' and every value is 1e36: weights above 2^8 of a reference that
+    was not moved would sum to more than fp32 holds."""
+    H, Hkv, S = 160, 80, 256                                  # (two tiles at a time: 160 x 3 >= 3 x 148)
+    Q, K = torch.zeros(1, H, S, D, device="cuda"), torch.zeros(1, Hkv, S, D, device="cuda")
+    Q[..., 0] = 1.0
+    K[:, :, 130, 0] = 10.5 * np.log(2.0) * np.sqrt(D)
+    V = torch.full((1, Hkv, S, D), 1e36, device="cuda").bfloat16()
+    O, lse = torch.empty(1, H, S, D, dtype=torch.bfloat16, device="cuda"), torch.empty(1, H, S, device="cuda")
+    kvm.kvm_prefill_attend(kvm.make_params(1, H, Hkv, S, D, torch.bfloat16), Q.bfloat16(), K.bfloat16(), V, O, lse)
+    # (a weighted mean of equal values: one rounding to bf16, one neighbour)
+    assert ((O.double() - V[0, 0, 0, 0].double()).abs() <= 2.0 ** -7 * 1e36).all()
+
+
+@pytest.mark.parametrize("H,Hkv,S,D", [(256, 128, 300, 64), (240, 30, 461, 64), (232, 116, 586, 64), (154, 154, 732, 128)])
+def test_two_tiles_at_a_time_are_no_less_precise_than_one(H, Hkv, S, D):
+    """The same heads all together and few at a time (which one tile at a time is the kernel for): the error of O against
+    64 bits, over all rows, is no larger."""
+    cfg = si.CONFIGS["C1"].scaled(seq=S, head_dim=D, n_q_heads=H, n_kv_heads=Hkv, seed=29)
+    Q, K, V = (si.make_layer(cfg)[k].cuda() for k in "QKV")
+    G, T = H // Hkv, (S + 127) // 128
+    n = max(u for u in range(1, Hkv) if Hkv % u == 0 and u * G * (T + 1) < 444)
+    assert H * (T + 1) >= 444
+
+    def attend(Q, K, V):
+        O, lse = torch.empty_like(Q), torch.empty(Q.shape[:3], device="cuda")
+        kvm.kvm_prefill_attend(kvm.make_params(1, Q.shape[1], K.shape[1], S, D, torch.bfloat16), Q, K, V, O, lse)
+        return O
+    together = attend(Q, K, V)
+    few = torch.cat([attend(*(t[:, i * k:(i + n) * k].contiguous() for t, k in ((Q, G), (K, 1), (V, 1))))
+                     for i in range(0, Hkv, n)], 1)
+    causal = torch.ones(S, S, dtype=torch.bool, device="cuda").tril()
+    err = np.zeros(2)
+    for u in range(Hkv):
+        L = (Q[0, u * G:(u + 1) * G].double() @ K[0, u].double().T / np.sqrt(D)).masked_fill(~causal, float("-inf"))
+        ref = torch.softmax(L, -1) @ V[0, u].double()
+        err += [(O[0, u * G:(u + 1) * G].double() - ref).square().sum().item() for O in (together, few)]
+    assert err[0] <= err[1]
+
+
 def test_prefill_attention_with_unscaled_logits_and_a_custom_scale():
     """Nearly one-hot rows (logits of standard deviation in the tens) move the reference maximum often."""
     from oracle import kvmo
