@@ -30,7 +30,7 @@
 // 32 heads x 4096 x 128 351 / 377; 4 heads x 512 x 64 100 / 74 -> 9 / 9.  What bounds a step now is its 48 products: 3,340 of
 // 3,960 clocks, at the clock that so busy a tensor pipe is left by the power limit.  Before, the epilogue did (two steps in
 // 10,900 clocks, 5,000 of a step's 10,000 spent on joining the row pass's states): now those are joined by a kernel between
-// the passes, asked for a step ahead, and the exponentials are single instructions.
+// the passes where a step would read many, asked for a step ahead, and the exponentials are single instructions.
 // Tried without gain: eleven converter warps, a barrier per plane, planes split beforehand and fetched by TMA (the extra pass
 // costs what the conversion costs here).
 //
@@ -63,6 +63,16 @@ constexpr int NEPI = 8, NCONV = 7;                // warps; with the MMA warp si
 constexpr int NTHREADS = (NEPI + NCONV + 1) * 32;
 constexpr int SIM_RUN = 8;                         // consecutive tokens per lane group (similarities)
 constexpr int NSLOT = 8;                           // piece-end buffers in rotation
+// The row pass's states are joined by a kernel between the passes where an epilogue group would read this many of them one after
+// the other (steps of a CTA / 2, by the pieces of a row): the launch takes 1.2 us, a state 0.2-0.4 us of every step, of which the
+// step's own products hide a part (twice the channels, or a second step under way, hide more).  us a kvm_score call, read by the
+// steps / joined between; D = 64: 1 head x 256 tokens (2 states) 16.2 / 17.5, 16 / 8 x 512 (3, two steps) 21.3 / 22.5, 8 / 4 x 1024 (5,
+// two steps) 24.0 / 24.6, 32 x 512 (4, three steps) 28.3 / 27.6, 4 x 512 (4) 19.7 / 19.1, 1 x 700 (6) 21.7 / 19.5; D = 128: 4 x 512 (4)
+// 21.5 / 22.5, 32 x 512 (4, three steps) 35.9 / 37.0, 8 / 4 x 1024 (5, two steps) 28.9 / 30.4, 16 / 8 x 700 (6) 34.6 / 34.7, 32 x 700 (6)
+// 50.0 / 49.2, 4 x 2048 (10) 45.2 / 43.0, 16 / 8 x 2999 (34) 212.9 / 200.8.
+bool join_between(const Plan& p, int D) {
+    return (p.q + 1) / 2 * (unsigned)p.pr >= (D == 64 && p.q != 2 ? 4u : 6u);
+}
 constexpr size_t SPLIT_BYTES_MAX = (size_t)KVM_STATIC_SCORE_ROWS * sizeof(float);
 constexpr float LOG2E = 1.4426950408889634f, LN2 = 0.6931471805599453f;
 
@@ -166,12 +176,13 @@ struct Feed {
     }
 };
 
-// flat (nullable): the rows' log-sum-exp, times flat_mul in log2 units; else the row pass's states are combined.
+// flat (nullable): the rows' log-sum-exp, times flat_mul in log2 units; else joined: states hold it (join_states_kernel), or the
+// row pass's states are combined here.
 template <int KCH, int PASS>
 __global__ void __launch_bounds__(NTHREADS, 1)
 score_f32_kernel(const float* __restrict__ Q, const float* __restrict__ K, float2* __restrict__ states,
                  const float* __restrict__ flat, float flat_mul, float* __restrict__ out, kvm_stats* stats,
-                 const Plan plan, int Hq, int Hkv, int S, float scale2, float* __restrict__ sim_out) {
+                 const Plan plan, int Hq, int Hkv, int S, float scale2, int joined, float* __restrict__ sim_out) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* sA = smem_raw + (base - smem_u32(smem_raw));     // [KCH][plane][128 rows][128 B]
@@ -304,8 +315,8 @@ score_f32_kernel(const float* __restrict__ Q, const float* __restrict__ K, float
         const uint64_t sc2 = pack2(scale2, scale2);
         uint32_t cnt = 0, own = 0;
         const size_t rows = (size_t)plan.NH * S;
-        // The log-sum-exp (log2 units) of four of the 128 queries of tile t of the group's query head h: the caller's, the row
-        // pass's, or what join_states_kernel made of its states.  Queries past the end weigh nothing.
+        // The log-sum-exp (log2 units) of four of the 128 queries of tile t of the group's query head h: the caller's or the row
+        // pass's, what join_states_kernel left, or made of the row pass's states here.  Queries past the end weigh nothing.
         auto ask = [&](float (&v)[4], int h, int t) {
             const int qh = (w.head / Hkv) * Hq + (w.head % Hkv) * plan.G + h;
             const size_t r = (size_t)qh * S + t * TILE + lane;
@@ -313,9 +324,22 @@ score_f32_kernel(const float* __restrict__ Q, const float* __restrict__ K, float
             if (flat) {
 #pragma unroll
                 for (int e = 0; e < 4; ++e) v[e] = e * 32 < left ? flat[r + e * 32] * flat_mul : INFINITY;
-            } else {
+            } else if (joined) {
 #pragma unroll
                 for (int e = 0; e < 4; ++e) v[e] = e * 32 < left ? __ldcg(&states[r + e * 32].x) : INFINITY;
+            } else {
+                const int np = plan.row_pieces(qh, t);
+                float M[4], L[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) { M[e] = -INFINITY; L[e] = 0.f; }
+#pragma unroll 1
+                for (int x = 0; x < np; ++x) {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        if (e * 32 < left) add_state(M[e], L[e], __ldcg(states + (size_t)x * rows + r + e * 32));
+                }
+#pragma unroll
+                for (int e = 0; e < 4; ++e) v[e] = e * 32 < left ? M[e] + log2f(L[e]) : INFINITY;
             }
         };
         float ahead[4] = {0.f, 0.f, 0.f, 0.f};
@@ -347,7 +371,7 @@ score_f32_kernel(const float* __restrict__ Q, const float* __restrict__ K, float
                 ++own;
                 if (ok) tc_fence_after();
                 if (PASS == 2) {
-                    asked = i + 2 < w.n;
+                    asked = (flat || joined) && i + 2 < w.n;
                     if (asked) {
                         const int bn = bt + 1 == plan.T ? w.tile : bt + 1, gn = bt + 1 == plan.T ? g + 1 : g;
                         ask(ahead, gn, bn);
@@ -503,9 +527,7 @@ __global__ void __launch_bounds__(256) combine_kernel(const float* __restrict__ 
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j < S) scores[(size_t)blockIdx.y * S + j] = plan::column_sum(part, plan, S, blockIdx.y, j);
 }
-// The row pass's states of cut items -> the rows' log-sum-exp (log2 units), in the place of their first states.  (Joined by
-// every step of the column pass that reads them instead of by this launch, us a call joined / not: 4 heads x 512 x 64, one step
-// per CTA, 30.6 / 31.6; 4 x 1024 34.3 / 38.4; 18 / 9 x 1000, five steps, 49.7 / 52.5; 16 / 8 x 2999 x 128 232 / 238.)
+// The row pass's states of cut items -> the rows' log-sum-exp (log2 units), in the place of their first states.
 __global__ void __launch_bounds__(256) join_states_kernel(float2* __restrict__ states, const Plan plan, int S) {
     grid_dependency_wait();
     const size_t rows = (size_t)plan.NH * S, r = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -551,7 +573,7 @@ cudaError_t launch_t(const Dims& d, const Plan& plan, const float* Q, const floa
     const float scale2 = d.scale * LOG2E;
     if (!lse_in) {
         e = launch_dependent(score_f32_kernel<KCH, 1>, rgrid, block, smem, st, Q, K, states, (const float*)nullptr,
-                             1.f, flat, stats, plan, d.Hq, d.Hkv, d.S, scale2, (float*)nullptr);
+                             1.f, flat, stats, plan, d.Hq, d.Hkv, d.S, scale2, 0, (float*)nullptr);
         if (e != cudaSuccess) return e;
     }
     if (lse_out) {
@@ -560,13 +582,14 @@ cudaError_t launch_t(const Dims& d, const Plan& plan, const float* Q, const floa
         if (e != cudaSuccess) return e;
     }
     if (!scores) return cudaSuccess;
-    if (!lse_in && plan.split_row) {
+    const bool join = !lse_in && plan.split_row && join_between(plan, d.D);
+    if (join) {
         e = launch_dependent(join_states_kernel, dim3((unsigned)((rows + 255) / 256)), dim3(256), 0, st, states, plan, d.S);
         if (e != cudaSuccess) return e;
     }
     e = launch_dependent(score_f32_kernel<KCH, 2>, cgrid, block, smem, st, Q, K, states,
                          lse_in ? lse_in : (const float*)flat, lse_in ? LOG2E : 1.f, plan.split_col ? part : scores, stats, plan,
-                         d.Hq, d.Hkv, d.S, scale2, sim_out);
+                         d.Hq, d.Hkv, d.S, scale2, (int)join, sim_out);
     if (e != cudaSuccess || !plan.split_col) return e;
     if (parts) {                                      // the caller's next kernel adds the pieces up
         parts->part = part;

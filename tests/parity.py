@@ -390,3 +390,27 @@ def host_groups(units, unit_bytes):
         e = int(acc / total * units + 0.5)
         first.append(units if c + 1 == n else min(max(e, first[c] + 1), units - (n - 1 - c)))
     return [b - a for a, b in zip(first, first[1:])]
+
+
+def launched(fn):
+    """What `fn` enqueues on the current stream: the kernels' names, in order, and "memset" or the like for other nodes."""
+    from cuda.bindings import driver as cu
+    fn()                                       # (attributes are set, modules loaded)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(g):
+        fn()
+    graph = cu.CUgraph(g.raw_cuda_graph())
+    _, _, n = cu.cuGraphGetNodes(graph, 0)
+    err, nodes, n = cu.cuGraphGetNodes(graph, n)
+    assert err == cu.CUresult.CUDA_SUCCESS
+    names = []
+    for node in nodes[:n]:
+        kind = cu.cuGraphNodeGetType(node)[1]
+        if kind != cu.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL:
+            names.append(kind.name.replace("CU_GRAPH_NODE_TYPE_", "").lower())
+            continue
+        params = cu.cuGraphKernelNodeGetParams(node)[1]
+        name = cu.cuKernelGetName(params.kern)[1] if int(params.kern) else cu.cuFuncGetName(params.func)[1]
+        names.append(name.decode())
+    return names

@@ -49,6 +49,33 @@ def test_scores_and_row_lse_against_fp64(B, Hq, Hkv, S, D):
                 assert ((got[b, u].double() - ref).abs() / ref).max().item() <= 2.1 * delta + 2.0 ** -17
 
 
+@pytest.mark.parametrize("Hq,Hkv,S,D,joined", [
+    (1, 1, 130, 64, False),        # two states a row, one step a CTA
+    (4, 4, 512, 128, False),       # four states, one step
+    (4, 4, 512, 64, True),         # ... of half the channels
+    (8, 4, 1024, 64, False),       # five, two steps
+    (1, 1, 700, 128, True),        # six, one step
+    (32, 32, 389, 64, True),       # two, three steps
+    (32, 32, 700, 128, True),      # two, five steps
+])
+def test_row_states_are_joined_by_a_launch_where_steps_would_read_many(Hq, Hkv, S, D, joined):
+    """A launch between the passes costs a small call more than its steps' few reads; both forms give the same bits as the
+    column pass fed with the row log-sum-exp (which joins the states by a kernel of its own) to the rounding of the units."""
+    from parity import launched
+    g = torch.Generator().manual_seed(S)
+    Q, K = torch.randn(1, Hq, S, D, generator=g).cuda(), torch.randn(1, Hkv, S, D, generator=g).cuda()
+    p = kvm.make_params(1, Hq, Hkv, S, D, torch.float32, budget=1.0, recent_ratio=0.0, heavy_ratio=0.0)
+    ws = torch.empty(kvm.kvm_workspace_bytes(p), dtype=torch.uint8, device="cuda")
+    scores, with_lse, lse = torch.empty(1, Hkv, S, device="cuda"), torch.empty(1, Hkv, S, device="cuda"), torch.empty(1, Hq, S, device="cuda")
+    kvm.kvm_score(p, Q, K, None, scores, ws)
+    kvm.kvm_row_lse(p, Q, K, lse, ws)
+    kvm.kvm_score(p, Q, K, lse, with_lse, ws)
+    # (log2 units to natural and back: two roundings of a number below 64, 2^-24 of it each)
+    assert ((scores - with_lse).abs() <= 2.0 ** -17 * with_lse).all()
+    names = launched(lambda: kvm.kvm_score(p, Q, K, None, scores, ws))
+    assert sum("join_states_kernel" in n for n in names) == int(joined) and sum("score_f32_kernel" in n for n in names) == 2
+
+
 def _reference(Q, K, allowed):
     L = (Q.double() @ K.double().transpose(-1, -2) / math.sqrt(Q.shape[-1])).masked_fill(~allowed, float("-inf"))
     return torch.nan_to_num(torch.softmax(L, -1)).sum(-2)          # (rows without any key weigh nothing)
