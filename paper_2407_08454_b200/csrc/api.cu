@@ -133,7 +133,7 @@ int run_chain(const Dims& d, const Layers& L, const float* lse_in, float* scores
     if (launch_segment(d, L, scores, parts, w.sim, w.set_id, w.set_start, stats, st) != cudaSuccess) return KVM_E_CUDA;
     const cudaError_t e =
         d.weight_rule == KVM_WEIGHT_PIVOT_ONLY
-            ? launch_gather(d, L.K[0], L.V[0], w.set_start, L.pivot[0], L.out_len[0], L.K_out[0], L.V_out[0], nullptr, st)
+            ? launch_gather(d, L.K[0], L.V[0], w.set_start, L.pivot[0], L.out_len[0], L.K_out[0], L.V_out[0], nullptr, L.zero_rest ? L.pivot[0] : nullptr, st)
             : launch_merge(d, L, w.set_start, w.set_id, nullptr, w.merge_part, w.sim, w.scores, stats, st);
     return e == cudaSuccess ? KVM_OK : KVM_E_CUDA;
 }
@@ -331,7 +331,7 @@ int kvm_merge_compact(const kvm_params* p, const void* K, const void* V, const i
     if ((rc = check_ws(d, ws, ws_bytes, w)) != KVM_OK) return rc;
     cudaStream_t st = (cudaStream_t)cuda_stream;
     if (d.weight_rule == KVM_WEIGHT_PIVOT_ONLY)
-        return launch_gather(d, K, V, set_start, pivot, out_len, K_out, V_out, out_size, st) == cudaSuccess
+        return launch_gather(d, K, V, set_start, pivot, out_len, K_out, V_out, out_size, nullptr, st) == cudaSuccess
                    ? KVM_OK
                    : KVM_E_CUDA;
     if (launch_token_sets(d, set_start, out_len, w.set_id, st) != cudaSuccess) return KVM_E_CUDA;
@@ -412,13 +412,6 @@ static int compress_layers(int zero_rest, const kvm_params* p, int32_t n_layers,
         }
         const Dims dn = times_batch(d, n);
         const Workspace wn = carve(dn, ws);
-        if (zero_rest && d.weight_rule == KVM_WEIGHT_PIVOT_ONLY) {       // (a gather, no merge: one layer at a time)
-            const size_t kv = (size_t)d.U * d.cap * d.D * (d.dtype == KVM_BF16 ? 2 : 4);
-            cudaStream_t st = (cudaStream_t)cuda_stream;
-            if (cudaMemsetAsync(L.K_out[0], 0, kv, st) != cudaSuccess || cudaMemsetAsync(L.V_out[0], 0, kv, st) != cudaSuccess ||
-                cudaMemsetAsync(L.pivot[0], 0, (size_t)d.U * d.cap * sizeof(int32_t), st) != cudaSuccess)
-                return KVM_E_CUDA;
-        }
         rc = run_chain(dn, L, nullptr, wn.scores, wn, stats, (cudaStream_t)cuda_stream);
         if (rc != KVM_OK) return rc;
         l0 += n;

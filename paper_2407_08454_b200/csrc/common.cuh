@@ -32,7 +32,7 @@ template <int NL> struct LayersOf {
     void *K_out[NL], *V_out[NL];
     int32_t *out_len[NL], *pivot[NL];
     float eps[NL];
-    int zero_rest;                                 // the merge also zero-fills the rows and positions past a unit's length
+    int zero_rest;                                 // the merge or gather also zero-fills the rows and positions past a unit's length
 };
 using Layers = LayersOf<MAX_LAYERS>;
 inline LayersOf<1> first_of(const Layers& L) {
@@ -146,10 +146,11 @@ cudaError_t launch_token_sets(const Dims& d, const int32_t* set_start, const int
                               cudaStream_t st);
 cudaError_t launch_merge(const Dims& d, const Layers& L, const int32_t* set_start, const int32_t* set_id, int32_t* out_size,
                          float* scratch, float* set_coef, float* token_d2, kvm_stats* stats, cudaStream_t st);
-// Rows that are one input state each (pivot-only weights, eviction): a gather.
+// Rows that are one input state each (pivot-only weights, eviction): a gather.  zero_pos (nullable: pivot): rows and positions
+// past the lengths become zero.
 cudaError_t launch_gather(const Dims& d, const void* K, const void* V, const int32_t* set_start,
                           const int32_t* pivot, const int32_t* out_len, void* K_out, void* V_out, int32_t* out_size,
-                          cudaStream_t st);
+                          int32_t* zero_pos, cudaStream_t st);
 
 // Decode-step attention over a ragged cache and the full-vs-compressed output difference.
 size_t attend_scratch_floats(const Dims& d);

@@ -354,25 +354,35 @@ __global__ void __launch_bounds__(256) set_coef_kernel(const float* __restrict__
 }
 
 // Output rows that are a single input state: row s = K[pivot[s]], V[pivot[s]] (V times the set size when
-// asked and the sets are real ones).  One lane group per (row, tensor), 16-byte copies.
+// asked and the sets are real ones).  One lane group per (row, tensor), 16-byte copies.  zero_pos (nullable: pivot): rows and
+// positions past a unit's length become zero.  (By memsets before the chain, three a layer: 363 us for 8 layers of
+// 32 / 8 heads x 512 tokens; with one fill of all of them before the first layer 308; so 300.)
 template <typename T, int D>
 __global__ void __launch_bounds__(256) gather_rows_kernel(const T* __restrict__ K, const T* __restrict__ V,
                                                           const int32_t* __restrict__ set_start,
                                                           const int32_t* __restrict__ pivot,
                                                           const int32_t* __restrict__ out_len, T* __restrict__ K_out,
                                                           T* __restrict__ V_out, int32_t* __restrict__ out_size,
-                                                          int S, int cap, int scale_v, int singletons) {
+                                                          int S, int cap, int scale_v, int singletons,
+                                                          int32_t* __restrict__ zero_pos) {
     constexpr int N = Vec<T>::N, LPR = D / N, ROWS = 256 / LPR / 2;
     grid_dependency_wait();     // sets and pivots come from the kernel before this one
     const long long u = blockIdx.y;
     const int g = threadIdx.x / LPR, lane = threadIdx.x % LPR;
     const int s = blockIdx.x * ROWS + (g >> 1), which = g & 1;
-    if (s >= min(__ldcg(out_len + u), cap)) return;
+    if (s >= cap) return;
+    T* dst = (which ? V_out : K_out) + ((size_t)u * cap + s) * D + lane * N;
+    if (s >= __ldcg(out_len + u)) {
+        if (zero_pos) {
+            *reinterpret_cast<uint4*>(dst) = make_uint4(0u, 0u, 0u, 0u);
+            if (which == 0 && lane == 0) zero_pos[(size_t)u * cap + s] = 0;
+        }
+        return;
+    }
     const int p = __ldcg(pivot + (size_t)u * cap + s);
     const int32_t* st = set_start + (size_t)u * (cap + 1);
     const int n = singletons ? 1 : __ldcg(st + s + 1) - __ldcg(st + s);
     const T* src = (which ? V : K) + ((size_t)u * S + p) * D + lane * N;
-    T* dst = (which ? V_out : K_out) + ((size_t)u * cap + s) * D + lane * N;
     uint4 r = ldg16(src);
     if (which && scale_v && n > 1) {
         float x[N];
@@ -388,11 +398,11 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const T* __restrict__ 
 template <typename T, int D>
 cudaError_t launch_gather_t(const Dims& d, const void* K, const void* V, const int32_t* set_start,
                             const int32_t* pivot, const int32_t* out_len, void* K_out, void* V_out,
-                            int32_t* out_size, cudaStream_t st) {
+                            int32_t* out_size, int32_t* zero_pos, cudaStream_t st) {
     constexpr int ROWS = 256 / (D / Vec<T>::N) / 2;
     return launch_dependent(gather_rows_kernel<T, D>, dim3((d.cap + ROWS - 1) / ROWS, d.U), dim3(256), 0, st,
                             (const T*)K, (const T*)V, set_start, pivot, out_len, (T*)K_out, (T*)V_out, out_size, d.S,
-                            d.cap, d.scale_v, d.set_rule == KVM_SETS_CONSERVED_ONLY ? 1 : 0);
+                            d.cap, d.scale_v, d.set_rule == KVM_SETS_CONSERVED_ONLY ? 1 : 0, zero_pos);
 }
 
 template <typename T, int D, int TOK, int NL>
@@ -456,14 +466,14 @@ cudaError_t launch_token_sets(const Dims& d, const int32_t* set_start, const int
 
 cudaError_t launch_gather(const Dims& d, const void* K, const void* V, const int32_t* set_start,
                           const int32_t* pivot, const int32_t* out_len, void* K_out, void* V_out, int32_t* out_size,
-                          cudaStream_t st) {
+                          int32_t* zero_pos, cudaStream_t st) {
     if (d.dtype == KVM_BF16) {
         return d.D == 128
-                   ? launch_gather_t<__nv_bfloat16, 128>(d, K, V, set_start, pivot, out_len, K_out, V_out, out_size, st)
-                   : launch_gather_t<__nv_bfloat16, 64>(d, K, V, set_start, pivot, out_len, K_out, V_out, out_size, st);
+                   ? launch_gather_t<__nv_bfloat16, 128>(d, K, V, set_start, pivot, out_len, K_out, V_out, out_size, zero_pos, st)
+                   : launch_gather_t<__nv_bfloat16, 64>(d, K, V, set_start, pivot, out_len, K_out, V_out, out_size, zero_pos, st);
     }
-    return d.D == 128 ? launch_gather_t<float, 128>(d, K, V, set_start, pivot, out_len, K_out, V_out, out_size, st)
-                      : launch_gather_t<float, 64>(d, K, V, set_start, pivot, out_len, K_out, V_out, out_size, st);
+    return d.D == 128 ? launch_gather_t<float, 128>(d, K, V, set_start, pivot, out_len, K_out, V_out, out_size, zero_pos, st)
+                      : launch_gather_t<float, 64>(d, K, V, set_start, pivot, out_len, K_out, V_out, out_size, zero_pos, st);
 }
 
 // set_coef [U, cap] and token_d2 [U, S]: fp32 scratch, used only by the per-set bandwidth rule.

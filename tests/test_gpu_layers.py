@@ -67,6 +67,48 @@ def test_rows_past_a_units_length_are_zero(n, S, Hkv, D, dtype, rules):
         if n == 2:                                    # (alone: the same bits)
             assert all(torch.equal(getattr(c, k), getattr(ref, k)) for k in ("K_out", "V_out", "out_pos"))
 
+def _call_layers(name, p, layers, outs, ws, eps=None):
+    """kvm_compress_layers or kvm_compress_layers_filled on the caller's buffers (K_out, V_out, out_len, out_pos per layer)."""
+    import ctypes
+    array = ctypes.c_void_p * len(layers)
+    q, k, v = (array(*[l[i].data_ptr() for l in layers]) for i in range(3))
+    ko, vo, ln, pos = (array(*[o[i].data_ptr() for o in outs]) for i in range(4))
+    binding._call(name, p, len(layers), eps and (ctypes.c_float * len(layers))(*eps), q, k, v, ko, vo, ln, pos, None,
+                  ws.data_ptr(), ws.nbytes, binding._stream(None))
+
+
+def _dirty_outputs(n, Hkv, cap, D, dtype):
+    def full(shape, dt):
+        t = torch.empty(shape, dtype=dt, device="cuda")
+        t.view(torch.uint8).fill_(0xFF)
+        return t
+    return [(full((1, Hkv, cap, D), dtype), full((1, Hkv, cap, D), dtype), full((1, Hkv), torch.int32),
+             full((1, Hkv, cap), torch.int32)) for _ in range(n)]
+
+
+@pytest.mark.parametrize("S,Hkv,D,dtype,rules", [
+    (700, 2, 64, torch.bfloat16, {"set_rule": kvm.KVM_SETS_CONSERVED_ONLY}),
+    (129, 3, 128, torch.float32, {"set_rule": kvm.KVM_SETS_CONSERVED_ONLY}),
+    (500, 2, 128, torch.bfloat16, {"weight_rule": kvm.KVM_WEIGHT_PIVOT_ONLY}),
+])
+def test_gathered_layers_are_zero_past_their_length_without_further_launches(S, Hkv, D, dtype, rules):
+    from parity import launched
+    p = kvm.make_params(1, Hkv, Hkv, S, D, dtype, **rules)
+    # (neighbours alike, so that there are fewer sets than rows)
+    layers = [tuple(torch.randn(1, Hkv, S // 8 + 1, D, device="cuda").repeat_interleave(8, 2)[:, :, :S].to(dtype).contiguous()
+                    for _ in "QKV") for _ in range(3)]
+    cap = kvm.kvm_sizes(p)[0]
+    ws = torch.empty(binding.kvm_layers_workspace_bytes(p, 3), dtype=torch.uint8, device="cuda")
+    outs = _dirty_outputs(3, Hkv, cap, D, dtype)
+    filled = launched(lambda: _call_layers("kvm_compress_layers_filled", p, layers, outs, ws))
+    other = _dirty_outputs(3, Hkv, cap, D, dtype)
+    assert filled == launched(lambda: _call_layers("kvm_compress_layers", p, layers, other, ws))
+    for (ko, vo, n, pos), (Q, K, V) in zip(outs, layers):
+        ref = kvm.Compressor(p)(Q, K, V)              # (its buffers start at zero)
+        assert int(n.max()) < cap and torch.equal(n, ref.out_len)
+        assert torch.equal(ko, ref.K_out) and torch.equal(vo, ref.V_out) and torch.equal(pos, ref.out_pos)
+
+
 def test_a_layer_that_is_dropped_is_freed():
     p = kvm.make_params(1, 4, 4, 1024, 128, torch.bfloat16)
     layers = [tuple(torch.randn(1, 4, 1024, 128, device="cuda").bfloat16() for _ in "QKV") for _ in range(4)]
