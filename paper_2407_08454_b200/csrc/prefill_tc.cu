@@ -491,7 +491,8 @@ struct alignas(16) PairShared {
     int abort_flag;
 };
 
-// Item i of a CTA: tile[g] of query head[g] (n[g] key tiles; 0: none), longest first, boustrophedon.
+// Item i of a CTA: tile[g] of query head[g] (n[g] key tiles; 0: none), longest first, boustrophedon.  Of an odd number of tiles
+// it is the first, shortest one that stays alone.
 struct PairSched {
     int P, c, NH, T, by_head;
     __device__ __forceinline__ bool item(int i, int (&head)[2], int (&tile)[2], int (&n)[2]) const {
@@ -501,8 +502,8 @@ struct PairSched {
         const unsigned r = k / per, h = k - r * per, t = rows - 1 - r;
         for (int g = 0; g < 2; ++g) {
             head[g] = (int)(by_head ? 2 * h + g : h);
-            tile[g] = (int)(by_head ? t : 2 * t + g);
-            n[g] = tile[g] < T ? tile[g] + 1 : 0;
+            tile[g] = by_head ? (int)t : 2 * (int)t + g - (T & 1);
+            n[g] = tile[g] + 1;
         }
         return true;
     }
