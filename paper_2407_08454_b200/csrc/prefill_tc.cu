@@ -845,12 +845,23 @@ cudaError_t launch_t(const Dims& d, const CUtensorMap& mq, const CUtensorMap& mk
     const long long items = (long long)d.B * d.Hq * T;
     if (items + sms >= (1ll << 31)) return cudaErrorInvalidValue;   // the schedule counts items in 32 bits
     const int G = d.Hq / d.Hkv;
-    const long long pairs = G % 2 == 0 ? items / 2 : (long long)d.B * d.Hq * ((T + 1) / 2);
+    const long long heads = (long long)d.B * d.Hq, pairs = G % 2 == 0 ? items / 2 : heads * ((T + 1) / 2);
     // Two tiles at a time where the longest pair is not what a CTA's share is made of: its two tiles take turns where single ones
     // would run beside one another.  (us, single tiles / pairs, steps over T x 148 beside them; D = 128: 8 heads x 4096 tokens 0.9
-    // 40.9 / 57.8, 10 heads 1.1 52.3 / 58.7, 12 heads 1.3 62.2 / 59.0, 14 heads 1.6 69.6 / 59.5, 32 heads 3.6 147.6 / 127; 32 x 1024 1.0
-    // 24.7 / 23.4, 48 x 1024 1.5 25.8 / 19.9; D = 64: 100 x 500 1.7 16.5 / 16.2, 32 / 8 x 10007 8.6 703 / 558.)
-    if ((long long)d.B * d.Hq * T * (T + 1) >= 3ll * sms * T)
+    // 40.9 / 57.8, 10 heads 1.1 52.3 / 58.7, 12 heads 1.3 62.2 / 59.0, 14 heads 1.6 69.6 / 59.5, 32 heads 3.6 146 / 130; 32 x 1024 1.0
+    // 24.7 / 23.4, 48 x 1024 1.5 25.8 / 19.9; D = 64: 100 x 500 1.7 16.5 / 16.2, 32 / 8 x 10007 8.6 695 / 572.)
+    bool two = heads * T * (T + 1) >= 3ll * sms * T;
+    // Neighbouring tiles of a head are no pair where there is one tile (D = 64: 512 heads 14.4 / 15.5, 1024 heads 23.0 / 24.2; with
+    // 128 channels the output's way through shared memory is worth more: 444 heads 15.2 / 14.7, 512 17.4 / 17.6, 1024 31.3 / 28.1),
+    // and single tiles are faster where a few CTAs have a second pair (2 tiles, D = 128: 148 heads 13.1 / 11.0, 157 15.2 / 16.0, 193
+    // 15.7 / 17.1, 202 17.5 / 16.8; D = 64: 11.0 / 9.1, 12.4 / 13.9, 12.5 / 14.6, 14.4 / 14.7) or a short one beside the longest
+    // (4 tiles, D = 64: 94 heads 16.3 / 14.9, 99 16.4 / 17.0, 109 17.0 / 18.0, 114 18.8 / 17.8; D = 128: 104 20.7 / 20.1).
+    if (G % 2 != 0) {
+        if (T == 1) two = two && KCH == 2;
+        if (T == 2) two = two && (heads <= sms || 3 * heads > 4ll * sms);
+        if (T == 4) two = two && (KCH == 2 || 3 * heads <= 2ll * sms || 4 * heads > 3ll * sms);
+    }
+    if (two)
         return launch_dependent(prefill_pair_kernel<KCH>, dim3((unsigned)(pairs < sms ? pairs : sms)), dim3(NTHREADS), pair_smem, st, mq, mk,
                                 mv, mo, O, lse, stats, d.B * d.Hq, G, d.S, d.scale * LOG2E);
     const int grid = (int)(items < sms ? items : sms);

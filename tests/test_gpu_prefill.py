@@ -78,6 +78,34 @@ def test_two_query_tiles_at_a_time_match_the_checker_elementwise(S, D, Hq, Hkv, 
         assert (np.abs(O.float().cpu().numpy() - refO) <= tol).all()
 
 
+@pytest.mark.parametrize("S,D,Hq,Hkv,pairs", [
+    (100, 64, 256, 256, False),       # one tile a head: no pair
+    (128, 128, 456, 152, True),       # ... whose output is written the pairs' way (half of a block idle in every item)
+    (100, 64, 256, 128, True),        # two heads of a group
+    (250, 128, 148, 148, True),       # two tiles, a pair for every CTA
+    (250, 64, 166, 166, False),       # ... and a second one for few
+    (129, 128, 192, 64, False),
+    (255, 64, 231, 231, True),
+    (500, 64, 99, 33, False),         # four tiles: the longest pair and a short one
+    (500, 128, 99, 33, True),
+    (385, 64, 114, 114, True),
+    (300, 64, 111, 111, True),        # three: the first one alone, twice per CTA
+    (640, 64, 74, 74, True),          # five
+])
+def test_tiles_go_in_pairs_where_that_is_faster(S, D, Hq, Hkv, pairs):
+    from parity import launched
+    cfg = si.CONFIGS["C1"].scaled(seq=S, head_dim=D, n_q_heads=Hq, n_kv_heads=Hkv, seed=34)
+    d = si.make_layer(cfg)
+    p, Q, K, V, O, lse = _run(cfg, d)
+    names = launched(lambda: kvm.kvm_prefill_attend(p, Q, K, V, O, lse))
+    assert len(names) == 1 and ("prefill_pair_kernel" in names[0]) == pairs
+    G = Hq // Hkv
+    causal = torch.ones(S, S, dtype=torch.bool, device="cuda").tril()
+    L = (Q[0].double() @ K[0].repeat_interleave(G, 0).double().transpose(-1, -2) / np.sqrt(D)).masked_fill(~causal, float("-inf"))
+    refO = torch.softmax(L, -1) @ V[0].repeat_interleave(G, 0).double()
+    _check(O, lse, refO[None].cpu().numpy(), torch.logsumexp(L, -1)[None].cpu().numpy(), d["V"], G)
+
+
 @pytest.mark.parametrize("D", [64, 128])
 def test_large_values_stay_finite_when_a_maximum_grows(D):
     """A late key's logit is 10.5 (log2 units) above the others' and every value is 1e36: weights above 2^8 of a reference that
