@@ -296,7 +296,9 @@ class Compressor:
 def compress_layers(p: KvmParams, layers, sim_thresholds=None, device="cuda", stream=None):
     """Compress a stack of layers, each an (Q, K, V) triple of CUDA tensors of the shape `p` describes, with one
     similarity threshold per layer (Section 3.2: thresholds chosen layer by layer), through kvm_compress_layers_filled.
-    Returns, per layer, a `Compressed` holding the outputs, and the layer's compression ratio mean(out_len) / S."""
+    Returns, per layer, a `Compressed` holding the outputs, and the layer's compression ratio mean(out_len) / S.
+    `stream`: the one the kernels run on, after what the current stream has been given so far; the results are there when
+    the function returns."""
     # (the GPU waits for this function: whatever its results do not need is left until the kernels are enqueued, and the
     # addresses are worked out from the bases)
     n = len(layers)
@@ -318,12 +320,22 @@ def compress_layers(p: KvmParams, layers, sim_thresholds=None, device="cuda", st
         assert len(sim_thresholds) == n
         eps = (ctypes.c_float * n)(*[float(e) for e in sim_thresholds])
     bases, len_base = [b.data_ptr() for b in blobs], out_len.data_ptr()
+    handle, other = _stream(stream), None
+    if stream is not None and handle != _stream(None):
+        # (the buffers are the current stream's: what it last did with their memory comes before the kernels, and the
+        # workspace is not handed out again before they are through)
+        other = torch.cuda.ExternalStream(handle, device=out_len.device)
+        other.wait_stream(torch.cuda.current_stream(out_len.device))
+        for t in (*blobs, out_len, ws):
+            t.record_stream(other)
     _call("kvm_compress_layers_filled", p, n, eps, q, k, v, array(*bases), array(*[b + kv_bytes for b in bases]),
           array(*range(len_base, len_base + 4 * n * units, 4 * units)), array(*[b + 2 * kv_bytes for b in bases]), None,
-          ws.data_ptr(), ws.nbytes, _stream(stream))
+          ws.data_ptr(), ws.nbytes, handle)
     out = []
-    for blob, lengths in zip(blobs, out_len.unbind(0)):
+    for blob, layer_len in zip(blobs, out_len.unbind(0)):
         K_out, V_out = blob[:2 * kv_bytes].view(dtype).view(2, B, H, cap, D).unbind(0)
-        out.append(Compressed(K_out, V_out, lengths, blob[2 * kv_bytes:].view(torch.int32).view(B, H, cap), None, cap))
-    ratios = (out_len.cpu().float().mean((1, 2)) / p.seq).tolist()      # the one read-back of the call
+        out.append(Compressed(K_out, V_out, layer_len, blob[2 * kv_bytes:].view(torch.int32).view(B, H, cap), None, cap))
+    with torch.cuda.stream(other):                                      # (None: the current one)
+        lengths = out_len.cpu()                                         # the one read-back of the call
+    ratios = (lengths.float().mean((1, 2)) / p.seq).tolist()
     return out, ratios

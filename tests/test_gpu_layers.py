@@ -109,6 +109,24 @@ def test_gathered_layers_are_zero_past_their_length_without_further_launches(S, 
         assert torch.equal(ko, ref.K_out) and torch.equal(vo, ref.V_out) and torch.equal(pos, ref.out_pos)
 
 
+@pytest.mark.parametrize("as_handle", [False, True])
+def test_on_a_stream_that_is_not_the_current_one(as_handle):
+    """The ratios are read where the kernels run, the results and the freed workspace belong to the current stream."""
+    n, H, S, D = 3, 4, 600, 64
+    layers = [tuple(torch.randn(1, H, S // 8, D, device="cuda").repeat_interleave(8, 2).bfloat16() for _ in "QKV") for _ in range(n)]
+    p = kvm.make_params(1, H, H, S, D, torch.bfloat16)
+    want, ratios = kvm.compress_layers(p, layers)
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        torch.cuda._sleep(50_000_000)                 # (the kernels begin some 25 ms after the call)
+    got, got_ratios = kvm.compress_layers(p, layers, stream=s.cuda_stream if as_handle else s)
+    scratch = [torch.full((1 << 20,), -1, dtype=torch.int32, device="cuda") for _ in range(16)]      # (the freed workspace's memory, among others)
+    assert got_ratios == ratios and s.query()
+    for a, b in zip(got, want):
+        assert all(torch.equal(getattr(a, k), getattr(b, k)) for k in ("K_out", "V_out", "out_len", "out_pos"))
+    del scratch
+
+
 def test_a_layer_that_is_dropped_is_freed():
     p = kvm.make_params(1, 4, 4, 1024, 128, torch.bfloat16)
     layers = [tuple(torch.randn(1, 4, 1024, 128, device="cuda").bfloat16() for _ in "QKV") for _ in range(4)]
