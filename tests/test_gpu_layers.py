@@ -45,28 +45,6 @@ def test_layers_together_match_layers_alone(n, S, Hq, Hkv, D, dtype, monkeypatch
         assert same >= 0.97 * rows
 
 
-@pytest.mark.parametrize("n,S,Hkv,D,dtype,rules", [
-    (3, 389, 4, 128, "bf16", {}),                     # layers together; the last tile's share of the rows is cut
-    (2, 33, 3, 64, "f32", {}),                        # two tiles, capacity 16
-    (2, 700, 2, 64, "bf16", {"set_rule": kvm.KVM_SETS_CONSERVED_ONLY}),     # a gather instead of the merge
-    (2, 640, 2, 128, "bf16", {"weight_rule": kvm.KVM_WEIGHT_SET_SIGMA}),
-])
-def test_rows_past_a_units_length_are_zero(n, S, Hkv, D, dtype, rules):
-    cfg = si.CONFIGS["C1"].scaled(seq=S, head_dim=D, n_q_heads=Hkv, n_kv_heads=Hkv, dtype=dtype, seed=S)
-    layers = [tuple(si.make_layer(cfg, l)[k].cuda() for k in "QKV") for l in range(n)]
-    p = kvm.make_params(1, Hkv, Hkv, S, D, cfg.torch_dtype, **rules)
-    dirty = [torch.full((1 << 20,), -1, dtype=torch.int32, device="cuda") for _ in range(8)]
-    del dirty                                         # (what the results are allocated from is not zero)
-    out, _ = kvm.compress_layers(p, layers)
-    for c, (Q, K, V) in zip(out, layers):
-        ref = kvm.Compressor(p)(Q, K, V)              # (its buffers start at zero)
-        assert int(c.out_len.min()) < c.cap and torch.equal(c.out_len, ref.out_len)
-        rest = torch.arange(c.cap, device="cuda") >= c.out_len[..., None]
-        for t in (c.K_out, c.V_out, c.out_pos):
-            assert not t[rest].any()
-        if n == 2:                                    # (alone: the same bits)
-            assert all(torch.equal(getattr(c, k), getattr(ref, k)) for k in ("K_out", "V_out", "out_pos"))
-
 def _call_layers(name, p, layers, outs, ws, eps=None):
     """kvm_compress_layers or kvm_compress_layers_filled on the caller's buffers (K_out, V_out, out_len, out_pos per layer)."""
     import ctypes
@@ -84,6 +62,40 @@ def _dirty_outputs(n, Hkv, cap, D, dtype):
         return t
     return [(full((1, Hkv, cap, D), dtype), full((1, Hkv, cap, D), dtype), full((1, Hkv), torch.int32),
              full((1, Hkv, cap), torch.int32)) for _ in range(n)]
+
+
+@pytest.mark.parametrize("n,S,Hkv,D,dtype,rules", [
+    (3, 389, 4, 128, "bf16", {}),                     # layers together; the last tile's share of the rows is cut
+    (9, 1500, 8, 128, "bf16", {}),                    # two groups of layers, megabytes each
+    (2, 33, 3, 64, "f32", {}),                        # two tiles, capacity 16
+    (2, 700, 2, 64, "bf16", {"set_rule": kvm.KVM_SETS_CONSERVED_ONLY}),     # a gather instead of the merge
+    (2, 640, 2, 128, "bf16", {"weight_rule": kvm.KVM_WEIGHT_SET_SIGMA}),
+])
+def test_rows_past_a_units_length_are_zero(n, S, Hkv, D, dtype, rules, monkeypatch):
+    """kvm_compress_layers_filled zeroes what lies past the lengths, kvm_compress_layers leaves it, both give the same rows; the
+    buffers start as 0xFF bytes, those that compress_layers allocates too."""
+    cfg = si.CONFIGS["C1"].scaled(seq=S, head_dim=D, n_q_heads=Hkv, n_kv_heads=Hkv, dtype=dtype, seed=S)
+    layers = [tuple(si.make_layer(cfg, l)[k].cuda() for k in "QKV") for l in range(n)]
+    p = kvm.make_params(1, Hkv, Hkv, S, D, cfg.torch_dtype, **rules)
+    cap = kvm.kvm_sizes(p)[0]
+    ws = torch.empty(binding.kvm_layers_workspace_bytes(p, n), dtype=torch.uint8, device="cuda")
+    filled, left = (_dirty_outputs(n, Hkv, cap, D, cfg.torch_dtype) for _ in range(2))
+    _call_layers("kvm_compress_layers_filled", p, layers, filled, ws)
+    _call_layers("kvm_compress_layers", p, layers, left, ws)
+    empty = torch.empty
+    with monkeypatch.context() as m:
+        m.setattr(torch, "empty", lambda *a, **k: empty(*a, **k).view(torch.uint8).fill_(0xFF).view(k["dtype"]))
+        out, _ = kvm.compress_layers(p, layers)
+    for (ko, vo, ln, pos), (lko, lvo, lln, lpos), c, (Q, K, V) in zip(filled, left, out, layers):
+        assert 0 < int(ln.min()) < cap and torch.equal(ln, lln)
+        rest = torch.arange(cap, device="cuda") >= ln[..., None]
+        for t, u in ((ko, lko), (vo, lvo), (pos, lpos)):
+            assert torch.equal(t[~rest], u[~rest])
+            assert not t[rest].any() and (u[rest].view(torch.uint8) == 0xFF).all()
+        assert all(torch.equal(a, b) for a, b in ((c.K_out, ko), (c.V_out, vo), (c.out_len, ln), (c.out_pos, pos)))
+        if n == 2:                                    # (alone: the same bits; its buffers start at zero)
+            ref = kvm.Compressor(p)(Q, K, V)
+            assert all(torch.equal(getattr(c, k), getattr(ref, k)) for k in ("K_out", "V_out", "out_len", "out_pos"))
 
 
 @pytest.mark.parametrize("S,Hkv,D,dtype,rules", [

@@ -106,6 +106,20 @@ def test_tiles_go_in_pairs_where_that_is_faster(S, D, Hq, Hkv, pairs):
     _check(O, lse, refO[None].cpu().numpy(), torch.logsumexp(L, -1)[None].cpu().numpy(), d["V"], G)
 
 
+@pytest.mark.parametrize("S,D,Hq,Hkv", [(2000, 64, 64, 32), (2000, 128, 64, 32), (1900, 64, 39, 39), (1900, 128, 39, 39)])
+def test_two_tiles_at_a_time_repeat_themselves_bit_for_bit(S, D, Hq, Hkv):
+    """The logits of a tile's next step land on the columns that its weights are read from: products that overtook one another
+    would show as results that differ from run to run (hundreds of blocks' items, 15 steps each, under other work's noise)."""
+    g = torch.Generator(device="cuda").manual_seed(S + D)
+    Q, K, V = (torch.randn(1, h, S, D, generator=g, device="cuda").bfloat16() for h in (Hq, Hkv, Hkv))
+    p = kvm.make_params(1, Hq, Hkv, S, D, torch.bfloat16)
+    O, lse, O2, lse2 = torch.empty_like(Q), torch.empty(1, Hq, S, device="cuda"), torch.empty_like(Q), torch.empty(1, Hq, S, device="cuda")
+    kvm.kvm_prefill_attend(p, Q, K, V, O, lse)
+    for _ in range(50):
+        kvm.kvm_prefill_attend(p, Q, K, V, O2, lse2)
+        assert torch.equal(O, O2) and torch.equal(lse, lse2)
+
+
 @pytest.mark.parametrize("D", [64, 128])
 def test_large_values_stay_finite_when_a_maximum_grows(D):
     """A late key's logit is 10.5 (log2 units) above the others' and every value is 1e36: weights above 2^8 of a reference that
