@@ -14,17 +14,18 @@
 //   warps 8-14  converters: read fp32 rows (L2 for all but the first touch), split them and write the three planes
 //               in the layout the tensor core reads (128-byte rows, 128-byte swizzle); no split copy of Q or K ever
 //               exists in global memory, so the pass needs no workspace for it and moves no extra bytes
-//   warp  15    MMA issue: one thread; owns tensor memory
+//   warp  15    MMA issue: the warp walks and waits together, one elected lane issues; owns tensor memory
 // As in the bf16 kernel a work item is a 128-row A tile (queries in pass 1, keys in pass 2) with all the B tiles it
 // meets under the causal mask, A rows are TMEM lanes, and a thread owns a row (pass 1) or column (pass 2) of the map.
 //
 // Split of the work: a step (one 128 x 128 logit tile) costs ~24 D clocks and there are few of them in the sizes
 // fp32 layers come in (40 for 4 heads x 512 tokens, 4800 for 16 x 2999), so items are not dealt whole: the steps of all
 // items form one list and every CTA takes q = ceil(steps / 148) consecutive ones, which is balanced to one step.  An
-// item that is cut leaves one partial state per piece: (max, sum) per query row, combined by whoever reads it, or a
-// partial column sum per key, added in piece order by combine_kernel (or by the segment kernel that follows in a
-// compress call).  Where the pieces' states would not fit 4 MiB (large problems, where whole items balance well
-// anyway) items stay whole and the states are final.  The rule depends on the shape only: results are reproducible.
+// item that is cut leaves one partial state per piece: (max, sum) per query row, joined by a kernel between the passes or, where
+// those are few, by the steps that read them (join_between below), or a partial column sum per key, added in piece order
+// by combine_kernel (or by the segment kernel that follows in a compress call).  Where the pieces' states would not fit
+// 4 MiB (large problems, where whole items balance well anyway) items stay whole and the states are final.  The rule
+// depends on the shape only: results are reproducible.
 //
 // Measured on a B200 (us, row / column pass; FMA tiles before): 16 / 8 heads x 2999 tokens x 128 1300 / 1890 -> 105 / 107;
 // 32 heads x 4096 x 128 351 / 377; 4 heads x 512 x 64 100 / 74 -> 9 / 9.  What bounds a step now is its 48 products: 3,340 of
@@ -99,7 +100,7 @@ struct alignas(16) Shared {
     alignas(16) float nl[NEPI][TILE];   // per epilogue warp: minus the log-sum-exp (log2 units) of the step's queries
 };
 
-static_assert(offsetof(Shared, nl) % 16 == 0, "read four at a time");
+static_assert(offsetof(Shared, nl) % 16 == 0, "read two at a time, in 8 bytes");
 
 // A 128-row x 64-channel chunk of a [S, D] fp32 matrix on its way to three bf16 planes, in units of eight channels:
 // unit u = t + k * (converter threads) is the eight channels u % 8 of row u / 8.
@@ -176,13 +177,13 @@ struct Feed {
     }
 };
 
-// flat (nullable): the rows' log-sum-exp, times flat_mul in log2 units; else joined: states hold it (join_states_kernel), or the
-// row pass's states are combined here.
-template <int KCH, int PASS>
+// flat (nullable): the rows' log-sum-exp, times flat_mul in log2 units; else states hold it (join_states_kernel) or, with JOIN, the
+// row pass's states are joined here (a kernel of its own: 0.4 % of the others' time).
+template <int KCH, int PASS, bool JOIN = false>
 __global__ void __launch_bounds__(NTHREADS, 1)
 score_f32_kernel(const float* __restrict__ Q, const float* __restrict__ K, float2* __restrict__ states,
                  const float* __restrict__ flat, float flat_mul, float* __restrict__ out, kvm_stats* stats,
-                 const Plan plan, int Hq, int Hkv, int S, float scale2, int joined, float* __restrict__ sim_out) {
+                 const Plan plan, int Hq, int Hkv, int S, float scale2, float* __restrict__ sim_out) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* sA = smem_raw + (base - smem_u32(smem_raw));     // [KCH][plane][128 rows][128 B]
@@ -321,10 +322,10 @@ score_f32_kernel(const float* __restrict__ Q, const float* __restrict__ K, float
             const int qh = (w.head / Hkv) * Hq + (w.head % Hkv) * plan.G + h;
             const size_t r = (size_t)qh * S + t * TILE + lane;
             const int left = S - t * TILE - lane;
-            if (flat) {
+            if (!JOIN && flat) {
 #pragma unroll
                 for (int e = 0; e < 4; ++e) v[e] = e * 32 < left ? flat[r + e * 32] * flat_mul : INFINITY;
-            } else if (joined) {
+            } else if (!JOIN) {
 #pragma unroll
                 for (int e = 0; e < 4; ++e) v[e] = e * 32 < left ? __ldcg(&states[r + e * 32].x) : INFINITY;
             } else {
@@ -371,7 +372,7 @@ score_f32_kernel(const float* __restrict__ Q, const float* __restrict__ K, float
                 ++own;
                 if (ok) tc_fence_after();
                 if (PASS == 2) {
-                    asked = (flat || joined) && i + 2 < w.n;
+                    asked = !JOIN && i + 2 < w.n;
                     if (asked) {
                         const int bn = bt + 1 == plan.T ? w.tile : bt + 1, gn = bt + 1 == plan.T ? g + 1 : g;
                         ask(ahead, gn, bn);
@@ -560,6 +561,8 @@ cudaError_t launch_t(const Dims& d, const Plan& plan, const float* Q, const floa
             if (e != cudaSuccess) return e;
             e = cudaFuncSetAttribute(score_f32_kernel<KCH, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
+            e = cudaFuncSetAttribute(score_f32_kernel<KCH, 2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
             done[dev] = true;
         }
     }
@@ -573,7 +576,7 @@ cudaError_t launch_t(const Dims& d, const Plan& plan, const float* Q, const floa
     const float scale2 = d.scale * LOG2E;
     if (!lse_in) {
         e = launch_dependent(score_f32_kernel<KCH, 1>, rgrid, block, smem, st, Q, K, states, (const float*)nullptr,
-                             1.f, flat, stats, plan, d.Hq, d.Hkv, d.S, scale2, 0, (float*)nullptr);
+                             1.f, flat, stats, plan, d.Hq, d.Hkv, d.S, scale2, (float*)nullptr);
         if (e != cudaSuccess) return e;
     }
     if (lse_out) {
@@ -582,14 +585,15 @@ cudaError_t launch_t(const Dims& d, const Plan& plan, const float* Q, const floa
         if (e != cudaSuccess) return e;
     }
     if (!scores) return cudaSuccess;
-    const bool join = !lse_in && plan.split_row && join_between(plan, d.D);
-    if (join) {
+    const bool states_in = !lse_in && plan.split_row, between = states_in && join_between(plan, d.D);
+    if (between) {
         e = launch_dependent(join_states_kernel, dim3((unsigned)((rows + 255) / 256)), dim3(256), 0, st, states, plan, d.S);
         if (e != cudaSuccess) return e;
     }
-    e = launch_dependent(score_f32_kernel<KCH, 2>, cgrid, block, smem, st, Q, K, states,
+    const auto columns = states_in && !between ? score_f32_kernel<KCH, 2, true> : score_f32_kernel<KCH, 2>;
+    e = launch_dependent(columns, cgrid, block, smem, st, Q, K, states,
                          lse_in ? lse_in : (const float*)flat, lse_in ? LOG2E : 1.f, plan.split_col ? part : scores, stats, plan,
-                         d.Hq, d.Hkv, d.S, scale2, (int)join, sim_out);
+                         d.Hq, d.Hkv, d.S, scale2, sim_out);
     if (e != cudaSuccess || !plan.split_col) return e;
     if (parts) {                                      // the caller's next kernel adds the pieces up
         parts->part = part;
