@@ -473,9 +473,12 @@ prefill_attend_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
 // reference moved, by 12 (x 1e-3; rounding O alone 1.64-1.66): 32 heads x 4096 x 128 1.996 / 1.924 / 1.970 (146 / 130.4 / 129.2 us),
 // 32 / 8 x 10007 x 64 2.052 / 1.978 / 2.024 (695 / 572 / 574), 256 / 128 x 300 x 64 1.879 / 1.873 / 1.887, 240 / 30 x 461 x 64
 // 1.897 / 1.888 / 1.913.
-// A tile's products are issued in the order P V (j), Q K^T (j + 1) by one thread and run in that order (a CTA's products pass
-// the tensor pipe one after the other), so S may take P's place, and an S that is there says that the last P V is done (a
-// commit covers all that its thread issued before): O may be rescaled, and P written, without another barrier.
+// A tile's products are issued in the order P V (j), Q K^T (j + 1) by one thread.  An S that is there says that the last P V is
+// done (a commit covers all that its thread issued before): O may be rescaled, and P written, without another barrier.  That Q K^T
+// may take the place of the P that P V reads, with no wait between them, rests on a CTA's products passing its tensor pipe in the
+// order of their issue.  PTX promises this for products of one accumulator and shape only; here the accumulators differ (and with
+// 64 channels the shape).  Published attention kernels for this architecture write their logits over the weights in the same
+// way, and the tests compare the bits of many runs; a wait in between would cost the 1,200 clocks that it hides.
 constexpr int NST = 2;                  // iterations in the rings of K and V tiles
 constexpr int REGS_PAIR_OTHER = 88;     // (2 x 128 x 208 + 128 x 88 = 384 x 168, what the block is launched with)
 constexpr int P_FIRST = 96;             // keys of a step whose P is handed over first
