@@ -477,8 +477,8 @@ prefill_attend_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
 // done (a commit covers all that its thread issued before): O may be rescaled, and P written, without another barrier.  That Q K^T
 // may take the place of the P that P V reads, with no wait between them, rests on a CTA's products passing its tensor pipe in the
 // order of their issue.  PTX promises this for products of one accumulator and shape only; here the accumulators differ (and with
-// 64 channels the shape).  Published attention kernels for this architecture write their logits over the weights in the same
-// way, and the tests compare the bits of many runs; a wait in between would cost the 1,200 clocks that it hides.
+// 64 channels the shape).  Published attention kernels for this architecture rely on it likewise, and the tests compare the bits
+// of many runs.
 constexpr int NST = 2;                  // iterations in the rings of K and V tiles
 constexpr int REGS_PAIR_OTHER = 88;     // (2 x 128 x 208 + 128 x 88 = 384 x 168, what the block is launched with)
 constexpr int P_FIRST = 96;             // keys of a step whose P is handed over first
