@@ -332,10 +332,10 @@ def compress_layers(p: KvmParams, layers, sim_thresholds=None, device="cuda", st
           array(*range(len_base, len_base + 4 * n * units, 4 * units)), array(*[b + 2 * kv_bytes for b in bases]), None,
           ws.data_ptr(), ws.nbytes, handle)
     out = []
-    for blob, layer_len in zip(blobs, out_len.unbind(0)):
+    for blob, lengths in zip(blobs, out_len.unbind(0)):
         K_out, V_out = blob[:2 * kv_bytes].view(dtype).view(2, B, H, cap, D).unbind(0)
-        out.append(Compressed(K_out, V_out, layer_len, blob[2 * kv_bytes:].view(torch.int32).view(B, H, cap), None, cap))
-    with torch.cuda.stream(other):                                      # (None: the current one)
-        lengths = out_len.cpu()                                         # the one read-back of the call
-    ratios = (lengths.float().mean((1, 2)) / p.seq).tolist()
+        out.append(Compressed(K_out, V_out, lengths, blob[2 * kv_bytes:].view(torch.int32).view(B, H, cap), None, cap))
+    if other is not None:
+        other.synchronize()
+    ratios = (out_len.cpu().float().mean((1, 2)) / p.seq).tolist()      # the one read-back of the call
     return out, ratios

@@ -123,7 +123,7 @@ def test_gathered_layers_are_zero_past_their_length_without_further_launches(S, 
 
 @pytest.mark.parametrize("as_handle", [False, True])
 def test_on_a_stream_that_is_not_the_current_one(as_handle):
-    """The ratios are read where the kernels run, the results and the freed workspace belong to the current stream."""
+    """The ratios are read when the kernels are through, the results and the freed workspace belong to the current stream."""
     n, H, S, D = 3, 4, 600, 64
     layers = [tuple(torch.randn(1, H, S // 8, D, device="cuda").repeat_interleave(8, 2).bfloat16() for _ in "QKV") for _ in range(n)]
     p = kvm.make_params(1, H, H, S, D, torch.bfloat16)
